@@ -41,29 +41,17 @@ FP64_NOMINAL_TFLOPS = 1.25   # GB300 dense FP64, nominal
 
 
 def kappa_flops(P, S, J, Nz):
-    """Algorithmic FP32 flops of one launch of the PF likelihood kernel: per (p, s, j)
-    two passes over Nz elements against the S-1 (eigen-whitened, orthogonal) basis
-    columns plus the residual column, 8 flops per complex multiply-add, the steering
-    vector and residual element work (40 per element) and the O(S) amplitude sums."""
-    per = 8 * Nz * S + 8 * Nz * (S - 1) + 40 * Nz + 16 * (S - 1)
-    return float(P) * S * J * per
+    """Algorithmic flops of one launch of the PF likelihood kernel: per (p, s, j) the steering
+    vector (6 per element) and its projections on the S-1 whitened basis columns and the
+    null residual, 8 flops per complex multiply-add."""
+    return float(P) * S * J * (8 * Nz * S + 6 * Nz)
 
 
-def kappa_tc_used(g, S, S_max):
-    """Whether the PF likelihood runs on the tensor cores (k_kappa_tc) with its built-in
-    tiles: a shape the kernel takes (autotune.tensor_core_shape) and a column bucket equal
-    to the basis stride (S > 32 at stride 64, S > 24 at stride 32)."""
-    from paper_2604_19723_gb300 import autotune
-    if not autotune.tensor_core_shape(g, S_max):
-        return False
-    width = autotune.basis_stride(S_max)
-    return S > (32 if width == 64 else 24)
-
-
-def kappa_contraction_flops(P, S, J, Nz):
-    """The two contractions of the PF likelihood (psi^H V over the S-1 basis columns and
-    r0, then V conj(h) over the S-1 basis columns), 8 flops per complex multiply-add."""
-    return float(P) * S * J * (8 * Nz * S + 8 * Nz * (S - 1))
+def kappa_mma_flops(P, S, J, Nz):
+    """BF16 flops the PF likelihood (k_kappa_x) issues on the tensor cores: ten digit products of
+    (P x 2 Nh) by (2 Nh x 2 SW) per (s, j), Nh = ceil(Nz / 2) elements of a symmetric layout, SW =
+    S rounded up to 8 columns."""
+    return float(P) * S * J * 10 * 2 * (2 * ((Nz + 1) // 2)) * (2 * ((S + 7) // 8 * 8))
 
 
 def iota_flops(P, S, J, Nf, My, Mz):
@@ -85,15 +73,10 @@ def iota_flops(P, S, J, Nf, My, Mz):
 # once per PF and then served from L2), so a record applies only to the workload and
 # particle count it was taken at, and only while the kernel sources hash to the recorded
 # value.
-TRAFFIC_RECORDS = {
-    "k_kappa_tc": {"workload": "scale_64x100k", "P": 100000, "bytes": 873119232 + 50664448,
-                   "sources_sha256": "1110bf0b1cfc98075cd47b06617919570f7d65d3df893ff6bb438e748e463a97",
-                   "how": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
-                          "--clock-control none -k regex:^k_kappa_tc$ -c 1 python bench.py --steps 2 "
-                          "--warmup 1 --no-matched --no-cpu-baseline"},
-}
-KERNEL_SOURCES = ("paper_2604_19723_gb300/csrc/k_like.cu", "paper_2604_19723_gb300/csrc/bp_kernels.cuh",
-                  "paper_2604_19723_gb300/csrc/bp_internal.cuh", "paper_2604_19723_gb300/csrc/tc_sm100.cuh")
+TRAFFIC_RECORDS = {}
+KERNEL_SOURCES = ("paper_2604_19723_gb300/csrc/k_kappa.cu", "paper_2604_19723_gb300/csrc/k_like.cu",
+                  "paper_2604_19723_gb300/csrc/bp_kernels.cuh", "paper_2604_19723_gb300/csrc/bp_internal.cuh",
+                  "paper_2604_19723_gb300/csrc/tc_sm100.cuh")
 
 
 def kernel_sources_sha256():
@@ -396,23 +379,16 @@ def run_gpu(args, rank, world):
             # the same algorithmic flops against the nominal FP64 rate, the precision class the
             # log determinant needs (the kernel emulates it with FP32 operations)
             r["vs_fp64_nominal"] = {"peak": FP64_NOMINAL_TFLOPS, "frac": a / FP64_NOMINAL_TFLOPS}
-        if name == "k_kappa" and kappa_tc_used(g, S, S_max):
-            # both contractions run on the tensor cores in 3xTF32: each algorithmic flop is
-            # three TF32 MMA flops, against the measured bf16 rate (sustained: the kernel runs
-            # inside a long step) times the nominal TF32/BF16 ratio (1.1 / 2.25 PFLOP/s)
-            tf32 = peaks.get("bf16_tflops_sustained", 1700.0) * (1.1 / 2.25)
-            eff = tf32 / 3.0
-            fc = kappa_contraction_flops(P, S, g.J, g.Nz)
-            ac = fc / (ms * 1e-3) / 1e12
-            r = {"bound": "tensor", "kernel": "k_kappa_tc (tcgen05 3xTF32, both contractions)", "achieved": ac,
-                 "peak": eff, "unit": "TFLOP/s", "frac": ac / eff,
-                 "traffic": traffic_for("k_kappa_tc", args.workload, P),
-                 "ms_per_launch": ms,
-                 "peak_basis": f"3xTF32 effective: MEASURED_PEAKS bf16_tflops_sustained {peaks.get('bf16_tflops_sustained')} "
-                               f"x 1.1/2.25 (nominal TF32/BF16) / 3 products",
-                 "cuda_core_part": {"flops": fl - fc, "achieved": (fl - fc) / (ms * 1e-3) / 1e12, "peak": peak_alu,
-                                    "note": "element-wise float-float residual and amplitude sums on the FP32 lanes, "
-                                            "whole-kernel time"}}
+        if name == "k_kappa":
+            # the digit products on the tensor cores against the measured bf16 rate (sustained:
+            # the kernel runs inside a long step)
+            bf16 = peaks.get("bf16_tflops_sustained", 1700.0)
+            ac = kappa_mma_flops(P, S, g.J, g.Nz) / (ms * 1e-3) / 1e12
+            r = {"bound": "tensor", "kernel": "k_kappa_x (tcgen05 kind::f16, ten exact BF16 digit products)",
+                 "achieved": ac, "peak": bf16, "unit": "TFLOP/s", "frac": ac / bf16,
+                 "traffic": traffic_for("k_kappa_x", args.workload, P), "ms_per_launch": ms,
+                 "peak_basis": f"MEASURED_PEAKS bf16_tflops_sustained {peaks.get('bf16_tflops_sustained')}",
+                 "algorithmic": {"flops": fl, "achieved": a}}
         return r
     dominant = max(per_kernel, key=lambda n: per_kernel[n][0])
     other = "k_iota_blk" if dominant == "k_kappa" else "k_kappa"

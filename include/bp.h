@@ -242,21 +242,12 @@ bp_status bp_get_profile(bp_handle* h, double* ms, int n);
  * (paper_2604_19723_gb300/autotune.py).  The paper has no counterpart; results
  * depend on them only through FP32 rounding.  0 in a field = the built-in
  * choice.
- *   kappa_sc      column bucket S~ of the CUDA-core PF likelihood (S~ - 1 basis
- *                 columns held per particle): 8, 16, 24, 32, 48 or 64.  Used
- *                 when S <= kappa_sc <= the filter's basis stride (32 for
- *                 S_max <= 32, else 64), otherwise the smallest bucket >= S.
- *   kappa_blocks  CUDA-core PF-likelihood blocks of 256 particles per SM: 1 or 2
- *                 (2 caps registers at 128 per thread and shrinks the staged
- *                 frequency chunk; buckets <= 32 only, else 1 is used).
- *   kappa_fch     frequencies of V staged in shared memory per chunk (the Nz
- *                 tile), clamped to what fits.
- *   kappa_tc      1: the tensor-core PF likelihood wherever the shape allows it,
- *                 at the bucket equal to the basis stride (Mz even, and either
- *                 64 basis columns with 2 My Mz in {8, 16, 32}, or 32 or 64
- *                 columns with My Mz a multiple of 16, at least 32; shared
- *                 memory within 227 KB); built-in (0): the same where the
- *                 bucket is the stride; -1: never.
+ *   kappa_tc      0 or 1: the PF likelihood on the tensor cores (every shape);
+ *                 -1: on the CUDA cores.
+ *   kappa_sc, kappa_blocks, kappa_fch  checked and stored, without effect: both
+ *                 PF-likelihood kernels size their tiles themselves.  Values:
+ *                 kappa_sc 8, 16, 24, 32, 48 or 64; kappa_blocks 1 or 2;
+ *                 kappa_fch >= 0.
  *   table_chunk   particles per shared-memory chunk of the message table: 16,
  *                 32, 64 or 128 (clamped to what fits; built-in 64).
  *   table_split   particle splits of the message-table grid (>= 1; clamped to

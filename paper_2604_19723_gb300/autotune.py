@@ -10,9 +10,8 @@ candidate with the whole table.  The scenarios' results do not depend on the cho
 (each scenario runs the same kernels in the same order).
 
 The tile tuner (tune_tiles, tune_batch_tiles) picks, per filter or per shape class of a
-batch, the kernels' tile shapes (bp_set_tiles): the PF likelihood's column bucket S~,
-its blocks per SM and staged frequency chunk (the Nz tile), tensor-core or CUDA-core
-kernel, and the message table's particle chunk.  Each candidate is timed on the same
+batch, the kernels' tile shapes (bp_set_tiles): the PF likelihood's tensor-core or
+CUDA-core kernel, and the message table's particle chunk.  Each candidate is timed on the same
 predicted state with the library's own per-stage CUDA events (the PF-likelihood and
 message-table stages), the median of a few updates.  Results depend on the tiles only
 through FP32 rounding.
@@ -66,24 +65,20 @@ BUCKETS = (8, 16, 24, 32, 48, 64)
 
 
 def basis_stride(S_max: int) -> int:
-    """Column stride of a filter's basis buffers (the largest usable bucket)."""
+    """Columns of a filter's basis buffer (the largest bucket of its PF counts)."""
     return 8 if S_max <= 8 else 16 if S_max <= 16 else 32 if S_max <= 32 else 64
 
 
 def tensor_core_large(geom) -> bool:
-    """The arrays whose tensor-core pass-1 rounds lie within one frequency (My Mz a
-    multiple of 16, at least 32); their kernel forms the steering elements as (hi, lo)
-    pairs in pass 2."""
+    """Arrays of at least 32 elements, a multiple of 16."""
     nm = geom.My * geom.Mz
     return nm >= 32 and nm % 16 == 0
 
 
 def tensor_core_smem(geom, width: int) -> int:
-    """Dynamic shared memory of the tensor-core PF likelihood (one 128-particle tile per
-    block; width = basis columns incl. r0): the operand region of either pass, barriers,
-    r0 per element, 1/lambda and y~0, the factors (frequency factors kept up to 16, and
-    never for the large arrays), and for the large arrays the low parts of a_z and the
-    (hi, lo) cis table."""
+    """The shared-memory figure of the shape-class rule, in bytes: 32-element operand tiles of
+    128 particles at `width` basis columns, the residual and the steering factors.  (The kernel
+    sizes its own ring; every shape fits.)"""
     large = tensor_core_large(geom)
     region = max(2 * 128 * 32 + 2 * (2 * width) * 32, 2 * 128 * 32 + 2 * 2 * 64 * 32)
     nfac = (geom.Nf if geom.Nf <= 16 and not large else 0) + geom.My + geom.Mz
@@ -92,10 +87,10 @@ def tensor_core_smem(geom, width: int) -> int:
 
 
 def tensor_core_shape(geom, S_max: int) -> bool:
-    """Whether the tensor-core PF likelihood applies to this shape: Mz even and either
-    64 basis columns with 2 My Mz in {8, 16, 32} (a pass-1 round is whole frequencies) or
-    64 or 32 columns with My Mz a multiple of 16, at least 32 (a round is part of one
-    frequency); its shared memory within 227 KB.  It runs at the basis stride's width."""
+    """Part of the shape class: whether rounds of 16 elements divide the array evenly (Mz even
+    and 64 basis columns with 2 My Mz in {8, 16, 32}, or 64 or 32 columns with My Mz a
+    multiple of 16, at least 32) within 227 KB.  The PF likelihood runs on the tensor cores at
+    every shape."""
     width, nm = basis_stride(S_max), geom.My * geom.Mz
     if geom.Mz % 2:
         return False
@@ -105,23 +100,9 @@ def tensor_core_shape(geom, S_max: int) -> bool:
 
 
 def kappa_candidates(S: int, S_max: int, geom) -> List[Dict[str, int]]:
-    """Tile candidates of the PF likelihood: the two smallest buckets that hold S (within
-    the basis stride), two blocks per SM where the bucket allows it (<= 32), half the
-    staged frequency chunk, and the tensor-core kernel on or off where the shape allows."""
-    top = basis_stride(S_max)
-    bks = [b for b in BUCKETS if S <= b <= top][:2]
-    out = []
-    for b in bks:
-        if b == top and tensor_core_shape(geom, S_max):
-            out.append(dict(kappa_sc=b, kappa_tc=1, kappa_blocks=0, kappa_fch=0))
-        if b == 64 and tensor_core_shape(geom, S_max):
-            out.append(dict(kappa_sc=64, kappa_tc=-1, kappa_blocks=0, kappa_fch=0))
-            continue
-        for mb in ((1, 2) if b in (24, 32) else (0,)):
-            out.append(dict(kappa_sc=b, kappa_tc=-1, kappa_blocks=mb, kappa_fch=0))
-        if geom.Nf >= 4:
-            out.append(dict(kappa_sc=b, kappa_tc=-1, kappa_blocks=0, kappa_fch=(geom.Nf + 3) // 4))
-    return out
+    """Tile candidates of the PF likelihood: the built-in tensor-core kernel and the CUDA-core one."""
+    b = next(x for x in BUCKETS if x >= S)
+    return [dict(kappa_sc=b, kappa_tc=tc, kappa_blocks=0, kappa_fch=0) for tc in (0, -1)]
 
 
 def table_candidates() -> List[Dict[str, int]]:

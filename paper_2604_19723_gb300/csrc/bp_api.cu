@@ -102,6 +102,12 @@ void fill_geom(DevGeom& G, const bp_geometry* g) {
         G.pz_lo[m] = (float)(v - (double)G.pz_l[m]);
     }
     G.amp_c = (float)(G.lam / (4.0 * M_PI));
+    auto symmetric = [](const double* v, int n) {
+        double m = 0.0, a = 0.0;
+        for (int i = 0; i < n; ++i) { m = std::max(m, std::fabs(v[i])); a = std::max(a, std::fabs(v[i] + v[n - 1 - i])); }
+        return a <= 1e-13 * m;
+    };
+    G.sym = symmetric(G.f, g->Nf) && symmetric(G.py, g->My) && symmetric(G.pz, g->Mz);
 }
 
 extern "C" {
@@ -442,9 +448,7 @@ WsPlan ws_plan(const DevGeom& G, const DevParams& Pm, int SCA, int nsplit_max) {
     w.isel = take(256 + PP * sizeof(float));
     w.tab = take(4 * SM * J * Nz * 2 * sizeof(double));
     w.tab_part = take((size_t)nsplit_max * 3 * SM * J * Nz * 2 * sizeof(double));
-    w.kV = take(SM * J * Nz * (size_t)SCA * sizeof(float2));
-    w.kr0l = take(SM * J * Nz * sizeof(float2));
-    w.kB = kappa_tc_ok(G, SCA) ? take(kappa_btile_floats(G, S_max, SCA) * sizeof(float)) : take(0);
+    w.kB = take(kappa_operand_bytes(G, S_max));
     w.red_part = take(nbel * 64 * RED_W * 2 * sizeof(double));
     w.gram = take(J * SM * SM * 2 * sizeof(double));
     w.V64 = take(SM * J * Nz * (size_t)SCA * 2 * sizeof(double));
@@ -472,9 +476,7 @@ void ws_bind(bp_handle* h, char* base) {
     D.iota_err = reinterpret_cast<float*>(base + w.isel + 256);
     D.tab = reinterpret_cast<double*>(base + w.tab);
     D.tab_part = reinterpret_cast<double*>(base + w.tab_part);
-    D.kV = reinterpret_cast<float2*>(base + w.kV);
-    D.kr0l = reinterpret_cast<float2*>(base + w.kr0l);
-    D.kB = kappa_tc_ok(h->G, h->SCA) ? reinterpret_cast<float*>(base + w.kB) : nullptr;
+    D.kB = reinterpret_cast<unsigned char*>(base + w.kB);
     D.red_part = reinterpret_cast<double*>(base + w.red_part);
     h->gram = reinterpret_cast<double*>(base + w.gram);
     h->V64 = reinterpret_cast<double*>(base + w.V64);
@@ -553,10 +555,10 @@ bp_status handle_create(const bp_geometry* geom, const bp_params* prm, int P, in
     ok &= dalloc(h, &D.llr_w, (size_t)S_max * J);
     ok &= dalloc(h, &D.W, (size_t)S_max);
     ok &= dalloc(h, &D.eta_bar, (size_t)J);
-    ok &= dalloc(h, &D.kdl, (size_t)S_max * J * SCA);
+    ok &= dalloc(h, &D.kSc, (size_t)S_max * J * 64);
+    ok &= dalloc(h, &D.kC, (size_t)S_max * J);
+    ok &= dalloc(h, &D.ctab, 256);
     ok &= dalloc(h, &D.kerr, 1);
-    ok &= dalloc(h, &D.ky0, (size_t)S_max * J * SCA);
-    ok &= dalloc(h, &D.kJ0, (size_t)S_max * J);
     ok &= dalloc(h, &D.nu_T, (size_t)J * 4 * S_max);
     ok &= dalloc(h, &D.nu_c, (size_t)J * 2);
     const int nbel = bel_count(S_max, J);
@@ -601,7 +603,8 @@ bp_status handle_create(const bp_geometry* geom, const bp_params* prm, int P, in
     }
     D.cur = 0;
     launch_init(h->G, h->Pm, D, S0, h->st);
-    h->launches += 1;
+    launch_cis_table(D, h->st);
+    h->launches += 2;
     h->S = S0; h->S_upd = S0; h->n = 0; h->phase = 0;
     if (cudaStreamSynchronize(h->st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
         *err = std::string("bp_init: ") + cudaGetErrorString(cudaGetLastError());
@@ -647,12 +650,10 @@ void update_enqueue(bp_handle* h, const float* z_dev) {
     launch_geom(h->G, h->Pm, D, S, h->st);
     launch_table(h->G, h->Pm, D, S, nsplit, h->tiles.table_chunk, h->st);
     mark(h, 3);
-    launch_stage(h->G, h->Pm, D, S, h->SCA, z_dev, h->gram, h->nu_b, h->V64, h->st, h->st_side, h->ev_fork, h->ev_join);
-    const KappaPlan kp = plan_kappa(h->G, D, S, h->SCA, h->tiles.kappa_sc, h->tiles.kappa_blocks, h->tiles.kappa_fch,
-                                    h->tiles.kappa_tc);
-    if (kp.tc) h->launches += launch_kappa_btile(h->G, D, S, h->SCA, h->st);   // B tiles of the tensor-core kernel
+    launch_stage(h->G, h->Pm, D, S, h->SCA, z_dev, h->gram, h->nu_b, h->V64, h->st);
     mark(h, 4);
-    launch_kappa(h->G, h->Pm, D, S, h->SCA, kp, h->st);
+    const int kappa_launches = launch_kappa(h->G, h->Pm, D, S, h->SCA, h->tiles.kappa_tc >= 0, h->V64, h->st);
+    launch_nu_tridiag(h->G, h->Pm, D, S, h->gram, h->nu_b, h->st, h->st_side, h->ev_fork, h->ev_join);
     mark(h, 5);
     const int iota_launches = launch_iota(h->G, h->Pm, D, S, z_dev, h->st) + 1;
     launch_iota_repair(h->G, h->Pm, D, S, z_dev, h->st);
@@ -667,7 +668,7 @@ void update_enqueue(bp_handle* h, const float* z_dev) {
         cudaEventRecord(h->ev[BP_PROF_STAGES], h->st);
         for (int i = 1; i < BP_PROF_STAGES; ++i) h->ev_valid[i] = true;
     }
-    h->launches += 1 + 3 + 3 + 1 + iota_launches + 1 + 5 + 3;
+    h->launches += 1 + 3 + 3 + kappa_launches + iota_launches + 1 + 5 + 3;
     h->D.cur = 1 - h->D.cur;
     h->S_upd = S;
     h->phase = 0;

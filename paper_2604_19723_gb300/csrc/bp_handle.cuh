@@ -14,7 +14,7 @@
 // filter on its own owns one; filters of a batch that run one after another on the
 // same stream share one, sized for the largest of them.
 struct WsPlan {
-    size_t lw_x, lw_y, lw_eta, geo, geo_lo, flags, isel, tab, tab_part, kV, kr0l, kB, red_part, gram, V64, cdf, wn, idx;
+    size_t lw_x, lw_y, lw_eta, geo, geo_lo, flags, isel, tab, tab_part, kB, red_part, gram, V64, cdf, wn, idx;
     size_t bprop, bprop_c;   // birth proposal scratch (empty unless enabled)
     size_t total;
 };
@@ -25,11 +25,11 @@ struct bp_handle {
     bp::DevState D;
     cudaStream_t st;
     // single filters: a side stream for the noise-likelihood tridiagonalisation, which
-    // runs beside the PF basis stage (fork after the Gram, join before its consumer)
+    // runs beside the MT likelihood (fork after the PF likelihood, join before its consumer)
     cudaStream_t st_side;
     cudaEvent_t ev_fork, ev_join;
     int P, S_max, J, Nz;
-    int SCA;            // column stride of the per-(s,j) basis buffers
+    int SCA;            // columns of the per-(s,j) basis buffer (r0 in the last)
     int S;              // current number of PFs (host copy)
     int S_legacy;       // PFs before the births of the current prediction
     int S_upd;          // S of the last bp_update

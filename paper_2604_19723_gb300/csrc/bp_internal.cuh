@@ -19,6 +19,7 @@ constexpr int S_CAP_MAX = 64;
 // Geometry and parameters, passed to kernels by value (constant bank).
 struct DevGeom {
     int J, Nf, My, Mz, Nz;
+    int sym;                 // frequencies and element positions symmetric about 0 (to rounding)
     double fc, c, lam, B;
     double p_pa[J_MAX][3];
     double R[J_MAX][9];      // row-major, columns = local axes (global coords)
@@ -396,15 +397,12 @@ struct DevState {
     double* tab_part; // table partial sums [nsplit][3][S_max][J][Nz] double2
     double* W;        // S_max    sum_p w_alpha
     double* eta_bar;  // J
-    // kappa stage outputs (per (s,j))
-    float2* kV;       // [S_max][J][Nz][S_cap]   whitened basis, column S_cap-1 = r0 (FP32 part)
-    float2* kr0l;     // [S_max][J][Nz]          low part of r0 (r0 = FP32 part + low part)
-    float2* kdl;      // [S_max][J][S_cap]       1/lambda_c of the eigen-whitened basis (.x; zero-padded)
-    float* kB;        // TF32 B tiles of the tensor-core PF likelihood (or null): pass 1
-                      // [S][J][rounds][hi, lo][2 S_cap x 32], then pass 2 [S][J][groups][S_cap/16][hi, lo][64 x 32]
-    int* kerr;        // nonzero after a bounded wait of a kernel gave up (reported by bp_estimate)
-    float2* ky0;      // [S_max][J][S_cap]       y~0 = V^H e0 / eta_bar (zero-padded)
-    double* kJ0;      // [S_max][J]              |r0|^2/eta_bar
+    // PF likelihood (k_kappa.cu), per (s, j)
+    unsigned char* kB; // BF16 digit slices of the whitened basis and r0: [S][J][chunks][4][2 SW x 32]
+    float* kSc;        // [S_max][J][64] power-of-two scales of the columns
+    float4* kC;        // [S_max][J] 1/eta_bar and zeta as (hi, lo) pairs
+    float4* ctab;      // [256] e^{i 2 pi n / 256} as (hi, lo) pairs
+    int* kerr;         // nonzero after a bounded wait of a kernel gave up (reported by bp_estimate)
     // nu stage outputs (per j)
     double* nu_T;     // [J][S_max] diag a_k, [J][S_max] |offdiag|^2, [J][S_max] double2 b'
     double* nu_c;     // [J][2] |e|^2, constant

@@ -31,6 +31,8 @@ int launch_birth_proposal(const DevGeom& G, const DevParams& Pm, const DevState&
 
 // Largest dynamic shared memory a block may opt in to on the current device.
 int smem_optin();
+// Streaming multiprocessors of the device.
+int sm_count();
 // Raises a kernel's dynamic shared-memory limit to the opt-in maximum less its static
 // shared memory (once per kernel), not to one launch's need: launches of one kernel
 // with different sizes from several streams, or replayed from a captured graph, then
@@ -211,22 +213,20 @@ void launch_row_sums(const DevParams& Pm, const DevState& D, int S, int J, cudaS
 // chunk_req: particles per shared-memory chunk (16, 32, 64, 128; 0 = 64), halved to fit
 void launch_table(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int nsplit, int chunk_req,
                   cudaStream_t st);
-// the PF basis stage; with a side stream the noise-likelihood tridiagonalisation runs there
-// (forked after the Gram through ev_fork, ev_join recorded after it)
-void launch_stage(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SC, const float* z,
-                  double* gram, double* nu_b, double* V64, cudaStream_t st, cudaStream_t side = nullptr,
-                  cudaEvent_t ev_fork = nullptr, cudaEvent_t ev_join = nullptr);
-// the PF-likelihood launch chosen from S, the shape and the tile requests (0 = built-in):
-// column bucket sc, tensor-core kernel or CUDA-core one with mb blocks per SM and fch
-// frequencies staged per chunk (smem bytes)
-struct KappaPlan { int sc, mb, fch; bool tc; size_t smem; };
-KappaPlan plan_kappa(const DevGeom& G, const DevState& D, int S, int SCA, int t_sc, int t_mb, int t_fch, int t_tc);
-void launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, const KappaPlan& k,
-                  cudaStream_t st);
-bool kappa_tc_ok(const DevGeom& G, int SCA);
-size_t kappa_btile_floats(const DevGeom& G, int S_max, int SCA);
-// operand tiles of both tensor-core passes of the PF likelihood; returns launches
-int launch_kappa_btile(const DevGeom& G, const DevState& D, int S, int SCA, cudaStream_t st);
+// the Gram matrices, the PF basis V64 and the existence tests
+void launch_stage(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, const float* z,
+                  double* gram, double* nu_b, double* V64, cudaStream_t st);
+// the noise likelihood's tridiagonal forms; with a side stream they run there (forked from st
+// through ev_fork, ev_join recorded after them)
+void launch_nu_tridiag(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const double* gram,
+                       const double* nu_b, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join);
+// the PF likelihood from the stage's basis V64 [S][J][SCA][Nz] (k_kappa.cu): operand digits,
+// then the tensor-core kernel, or the CUDA-core one where a tile request declines it; returns
+// launches.  launch_cis_table fills D.ctab once per handle.
+int launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, bool tensor,
+                 const double* V64, cudaStream_t st);
+size_t kappa_operand_bytes(const DevGeom& G, int S_max);
+void launch_cis_table(const DevState& D, cudaStream_t st);
 // MT likelihood of every particle (returns its launches): the FP32 warp kernel with
 // ratio flags below IOTA_FF_ALL_S PFs, else k_iota_bulk and the selection of the particles
 // whose weights need the float-float evaluation; launch_iota_repair then evaluates the

@@ -1,4 +1,5 @@
-// Per-particle update messages (Supplementary Sec. S-V), the hot loop.
+// Per-particle update messages iota~ and nu~ (Supplementary Sec. S-V); the PF message
+// kappa~ is in k_kappa.cu.
 //
 // Every message is a complex Gaussian whose quadratic form is evaluated in
 // its variational (regularised least-squares) form,
@@ -8,12 +9,6 @@
 // noise floor) rather than to the signal energy, and errors in y* enter
 // only at second order.
 //
-//  kappa~(phi_s^p, 1)/kappa~(., 0) for every (s, p), summed over j:
-//     Delta = J0 - J(tau*) - log(1 + q alpha),
-//     J(tau) = |r0 - tau psi_perp|^2/eta_bar + |y0 - tau Lambda^-1/2 V^H psi/eta_bar|^2 + |tau - a|^2/q
-//     (amplitudes in the eigenbasis of I + M^H M/eta_bar, V its whitened basis),
-//     psi_perp = psi - V V^H psi/eta_bar, a = zeta mu^p, q = (gamma^p + |mu^p|^2 (1 - zeta)) zeta,
-//     alpha = psi^H A_s^-1 psi, tau* = (psi^H r0/eta_bar + a/q)/(alpha + 1/q).
 //  iota~(x^p) for every p, summed over j (columns sqrt(pi (gamma + |mu|^2 (1 - pi))) psi_s):
 //     log iota = -|r|^2/eta_bar - |y|^2 - log det(I + D G D/eta_bar) - Nz log(pi eta_bar).
 //  nu~(eta^(j,p)) for every (j, p) through the tridiagonal form of G = M^H M.
@@ -23,895 +18,8 @@
 // per-(p, s, j) geometry records of k_geom (FP64 distance and direction).
 #include "bp_internal.cuh"
 #include "bp_kernels.cuh"
-#include "tc_sm100.cuh"
 
 namespace bp {
-
-// ---------------------------------------------------------------- kappa
-// block = (particle tile of KT threads, s); loop over j; V_{s,j} staged in shared
-// memory as rows of SC complex values (columns 0..SC-2 the eigen-whitened basis,
-// column SC-1 the null residual r0), read two columns per 128-bit broadcast load;
-// 1/lambda_c and y~0_c = (V^H e0)_c/eta_bar beside it.  The basis columns are orthogonal,
-// so every amplitude term is a diagonal sum over the columns.
-
-// The amplitude terms of the PF likelihood in the eigenbasis, with x_c = conj(h_c) =
-// (V^H psi)_c, y~0 = V^H e0/eta_bar and v_c = tau x_c/eta_bar:
-//     |y0|^2 - |y(tau)|^2 = sum_c (|y~0_c|^2 - |y~0_c - v_c|^2)/lambda_c
-//                        = sum_c Re(conj(v_c) (2 y~0_c - v_c))/lambda_c = sum_c g_c.
-// Each g_c is small where v_c is, and the sum has no constant of the size of |y~0|^2 to
-// cancel.  A column whose terms reach KAPPA_AMP_FF (l (|y~0_c| + |v_c|)^2, l = 1/lambda_c)
-// is summed in float-float from exact sums and products of its FP32 operands (a strong
-// path, or a PF whose steering vector lies largely in the others' span: FP32 would put
-// ~1e-7 of the term on the result, and the term varies from particle to particle); the
-// others in FP32, each within ~2e-7 nats.  v_c is rounded to FP32 first: the evaluation
-// point then moves by a rounding, which J, minimal there, feels only at second order.
-// Also gg = sum_c |h_c|^2/lambda_c, the eigenbasis part of alpha.
-// yt: y~0_c, il: 1/lambda_c (.x), u = tau/eta_bar; padded columns have yt = il = 0.
-constexpr float KAPPA_AMP_FF = 1.0f;
-
-__device__ __forceinline__ void kappa_amp_ff_term(ff& G, float l, float2 y, float vx, float vy) {
-    float ax, axl, ay, ayl;
-    two_sum(2.0f * y.x, -vx, ax, axl);   // 2 y~0 - v exactly (2 y~0 is exact)
-    two_sum(2.0f * y.y, -vy, ay, ayl);
-    const float p1 = __fmul_rn(vx, ax), e1 = fmaf(vx, ax, -p1);
-    const float p2 = __fmul_rn(vy, ay), e2 = fmaf(vy, ay, -p2);
-    float sh, sl;
-    two_sum(p1, p2, sh, sl);
-    const float lo = __fadd_rn(__fadd_rn(sl, __fadd_rn(e1, e2)), fmaf(vx, axl, __fmul_rn(vy, ayl)));
-    const float q = __fmul_rn(l, sh), eq = fmaf(l, sh, -q);
-    float t, et;
-    two_sum(G.hi, q, t, et);
-    G.hi = t;
-    G.lo = __fadd_rn(G.lo, __fadd_rn(et, fmaf(l, lo, eq)));
-}
-
-// column c's g_c into G (float-float) or g (FP32), and |h_c|^2/lambda_c into q
-__device__ __forceinline__ void kappa_amp_col(ff& G, float& g, float& q, float2 y, float l, float2 hc, float2 u) {
-    const float vx = fmaf(u.x, hc.x, u.y * hc.y);     // v = u conj(h)
-    const float vy = fmaf(u.y, hc.x, -(u.x * hc.y));
-    const float m = fabsf(y.x) + fabsf(y.y) + fabsf(vx) + fabsf(vy);
-    if (l * m * m > KAPPA_AMP_FF) kappa_amp_ff_term(G, l, y, vx, vy);
-    else g += l * fmaf(vx, fmaf(2.0f, y.x, -vx), vy * fmaf(2.0f, y.y, -vy));
-    q = fmaf(l, fmaf(hc.x, hc.x, hc.y * hc.y), q);
-}
-
-template <int NC>
-__device__ inline void kappa_amp_terms(const float2* yt, const float2* il, const float2 (&h)[NC], float2 u,
-                                       double& dyd, float& gg) {
-    float g0 = 0.f, g1 = 0.f, q0 = 0.f, q1 = 0.f;
-    ff G{0.f, 0.f};
-    #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        if (c & 1) kappa_amp_col(G, g1, q1, yt[c], il[c].x, h[c], u);
-        else       kappa_amp_col(G, g0, q0, yt[c], il[c].x, h[c], u);
-    }
-    dyd = (double)G.hi + (double)G.lo + (double)(g0 + g1);
-    gg = q0 + q1;
-}
-
-// MB blocks per SM (register cap 65536 / (256 MB) per thread)
-template <int SC, int MB>
-__global__ void __launch_bounds__(256, MB) k_kappa(DevGeom G, DevParams Pm, DevState D, int S, int SCA, int fch) {
-    constexpr int KT = 256;
-    constexpr int NC = SC - 1;           // basis columns (zero beyond S-2)
-    constexpr int NP = SC / 2;           // column pairs per row
-    extern __shared__ __align__(1024) float4 sm4[];
-    const int s = blockIdx.y;
-    const int P = Pm.P, J = G.J, Nz = G.Nz, Nm = G.My * G.Mz;
-    float4* Vs = sm4;                                                  // [fch * Nm][NP] rows staged
-    float2* dls = reinterpret_cast<float2*>(Vs + (size_t)fch * Nm * NP); // [SC] 1/lambda_c (.x)
-    float2* y0s = dls + SC;                                            // [SC] y~0_c
-    float2* fac = y0s + SC;                                            // [nfac][KT] factors (high parts)
-    float2* r0ls = fac + (size_t)(G.Nf + G.My + G.Mz) * KT;           // [fch * Nm] low part of r0
-    float2* facl = r0ls + (size_t)fch * Nm;                            // [My + Mz][KT] low parts of a_y, a_z
-    // [256] e^{i 2 pi n / 256} as (hi, lo) pairs, on a 16-byte boundary
-    float4* ctab = reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(facl + (size_t)(G.My + G.Mz) * KT) + 15) &
-                                             ~(uintptr_t)15);
-    float* rn = reinterpret_cast<float*>(ctab + 256);                  // [fch * Nm] |V_k|^2 over the basis columns
-    const int tid = threadIdx.x;
-    cis_table_fill(ctab, tid, KT);
-    const int p = blockIdx.x * KT + tid;
-    const bool act = p < P;
-    const int pp = act ? p : 0;
-    const float* ph = D.phi[D.cur] + (size_t)s * 6 * P;
-    const float4* geo_s = D.geo + (size_t)s * J * P;
-    const float2* geol_s = D.geo_lo + (size_t)s * J * P;
-    const float gmf = ph[3 * P + pp];
-    const float mrf = ph[4 * P + pp], mif = ph[5 * P + pp];
-    const double mr = mrf, mi = mif;
-    double delta_sum = 0.0;
-    for (int j = 0; j < J; ++j) {
-        const float2* gV = D.kV + ((size_t)s * J + j) * Nz * SCA;
-        const float2* gr0l = D.kr0l + ((size_t)s * J + j) * Nz;
-        // rows of frequencies [f0, f0 + fch) -> Vs, r0ls (called by all threads)
-        auto stage_rows = [&](int f0) {
-            float2* Vs2 = reinterpret_cast<float2*>(Vs);
-            const int nrow = min(fch, G.Nf - f0) * Nm;
-            for (int t = tid; t < nrow * SC; t += KT) {
-                const int k = f0 * Nm + t / SC, c = t % SC;
-                Vs2[t] = (c < NC) ? gV[(size_t)k * SCA + c] : gV[(size_t)k * SCA + SCA - 1];
-            }
-            for (int t = tid; t < nrow; t += KT) {
-                r0ls[t] = gr0l[f0 * Nm + t];
-                const float2* vr = gV + (size_t)(f0 * Nm + t) * SCA;
-                float n2 = 0.f;
-                for (int c = 0; c < NC; ++c) n2 = fmaf(vr[c].x, vr[c].x, fmaf(vr[c].y, vr[c].y, n2));
-                rn[t] = n2;
-            }
-        };
-        __syncthreads();
-        {
-            if (fch >= G.Nf) stage_rows(0);
-            const float2* gd = D.kdl + ((size_t)s * J + j) * SCA;
-            const float2* gy = D.ky0 + ((size_t)s * J + j) * SCA;
-            for (int t = tid; t < SC; t += KT) { dls[t] = gd[t]; y0s[t] = gy[t]; }
-        }
-        __syncthreads();
-        const double eb = D.eta_bar[j];
-        const float ebf = (float)eb;
-        const double ieb64 = 1.0 / eb;
-        const double zeta = D.zeta[s * J + j];
-        const double J0r = D.kJ0[s * J + j];   // |r0|^2 / eta_bar
-        float2* fb = fac + tid;
-        float2* fy = fb + G.Nf * KT;
-        float2* fz = fy + G.My * KT;
-        float2* fyl = facl + tid;
-        float2* fzl = fyl + G.My * KT;
-        // steering factors with the carrier folded into b', evaluated as (hi, lo) pairs; the high
-        // parts feed pass 1 (whose rounding only shifts the fitted amplitudes: second order),
-        // pass 2 takes the pairs (the low parts of b' are recomputed there per frequency)
-        const float4 grec = geo_s[(size_t)j * P + pp];
-        const float2 grl = geol_s[(size_t)j * P + pp];
-        const float Aamp = G.amp_c / (grec.x + grec.y);
-        float ch0, cl0;
-        ff_frac_mul2(grec.x, grec.y, G.inv_lam_hi, G.inv_lam_lo, ch0, cl0);
-        {
-            float2 lo_unused;
-            for (int f = 0; f < G.Nf; ++f) bprime_pair(G, ctab, grec.x, grec.y, ch0, cl0, f, fb[f * KT], lo_unused);
-            for (int y = 0; y < G.My; ++y) {
-                const float p = __fmul_rn(G.py_l[y], grec.z);
-                const float e = fmaf(G.py_l[y], grl.x, fmaf(G.py_lo[y], grec.z, fmaf(G.py_l[y], grec.z, -p)));
-                cis_pair(ctab, p, e, fy[y * KT], fyl[y * KT]);
-            }
-            for (int m = 0; m < G.Mz; ++m) {
-                const float p = __fmul_rn(G.pz_l[m], grec.w);
-                const float e = fmaf(G.pz_l[m], grl.y, fmaf(G.pz_lo[m], grec.w, fmaf(G.pz_l[m], grec.w, -p)));
-                cis_pair(ctab, p, e, fz[m * KT], fzl[m * KT]);
-            }
-        }
-        // pass 1: h = psi^H V, pr = psi^H r0
-        float2 h[NC];
-        #pragma unroll
-        for (int c = 0; c < NC; ++c) h[c] = make_float2(0.f, 0.f);
-        float2 pr = make_float2(0.f, 0.f);
-        float nps = 0.f;
-        for (int f0 = 0; f0 < G.Nf; f0 += fch) {
-          if (fch < G.Nf) { __syncthreads(); stage_rows(f0); __syncthreads(); }
-          for (int f = f0; f < min(G.Nf, f0 + fch); ++f) {
-            const float2 cb = make_float2(Aamp * fb[f * KT].x, Aamp * fb[f * KT].y);
-            for (int y = 0; y < G.My; ++y) {
-                const float2 w = cmul(cb, fy[y * KT]);
-                for (int m = 0; m < G.Mz; ++m) {
-                    const float2 ps = cmul(w, fz[m * KT]);
-                    const float4* row = Vs + (size_t)((f - f0) * Nm + y * G.Mz + m) * NP;
-                    #pragma unroll
-                    for (int c2 = 0; c2 < NP; ++c2) {
-                        // conj(psi) v as explicit FMA chains (4 FMA per complex term)
-                        const float4 v = row[c2];
-                        h[2 * c2].x = fmaf(ps.x, v.x, fmaf(ps.y, v.y, h[2 * c2].x));
-                        h[2 * c2].y = fmaf(ps.x, v.y, fmaf(-ps.y, v.x, h[2 * c2].y));
-                        if (2 * c2 + 1 < NC) {
-                            h[2 * c2 + 1].x = fmaf(ps.x, v.z, fmaf(ps.y, v.w, h[2 * c2 + 1].x));
-                            h[2 * c2 + 1].y = fmaf(ps.x, v.w, fmaf(-ps.y, v.z, h[2 * c2 + 1].y));
-                        } else {
-                            pr.x = fmaf(ps.x, v.z, fmaf(ps.y, v.w, pr.x));
-                            pr.y = fmaf(ps.x, v.w, fmaf(-ps.y, v.z, pr.y));
-                        }
-                    }
-                    nps += ps.x * ps.x + ps.y * ps.y;
-                }
-            }
-          }
-        }
-        float hh = 0.f;   // alpha here only places tau (the objective is evaluated exactly at it)
-        #pragma unroll
-        for (int c = 0; c < NC; ++c) hh = fmaf(h[c].x, h[c].x, fmaf(h[c].y, h[c].y, hh));
-        // tau in FP32: J is evaluated exactly at the tau used, so its rounding
-        // enters Delta at second order only
-        const float ieb = 1.0f / ebf;
-        const float alpha = (nps - hh * ieb) * ieb;
-        // a PF whose steering vector lies mostly in the span of the others' m-vectors (more
-        // than 3/4 of its energy) makes psi_perp a small difference: V conj(h) is then summed
-        // exactly (products on a grid fixed per element, 2^E > 8 |V_k| |h|), else in FP32 chains
-        const bool vh_exact = hh * ieb > 0.75f * nps;
-        const float hnorm = sqrtf(hh);
-        const float zf = (float)zeta;
-        const float2 af = make_float2(zf * mrf, zf * mif);
-        const float q = (gmf + (mrf * mrf + mif * mif) * (1.0f - zf)) * zf;
-        const float iq = (q > 0.f) ? 1.0f / q : 0.f;
-        float2 tf = af;
-        if (q > 0.f) {
-            const float den = alpha + iq;
-            tf = make_float2((pr.x * ieb + af.x * iq) / den, (pr.y * ieb + af.y * iq) / den);
-        }
-        // pass 2: r = r0 - tau (psi - V V^H psi / eta_bar), |r|^2 and |psi_perp|^2.
-        // |r|^2/eta_bar can reach ~1e4 (unmodelled paths), so r is formed in
-        // float-float from the exact product tau psi_perp and the two parts of r0,
-        // and its squares are summed exactly; V V^H psi runs in eight FP32 chains of
-        // an eighth of the columns each, added pairwise.
-        ff rr{0.f, 0.f};
-        float pn = 0.f;
-        for (int f0 = 0; f0 < G.Nf; f0 += fch) {
-          if (fch < G.Nf) { __syncthreads(); stage_rows(f0); __syncthreads(); }
-          for (int f = f0; f < min(G.Nf, f0 + fch); ++f) {
-            // the steering element psi = A b' a_y a_z as a (hi, lo) pair (~1e-9): its error
-            // enters the residual at first order
-            float2 bh, bl;
-            bprime_pair(G, ctab, grec.x, grec.y, ch0, cl0, f, bh, bl);
-            const float2 cbh = make_float2(Aamp * bh.x, Aamp * bh.y);
-            const float2 cbl = make_float2(fmaf(Aamp, bh.x, -cbh.x) + Aamp * bl.x, fmaf(Aamp, bh.y, -cbh.y) + Aamp * bl.y);
-            for (int y = 0; y < G.My; ++y) {
-                const float4 wp = cpair_mul(cbh, cbl, fy[y * KT], fyl[y * KT]);
-                const float2 wh = make_float2(wp.x, wp.y), wl = make_float2(wp.z, wp.w);
-                for (int m = 0; m < G.Mz; ++m) {
-                    const float4 psp = cpair_mul(wh, wl, fz[m * KT], fzl[m * KT]);
-                    const int kr = (f - f0) * Nm + y * G.Mz + m;
-                    const float4* row = Vs + (size_t)kr * NP;
-                    constexpr int NCH = NP >= 8 ? 8 : NP;
-                    float2 r0 = make_float2(row[NP - 1].z, row[NP - 1].w);
-                    float vsx = 0.f, vsy = 0.f, vlx = 0.f, vly = 0.f;   // V conj(h) = (vsx + vlx, vsy + vly)
-                    if (vh_exact) {
-                        int gE;
-                        frexpf(8.0f * sqrtf(rn[kr]) * hnorm + 1e-30f, &gE);
-                        const float GM = ldexpf(1.5f, gE);
-                        auto grid = [&](float a, float b, float& g, float& q) {
-                            const float t = __fsub_rn(fmaf(a, b, GM), GM);
-                            g = __fadd_rn(g, t);
-                            q += fmaf(a, b, -t);
-                        };
-                        #pragma unroll
-                        for (int c2 = 0; c2 < NP; ++c2) {
-                            const float4 v = row[c2];
-                            grid(v.x, h[2 * c2].x, vsx, vlx);
-                            grid(v.y, h[2 * c2].y, vsx, vlx);
-                            grid(v.y, h[2 * c2].x, vsy, vly);
-                            grid(-v.x, h[2 * c2].y, vsy, vly);
-                            if (2 * c2 + 1 < NC) {
-                                grid(v.z, h[2 * c2 + 1].x, vsx, vlx);
-                                grid(v.w, h[2 * c2 + 1].y, vsx, vlx);
-                                grid(v.w, h[2 * c2 + 1].x, vsy, vly);
-                                grid(-v.z, h[2 * c2 + 1].y, vsy, vly);
-                            }
-                        }
-                    } else {
-                        float2 va[NCH];
-                        #pragma unroll
-                        for (int i = 0; i < NCH; ++i) va[i] = make_float2(0.f, 0.f);
-                        #pragma unroll
-                        for (int c2 = 0; c2 < NP; ++c2) {
-                            const int ch = (NCH * c2) / NP;
-                            const float4 v = row[c2];
-                            va[ch].x = fmaf(v.x, h[2 * c2].x, fmaf(v.y, h[2 * c2].y, va[ch].x));
-                            va[ch].y = fmaf(v.y, h[2 * c2].x, fmaf(-v.x, h[2 * c2].y, va[ch].y));
-                            if (2 * c2 + 1 < NC) {
-                                va[ch].x = fmaf(v.z, h[2 * c2 + 1].x, fmaf(v.w, h[2 * c2 + 1].y, va[ch].x));
-                                va[ch].y = fmaf(v.w, h[2 * c2 + 1].x, fmaf(-v.z, h[2 * c2 + 1].y, va[ch].y));
-                            }
-                        }
-                        #pragma unroll
-                        for (int w2 = NCH / 2; w2 >= 1; w2 /= 2) {   // pairwise sum of the chains
-                            #pragma unroll
-                            for (int i = 0; i < w2; ++i) { va[i].x += va[i + w2].x; va[i].y += va[i + w2].y; }
-                        }
-                        vsx = va[0].x; vsy = va[0].y;
-                    }
-                    // psi_perp = psi - V V^H psi / eta_bar with the product by 1/eta_bar and the
-                    // subtraction taken exactly
-                    const float dxh = vsx * ieb, dyh = vsy * ieb;
-                    const float dxl = fmaf(vsx, ieb, -dxh) + vlx * ieb, dyl = fmaf(vsy, ieb, -dyh) + vly * ieb;
-                    float2 pp2, ppl;
-                    two_sum(psp.x, -dxh, pp2.x, ppl.x);
-                    two_sum(psp.y, -dyh, pp2.y, ppl.y);
-                    ppl.x += psp.z - dxl;
-                    ppl.y += psp.w - dyl;
-                    pn += pp2.x * pp2.x + pp2.y * pp2.y;
-                    // t = tau pp2 exactly: re = p1 - p2, im = p3 + p4 (+ FMA errors)
-                    const float p1 = __fmul_rn(tf.x, pp2.x), e1 = fmaf(tf.x, pp2.x, -p1);
-                    const float p2 = __fmul_rn(tf.y, pp2.y), e2 = fmaf(tf.y, pp2.y, -p2);
-                    const float p3 = __fmul_rn(tf.x, pp2.y), e3 = fmaf(tf.x, pp2.y, -p3);
-                    const float p4 = __fmul_rn(tf.y, pp2.x), e4 = fmaf(tf.y, pp2.x, -p4);
-                    const float2 rl = r0ls[kr];
-                    float sx, ex1, ex2, sy, ey1, ey2;
-                    ff rx, ry;
-                    two_sum(r0.x, -p1, sx, ex1);
-                    two_sum(sx, p2, rx.hi, ex2);
-                    rx.lo = __fadd_rn(__fadd_rn(rl.x, __fsub_rn(e2, e1)), __fadd_rn(ex1, ex2));
-                    rx.lo = fmaf(-tf.x, ppl.x, fmaf(tf.y, ppl.y, rx.lo));   // - Re(tau psi_perp,lo)
-                    two_sum(r0.y, -p3, sy, ey1);
-                    two_sum(sy, -p4, ry.hi, ey2);
-                    ry.lo = __fsub_rn(__fadd_rn(rl.y, __fadd_rn(ey1, ey2)), __fadd_rn(e3, e4));
-                    ry.lo = fmaf(-tf.x, ppl.y, fmaf(-tf.y, ppl.x, ry.lo));  // - Im(tau psi_perp,lo)
-                    ff_acc_sq(rr, make_float2(rx.hi, ry.hi));
-                    rr.lo = fmaf(2.0f * rx.hi, rx.lo, fmaf(2.0f * ry.hi, ry.lo, rr.lo));
-                }
-            }
-          }
-        }
-        // amplitude terms in the eigenbasis, column by column (kappa_amp_terms)
-        double dyd;
-        float gg;
-        kappa_amp_terms<NC>(y0s, dls, h, make_float2(tf.x * ieb, tf.y * ieb), dyd, gg);
-        double dlt = J0r - ((double)rr.hi + (double)rr.lo) * ieb64 + dyd;
-        if (q > 0.f) {
-            // prior term |tau - a|^2 / q with the difference taken in FP64 (a may be
-            // much larger than the innovation)
-            const double dx = (double)tf.x - zeta * mr, dyt = (double)tf.y - zeta * mi;
-            dlt -= (dx * dx + dyt * dyt) * (double)iq;
-            // alpha = psi^H A^-1 psi = |psi_perp|^2/eta_bar + |R^-1 V^H psi|^2/eta_bar^2 (non-negative terms)
-            const float alpha_acc = pn * ieb + gg * ieb * ieb;
-            dlt -= (double)log1pf(q * alpha_acc);
-        }
-        delta_sum += dlt;
-    }
-    if (act) D.lw_y[(size_t)s * P + p] = delta_sum;
-}
-
-// ---------------------------------------------------------------- kappa on the tensor cores
-// Both contractions of k_kappa run as tcgen05.mma kind::tf32 in 3xTF32 (hi.hi + hi.lo +
-// lo.hi: FP32-level products, FP32 accumulation) with the 128 NT particles of a block as NT
-// 128-row M tiles and TMEM accumulators whose lane is the particle.  SW = 64 or 32 basis
-// columns (SW - 1 eigen-whitened columns and r0):
-//   pass 1, per round of 16 elements: A = psi (Re/Im interleaved), B = rows of
-//     [[Re V, Im V], [Im V, -Re V]] -> h = psi^H V (SW - 1 columns) and psi^H r0 in
-//     2 SW TMEM columns;
-//   pass 2, per group of 32 elements (up to 64 real outputs) and K chunk of 32:
-//     A = [Re h, Im h] (from registers), B = rows [[Re V, Im V]; [Im V, -Re V]] over the
-//     basis columns (r0 excluded) -> the chunk's part of V conj(h) = V V^H psi for the
-//     group's elements, real parts in columns [0, nk), imaginary parts in [nk, 2 nk) of
-//     the chunk's own 64-column accumulator.
-// Pass 2 is the one contraction whose rounding enters the likelihood at first order, so
-// its SW / 16 K chunks accumulate apart (12 MMA accumulations each) and are added pairwise
-// in FP32 when the element-wise float-float residual r = r0 - tau (psi - V V^H psi /
-// eta_bar) reads them back from TMEM, 8 elements at a time.  Operand tiles of B come
-// prebuilt (k_kappa_btile, k_kappa_btile2) by bulk copy; every mbarrier wait is bounded
-// (KAPPA_TC_WAIT polls), after which the kernel flags D.kerr, lets copies and MMAs in
-// flight land, frees TMEM and ends.
-constexpr int KAPPA_TC_WAIT = 1 << 20;
-constexpr int KAPPA_TC_KC2 = 32;   // real K per pass-2 chunk (16 basis columns)
-constexpr int KAPPA_TC_N2 = 64;    // pass-2 accumulator columns per chunk (SW / 16 chunks x 64 per tile)
-
-// The elements k = f Nm + y Mz + m (Nm = My Mz) are taken in ranges: pass 1 in rounds of
-// 16 (KAPPA_TC_KR real K), pass 2 in groups of 32 (up to 64 real outputs).  With
-// 2 My Mz in {8, 16, 32} a round is KR / (2 Nm) whole frequencies and a group 32 / Nm;
-// with Nm a multiple of 16 a round is part of one frequency.
-__host__ __device__ inline int kappa_tc_groups(int Nf, int Nm) { return (Nf * Nm + 31) / 32; }
-__host__ __device__ inline int round16(int x) { return (x + 15) & ~15; }
-// Pass 1's two accumulators alternate by round; every KAPPA_TC_SEG rounds of one (five
-// when a round is one frequency of the 4 x 4 URA, as validated at full size; else two,
-// i.e. 24 MMA accumulations, the chain that stayed within 1e-4) it is added into
-// registers and restarted.  Above KAPPA_TC_FLY_NF frequencies the frequency factors are
-// formed when used instead of being kept in shared memory.
-constexpr int KAPPA_TC_KR = 32;
-constexpr int KAPPA_TC_FLY_NF = 16;
-__host__ __device__ inline int kappa_tc_f1(int Nm) { return KAPPA_TC_KR / (2 * Nm); }   // 0 when Nm > 16
-__host__ __device__ inline int kappa_tc_r1(int Nf, int Nm) { return (Nf * Nm + 15) / 16; }
-__host__ __device__ inline int kappa_tc_seg(int Nm) { return 2 * Nm == KAPPA_TC_KR ? 5 : 2; }
-// operand region in floats for SW basis columns (incl. r0): pass 1 A [NT][hi, lo][128 x KR]
-// and one B slot [hi, lo][2 SW x KR]; pass 2 A [NT][hi, lo][128 x KC2] and two B slots
-// [hi, lo][64 x KC2]
-__host__ __device__ inline int kappa_tc_region_floats(int SW, int NT) {
-    const int r1 = 2 * NT * 128 * KAPPA_TC_KR + 2 * (2 * SW) * KAPPA_TC_KR;
-    const int r2 = 2 * NT * 128 * KAPPA_TC_KC2 + 2 * 2 * KAPPA_TC_N2 * KAPPA_TC_KC2;
-    return r1 > r2 ? r1 : r2;
-}
-
-// NT 128-particle M tiles per block (threads 128 NT, TMEM columns 256 NT): NT = 1 lets two
-// blocks share an SM, so that one block's MMAs run while the other writes operands or
-// evaluates its residuals.
-// LARGE: the arrays of My Mz >= 32 elements (a multiple of 16): pass-1 rounds within one
-// frequency, and pass 2 forms psi as a (hi, lo) pair (~1e-9) from factors evaluated by
-// cis_pair, with psi - V conj(h) / eta_bar taken exactly; at Nz = 1024 and 30 dB the FP32
-// steering values' few ulps, which enter the residual at first order, put 1.2e-4 on the PF
-// weights.  Its frequency factors are formed when used.
-template <int NT, int SW, bool LARGE>
-__global__ void __launch_bounds__(128 * NT, NT == 1 ? 2 : 1) k_kappa_tc(DevGeom G, DevParams Pm, DevState D, int S, int SCA,
-                                                                     const float* __restrict__ Bt1,
-                                                                     const float* __restrict__ Bt2) {
-    static_assert(SW == 64 || SW == 32, "basis width");
-    static_assert(SW == 64 || LARGE, "32 columns only for the large arrays");
-    constexpr int KT = 128 * NT, NC = SW - 1, KC2 = KAPPA_TC_KC2;
-    constexpr int N1 = 2 * SW;                                 // pass-1 accumulator columns
-    constexpr int NCH = SW / 16;                               // pass-2 K chunks
-    extern __shared__ __align__(1024) float4 sm4[];
-    const int s = blockIdx.y;
-    const int P = Pm.P, J = G.J, Nz = G.Nz, Nm = G.My * G.Mz, Nf = G.Nf;
-    const int KC = 2 * Nm;                                     // pass-1 real K per frequency
-    constexpr int KR = KAPPA_TC_KR;                            // pass-1 real K per round
-    const int F1 = kappa_tc_f1(Nm), R1 = kappa_tc_r1(Nf, Nm), SEG = kappa_tc_seg(Nm);
-    const bool fly = LARGE || Nf > KAPPA_TC_FLY_NF;            // frequency factors formed when used
-    const int NG = kappa_tc_groups(Nf, Nm);
-    const int RF = kappa_tc_region_floats(SW, NT);            // operand region (floats)
-    float* sR = reinterpret_cast<float*>(sm4);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(sR + RF);    // [3]: MMAs done, B slot 0, B slot 1 arrived
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 3);
-    float4* r0s = reinterpret_cast<float4*>(sR + RF + 8);    // [Nz] r0 (hi.x, hi.y, lo.x, lo.y)
-    float2* dls = reinterpret_cast<float2*>(r0s + Nz);        // [SW] 1/lambda_c (.x)
-    float2* y0s = dls + SW;                                   // [SW] y~0_c
-    float2* fac = y0s + SW;                                   // [nfac][KT]
-    // LARGE: [Mz][KT] low parts of a_z, then the (hi, lo) cis table [256] on a 16-byte boundary
-    float2* facl = fac + (size_t)((fly ? 0 : Nf) + G.My + G.Mz) * KT;
-    float4* ctab = reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(facl + (size_t)G.Mz * KT) + 15) &
-                                             ~(uintptr_t)15);
-    const int tid = threadIdx.x, warp = tid >> 5, tile = tid >> 7, row = tid & 127;
-    if (LARGE) cis_table_fill(ctab, tid, KT);   // read after the first barrier of the j loop
-    const int p = blockIdx.x * KT + tid;
-    const bool act = p < P;
-    const int pp = act ? p : 0;
-    const uint32_t mb_mma = tc::smem_u32(&mbar[0]), mb_b0 = tc::smem_u32(&mbar[1]);   // slot sl: mb_b0 + 8 sl
-    uint32_t n_commit = 0;
-    uint32_t b_pend = 0, b_par = 0;   // thread 0: per B slot, a copy in flight / the parity of its next wait
-    bool bad = false;
-    if (warp == 0) tc::tmem_alloc(tslot, 256 * NT);
-    if (tid == 0) { tc::mbar_init(mb_mma, 1); tc::mbar_init(mb_b0, 1); tc::mbar_init(mb_b0 + 8, 1); tc::mbar_init_fence(); }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    // B operand stream (thread 0): pass 1 takes one slot of 2 x N1 x KR floats at
-    // sR + 2 NT 128 KR; pass 2 two slots of 2 x 64 x KC2 floats after its A tiles, so that
-    // the copy of the next round's B runs under this round's MMAs.  A copy into a slot is
-    // issued only once the MMAs that read the slot's previous contents have completed.
-    const size_t bchunk1 = (size_t)2 * N1 * KR;
-    const size_t bslot2 = (size_t)2 * KAPPA_TC_N2 * KC2;
-    const int NQ = NCH * NG;   // pass-2 rounds per j
-    float* sB1 = sR + 2 * NT * 128 * KR;
-    float* sB2 = sR + 2 * NT * 128 * KC2;
-    auto issueB = [&](int sl, float* dst, const float* src, uint32_t bytes) {
-        if (tid != 0 || bad) return;
-        const uint32_t mb = mb_b0 + 8u * (uint32_t)sl;
-        tc::mbar_expect_tx(mb, bytes);
-        tc::bulk_g2s(tc::smem_u32(dst), src, bytes, mb);
-        b_pend |= 1u << sl;
-    };
-    auto waitB = [&](int sl) -> bool {   // thread 0
-        const uint32_t mb = mb_b0 + 8u * (uint32_t)sl;
-        if (!tc::mbar_wait(mb, (b_par >> sl) & 1u, KAPPA_TC_WAIT)) return false;
-        b_par ^= 1u << sl;
-        b_pend &= ~(1u << sl);
-        return true;
-    };
-    auto b1_src = [&](int j, int r) { return Bt1 + (((size_t)s * J + j) * R1 + r) * bchunk1; };
-    auto b2_src = [&](int j, int q) { return Bt2 + (((size_t)s * J + j) * NQ + q) * bslot2; };
-    auto b2_bytes = [&](int q) {
-        const int g = q / NCH, nk = min(32, Nz - 32 * g);
-        return (uint32_t)(2 * (2 * round16(nk)) * KC2 * 4);
-    };
-    issueB(0, sB1, b1_src(0, 0), (uint32_t)(bchunk1 * 4));   // the first round's B, under the factor set-up
-    const uint32_t tmem = *tslot;
-    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(tile * 256);   // this thread's row
-    const float* ph = D.phi[D.cur] + (size_t)s * 6 * P;
-    const float4* geo_s = D.geo + (size_t)s * J * P;
-    const float2* geol_s = D.geo_lo + (size_t)s * J * P;
-    const float gmf = ph[3 * P + pp];
-    const float mrf = ph[4 * P + pp], mif = ph[5 * P + pp];
-    const double mr = mrf, mi = mif;
-    // one round: once the previous round's MMAs are done, issueNext() starts a B copy
-    // (thread 0) and every thread writes A (writeA); after the barrier thread 0 waits for
-    // this round's B (slot sl) and issues the 3xTF32 MMAs of both tiles (K in steps of 8)
-    auto round = [&](int sl, float* sA, float* sB, int Kt, uint32_t bLoOff, uint32_t idesc, uint32_t dcol,
-                     bool accum0, auto&& issueNext, auto&& writeA) {
-        if (n_commit > 0 && !bad && !tc::mbar_wait(mb_mma, (n_commit - 1) & 1u, KAPPA_TC_WAIT)) bad = true;
-        issueNext();
-        writeA();
-        tc::fence_async_smem();
-        tc::fence_before_sync();
-        __syncthreads();
-        tc::fence_after_sync();
-        if (tid == 0 && !bad) {
-            if (!waitB(sl)) bad = true;
-            if (!bad) {
-                const uint32_t sbo = (uint32_t)(Kt / 4) * 128u;
-                const uint32_t bH = tc::smem_u32(sB), bL = bH + bLoOff;
-                for (int t = 0; t < NT; ++t) {
-                    const uint32_t aH = tc::smem_u32(sA + (size_t)(t * 2) * 128 * Kt);
-                    const uint32_t aL = tc::smem_u32(sA + (size_t)(t * 2 + 1) * 128 * Kt);
-                    for (int ks = 0; ks < Kt / 8; ++ks) {
-                        const uint32_t o = (uint32_t)ks * 256u;
-                        const uint64_t dAH = tc::smem_desc(aH + o, 128, sbo), dAL = tc::smem_desc(aL + o, 128, sbo);
-                        const uint64_t dBH = tc::smem_desc(bH + o, 128, sbo), dBL = tc::smem_desc(bL + o, 128, sbo);
-                        const uint32_t d = tmem + (uint32_t)(t * 256) + dcol;
-                        tc::mma_tf32(d, dAH, dBH, idesc, accum0 || ks > 0);
-                        tc::mma_tf32(d, dAH, dBL, idesc, true);
-                        tc::mma_tf32(d, dAL, dBH, idesc, true);
-                    }
-                }
-                tc::mma_commit(mb_mma);
-            }
-        }
-        ++n_commit;
-    };
-    auto wait_mma = [&]() {
-        if (!bad && !tc::mbar_wait(mb_mma, (n_commit - 1) & 1u, KAPPA_TC_WAIT)) bad = true;
-        tc::fence_after_sync();
-    };
-    double delta_sum = 0.0;
-    for (int j = 0; j < J; ++j) {
-        const float2* gV = D.kV + ((size_t)s * J + j) * Nz * SCA;
-        const float2* gr0l = D.kr0l + ((size_t)s * J + j) * Nz;
-        __syncthreads();
-        for (int k = tid; k < Nz; k += KT) {
-            const float2 hi = gV[(size_t)k * SCA + SCA - 1], lo = gr0l[k];
-            r0s[k] = make_float4(hi.x, hi.y, lo.x, lo.y);
-        }
-        {
-            const float2* gd = D.kdl + ((size_t)s * J + j) * SCA;
-            const float2* gy = D.ky0 + ((size_t)s * J + j) * SCA;
-            for (int t = tid; t < SW; t += KT) { dls[t] = gd[t]; y0s[t] = gy[t]; }
-        }
-        __syncthreads();
-        const double eb = D.eta_bar[j];
-        const float ebf = (float)eb;
-        const double ieb64 = 1.0 / eb;
-        const double zeta = D.zeta[s * J + j];
-        const double J0r = D.kJ0[s * J + j];
-        float2* fb = fac + tid;                                // [Nf][KT] unless fly
-        float2* fy = fb + (fly ? 0 : Nf) * KT;
-        float2* fz = fy + G.My * KT;
-        const float4 grec = geo_s[(size_t)j * P + pp];
-        const float2 grl = geol_s[(size_t)j * P + pp];
-        float2 Fc;
-        float Aamp = 0.f, ch0 = 0.f, cl0 = 0.f;   // LARGE: psi = A (b' kron a_y kron a_z), carrier in b'
-        float2* fzl = facl + tid;
-        // the phase of a_y (cycles, float-float) and its (hi, lo) pair
-        auto ay_phase = [&](int y, float& p, float& e) {
-            p = __fmul_rn(G.py_l[y], grec.z);
-            e = fmaf(G.py_l[y], grl.x, fmaf(G.py_lo[y], grec.z, fmaf(G.py_l[y], grec.z, -p)));
-        };
-        if (LARGE) {
-            Aamp = G.amp_c / (grec.x + grec.y);
-            ff_frac_mul2(grec.x, grec.y, G.inv_lam_hi, G.inv_lam_lo, ch0, cl0);
-            Fc = make_float2(Aamp, 0.f);   // cmul(Fc, b') = A b' exactly
-            float2 lo_unused;
-            for (int y = 0; y < G.My; ++y) {
-                float p, e;
-                ay_phase(y, p, e);
-                cis_pair(ctab, p, e, fy[y * KT], lo_unused);
-            }
-            for (int m = 0; m < G.Mz; ++m) {
-                const float p = __fmul_rn(G.pz_l[m], grec.w);
-                const float e = fmaf(G.pz_l[m], grl.y, fmaf(G.pz_lo[m], grec.w, fmaf(G.pz_l[m], grec.w, -p)));
-                cis_pair(ctab, p, e, fz[m * KT], fzl[m * KT]);
-            }
-        } else if (fly) {
-            Fc = carrier_factor(G, grec);
-            array_factors(G, grec, grl, fy, fz, KT);
-        } else {
-            Fc = factors_from_geo(G, grec, grl, fb, fy, fz, KT);
-        }
-        // b_f as pass 1 and pass 2 both take it (the shared copy holds the same values);
-        // LARGE: the high part of b'_f
-        auto bfac = [&](int f) {
-            if (LARGE) {
-                float2 bh, bl;
-                bprime_pair(G, ctab, grec.x, grec.y, ch0, cl0, f, bh, bl);
-                return bh;
-            }
-            return fly ? freq_factor(G, grec, f) : fb[f * KT];
-        };
-        // h = psi^H V and pr = psi^H r0, summed over the pass-1 accumulator segments
-        float2 h[NC];
-        float2 pr = make_float2(0.f, 0.f);
-        #pragma unroll
-        for (int c = 0; c < NC; ++c) h[c] = make_float2(0.f, 0.f);
-        // adds the pass-1 accumulator at TMEM column base (N1 columns: Re h 0..NC-1, Re pr,
-        // Im h 0..NC-1, Im pr) into h and pr, 32 columns at a time
-        auto absorb = [&](uint32_t base) {
-            #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                #pragma unroll
-                for (int c0 = 0; c0 < SW; c0 += 32) {
-                    uint32_t v[32];
-                    tc::tmem_ld32(tlane + base + (uint32_t)(part * SW + c0), v);
-                    tc::tmem_ld_wait();
-                    #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const float a = __uint_as_float(v[i]);
-                        if (c0 + i < NC) { if (part == 0) h[c0 + i].x += a; else h[c0 + i].y += a; }
-                        else             { if (part == 0) pr.x += a; else pr.y += a; }
-                    }
-                }
-            }
-        };
-        // ---- pass 1: h = psi^H V, pr = psi^H r0, 16 elements per round
-        float nps = 0.f;
-        {
-            float* sA = sR;
-            float* aHi = sA + (size_t)(tile * 2 + 0) * 128 * KR;
-            float* aLo = sA + (size_t)(tile * 2 + 1) * 128 * KR;
-            const uint32_t idesc = tc::idesc_tf32_f32(128, N1);
-            // even rounds accumulate in columns 0..N1-1, odd ones in N1..2 N1-1; a segment of
-            // SEG rounds of one accumulator is added into h (after the MMAs of the previous
-            // round are done, before this round overwrites it); the first round's B was
-            // issued before this j began
-            for (int r = 0; r < R1; ++r) {
-                const int q = r & 1;
-                const bool seg_start = ((r >> 1) % SEG) == 0;
-                round(0, sA, sB1, KR, (uint32_t)(N1 * KR * 4), idesc, (uint32_t)(q * N1), !seg_start,
-                      [&]() {
-                    if (seg_start && r >= 2) absorb((uint32_t)(q * N1));
-                    if (r > 0) issueB(0, sB1, b1_src(j, r), (uint32_t)(bchunk1 * 4));
-                }, [&]() {
-                    if constexpr (LARGE) {
-                        // Nm a multiple of 16: the round is elements 16 r .. 16 r + 15 of one
-                        // frequency, walked in pairs (m, m + 1) of a row (Mz even)
-                        const int k0 = r * 16, f = k0 / Nm, e0 = k0 - f * Nm;
-                        const float2 cb = cmul(Fc, bfac(f));
-                        int y = e0 / G.Mz, m = e0 - y * G.Mz;
-                        float2 w = cmul(cb, fy[y * KT]);
-                        #pragma unroll 1
-                        for (int l = 0; l < 16; l += 2) {
-                            const float2 p0 = cmul(w, fz[m * KT]), p1 = cmul(w, fz[(m + 1) * KT]);
-                            nps += p0.x * p0.x + p0.y * p0.y + p1.x * p1.x + p1.y * p1.y;
-                            const float4 hi = make_float4(tc::tf32_rn(p0.x), tc::tf32_rn(p0.y), tc::tf32_rn(p1.x),
-                                                          tc::tf32_rn(p1.y));
-                            const float4 lo = make_float4(tc::tf32_rn(p0.x - hi.x), tc::tf32_rn(p0.y - hi.y),
-                                                          tc::tf32_rn(p1.x - hi.z), tc::tf32_rn(p1.y - hi.w));
-                            const int off = tc::core_off(row, 2 * l, KR) >> 2;
-                            *reinterpret_cast<float4*>(aHi + off) = hi;
-                            *reinterpret_cast<float4*>(aLo + off) = lo;
-                            m += 2;
-                            if (m == G.Mz && l + 2 < 16) { m = 0; ++y; w = cmul(cb, fy[y * KT]); }
-                        }
-                    } else {
-                    for (int i = 0; i < F1; ++i) {
-                        const int f = r * F1 + i;
-                        if (f >= Nf) {   // past the last frequency: zero operands
-                            for (int kk = i * KC; kk < (i + 1) * KC; kk += 4) {
-                                const int off = tc::core_off(row, kk, KR) >> 2;
-                                *reinterpret_cast<float4*>(aHi + off) = make_float4(0.f, 0.f, 0.f, 0.f);
-                                *reinterpret_cast<float4*>(aLo + off) = make_float4(0.f, 0.f, 0.f, 0.f);
-                            }
-                            continue;
-                        }
-                        const float2 cb = cmul(Fc, bfac(f));
-                        for (int y = 0; y < G.My; ++y) {
-                            const float2 w = cmul(cb, fy[y * KT]);
-                            for (int m = 0; m < G.Mz; m += 2) {
-                                const float2 p0 = cmul(w, fz[m * KT]), p1 = cmul(w, fz[(m + 1) * KT]);
-                                nps += p0.x * p0.x + p0.y * p0.y + p1.x * p1.x + p1.y * p1.y;
-                                const float4 hi = make_float4(tc::tf32_rn(p0.x), tc::tf32_rn(p0.y), tc::tf32_rn(p1.x),
-                                                              tc::tf32_rn(p1.y));
-                                const float4 lo = make_float4(tc::tf32_rn(p0.x - hi.x), tc::tf32_rn(p0.y - hi.y),
-                                                              tc::tf32_rn(p1.x - hi.z), tc::tf32_rn(p1.y - hi.w));
-                                const int off = tc::core_off(row, i * KC + 2 * (y * G.Mz + m), KR) >> 2;
-                                *reinterpret_cast<float4*>(aHi + off) = hi;
-                                *reinterpret_cast<float4*>(aLo + off) = lo;
-                            }
-                        }
-                    }
-                    }
-                });
-            }
-        }
-        wait_mma();
-        // pass 2's first two B tiles, under the read-back of h and the amplitude sums
-        issueB(0, sB2, b2_src(j, 0), b2_bytes(0));
-        issueB(1, sB2 + bslot2, b2_src(j, 1), b2_bytes(1));
-        absorb(0);                       // the segments still in TMEM
-        if (R1 > 1) absorb((uint32_t)N1);
-        // h and pr back into columns 0..N1-1 (the accumulator layout), where the amplitude
-        // loop reads them
-        #pragma unroll
-        for (int part = 0; part < 2; ++part) {
-            #pragma unroll
-            for (int c0 = 0; c0 < SW; c0 += 32) {
-                uint32_t v[32];
-                #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const float2 a = (c0 + i < NC) ? h[c0 + i] : pr;
-                    v[i] = __float_as_uint(part == 0 ? a.x : a.y);
-                }
-                tc::tmem_st32(tlane + (uint32_t)(part * SW + c0), v);
-            }
-        }
-        tc::tmem_st_wait();
-        // tau (FP32; J is evaluated exactly at the tau used) and the O(S) amplitude sums
-        float hh = 0.f;
-        #pragma unroll
-        for (int c = 0; c < NC; ++c) hh = fmaf(h[c].x, h[c].x, fmaf(h[c].y, h[c].y, hh));
-        const float ieb = 1.0f / ebf;
-        const float alpha = (nps - hh * ieb) * ieb;
-        const float zf = (float)zeta;
-        const float2 af = make_float2(zf * mrf, zf * mif);
-        const float q = (gmf + (mrf * mrf + mif * mif) * (1.0f - zf)) * zf;
-        const float iq = (q > 0.f) ? 1.0f / q : 0.f;
-        float2 tf = af;
-        if (q > 0.f) {
-            const float den = alpha + iq;
-            tf = make_float2((pr.x * ieb + af.x * iq) / den, (pr.y * ieb + af.y * iq) / den);
-        }
-        // amplitude terms in the eigenbasis (kappa_amp_terms), h read again from TMEM columns
-        // 0..N1-1 (written back above) eight columns at a time: a rolled loop keeps the
-        // per-column code out of the instruction cache's way
-        double dyd;
-        float gg;
-        {
-            const float2 u = make_float2(tf.x * ieb, tf.y * ieb);
-            float g0 = 0.f, g1 = 0.f, q0 = 0.f, q1 = 0.f;
-            ff G{0.f, 0.f};
-            #pragma unroll 1
-            for (int c0 = 0; c0 < SW; c0 += 8) {
-                uint32_t a[8], b[8];
-                float hx[8], hy[8];
-                tc::tmem_ld8(tlane + (uint32_t)c0, a);
-                tc::tmem_ld8(tlane + (uint32_t)(SW + c0), b);
-                tc::tmem_ld_wait();
-                #pragma unroll
-                for (int i = 0; i < 8; ++i) { hx[i] = __uint_as_float(a[i]); hy[i] = __uint_as_float(b[i]); }
-                #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int c = c0 + i;
-                    if (c < NC) {   // column NC holds psi^H r0
-                        if (i & 1) kappa_amp_col(G, g1, q1, y0s[c], dls[c].x, make_float2(hx[i], hy[i]), u);
-                        else       kappa_amp_col(G, g0, q0, y0s[c], dls[c].x, make_float2(hx[i], hy[i]), u);
-                    }
-                }
-            }
-            dyd = (double)G.hi + (double)G.lo + (double)(g0 + g1);
-            gg = q0 + q1;
-        }
-        // ---- pass 2: V V^H psi per group of frequencies, then the element-wise residual
-        ff rr{0.f, 0.f};
-        float pn = 0.f;
-        tc::fence_before_sync();   // TMEM reads of h complete before pass 2 reuses the columns
-        for (int g = 0; g < NG; ++g) {
-            const int k0 = 32 * g, nk = min(32, Nz - k0), nkp = round16(nk), N2 = 2 * nkp;
-            float* sA = sR;
-            float* aHi = sA + (size_t)(tile * 2 + 0) * 128 * KC2;
-            float* aLo = sA + (size_t)(tile * 2 + 1) * 128 * KC2;
-            const uint32_t idesc = tc::idesc_tf32_f32(128, N2);
-            #pragma unroll
-            for (int kc = 0; kc < NCH; ++kc) {
-                // round q = NCH g + kc reads slot q & 1 = kc & 1 (NCH is even); the copy of
-                // round q + 1 goes to the slot that round q - 1 read
-                const int q = NCH * g + kc;
-                round(kc & 1, sA, sB2 + (size_t)(kc & 1) * bslot2, KC2, (uint32_t)(N2 * KC2 * 4), idesc,
-                      (uint32_t)(kc * KAPPA_TC_N2), false, [&]() {
-                    if (q >= 1 && q + 1 < NQ)
-                        issueB((q + 1) & 1, sB2 + (size_t)((q + 1) & 1) * bslot2, b2_src(j, q + 1), b2_bytes(q + 1));
-                }, [&]() {
-                    #pragma unroll
-                    for (int c2 = 0; c2 < KC2 / 4; ++c2) {       // basis columns c, c + 1
-                        const int c = kc * 16 + 2 * c2;
-                        const float2 u0 = h[c];
-                        const float2 u1 = (c + 1 < NC) ? h[c + 1] : make_float2(0.f, 0.f);
-                        const float4 hi = make_float4(tc::tf32_rn(u0.x), tc::tf32_rn(u0.y), tc::tf32_rn(u1.x), tc::tf32_rn(u1.y));
-                        const float4 lo = make_float4(tc::tf32_rn(u0.x - hi.x), tc::tf32_rn(u0.y - hi.y),
-                                                      tc::tf32_rn(u1.x - hi.z), tc::tf32_rn(u1.y - hi.w));
-                        const int off = tc::core_off(row, 4 * c2, KC2) >> 2;
-                        *reinterpret_cast<float4*>(aHi + off) = hi;
-                        *reinterpret_cast<float4*>(aLo + off) = lo;
-                    }
-                });
-            }
-            wait_mma();
-            // every MMA of this j is done: the next j's first B tile, under the residuals
-            if (g == NG - 1 && j + 1 < J) issueB(0, sB1, b1_src(j + 1, 0), (uint32_t)(bchunk1 * 4));
-            // element (f, y, m) of the group walked in order from k0; w = Fc b_f a_y formed as
-            // pass 1 formed it (LARGE: the pair (wh, wl) = A b'_f a_y from cis_pair factors)
-            int cf = k0 / Nm, cy = (k0 - cf * Nm) / G.Mz, cm = k0 - cf * Nm - cy * G.Mz;
-            float2 w = make_float2(0.f, 0.f), wh = w, wl = w;
-            auto set_w = [&]() {
-                if (LARGE) {
-                    float2 bh, bl, ayh, ayl;
-                    bprime_pair(G, ctab, grec.x, grec.y, ch0, cl0, cf, bh, bl);
-                    const float2 cbh = make_float2(Aamp * bh.x, Aamp * bh.y);
-                    const float2 cbl = make_float2(fmaf(Aamp, bh.x, -cbh.x) + Aamp * bl.x,
-                                                   fmaf(Aamp, bh.y, -cbh.y) + Aamp * bl.y);
-                    float p, e;
-                    ay_phase(cy, p, e);
-                    cis_pair(ctab, p, e, ayh, ayl);
-                    const float4 wp = cpair_mul(cbh, cbl, ayh, ayl);
-                    wh = make_float2(wp.x, wp.y);
-                    wl = make_float2(wp.z, wp.w);
-                } else {
-                    w = cmul(cmul(Fc, bfac(cf)), fy[cy * KT]);
-                }
-            };
-            set_w();
-            for (int b = 0; b < nk; b += 8) {
-                // the chunk accumulators, added pairwise: (a0 + a1) [+ (a2 + a3)]
-                float vre[8], vim[8];
-                #pragma unroll
-                for (int c2 = 0; c2 < NCH; c2 += 2) {
-                    uint32_t r0[8], r1[8], i0[8], i1[8];
-                    tc::tmem_ld8(tlane + (uint32_t)(c2 * KAPPA_TC_N2 + b), r0);
-                    tc::tmem_ld8(tlane + (uint32_t)((c2 + 1) * KAPPA_TC_N2 + b), r1);
-                    tc::tmem_ld8(tlane + (uint32_t)(c2 * KAPPA_TC_N2 + nkp + b), i0);
-                    tc::tmem_ld8(tlane + (uint32_t)((c2 + 1) * KAPPA_TC_N2 + nkp + b), i1);
-                    tc::tmem_ld_wait();
-                    #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float ar = __uint_as_float(r0[i]) + __uint_as_float(r1[i]);
-                        const float ai = __uint_as_float(i0[i]) + __uint_as_float(i1[i]);
-                        if (c2 == 0) { vre[i] = ar; vim[i] = ai; }
-                        else         { vre[i] += ar; vim[i] += ai; }
-                    }
-                }
-                #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int kl = b + i;
-                    if (kl >= nk) break;
-                    const int k = k0 + kl;
-                    float2 ps;         // psi_k exactly as pass 1 formed it
-                    float4 psp;        // LARGE: psi_k as a (hi, lo) pair
-                    if (LARGE) psp = cpair_mul(wh, wl, fz[cm * KT], fzl[cm * KT]);
-                    else       ps = cmul(w, fz[cm * KT]);
-                    if (++cm == G.Mz) {
-                        cm = 0;
-                        if (++cy == G.My) { cy = 0; ++cf; }
-                        if (kl + 1 < nk) set_w();
-                    }
-                    const float vsx = vre[i], vsy = vim[i];
-                    float2 pp2, ppl = make_float2(0.f, 0.f);
-                    if (LARGE) {
-                        // psi_perp = psi - V V^H psi / eta_bar with the product by 1/eta_bar and
-                        // the subtraction taken exactly; its low part ppl
-                        const float dxh = vsx * ieb, dyh = vsy * ieb;
-                        const float dxl = fmaf(vsx, ieb, -dxh), dyl = fmaf(vsy, ieb, -dyh);
-                        two_sum(psp.x, -dxh, pp2.x, ppl.x);
-                        two_sum(psp.y, -dyh, pp2.y, ppl.y);
-                        ppl.x += psp.z - dxl;
-                        ppl.y += psp.w - dyl;
-                    } else {
-                        pp2 = make_float2(ps.x - vsx * ieb, ps.y - vsy * ieb);
-                    }
-                    pn += pp2.x * pp2.x + pp2.y * pp2.y;
-                    // t = tau pp2 exactly: re = p1 - p2, im = p3 + p4 (+ FMA errors)
-                    const float p1 = __fmul_rn(tf.x, pp2.x), e1 = fmaf(tf.x, pp2.x, -p1);
-                    const float p2 = __fmul_rn(tf.y, pp2.y), e2 = fmaf(tf.y, pp2.y, -p2);
-                    const float p3 = __fmul_rn(tf.x, pp2.y), e3 = fmaf(tf.x, pp2.y, -p3);
-                    const float p4 = __fmul_rn(tf.y, pp2.x), e4 = fmaf(tf.y, pp2.x, -p4);
-                    const float4 r0 = r0s[k];
-                    float sx, ex1, ex2, sy, ey1, ey2;
-                    ff rx, ry;
-                    two_sum(r0.x, -p1, sx, ex1);
-                    two_sum(sx, p2, rx.hi, ex2);
-                    rx.lo = __fadd_rn(__fadd_rn(r0.z, __fsub_rn(e2, e1)), __fadd_rn(ex1, ex2));
-                    two_sum(r0.y, -p3, sy, ey1);
-                    two_sum(sy, -p4, ry.hi, ey2);
-                    ry.lo = __fsub_rn(__fadd_rn(r0.w, __fadd_rn(ey1, ey2)), __fadd_rn(e3, e4));
-                    if (LARGE) {
-                        rx.lo = fmaf(-tf.x, ppl.x, fmaf(tf.y, ppl.y, rx.lo));    // - Re(tau psi_perp,lo)
-                        ry.lo = fmaf(-tf.x, ppl.y, fmaf(-tf.y, ppl.x, ry.lo));   // - Im(tau psi_perp,lo)
-                    }
-                    ff_acc_sq(rr, make_float2(rx.hi, ry.hi));
-                    rr.lo = fmaf(2.0f * rx.hi, rx.lo, fmaf(2.0f * ry.hi, ry.lo, rr.lo));
-                }
-            }
-            tc::fence_before_sync();   // TMEM reads complete before the next group's MMAs
-        }
-        double dlt = J0r - ((double)rr.hi + (double)rr.lo) * ieb64 + dyd;
-        if (q > 0.f) {
-            const double dx = (double)tf.x - zeta * mr, dyt = (double)tf.y - zeta * mi;
-            dlt -= (dx * dx + dyt * dyt) * (double)iq;
-            const float alpha_acc = pn * ieb + gg * ieb * ieb;
-            dlt -= (double)log1pf(q * alpha_acc);
-        }
-        delta_sum += dlt;
-    }
-    if (act) D.lw_y[(size_t)s * P + p] = delta_sum;
-    if (bad && (tid & 31) == 0) atomicOr(D.kerr, 1);
-    if (tid == 0) {
-        // after a timeout: let the copies and MMAs still in flight land (bounded)
-        for (int sl = 0; sl < 2; ++sl)
-            if ((b_pend >> sl) & 1u) waitB(sl);
-        if (n_commit > 0) tc::mbar_wait(mb_mma, (n_commit - 1) & 1u, KAPPA_TC_WAIT);
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tmem, 256 * NT);
-}
 
 // ---------------------------------------------------------------- iota (warp per particle)
 // Fast path in FP32: factors from the geometry records, g = Psi^H z, the Gram
@@ -1575,187 +683,6 @@ __global__ void k_nu(DevGeom G, DevParams Pm, DevState D, int S) {
     const double e2 = D.nu_c[2 * j];
     const double lnu = -(e2 - quad) / eta - (G.Nz - S) * log(eta) - logdet - G.Nz * log(M_PI);
     D.lw_eta[(size_t)j * P + p] = lnu;
-}
-
-// B tiles of the tensor-core pass 1, once per (s, j, round r of elements 16 r .. 16 r + 15):
-// rows n of [[Re V, Im V], [Im V, -Re V]]^T (n < SW: Re h_n, n >= SW: Im h_{n-SW}, SW = SCA
-// basis columns incl. r0) against the real K index 2 e + part of the round's element e
-// (part 0 = Re psi, 1 = Im psi; zero past the last element), split into TF32 high and low
-// parts, in the K-major core-matrix layout; [hi, lo] per round.
-__global__ void k_kappa_btile(DevGeom G, DevState D, int SCA, float* __restrict__ Bt) {
-    constexpr int KR = KAPPA_TC_KR;
-    const int s = blockIdx.x, j = blockIdx.y, r = blockIdx.z;
-    const int J = G.J, Nz = G.Nz, Nm = G.My * G.Mz, N1 = 2 * SCA;
-    const int R1 = kappa_tc_r1(G.Nf, Nm);
-    const float2* V = D.kV + ((size_t)s * J + j) * Nz * SCA;
-    float* out = Bt + (((size_t)s * J + j) * R1 + r) * 2 * N1 * KR;
-    for (int t = threadIdx.x; t < N1 * KR; t += blockDim.x) {
-        const int n = t / KR, kk = t - n * KR;
-        const int k = r * 16 + (kk >> 1), part = kk & 1;
-        const int c = n < SCA ? n : n - SCA;
-        const float2 v = (k < Nz) ? V[(size_t)k * SCA + c] : make_float2(0.f, 0.f);
-        const float b = (n < SCA) ? (part == 0 ? v.x : v.y) : (part == 0 ? v.y : -v.x);
-        const float hi = tc::tf32_rn(b);
-        const int off = tc::core_off(n, kk, KR) >> 2;
-        out[off] = hi;
-        out[N1 * KR + off] = tc::tf32_rn(b - hi);
-    }
-}
-
-// B tiles of the tensor-core pass 2, once per (s, j, group g of elements 32 g .. 32 g + 31,
-// K chunk kc of SCA / 16): rows n < nkp are the real parts, rows nkp <= n < 2 nkp the
-// imaginary parts of the group's elements e (rows past the group's nk elements are zero),
-// against the real K index 2 (c - 16 kc) + part of basis columns c (part 0 = Re h_c,
-// 1 = Im h_c; the r0 column SCA - 1 excluded): Re row [Re V_ec, Im V_ec], Im row
-// [Im V_ec, -Re V_ec]; TF32 hi/lo, K-major core-matrix layout, [hi, lo] per slot of
-// 2 x 64 x 32 floats.
-__global__ void k_kappa_btile2(DevGeom G, DevState D, int SCA, float* __restrict__ Bt2) {
-    constexpr int KC2 = KAPPA_TC_KC2;
-    const int NCH = SCA / 16;
-    const int s = blockIdx.x, j = blockIdx.y, g = blockIdx.z / NCH, kc = blockIdx.z - g * NCH;
-    const int J = G.J, Nz = G.Nz, Nm = G.My * G.Mz, NG = kappa_tc_groups(G.Nf, Nm);
-    const int k0 = 32 * g, nk = min(32, Nz - k0), nkp = round16(nk), N2 = 2 * nkp;
-    const float2* V = D.kV + ((size_t)s * J + j) * Nz * SCA;
-    float* out = Bt2 + ((((size_t)s * J + j) * NG + g) * NCH + kc) * (size_t)(2 * KAPPA_TC_N2 * KC2);
-    for (int t = threadIdx.x; t < N2 * KC2; t += blockDim.x) {
-        const int n = t / KC2, kk = t - n * KC2;
-        const bool im = n >= nkp;
-        const int e = im ? n - nkp : n;
-        const int c = kc * 16 + (kk >> 1), part = kk & 1;
-        float2 v = make_float2(0.f, 0.f);
-        if (e < nk && c < SCA - 1) v = V[(size_t)(k0 + e) * SCA + c];
-        const float b = im ? (part == 0 ? v.y : -v.x) : (part == 0 ? v.x : v.y);
-        const float hi = tc::tf32_rn(b);
-        const int off = tc::core_off(n, kk, KC2) >> 2;
-        out[off] = hi;
-        out[N2 * KC2 + off] = tc::tf32_rn(b - hi);
-    }
-}
-
-// dynamic shared memory of k_kappa_tc: the operand region (pass 1: A [NT][hi, lo][128 x 32],
-// B [hi, lo][2 SW x 32]; pass 2: A [NT][hi, lo][128 x 32], two B slots [hi, lo][64 x 32]),
-// barriers, r0 (hi, lo) per element, 1/lambda_c and y~0_c, and the factors of 128 NT particles
-constexpr int KAPPA_TC_NT = 1;   // M tiles per block of the launched variant
-static bool kappa_tc_large(const DevGeom& G) {
-    const int Nm = G.My * G.Mz;
-    return Nm >= 32 && Nm % 16 == 0;
-}
-static size_t kappa_tc_smem(const DevGeom& G, int SW, int NT = KAPPA_TC_NT) {
-    const bool large = kappa_tc_large(G);
-    const size_t nfac = (size_t)(large || G.Nf > KAPPA_TC_FLY_NF ? 0 : G.Nf) + G.My + G.Mz;
-    const size_t rf = (size_t)kappa_tc_region_floats(SW, NT);
-    const size_t pairs = large ? (size_t)G.Mz * 128 * NT * sizeof(float2) + 16 + 256 * sizeof(float4) : 0;
-    return rf * sizeof(float) + 32 + (size_t)G.Nz * sizeof(float4) + 2 * (size_t)SW * sizeof(float2) +
-           nfac * 128 * NT * sizeof(float2) + pairs;
-}
-// The tensor-core variant applies to
-//   * 64 basis columns (SCA = 64) with 2 My Mz in {8, 16, 32} (a pass-1 round is whole
-//     frequencies), and
-//   * 64 or 32 basis columns with My Mz a multiple of 16, at least 32 (a round is part of
-//     one frequency; the large arrays, whose CUDA-core kernel stages few frequencies),
-// both with Mz even (a pass-1 round writes the pairs (m, m + 1) of a row) and the shared
-// memory within the opt-in limit.  The tensor core adds each MMA's result into its FP32
-// accumulator (no FMA chain): with 75 frequencies of the 2 x 2 URA in one pass-1
-// accumulator (225 accumulations) the PF weights moved by 1.7e-4 (measured), with 24 they
-// stayed within 1e-4; hence the segments of KAPPA_TC_SEG rounds.
-bool kappa_tc_ok(const DevGeom& G, int SCA) {
-    const int Nm = G.My * G.Mz, KC = 2 * Nm;
-    if (G.Mz % 2 != 0) return false;
-    const bool whole = SCA == 64 && (KC == 8 || KC == 16 || KC == 32);
-    const bool part = (SCA == 64 || SCA == 32) && kappa_tc_large(G);
-    return (whole || part) && kappa_tc_smem(G, SCA) <= 227 * 1024;
-}
-static size_t kappa_btile1_floats(const DevGeom& G, int S_max, int SCA) {
-    return (size_t)S_max * G.J * kappa_tc_r1(G.Nf, G.My * G.Mz) * 2 * (2 * SCA) * KAPPA_TC_KR;
-}
-size_t kappa_btile_floats(const DevGeom& G, int S_max, int SCA) {
-    const int Nm = G.My * G.Mz;
-    return kappa_btile1_floats(G, S_max, SCA) +
-           (size_t)S_max * G.J * kappa_tc_groups(G.Nf, Nm) * (SCA / 16) * (2 * KAPPA_TC_N2 * KAPPA_TC_KC2);
-}
-int launch_kappa_btile(const DevGeom& G, const DevState& D, int S, int SCA, cudaStream_t st) {
-    if (!D.kB || !kappa_tc_ok(G, SCA)) return 0;
-    const int Nm = G.My * G.Mz;
-    k_kappa_btile<<<dim3(S, G.J, kappa_tc_r1(G.Nf, Nm)), 256, 0, st>>>(G, D, SCA, D.kB);
-    k_kappa_btile2<<<dim3(S, G.J, kappa_tc_groups(G.Nf, Nm) * (SCA / 16)), 256, 0, st>>>(
-        G, D, SCA, D.kB + kappa_btile1_floats(G, S, SCA));
-    return 2;
-}
-
-// shared memory of the CUDA-core PF likelihood: 1/lambda, y~0 [2 SC], factors [nfac][256],
-// low parts of a_y, a_z [My + Mz][256] (float2), alignment slack and the (hi, lo) cis table
-// [256] (float4), then per staged frequency the V rows, the low part of r0 and |V_k|^2
-static size_t kappa_smem_fixed(const DevGeom& G, int SC) {
-    const size_t nfac = (size_t)G.Nf + G.My + G.Mz;
-    return (2 * (size_t)SC + (nfac + G.My + G.Mz) * 256) * sizeof(float2) + 16 + 256 * sizeof(float4);
-}
-static size_t kappa_smem_per_f(const DevGeom& G, int SC) {
-    const size_t Nm = (size_t)G.My * G.Mz;
-    return Nm * (SC + 1) * sizeof(float2) + Nm * sizeof(float);
-}
-// shared-memory budget per block: one block per SM, or two (228 KB per SM, 1 KB reserved each)
-static size_t kappa_smem_budget(int mb) { return mb == 2 ? 112 * 1024 : 200 * 1024; }
-
-static bool kappa_sc_valid(int sc) { return sc == 8 || sc == 16 || sc == 24 || sc == 32 || sc == 48 || sc == 64; }
-
-KappaPlan plan_kappa(const DevGeom& G, const DevState& D, int S, int SCA, int t_sc, int t_mb, int t_fch, int t_tc) {
-    KappaPlan k{};
-    // the bucket: the requested one where it holds S and fits the basis stride, else the
-    // smallest that holds S; the tensor-core kernel where allowed and not declined
-    // (the kernel's width is the basis stride: 64, or 32 for the large arrays)
-    const bool tc_shape = D.kB && kappa_tc_ok(G, SCA);
-    if (kappa_sc_valid(t_sc) && t_sc >= S && t_sc <= SCA) k.sc = t_sc;
-    else if (S > 32 && tc_shape && t_tc >= 0) k.sc = 64;
-    else k.sc = S <= 8 ? 8 : S <= 16 ? 16 : S <= 24 ? 24 : S <= 32 ? 32 : S <= 48 ? 48 : 64;
-    k.tc = k.sc == SCA && tc_shape && t_tc >= 0;
-    if (k.tc) return k;
-    k.mb = (k.sc <= 16) ? 2 : (t_mb == 2 && k.sc <= 32 ? 2 : 1);
-    const size_t fixed = kappa_smem_fixed(G, k.sc), per_f = kappa_smem_per_f(G, k.sc);
-    if (k.mb == 2 && k.sc > 16 && fixed + per_f > kappa_smem_budget(2)) k.mb = 1;
-    const size_t limit = kappa_smem_budget(k.mb);
-    int fch = G.Nf;
-    while (fch > 1 && fixed + fch * per_f > limit) fch = (fch + 1) / 2;
-    if (t_fch > 0 && t_fch < fch) fch = t_fch;
-    k.fch = fch;
-    k.smem = fixed + (size_t)fch * per_f;
-    return k;
-}
-
-template <int SC, int MB>
-static void launch_kappa_cc(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, int fch,
-                            size_t smem, cudaStream_t st) {
-    smem_allow_max((const void*)k_kappa<SC, MB>);
-    k_kappa<SC, MB><<<dim3((Pm.P + 255) / 256, S), 256, smem, st>>>(G, Pm, D, S, SCA, fch);
-}
-
-void launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, const KappaPlan& k,
-                  cudaStream_t st) {
-    if (k.tc) {
-        constexpr int NT = KAPPA_TC_NT;
-        const dim3 grid((Pm.P + 128 * NT - 1) / (128 * NT), S);
-        const float* bt2 = D.kB + kappa_btile1_floats(G, S, SCA);
-        if (!kappa_tc_large(G)) {
-            smem_allow_max((const void*)k_kappa_tc<NT, 64, false>);
-            k_kappa_tc<NT, 64, false><<<grid, 128 * NT, kappa_tc_smem(G, 64), st>>>(G, Pm, D, S, SCA, D.kB, bt2);
-        } else if (SCA == 64) {
-            smem_allow_max((const void*)k_kappa_tc<NT, 64, true>);
-            k_kappa_tc<NT, 64, true><<<grid, 128 * NT, kappa_tc_smem(G, 64), st>>>(G, Pm, D, S, SCA, D.kB, bt2);
-        } else {
-            smem_allow_max((const void*)k_kappa_tc<NT, 32, true>);
-            k_kappa_tc<NT, 32, true><<<grid, 128 * NT, kappa_tc_smem(G, 32), st>>>(G, Pm, D, S, SCA, D.kB, bt2);
-        }
-        return;
-    }
-    switch (k.sc * 4 + k.mb) {
-        case 8 * 4 + 2:  launch_kappa_cc<8, 2>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        case 16 * 4 + 2: launch_kappa_cc<16, 2>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        case 24 * 4 + 1: launch_kappa_cc<24, 1>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        case 24 * 4 + 2: launch_kappa_cc<24, 2>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        case 32 * 4 + 1: launch_kappa_cc<32, 1>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        case 32 * 4 + 2: launch_kappa_cc<32, 2>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        case 48 * 4 + 1: launch_kappa_cc<48, 1>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-        default:         launch_kappa_cc<64, 1>(G, Pm, D, S, SCA, k.fch, k.smem, st); break;
-    }
 }
 
 // S below which the FP32 path runs first and only flagged particles are redone

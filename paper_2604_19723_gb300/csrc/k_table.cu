@@ -9,13 +9,11 @@
 // FP32 accumulation over chunks of particles, FP64 across chunks.
 //
 // Stage per (s, j), FP64 (S-V "PF state update message", "PR state update
-// message", S-VI): A_s = eta_bar I + M_{-s} M_{-s}^H is represented by the
-// Cholesky-whitened basis V = M_{-s} R^-1 (R^H R = I + G_{-s}/eta_bar), so that
-// a^H A_s^-1 b = (a^H b - (V^H a)^H (V^H b)/eta_bar)/eta_bar (the inversion lemma
-// of S-V with the small inverse factored).  It also forms the regularised
-// null residual r0 = eta_bar A_s^-1 e0 (e0 = z - sum_{s'!=s} mu3_s'), the
-// coefficients y0 = (eta_bar I + G_{-s})^-1 M_{-s}^H e0, J0 = e0^H A_s^-1 e0,
-// and the PR existence test omega~(1)/omega~(0) -> p_s^(j) (eq. PR-normalization).
+// message", S-VI): A_s = eta_bar I + M_{-s} M_{-s}^H is represented by a
+// Cholesky-whitened basis V of M_{-s} (the inversion lemma of S-V with the small
+// inverse factored), which with the null residual r0 = eta_bar A_s^-1 e0
+// (e0 = z - sum_{s'!=s} mu3_s') is all the PF likelihood needs; the same forms give
+// the PR existence test omega~(1)/omega~(0) -> p_s^(j) (eq. PR-normalization).
 //
 // nu (S-V "Noise variance update message"): G = M^H M is reduced once per j
 // to a real symmetric tridiagonal T = Q^H G Q (Householder), with b = Q^H M^H e;
@@ -212,210 +210,28 @@ __global__ void k_gram(DevGeom G, DevParams Pm, DevState D, int S, const float* 
 }
 
 // ---------------------------------------------------------------- kappa / omega stage per (s, j), FP64
-// One block per (s, j).  The inverse of A_s = eta_bar I + M_{-s} M_{-s}^H (S-V) enters
-// through B = I + M_{-s}^H M_{-s}/eta_bar = U diag(lambda) U^H, found by cyclic Jacobi
-// rotations: the whitened basis V = M_{-s} U diag(lambda)^{-1/2} has orthogonal
-// columns and V V^H = M_{-s} B^{-1} M_{-s}^H, so A_s^{-1} = (I - V V^H/eta_bar)/eta_bar,
-// and the per-particle amplitude terms |B^{-1/2} U^H M^H psi|^2 become diagonal sums.
-// V is written to an FP64 scratch row by row (thread per row).
-
-// Hermitian eigen-decomposition of the n x n matrix A (row-major, shared) by cyclic
-// Jacobi with the round-robin parallel ordering: in each of the n2 - 1 rounds of a sweep
-// (n2 = n rounded up to even) the n2/2 disjoint pairs rotate at once.  For the pair
-// (p, q) with a_pq = |a_pq| e^{i phi}, zeta = (a_qq - a_pp)/(2|a_pq|) and
-// t = sign(zeta)/(|zeta| + sqrt(1 + zeta^2)) the unitary G (columns p, q:
-// (c, -s e^{-i phi}), (s, c e^{-i phi}), c = 1/sqrt(1 + t^2), s = t c) zeroes a_pq in
-// G^H A G.  U accumulates the G's (from the identity, or from a given start).  Sweeps
-// stop when every pair satisfies |a_pq|^2 (a_pp - shift)(a_qq - shift) <= tol (a_pp a_qq)^2,
-// after at most max_sweeps.  For B = I + G with G positive semi-definite (shift = 1,
-// g = lambda - 1) an off-diagonal a_pq left in the basis perturbs every form
-// x^H M B^-1 M^H x by at most |a_pq| sqrt(g_p g_q) / (lambda_p lambda_q) per unit of
-// whitened energy, so the test weighs each pair by what it contributes: pairs of large
-// eigenvalues converge to a relative accuracy, pairs inside the cluster of eigenvalues
-// near 1 (near-duplicate columns of M) are not chased.  A test of the off-diagonal
-// energy against the diagonal energy, which the largest eigenvalues dominate, stopped
-// with the small eigenvalues' pairs unresolved.  T is float or double; all threads of
-// the block call it.
-template <typename T> struct cplx;
-template <> struct cplx<float> { using t = float2; };
-template <> struct cplx<double> { using t = double2; };
-template <typename T> struct JRot { T c, s, er, ei; };   // cos, sin, e^{i phi}
-
-// Cyclic Jacobi on a Hermitian matrix held as its packed lower triangle (element (r, c),
-// r >= c, at r (r + 1)/2 + c), in T = float or double arithmetic (the convergence test in
-// FP64).  Each round of the round-robin ordering takes two barriers: the rotations of its
-// disjoint pairs, then one pass that applies them, to U by columns and to A by 2 x 2 blocks
-// between pairs (rows of pair i, columns of pair i', i >= i': block <- G_i^H block G_i'),
-// the diagonal blocks set to their exact diagonal form.  U is updated from its given
-// start.  A pair whose off-diagonal element already meets the convergence test is not
-// rotated (threshold Jacobi).
-__device__ inline int pk_idx(int r, int c) { return r * (r + 1) / 2 + c; }
-template <typename C>
-__device__ inline C pk_get(const C* A, int r, int c) {
-    if (r >= c) return A[pk_idx(r, c)];
-    C v = A[pk_idx(c, r)];
-    v.y = -v.y;
-    return v;
-}
-template <typename C>
-__device__ inline void pk_set(C* A, int r, int c, C v) {
-    if (r >= c) { A[pk_idx(r, c)] = v; return; }
-    v.y = -v.y;
-    A[pk_idx(c, r)] = v;
-}
-
-template <typename T>
-__device__ void jacobi_herm_packed(typename cplx<T>::t* A, typename cplx<T>::t* U, int n, JRot<T>* rot, double* red,
-                                   double tol, double shift, int max_sweeps) {
-    using C = typename cplx<T>::t;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    __syncthreads();
-    if (n < 2) return;
-    const int n2 = n + (n & 1), half = n2 / 2;
-    auto pair_of = [&](int r, int i, int& p, int& q) {
-        int a, b;
-        if (i == 0) { a = n2 - 1; b = r; }
-        else { a = (r + i) % (n2 - 1); b = (r - i + n2 - 1) % (n2 - 1); }
-        p = min(a, b); q = max(a, b);
-    };
-    auto cz = []() { C z; z.x = T(0); z.y = T(0); return z; };
-    const int nblk = half * (half + 1) / 2;
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        if (tid == 0) red[0] = 0.0;
-        __syncthreads();
-        bool viol = false;
-        for (int t = tid; t < n * (n - 1) / 2; t += nt) {   // strictly lower elements (r, c)
-            int r = (int)((sqrtf((float)(8 * t + 1)) + 1.0f) * 0.5f);
-            while (r * (r - 1) / 2 > t) --r;
-            while ((r + 1) * r / 2 <= t) ++r;
-            const int c = t - r * (r - 1) / 2;
-            const C v = A[pk_idx(r, c)];
-            const double m2 = (double)v.x * v.x + (double)v.y * v.y;
-            const double dr = fabs((double)A[pk_idx(r, r)].x), dc = fabs((double)A[pk_idx(c, c)].x);
-            const double gr = fmax(dr - shift, 0.0), gc = fmax(dc - shift, 0.0);
-            if (!(m2 * gr * gc <= tol * (dr * dc) * (dr * dc))) viol = true;
-        }
-        if (viol) red[0] = 1.0;
-        __syncthreads();
-        const bool done = (red[0] == 0.0);
-        __syncthreads();
-        if (done) break;
-        for (int r = 0; r < n2 - 1; ++r) {
-            for (int i = tid; i < half; i += nt) {
-                int p, q;
-                pair_of(r, i, p, q);
-                JRot<T> g{T(1), T(0), T(1), T(0)};
-                if (q < n) {
-                    const C apq = pk_get(A, p, q);
-                    const T m = sqrt(apq.x * apq.x + apq.y * apq.y);
-                    const double dp = fabs((double)A[pk_idx(p, p)].x), dq = fabs((double)A[pk_idx(q, q)].x);
-                    const double m2 = (double)m * (double)m;
-                    const bool small = m2 * fmax(dp - shift, 0.0) * fmax(dq - shift, 0.0) <= tol * (dp * dq) * (dp * dq);
-                    if (!small && m > T(1e-30)) {
-                        const T zeta = (A[pk_idx(q, q)].x - A[pk_idx(p, p)].x) / (T(2) * m);
-                        const T t = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
-                        const T c = T(1) / sqrt(T(1) + t * t);
-                        g = JRot<T>{c, t * c, apq.x / m, apq.y / m};
-                    }
-                }
-                rot[i] = g;
-            }
-            __syncthreads();
-            // U by columns: (u_p, u_q) <- (c u_p - s e^{-i phi} u_q, s u_p + c e^{-i phi} u_q)
-            for (int t = tid; t < half * n; t += nt) {
-                const int i = t / n, row = t - i * n;
-                int p, q;
-                pair_of(r, i, p, q);
-                if (q >= n) continue;
-                const JRot<T> g = rot[i];
-                if (g.s == T(0)) continue;
-                const C xp = U[row * n + p], xq = U[row * n + q];
-                const T eqx = g.er * xq.x + g.ei * xq.y, eqy = g.er * xq.y - g.ei * xq.x;
-                C np, nq;
-                np.x = g.c * xp.x - g.s * eqx; np.y = g.c * xp.y - g.s * eqy;
-                nq.x = g.s * xp.x + g.c * eqx; nq.y = g.s * xp.y + g.c * eqy;
-                U[row * n + p] = np;
-                U[row * n + q] = nq;
-            }
-            // A by 2 x 2 blocks: rows of pair i, columns of pair i' <= i
-            for (int b = tid; b < nblk; b += nt) {
-                int i = (int)((sqrtf((float)(8 * b + 1)) - 1.0f) * 0.5f);
-                while ((i + 1) * (i + 2) / 2 <= b) ++i;
-                while (i * (i + 1) / 2 > b) --i;
-                const int i2 = b - i * (i + 1) / 2;
-                const JRot<T> g1 = rot[i], g2 = rot[i2];
-                if (g1.s == T(0) && g2.s == T(0)) continue;
-                int p1, q1, p2, q2;
-                pair_of(r, i, p1, q1);
-                pair_of(r, i2, p2, q2);
-                const bool v1 = q1 < n, v2 = q2 < n;   // the ghost index of odd n pairs with one real index
-                if (i == i2) {
-                    if (!v1) continue;
-                    // G^H [[a_pp, a_pq], [a_qp, a_qq]] G: diagonal by construction of the rotation
-                    const C apq = pk_get(A, p1, q1);
-                    const T app = A[pk_idx(p1, p1)].x, aqq = A[pk_idx(q1, q1)].x;
-                    const T re = g1.er * apq.x + g1.ei * apq.y;      // Re(e^{-i phi} a_pq) = |a_pq|
-                    const T c = g1.c, s = g1.s;
-                    C dpp = cz(), dqq = cz();
-                    dpp.x = c * c * app - T(2) * c * s * re + s * s * aqq;
-                    dqq.x = s * s * app + T(2) * c * s * re + c * c * aqq;
-                    A[pk_idx(p1, p1)] = dpp;
-                    A[pk_idx(q1, q1)] = dqq;
-                    A[pk_idx(q1, p1)] = cz();
-                    continue;
-                }
-                // block X = [[x00, x01], [x10, x11]] at rows (p1, q1), columns (p2, q2)
-                C x00 = pk_get(A, p1, p2);
-                C x01 = v2 ? pk_get(A, p1, q2) : cz();
-                C x10 = v1 ? pk_get(A, q1, p2) : cz();
-                C x11 = (v1 && v2) ? pk_get(A, q1, q2) : cz();
-                if (g2.s != T(0)) {   // X G2: columns (c x_p - s e^{-i phi} x_q, s x_p + c e^{-i phi} x_q)
-                    auto colrot = [&](C& xp, C& xq) {
-                        const T ex = g2.er * xq.x + g2.ei * xq.y, ey = g2.er * xq.y - g2.ei * xq.x;
-                        C np, nq;
-                        np.x = g2.c * xp.x - g2.s * ex; np.y = g2.c * xp.y - g2.s * ey;
-                        nq.x = g2.s * xp.x + g2.c * ex; nq.y = g2.s * xp.y + g2.c * ey;
-                        xp = np; xq = nq;
-                    };
-                    colrot(x00, x01);
-                    colrot(x10, x11);
-                }
-                if (g1.s != T(0)) {   // G1^H X: rows (c a_p - s e^{i phi} a_q, s a_p + c e^{i phi} a_q)
-                    auto rowrot = [&](C& ap, C& aq) {
-                        const T ex = g1.er * aq.x - g1.ei * aq.y, ey = g1.er * aq.y + g1.ei * aq.x;
-                        C np, nq;
-                        np.x = g1.c * ap.x - g1.s * ex; np.y = g1.c * ap.y - g1.s * ey;
-                        nq.x = g1.s * ap.x + g1.c * ex; nq.y = g1.s * ap.y + g1.c * ey;
-                        ap = np; aq = nq;
-                    };
-                    rowrot(x00, x10);
-                    rowrot(x01, x11);
-                }
-                pk_set(A, p1, p2, x00);
-                if (v2) pk_set(A, p1, q2, x01);
-                if (v1) pk_set(A, q1, p2, x10);
-                if (v1 && v2) pk_set(A, q1, q2, x11);
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// 12 warps per block and two blocks per SM (106 KB of shared memory each): the FP64
-// rotation and product loops are latency bound
-constexpr int STAGE_THREADS = 384;
-
+// One block per (s, j).  With B = I + M_{-s}^H M_{-s}/eta_bar = L L^H (Cholesky) the whitened
+// basis V = M_{-s} L^{-H} satisfies V V^H = M_{-s} B^{-1} M_{-s}^H, so the inversion lemma gives
+// a^H A_s^{-1} b = (a^H b - (V^H a)^H (V^H b)/eta_bar)/eta_bar for every form of S-V, and
+// r0 = eta_bar A_s^{-1} e0 = e0 - V V^H e0/eta_bar.  V and r0 leave as columns of V64
+// [S][J][SCA][Nz] (r0 in column SCA - 1) for k_kappa_digits.
+// The forms of the existence test need V^H x = L^{-1} (M^H x) for x = e0, m^w, mu4 only: the
+// rows (M^H x)^H ride along the factorisation as rows K .. K + 2.
+// Bound: the FP64 pipe (2 FMA per clock and SM), 4 Nz K^2/2 FMA for V (the eigen-decomposition
+// that stood here before, which the element-wise likelihood needed for its diagonal sums, took
+// 13.4 ms at 64 PFs x 4 PAs x Nz = 160, most of it rotations and barriers; this takes 1.7 ms with
+// the Gram, and 5.6 -> 1.5 ms at 40 PFs x Nz = 300).
+constexpr int STAGE_THREADS = 256;
 constexpr int STAGE_WRED = 9;   // per-warp partial sums of the omega test's scalars
-__host__ __device__ inline size_t stage_kappa_rp(int K, int Nz) {   // the packed region, then e0 (Nz)
-    const size_t t = (size_t)K * (K + 1) / 2;
-    return t > (size_t)Nz ? t : (size_t)Nz;
+__host__ __device__ inline int stage_row(int K, int r) {   // start of row r of [L; three carried rows]
+    return r < K ? r * (r + 1) / 2 : K * (K + 1) / 2 + (r - K) * K;
 }
 __host__ __device__ inline size_t stage_kappa_smem(int K, int Nz) {
-    return ((size_t)K * K + stage_kappa_rp(K, Nz) + (size_t)(STAGE_THREADS / 32) * K) * sizeof(double2) +
-           8 * sizeof(double) + 32 * sizeof(JRot<double>) + (size_t)STAGE_WRED * (STAGE_THREADS / 32) * sizeof(double);
+    return ((size_t)K * (K + 1) / 2 + 3 * (size_t)K + (size_t)Nz) * sizeof(double2) +
+           ((size_t)K + STAGE_WRED * (STAGE_THREADS / 32) + 2) * sizeof(double);
 }
 
-__global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevParams Pm, DevState D, int S, int SC,
+__global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevParams Pm, DevState D, int S, int SCA,
                                                                   const float* z, const double* gram, double* V64) {
     const int s = blockIdx.x, j = blockIdx.y;
     const int J = G.J, Nz = G.Nz, SM = Pm.S_max;
@@ -423,112 +239,26 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
     const double eb = D.eta_bar[j];
     const size_t plane = (size_t)SM * J * Nz;
     const double2* tab = reinterpret_cast<const double2*>(D.tab);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = STAGE_THREADS / 32;
     extern __shared__ double2 sh[];
-    double2* Ue = sh;                            // K x K eigenvectors (columns), FP64
-    double2* Rp = Ue + (size_t)K * K;            // packed lower triangle of U^H B U, then the eigenvalues
-    float2* A32 = reinterpret_cast<float2*>(Ue); // the FP32 solve first: A32 in Ue's bytes, U32 in Rp's
-    float2* U32 = reinterpret_cast<float2*>(Rp); // (K^2 float2 <= K (K + 1)/2 double2)
-    double2* scr = Rp + stage_kappa_rp(K, Nz);  // [nw][K] columns of B U; then the projections below
-    double2* ye = scr;                           // V^H e0 / eb      (K)
-    double2* vm = ye + K;                        // V^H m^w          (K)
-    double2* v4 = vm + K;                        // V^H mu4          (K)
-    double* dinv = reinterpret_cast<double*>(v4 + K);   // lambda^{-1/2}  (K)
-    double2* pa = scr + 4 * (size_t)K;           // M^H e0, M^H m^w, M^H mu4 (3 K; nw >= 7)
-    double2* E0 = Rp;                            // e0 = z - sum_{t != s} mu3_t once Rp is free (Nz)
-    double* red = reinterpret_cast<double*>(scr + (size_t)nw * K);   // reduction scratch [8]
-    JRot<double>* rot = reinterpret_cast<JRot<double>*>(red + 8);   // Jacobi pair rotations [32]
-    double* wred = reinterpret_cast<double*>(rot + 32);              // [STAGE_WRED][nw]
-    JRot<float>* rot32 = reinterpret_cast<JRot<float>*>(rot);
+    double2* Lp = sh;                             // packed lower triangle, then three rows of K
+    double2* E0 = Lp + stage_row(K, K + 3);       // e0 = z - sum_{t != s} mu3_t (Nz)
+    double* il = reinterpret_cast<double*>(E0 + Nz);   // 1 / L_cc (K)
+    double* wred = il + K;                        // [STAGE_WRED][nw]
     const double2* Gm = reinterpret_cast<const double2*>(gram) + (size_t)j * SM * SM;
-    // column map c -> s'
-    auto col = [&](int c) { return c < s ? c : c + 1; };
-    // B = I + G_{-s}/eb (Hermitian), read from the Gram matrix in global memory (L2)
-    auto Bv = [&](int r, int c) {
-        double2 g = Gm[col(r) * SM + col(c)];
-        g.x /= eb; g.y /= eb;
-        if (r == c) { g.x += 1.0; g.y = 0.0; }
-        return g;
-    };
-    // eigenvectors to FP32 accuracy by FP32 sweeps, then B rotated into that basis in FP64
-    // (nearly diagonal) and finished by FP64 sweeps
-    for (int t = threadIdx.x; t < K * (K + 1) / 2; t += blockDim.x) {   // packed lower triangle
-        int r = (int)((sqrtf((float)(8 * t + 1)) - 1.0f) * 0.5f);
-        while ((r + 1) * (r + 2) / 2 <= t) ++r;
-        while (r * (r + 1) / 2 > t) --r;
-        const double2 g = Bv(r, t - r * (r + 1) / 2);
-        A32[t] = make_float2((float)g.x, (float)g.y);
-    }
-    for (int t = threadIdx.x; t < K * K; t += blockDim.x) U32[t] = make_float2(t / K == t % K ? 1.f : 0.f, 0.f);
-    jacobi_herm_packed<float>(A32, U32, K, rot32, red, 1e-13, 1.0, 10);
-    for (int t = threadIdx.x; t < K * K; t += blockDim.x) Ue[t] = make_double2((double)U32[t].x, (double)U32[t].y);
-    __syncthreads();
-    {   // the FP32 columns are orthonormal to ~1e-5 only: modified Gram-Schmidt in FP64, so
-        // that U^H B U below is a similarity transform of B
-        for (int c = 0; c < K; ++c) {
-            if (wid == 0) {
-                double a = 0.0;
-                for (int r = lane; r < K; r += 32) a += Ue[r * K + c].x * Ue[r * K + c].x + Ue[r * K + c].y * Ue[r * K + c].y;
-                a = warp_sum_d(a);
-                if (lane == 0) red[0] = 1.0 / sqrt(a);
-            }
-            __syncthreads();
-            const double inv = red[0];
-            for (int r = threadIdx.x; r < K; r += blockDim.x) { Ue[r * K + c].x *= inv; Ue[r * K + c].y *= inv; }
-            __syncthreads();
-            for (int c2 = c + 1 + wid; c2 < K; c2 += nw) {
-                double dx = 0.0, dy = 0.0;
-                for (int r = lane; r < K; r += 32) {
-                    const double2 u = zmulc(Ue[r * K + c], Ue[r * K + c2]);
-                    dx += u.x; dy += u.y;
-                }
-                dx = warp_sum_d(dx); dy = warp_sum_d(dy);
-                for (int r = lane; r < K; r += 32) {
-                    const double2 u = zmul(make_double2(dx, dy), Ue[r * K + c]);
-                    Ue[r * K + c2].x -= u.x; Ue[r * K + c2].y -= u.y;
-                }
-            }
-            __syncthreads();
+    auto col = [&](int c) { return c < s ? c : c + 1; };   // column c of M_{-s} is PF col(c)
+    // B = I + G_{-s}/eb, packed
+    for (int r = wid; r < K; r += nw)
+        for (int c = lane; c <= r; c += 32) {
+            double2 g = Gm[col(r) * SM + col(c)];
+            g.x /= eb; g.y /= eb;
+            if (r == c) { g.x += 1.0; g.y = 0.0; }
+            Lp[stage_row(K, r) + c] = g;
         }
-    }
-    // R = U^H B U (packed lower triangle), one column at a time per warp: v = B u_c, then
-    // R_rc = u_r^H v for r >= c
-    for (int c = wid; c < K; c += nw) {
-        double2* v = scr + (size_t)wid * K;
-        for (int m = lane; m < K; m += 32) {
-            // (B u_c)_m = u_mc + (G_{-s} u_c)_m / eb, with G_mn = conj(G_nm): the Gram is stored
-            // with both triangles, bitwise Hermitian, so lanes m read consecutive addresses
-            double2 acc = make_double2(0.0, 0.0);
-            for (int n = 0; n < K; ++n) {
-                const double2 g = Gm[col(n) * SM + col(m)];
-                const double2 u = zmulc(g, Ue[n * K + c]);
-                acc.x += u.x; acc.y += u.y;
-            }
-            const double2 um = Ue[m * K + c];
-            v[m] = make_double2(um.x + acc.x / eb, um.y + acc.y / eb);
-        }
-        __syncwarp();
-        for (int r = c + lane; r < K; r += 32) {
-            double2 acc = make_double2(0.0, 0.0);
-            for (int m = 0; m < K; ++m) {
-                const double2 u = zmulc(Ue[m * K + r], v[m]);
-                acc.x += u.x; acc.y += u.y;
-            }
-            Rp[pk_idx(r, c)] = (r == c) ? make_double2(acc.x, 0.0) : acc;
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    // typically 2-3 sweeps; the weighted test at 1e-18 leaves ~1e-8 nats on the PR test
-    // (emulated on 26- and 64-PF states)
-    jacobi_herm_packed<double>(Rp, Ue, K, rot, red, 1e-18, 1.0, 8);
-    for (int c = threadIdx.x; c < K; c += blockDim.x) dinv[c] = 1.0 / sqrt(fmax(Rp[pk_idx(c, c)].x, 1.0));
-    __syncthreads();
-    // e0 = z - sum_{t != s} mu3_t per element (into the freed packed region) and the
-    // block sums of |e0|^2, m^H e0, |m|^2, mu4^H e0, |mu4|^2, m^H mu4 (m = m^w_s)
+    // e0 and the block sums of |e0|^2, m^H e0, |m|^2, mu4^H e0, |mu4|^2, m^H mu4 (m = m^w_s)
     {
         double acc[STAGE_WRED] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int k = threadIdx.x; k < Nz; k += blockDim.x) {
+        for (int k = tid; k < Nz; k += STAGE_THREADS) {
             double2 e0 = make_double2((double)z[2 * (j * Nz + k)], (double)z[2 * (j * Nz + k) + 1]);
             for (int t = 0; t < S; ++t) {
                 if (t == s) continue;
@@ -553,12 +283,12 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
         }
     }
     __syncthreads();
-    if (threadIdx.x < STAGE_WRED) {
+    if (tid < STAGE_WRED) {
         double v = 0.0;
-        for (int w = 0; w < nw; ++w) v += wred[threadIdx.x * nw + w];
-        wred[threadIdx.x * nw] = v;   // the block sum in slot 0
+        for (int w = 0; w < nw; ++w) v += wred[tid * nw + w];
+        wred[tid * nw] = v;   // the block sum in slot 0
     }
-    // M^H e0, M^H m^w, M^H mu4 over the columns t of M_{-s}: one warp per column
+    // (M^H e0)^H, (M^H m^w)^H, (M^H mu4)^H: one warp per column t
     for (int t = wid; t < K; t += nw) {
         const double2* mt = tab + ((size_t)col(t) * J + j) * Nz;
         const double2* mwp = tab + 1 * plane + ((size_t)s * J + j) * Nz;
@@ -573,129 +303,114 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
         bx = warp_sum_d(bx); by = warp_sum_d(by);
         cx = warp_sum_d(cx); cy = warp_sum_d(cy);
         if (lane == 0) {
-            pa[t] = make_double2(ax, ay);
-            pa[K + t] = make_double2(bx, by);
-            pa[2 * K + t] = make_double2(cx, cy);
+            Lp[stage_row(K, K) + t] = make_double2(ax, -ay);
+            Lp[stage_row(K, K + 1) + t] = make_double2(bx, -by);
+            Lp[stage_row(K, K + 2) + t] = make_double2(cx, -cy);
         }
     }
     __syncthreads();
-    // V^H x = diag(lambda)^{-1/2} U^H (M^H x): V = M U diag(lambda)^{-1/2}
-    for (int c = threadIdx.x; c < K; c += blockDim.x) {
-        double2 a1 = make_double2(0, 0), a2 = make_double2(0, 0), a3 = make_double2(0, 0);
-        for (int t = 0; t < K; ++t) {
-            const double2 u = Ue[t * K + c];
-            const double2 q1 = zmulc(u, pa[t]), q2 = zmulc(u, pa[K + t]), q3 = zmulc(u, pa[2 * K + t]);
-            a1.x += q1.x; a1.y += q1.y; a2.x += q2.x; a2.y += q2.y; a3.x += q3.x; a3.y += q3.y;
+    // right-looking Cholesky of the K x K triangle with the three carried rows; every pivot of B
+    // is at least 1
+    for (int k = 0; k < K; ++k) {
+        if (tid == 0) il[k] = rsqrt(fmax(Lp[stage_row(K, k) + k].x, 1.0));
+        __syncthreads();
+        const double d = il[k];
+        for (int r = k + 1 + tid; r < K + 3; r += STAGE_THREADS) {
+            double2& v = Lp[stage_row(K, r) + k];
+            v.x *= d; v.y *= d;
         }
-        const double d = dinv[c];
-        ye[c] = make_double2(d * a1.x, d * a1.y);
-        vm[c] = make_double2(d * a2.x, d * a2.y);
-        v4[c] = make_double2(d * a3.x, d * a3.y);
+        __syncthreads();
+        for (int r = k + 1 + (tid >> 4); r < K + 3; r += STAGE_THREADS / 16) {
+            const int row = stage_row(K, r), end = min(r, K - 1);
+            const double2 x = Lp[row + k];
+            for (int c = k + 1 + (tid & 15); c <= end; c += 16) {
+                const double2 u = zmulc(Lp[stage_row(K, c) + k], x);   // l_rk conj(l_ck)
+                double2& v = Lp[row + c];
+                v.x -= u.x; v.y -= u.y;
+            }
+        }
+        __syncthreads();
     }
-    // V rows v_k = m_k U diag(lambda)^{-1/2} (FP64), eight columns per work item so that
-    // each m_t(k) is read once per item; consecutive threads take consecutive elements
-    double2* Vs = reinterpret_cast<double2*>(V64) + ((size_t)s * J + j) * Nz * SC;
-    {
-        constexpr int CB = 8;
-        const int nch = (K + CB - 1) / CB;
-        for (int it = threadIdx.x; it < Nz * nch; it += blockDim.x) {
-            const int k = it % Nz, c0 = (it / Nz) * CB;
+    const double2* ye = Lp + stage_row(K, K);     // conj of V^H e0, V^H m^w, V^H mu4
+    const double2* vm = ye + K;
+    const double2* v4 = vm + K;
+    if (wid == 0) {
+        double a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        for (int c = lane; c < K; c += 32) {
+            const double2 e = make_double2(ye[c].x, -ye[c].y), b = make_double2(vm[c].x, -vm[c].y),
+                          u = make_double2(v4[c].x, -v4[c].y);
+            const double2 t1 = zmulc(b, e), t2 = zmulc(u, e), t3 = zmulc(b, u);
+            a[0] += e.x * e.x + e.y * e.y;
+            a[1] += t1.x; a[2] += t1.y;
+            a[3] += b.x * b.x + b.y * b.y;
+            a[4] += t2.x;
+            a[6] += u.x * u.x + u.y * u.y;
+            a[7] += t3.x; a[8] += t3.y;
+        }
+        #pragma unroll
+        for (int q = 0; q < 9; ++q) a[q] = (wred[q * nw] - warp_sum_d(a[q]) / eb) / eb;   // forms x^H A^-1 y
+        if (lane == 0) {
+            // e0^H A^-1 e0, and with e1 = e0 - mu4: e1^H A^-1 e1
+            const double Q00 = a[0], Q11 = a[0] - 2.0 * a[4] + a[6];
+            // m^H A^-1 m >= 0 (A positive definite); a negative value is cancellation
+            // rounding of a PF whose m-vector lies in the span of the others: clamp it
+            const double mAm = fmax(a[3], 0.0);
+            // m^H A^-1 e1 = m^H A^-1 e0 - m^H A^-1 mu4
+            const double2 mAe1 = make_double2(a[1] - a[7], a[2] - a[8]);
+            const double llr = (mAe1.x * mAe1.x + mAe1.y * mAe1.y) / (1.0 + mAm) - Q11 + Q00 - log1p(mAm);
+            D.llr_w[s * J + j] = llr;
+            const double zeta = D.zeta[s * J + j];
+            double pr;
+            if (zeta >= 1.0) pr = 1.0;
+            else if (zeta <= 0.0) pr = 0.0;
+            else {
+                const double u = log(zeta) - log1p(-zeta) + llr;
+                pr = (u >= 0) ? 1.0 / (1.0 + exp(-u)) : exp(u) / (1.0 + exp(u));
+            }
+            D.bel[BEL_PPR + s * J + j] = pr;
+        }
+    }
+    // V rows v_k = m_k L^{-H} by forward substitution, eight columns at a time (finished columns
+    // are read back, coalesced, from V64); consecutive threads take consecutive elements
+    double2* Vs = reinterpret_cast<double2*>(V64) + ((size_t)s * J + j) * SCA * Nz;
+    constexpr int CB = 8;
+    for (int k = tid; k < Nz; k += STAGE_THREADS) {
+        double2 r0 = E0[k];
+        for (int c0 = 0; c0 < K; c0 += CB) {
             double2 acc[CB];
             #pragma unroll
-            for (int q = 0; q < CB; ++q) acc[q] = make_double2(0.0, 0.0);
-            for (int t = 0; t < K; ++t) {
-                const double2 m = tab[((size_t)col(t) * J + j) * Nz + k];
-                const double2* ut = Ue + (size_t)t * K + c0;
+            for (int q = 0; q < CB; ++q)
+                acc[q] = c0 + q < K ? tab[((size_t)col(c0 + q) * J + j) * Nz + k] : make_double2(0.0, 0.0);
+            for (int t = 0; t < c0; ++t) {
+                const double2 v = Vs[(size_t)t * Nz + k];
                 #pragma unroll
                 for (int q = 0; q < CB; ++q) {
                     if (c0 + q < K) {
-                        const double2 u = zmul(m, ut[q]);
-                        acc[q].x += u.x; acc[q].y += u.y;
+                        const double2 u = zmulc(Lp[stage_row(K, c0 + q) + t], v);
+                        acc[q].x -= u.x; acc[q].y -= u.y;
                     }
                 }
             }
             #pragma unroll
-            for (int q = 0; q < CB; ++q)
-                if (c0 + q < K) Vs[(size_t)k * SC + c0 + q] = make_double2(acc[q].x * dinv[c0 + q], acc[q].y * dinv[c0 + q]);
+            for (int q = 0; q < CB; ++q) {
+                if (c0 + q < K) {
+                    const double d = il[c0 + q];
+                    acc[q].x *= d; acc[q].y *= d;
+                    Vs[(size_t)(c0 + q) * Nz + k] = acc[q];
+                    #pragma unroll
+                    for (int p = q + 1; p < CB; ++p) {
+                        if (c0 + p < K) {
+                            const double2 u = zmulc(Lp[stage_row(K, c0 + p) + c0 + q], acc[q]);
+                            acc[p].x -= u.x; acc[p].y -= u.y;
+                        }
+                    }
+                    const double2 y = make_double2(ye[c0 + q].x / eb, -ye[c0 + q].y / eb);
+                    const double2 u = zmul(acc[q], y);
+                    r0.x -= u.x; r0.y -= u.y;
+                }
+            }
         }
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) red[threadIdx.x] = wred[threadIdx.x * nw];
-    __shared__ double mm4_im;
-    if (threadIdx.x == 0) mm4_im = wred[8 * nw];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double pe0 = 0, pme_r = 0, pme_i = 0, pmm = 0, pue_r = 0, pue_i = 0, puu = 0, pmu_r = 0, pmu_i = 0;
-        for (int c = 0; c < K; ++c) {
-            const double2 a = ye[c], b = vm[c], u = v4[c];
-            pe0 += a.x * a.x + a.y * a.y;
-            const double2 t1 = zmulc(b, a); pme_r += t1.x; pme_i += t1.y;
-            pmm += b.x * b.x + b.y * b.y;
-            const double2 t2 = zmulc(u, a); pue_r += t2.x; pue_i += t2.y;
-            puu += u.x * u.x + u.y * u.y;
-            const double2 t3 = zmulc(b, u); pmu_r += t3.x; pmu_i += t3.y;
-        }
-        // e0^H A^-1 e0
-        const double Q00 = (red[0] - pe0 / eb) / eb;
-        // e1 = e0 - mu4
-        const double e1e1 = red[0] - 2.0 * red[4] + red[6];
-        const double pe1 = pe0 - 2.0 * pue_r + puu;
-        const double Q11 = (e1e1 - pe1 / eb) / eb;
-        // m^H A^-1 m >= 0 (A positive definite); a negative value is cancellation
-        // rounding of a PF whose m-vector lies in the span of the others: clamp it
-        const double mAm = fmax((red[3] - pmm / eb) / eb, 0.0);
-        // m^H A^-1 e1 = m^H A^-1 e0 - m^H A^-1 mu4
-        const double2 mAe0 = make_double2((red[1] - pme_r / eb) / eb, (red[2] - pme_i / eb) / eb);
-        const double2 mAu = make_double2((red[7] - pmu_r / eb) / eb, (mm4_im - pmu_i / eb) / eb);
-        const double2 mAe1 = make_double2(mAe0.x - mAu.x, mAe0.y - mAu.y);
-        const double llr = (mAe1.x * mAe1.x + mAe1.y * mAe1.y) / (1.0 + mAm) - Q11 + Q00 - log1p(mAm);
-        D.llr_w[s * J + j] = llr;
-        const double zeta = D.zeta[s * J + j];
-        double pr;
-        if (zeta >= 1.0) pr = 1.0;
-        else if (zeta <= 0.0) pr = 0.0;
-        else {
-            const double u = log(zeta) - log1p(-zeta) + llr;
-            pr = (u >= 0) ? 1.0 / (1.0 + exp(-u)) : exp(u) / (1.0 + exp(u));
-        }
-        D.bel[BEL_PPR + s * J + j] = pr;
-        // y~0 = V^H e0 / eb -> store; y0 = R^-1 y~0 (back substitution)
-        for (int c = 0; c < K; ++c) ye[c] = make_double2(ye[c].x / eb, ye[c].y / eb);
-    }
-    __syncthreads();
-    // r0 = e0 - V y~0 (rows), |r0|^2; store V, r0 as FP32
-    float2* kV = D.kV + ((size_t)s * J + j) * Nz * SC;
-    double r2 = 0.0;   // |r0|^2, summed in a fixed order (warps, then warp slots)
-    for (int k = threadIdx.x; k < Nz; k += blockDim.x) {
-        double2 e0 = E0[k];
-        for (int c = 0; c < K; ++c) {
-            const double2 v = Vs[(size_t)k * SC + c];
-            const double2 u = zmul(v, ye[c]);
-            e0.x -= u.x; e0.y -= u.y;
-            kV[(size_t)k * SC + c] = make_float2((float)v.x, (float)v.y);
-        }
-        for (int c = K; c < SC - 1; ++c) kV[(size_t)k * SC + c] = make_float2(0.f, 0.f);
-        const float2 r0h = make_float2((float)e0.x, (float)e0.y);
-        kV[(size_t)k * SC + SC - 1] = r0h;   // r0 in the last column, its low part apart
-        D.kr0l[((size_t)s * J + j) * Nz + k] = make_float2((float)(e0.x - (double)r0h.x), (float)(e0.y - (double)r0h.y));
-        r2 += e0.x * e0.x + e0.y * e0.y;
-    }
-    r2 = warp_sum_d(r2);
-    if (lane == 0) wred[wid] = r2;
-    __syncthreads();
-    if (threadIdx.x == 0) {   // the |y|^2 part enters the particle kernel as a difference
-        double v = 0.0;
-        for (int w = 0; w < nw; ++w) v += wred[w];
-        D.kJ0[s * J + j] = v / eb;
-    }
-    // the particle kernels take y~0 = V^H e0/eb and 1/lambda_c (padded with zeros) and form
-    // the amplitude terms sum_c (|y~0_c|^2 - |y~0_c - tau x_c/eb|^2)/lambda_c column by column
-    float2* ky = D.ky0 + ((size_t)s * J + j) * SC;
-    float2* kd = D.kdl + ((size_t)s * J + j) * SC;
-    for (int c = threadIdx.x; c < SC; c += blockDim.x) {
-        const double il = (c < K) ? dinv[c] * dinv[c] : 0.0;
-        ky[c] = (c < K) ? make_float2((float)ye[c].x, (float)ye[c].y) : make_float2(0.f, 0.f);
-        kd[c] = make_float2((float)il, 0.f);
+        Vs[(size_t)(SCA - 1) * Nz + k] = r0;
     }
 }
 
@@ -836,27 +551,29 @@ void launch_table(const DevGeom& G, const DevParams& Pm, const DevState& D, int 
     k_table_final<<<(tot + 255) / 256, 256, 0, st>>>(G, Pm, D, S, nsplit);
 }
 
-void launch_stage(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SC, const float* z,
-                  double* gram, double* nu_b, double* V64, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
-                  cudaEvent_t ev_join) {
+void launch_stage(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, const float* z,
+                  double* gram, double* nu_b, double* V64, cudaStream_t st) {
     const int npair = S * (S + 1) / 2 + S + 1;
     const int gx = min(64, (npair + 7) / 8);
     k_gram<<<dim3(gx, G.J), 256, 0, st>>>(G, Pm, D, S, z, gram, nu_b);
-    // J blocks of tridiagonalisation: on the side stream they fill the SMs the S x J basis
-    // blocks leave free
+    const size_t sm = stage_kappa_smem(S - 1, G.Nz);
+    smem_allow_max((const void*)k_stage_kappa);
+    k_stage_kappa<<<dim3(S, G.J), STAGE_THREADS, sm, st>>>(G, Pm, D, S, SCA, z, gram, V64);
+}
+
+void launch_nu_tridiag(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const double* gram,
+                       const double* nu_b, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
+    // on the side stream the J blocks run beside the MT likelihood (whose blocks are short; the
+    // persistent PF likelihood before it would wait for the SMs they hold)
     const bool fork = side && ev_fork && ev_join;
     if (fork) {
         cudaEventRecord(ev_fork, st);
         cudaStreamWaitEvent(side, ev_fork, 0);
     }
-    const size_t sm2 = ((size_t)S * S + 3 * (size_t)S) * sizeof(double2);
+    const size_t sm = ((size_t)S * S + 3 * (size_t)S) * sizeof(double2);
     smem_allow_max((const void*)k_nu_tridiag);
-    k_nu_tridiag<<<G.J, 128, sm2, fork ? side : st>>>(Pm, D, S, gram, nu_b);
+    k_nu_tridiag<<<G.J, 128, sm, fork ? side : st>>>(Pm, D, S, gram, nu_b);
     if (fork) cudaEventRecord(ev_join, side);
-    const int K = S - 1;
-    const size_t sm1 = stage_kappa_smem(K, G.Nz);
-    smem_allow_max((const void*)k_stage_kappa);
-    k_stage_kappa<<<dim3(S, G.J), STAGE_THREADS, sm1, st>>>(G, Pm, D, S, SC, z, gram, V64);
 }
 
 void smem_allow_max(const void* kernel) {
@@ -867,6 +584,17 @@ void smem_allow_max(const void* kernel) {
     cudaFuncGetAttributes(&a, kernel);
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - (int)a.sharedSizeBytes);
     done.push_back(kernel);
+}
+
+int sm_count() {
+    static int v = 0;
+    if (v == 0) {
+        int dev = 0, a = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&a, cudaDevAttrMultiProcessorCount, dev);
+        v = a > 0 ? a : 1;
+    }
+    return v;
 }
 
 int smem_optin() {
