@@ -655,8 +655,8 @@ void update_enqueue(bp_handle* h, const float* z_dev) {
     const int kappa_launches = launch_kappa(h->G, h->Pm, D, S, h->SCA, h->tiles.kappa_tc >= 0, h->V64, h->st);
     launch_nu_tridiag(h->G, h->Pm, D, S, h->gram, h->nu_b, h->st, h->st_side, h->ev_fork, h->ev_join);
     mark(h, 5);
-    const int iota_launches = launch_iota(h->G, h->Pm, D, S, z_dev, h->st) + 1;
-    launch_iota_repair(h->G, h->Pm, D, S, z_dev, h->st);
+    int iota_launches = launch_iota(h->G, h->Pm, D, S, z_dev, h->st);
+    iota_launches += launch_iota_repair(h->G, h->Pm, D, S, z_dev, h->st);
     mark(h, 6);
     if (h->st_side) cudaStreamWaitEvent(h->st, h->ev_join, 0);   // the tridiagonal forms
     launch_nu(h->G, h->Pm, D, S, h->st);

@@ -286,6 +286,13 @@ __device__ inline ff ff_mul(ff x, ff y) {
     fast_two_sum(p, e, r.hi, r.lo);
     return r;
 }
+__device__ inline ff ff_mulf(ff x, float b) {
+    const float p = __fmul_rn(x.hi, b);
+    const float e = fmaf(x.lo, b, fmaf(x.hi, b, -p));
+    ff r;
+    fast_two_sum(p, e, r.hi, r.lo);
+    return r;
+}
 __device__ inline ff ff_prod(float a, float b) {       // exact product of two floats
     const float p = __fmul_rn(a, b);
     return ff{p, fmaf(a, b, -p)};

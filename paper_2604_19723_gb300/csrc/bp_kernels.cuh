@@ -204,8 +204,34 @@ __device__ inline float4 cpair_mul(float2 ah, float2 al, float2 bh, float2 bl) {
     return make_float4(rh, ih, rl, il);
 }
 
+// a b of unit-modulus pairs in fixed point: hi a multiple of 2^-22 (adding 3 rounds each product
+// onto that grid, where the sums are exact), lo the remainders and the low-order cross terms
+// (|lo| < 2^-20)
+__device__ __forceinline__ void pair_dot2_fx(float a, float b, float c, float d, float al, float bl, float cl, float dl,
+                                             float& hi, float& lo) {   // (a + al)(b + bl) + (c + cl)(d + dl)
+    const float t = fmaf(a, b, 3.0f), t2 = fmaf(c, d, t);
+    const float p = fmaf(a, b, __fsub_rn(3.0f, t)), q = fmaf(c, d, __fsub_rn(t, t2));
+    hi = __fsub_rn(t2, 3.0f);
+    lo = __fadd_rn(fmaf(a, bl, fmaf(al, b, p)), fmaf(c, dl, fmaf(cl, d, q)));
+}
+__device__ __forceinline__ float4 pair_mul_fx(float4 a, float4 b) {
+    float4 u;
+    pair_dot2_fx(a.x, b.x, -a.y, b.y, a.z, b.z, -a.w, b.w, u.x, u.z);
+    pair_dot2_fx(a.x, b.y, a.y, b.x, a.z, b.w, a.w, b.z, u.y, u.w);
+    return u;
+}
+// |v|^2 - 1 of a unit-modulus pair, without the rounding of 1 (Sterbenz: the larger square is at
+// least 1/2)
+__device__ __forceinline__ float pair_unit_dev(float2 hi, float2 lo) {
+    const float p = __fmul_rn(hi.x, hi.x), e = fmaf(hi.x, hi.x, -p);
+    const float q = __fmul_rn(hi.y, hi.y), f = fmaf(hi.y, hi.y, -q);
+    const float big = fmaxf(p, q), small = fminf(p, q);
+    const float d = __fsub_rn(small, __fsub_rn(1.0f, big));
+    return d + ((e + f) + 2.0f * fmaf(hi.x, lo.x, hi.y * lo.y));
+}
+
 void launch_geom(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, cudaStream_t st);
-void launch_iota_repair(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st);
+int launch_iota_repair(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st);
 
 void launch_init(const DevGeom& G, const DevParams& Pm, const DevState& D, int S0, cudaStream_t st);
 int launch_predict(const DevGeom& G, const DevParams& Pm, const DevState& D, int S_old, int S_new, cudaStream_t st);
@@ -227,6 +253,11 @@ int launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S
                  const double* V64, cudaStream_t st);
 size_t kappa_operand_bytes(const DevGeom& G, int S_max);
 void launch_cis_table(const DevState& D, cudaStream_t st);
+// symmetric layouts (k_iota_sym.cu): whether they apply, and the float-float evaluation of every
+// particle (below IOTA_FF_ALL_S PFs) or of the queued ones
+bool iota_sym_ok(const DevGeom& G, int S);
+bool launch_iota_bulk_sym(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st);
+void launch_iota_ff(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, bool all, cudaStream_t st);
 // MT likelihood of every particle (returns its launches): the FP32 warp kernel with
 // ratio flags below IOTA_FF_ALL_S PFs, else k_iota_bulk and the selection of the particles
 // whose weights need the float-float evaluation; launch_iota_repair then evaluates the

@@ -13,13 +13,6 @@ namespace bp {
 __device__ inline ff ffx(float a) { return ff{a, 0.f}; }
 __device__ inline ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
 __device__ inline ff ff_twice(ff x) { return ff{2.0f * x.hi, 2.0f * x.lo}; }   // exact
-__device__ inline ff ff_mulf(ff x, float b) {                                    // x b
-    const float p = __fmul_rn(x.hi, b);
-    const float e = fmaf(x.lo, b, fmaf(x.hi, b, -p));
-    ff r;
-    fast_two_sum(p, e, r.hi, r.lo);
-    return r;
-}
 __device__ inline ff ff_sqrt(ff x) {   // one correction of the FP32 root: s + (x - s^2) / (2 s)
     const float s = sqrtf(x.hi);
     const ff r = ff_sub(x, ff_prod(s, s));

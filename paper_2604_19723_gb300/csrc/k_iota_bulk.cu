@@ -382,7 +382,8 @@ static void launch_bulk_nb(const DevGeom& G, const DevParams& Pm, const DevState
 int launch_iota_bulk(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st) {
     cudaMemsetAsync(D.flags, 0, sizeof(int), st);
     cudaMemsetAsync(D.iota_key, 0, sizeof(unsigned long long), st);
-    if (S <= 32) launch_bulk_nb<4>(G, Pm, D, S, z, st);
+    if (launch_iota_bulk_sym(G, Pm, D, S, z, st)) {}   // the real form of a symmetric layout
+    else if (S <= 32) launch_bulk_nb<4>(G, Pm, D, S, z, st);
     else launch_bulk_nb<8>(G, Pm, D, S, z, st);
     const int nb = std::min((Pm.P + 255) / 256, 4 * 152);
     k_iota_maxlow<<<nb, 256, 0, st>>>(Pm, D);

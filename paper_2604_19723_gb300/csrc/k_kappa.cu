@@ -123,21 +123,6 @@ __device__ __forceinline__ KxU kx_mul(const KxW& w, const KxU& a) {
     kx_dot2(w.x, a.yh, w.y, a.xh, w.xl, a.yl, w.yl, a.xl, u.yh, u.yl);
     return u;
 }
-// the same for one element
-__device__ __forceinline__ void kx_dot1(float a, float b, float c, float d, float al, float bl, float cl, float dl,
-                                        float& hi, float& lo) {
-    const float t = fmaf(a, b, 3.0f), t2 = fmaf(c, d, t);
-    const float p = fmaf(a, b, __fsub_rn(3.0f, t)), q = fmaf(c, d, __fsub_rn(t, t2));
-    hi = __fsub_rn(t2, 3.0f);
-    lo = __fadd_rn(fmaf(a, bl, fmaf(al, b, p)), fmaf(c, dl, fmaf(cl, d, q)));
-}
-__device__ __forceinline__ float4 kx_mul1(float4 a, float4 b) {
-    float4 u;
-    kx_dot1(a.x, b.x, -a.y, b.y, a.z, b.z, -a.w, b.w, u.x, u.z);
-    kx_dot1(a.x, b.y, a.y, b.x, a.z, b.w, a.w, b.z, u.y, u.w);
-    return u;
-}
-
 // the four digits of two elements: adding 1.5 x 2^23 units rounds to a multiple of the unit, the
 // remainder is exact; digit i of element e in w[i][e] as the BF16 pair (Re, Im)
 __device__ __forceinline__ void kx_digits(const KxU& u, uint32_t (&w)[4][2]) {
@@ -156,38 +141,20 @@ __device__ __forceinline__ void kx_digits(const KxU& u, uint32_t (&w)[4][2]) {
         if (i == 1) { rx = f2_add(rx, u.xl); ry = f2_add(ry, u.yl); }
     }
 }
-// |v|^2 - 1 of a unit-modulus pair, without the rounding of 1 (Sterbenz: the larger square is at
-// least 1/2)
-__device__ __forceinline__ float kx_unit_dev(float2 hi, float2 lo) {
-    const float p = __fmul_rn(hi.x, hi.x), e = fmaf(hi.x, hi.x, -p);
-    const float q = __fmul_rn(hi.y, hi.y), f = fmaf(hi.y, hi.y, -q);
-    const float big = fmaxf(p, q), small = fminf(p, q);
-    const float d = __fsub_rn(small, __fsub_rn(1.0f, big));
-    return d + ((e + f) + 2.0f * fmaf(hi.x, lo.x, hi.y * lo.y));
-}
-
-__device__ __forceinline__ ff ff_mulf1(ff x, float b) {
-    const float p = __fmul_rn(x.hi, b);
-    const float e = fmaf(x.lo, b, fmaf(x.hi, b, -p));
-    ff r;
-    fast_two_sum(p, e, r.hi, r.lo);
-    return r;
-}
-
 // Delta of one (p, s, j): consts (1/eta_bar, zeta as pairs), amplitude A, gamma, mu, alpha_u =
 // |u|^2 - |h|^2 and pr = u^H r0
 __device__ inline ff kx_delta(float4 kc, float A, float gm, float mr, float mi, ff alpha_u, cff pr) {
     const ff ieb{kc.x, kc.y}, zeta{kc.z, kc.w};
-    const ff Aeb = ff_mulf1(ieb, A);                      // A / eta_bar
-    const ff alpha = ff_mul(ff_mulf1(Aeb, A), alpha_u);
+    const ff Aeb = ff_mulf(ieb, A);                      // A / eta_bar
+    const ff alpha = ff_mul(ff_mulf(Aeb, A), alpha_u);
     const cff b{ff_mul(Aeb, pr.re), ff_mul(Aeb, pr.im)};
-    const cff a{ff_mulf1(zeta, mr), ff_mulf1(zeta, mi)};
+    const cff a{ff_mulf(zeta, mr), ff_mulf(zeta, mi)};
     const cff d{ff_add(b.re, ff_neg(ff_mul(alpha, a.re))), ff_add(b.im, ff_neg(ff_mul(alpha, a.im)))};
     ff out = ff_add(ff_mul(a.re, ff_add(b.re, d.re)), ff_mul(a.im, ff_add(b.im, d.im)));
     const float zf = kc.z;
     const float q = (gm + (mr * mr + mi * mi) * (1.0f - zf)) * zf;
     if (q > 0.f) {
-        const ff qa = ff_mulf1(alpha, q);
+        const ff qa = ff_mulf(alpha, q);
         const ff g = ff_div(ff{q, 0.f}, ff_add(ff{1.0f, 0.f}, qa));
         const ff d2 = ff_add(ff_mul(d.re, d.re), ff_mul(d.im, d.im));
         out = ff_add(out, ff_mul(g, d2));
@@ -576,7 +543,7 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
                 cis_pair(ctab, -h, -l, hi, lo);
                 return make_float4(hi.x, hi.y, lo.x, lo.y);
             };
-            auto unit_dev = [&](float4 a) { return kx_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w)); };
+            auto unit_dev = [&](float4 a) { return pair_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w)); };
             const float fdup = G.sym ? 2.0f : 1.0f;
             kx_bar();                             // every group is done with the previous unit's factors
             const int hy = G.sym ? (My + 1) / 2 : My, hz = G.sym ? (Mz + 1) / 2 : Mz;
@@ -637,7 +604,7 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
                         return true;
                     };
                     set_b(0);
-                    float4 w = kx_mul1(b, fy[yy * 128 + row]);
+                    float4 w = pair_mul_fx(b, fy[yy * 128 + row]);
                     KxW w2;
                     if (VEC > 1) w2 = kx_w(w, w);
                     #pragma unroll
@@ -645,16 +612,16 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
                         KxU a;
                         if (VEC > 1) {
                             if (VEC == 2 && q == 1 && step(2, 2) && k + 2 < Nh) {
-                                w = kx_mul1(b, fy[yy * 128 + row]);
+                                w = pair_mul_fx(b, fy[yy * 128 + row]);
                                 w2 = kx_w(w, w);
                             }
                             const int m2 = VEC == 4 ? mm + 2 * q : mm;
                             const float4 h = fz[m2 * 128 + row], l = fz[(m2 + 1) * 128 + row];
                             a = KxU{f2_pack(h.x, h.y), f2_pack(h.z, h.w), f2_pack(l.x, l.y), f2_pack(l.z, l.w)};
                         } else {
-                            if (q == 1 && step(2, 1) && k + 2 < Nh) w = kx_mul1(b, fy[yy * 128 + row]);
+                            if (q == 1 && step(2, 1) && k + 2 < Nh) w = pair_mul_fx(b, fy[yy * 128 + row]);
                             const float4 a0 = fz[mm * 128 + row], w0 = w;
-                            if (step(2 * q + 1, 1) && k + 2 * q + 1 < Nh) w = kx_mul1(b, fy[yy * 128 + row]);
+                            if (step(2 * q + 1, 1) && k + 2 * q + 1 < Nh) w = pair_mul_fx(b, fy[yy * 128 + row]);
                             const float4 a1 = fz[mm * 128 + row];
                             w2 = kx_w(w0, w);
                             a = KxU{f2_pack(a0.x, a1.x), f2_pack(a0.y, a1.y), f2_pack(a0.z, a1.z), f2_pack(a0.w, a1.w)};
@@ -735,7 +702,7 @@ __global__ void __launch_bounds__(KCC_T) k_kappa_cc(DevGeom G, DevParams Pm, Dev
         float dev = 0.f, sg = 0.f, sr = 0.f;
         for (int i = 0; i < nant; ++i) {
             const float4 a = kx_antenna(G, ctab, path, i);
-            dev = fmaf((float)(i < My ? G.Nf * Mz : G.Nf * My), kx_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w)), dev);
+            dev = fmaf((float)(i < My ? G.Nf * Mz : G.Nf * My), pair_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w)), dev);
             fa[i * KCC_T + tid] = a;
         }
         cff pr{ff{0.f, 0.f}, ff{0.f, 0.f}};
@@ -768,7 +735,7 @@ __global__ void __launch_bounds__(KCC_T) k_kappa_cc(DevGeom G, DevParams Pm, Dev
                         float2 hi, lo;
                         bprime_pair(G, ctab, path.dh, path.dl, path.h0, path.l0, f, hi, lo);
                         b = make_float4(hi.x, hi.y, lo.x, lo.y);
-                        if (c0 == 0 && ym == 0) dev = fmaf((float)Nm, kx_unit_dev(hi, lo), dev);
+                        if (c0 == 0 && ym == 0) dev = fmaf((float)Nm, pair_unit_dev(hi, lo), dev);
                     }
                     if (m == 0 || e == 0) w = kx_pair_mul(b, fa[y * KCC_T + tid]);
                     const float4 u = kx_pair_mul(w, fa[(My + m) * KCC_T + tid]);
@@ -794,7 +761,7 @@ __global__ void __launch_bounds__(KCC_T) k_kappa_cc(DevGeom G, DevParams Pm, Dev
                     cff h;
             two_sum(ar[q], lr[q], h.re.hi, h.re.lo);
             two_sum(ai[q], li[q], h.im.hi, h.im.lo);
-            h = cff{ff_mulf1(h.re, sc), ff_mulf1(h.im, sc)};
+            h = cff{ff_mulf(h.re, sc), ff_mulf(h.im, sc)};
                 if (c == SW - 1) { pr = h; continue; }
                 const float v[2] = {h.re.hi, h.im.hi}, vl[2] = {h.re.lo, h.im.lo};
                 #pragma unroll

@@ -690,6 +690,10 @@ constexpr int IOTA_FF_ALL_S = 24;
 
 int launch_iota(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st) {
     if (S >= IOTA_FF_ALL_S) return launch_iota_bulk(G, Pm, D, S, z, st);
+    if (iota_sym_ok(G, S)) {   // float-float for every particle; nothing is left to repair
+        launch_iota_ff(G, Pm, D, S, z, true, st);
+        return 1;
+    }
     const int nfac = G.Nf + G.My + G.Mz;
     const size_t per_warp = iota32_warp_f2(S, nfac, G.Nf) * sizeof(float2);
     int wpb = 8;
@@ -701,7 +705,12 @@ int launch_iota(const DevGeom& G, const DevParams& Pm, const DevState& D, int S,
     return 1;
 }
 
-void launch_iota_repair(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st) {
+int launch_iota_repair(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st) {
+    if (iota_sym_ok(G, S)) {
+        if (S < IOTA_FF_ALL_S) return 0;
+        launch_iota_ff(G, Pm, D, S, z, false, st);
+        return 1;
+    }
     const int nfac = G.Nf + G.My + G.Mz;
     const size_t smem = iota_blk_smem(S, nfac, G.Nf, G.Nz);
     constexpr int NCG = IOTA_BLK_NCG;
@@ -711,6 +720,7 @@ void launch_iota_repair(const DevGeom& G, const DevParams& Pm, const DevState& D
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int wave = IOTA_BLK_PER_SM * std::max(sms, 1);
     k_iota_blk<NCG><<<wave, 32 * NCG, smem, st>>>(G, Pm, D, S, z, 0);
+    return 1;
 }
 
 void launch_nu(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, cudaStream_t st) {
