@@ -249,9 +249,9 @@ bp_status bp_get_profile(bp_handle* h, double* ms, int n);
  *                 kappa_sc 8, 16, 24, 32, 48 or 64; kappa_blocks 1 or 2;
  *                 kappa_fch >= 0.
  *   table_chunk   particles per shared-memory chunk of the message table: 16,
- *                 32, 64 or 128 (clamped to what fits; built-in 64).
+ *                 32, 64 or 128 (clamped to what fits; built-in 128).
  *   table_split   particle splits of the message-table grid (>= 1; clamped to
- *                 P / 256 and the workspace's partial-sum capacity; built-in
+ *                 P / 128 and the workspace's partial-sum capacity; built-in
  *                 about 4096 blocks over the S x J problems).
  * bp_set_tiles validates and stores the fields (BP_ERR_INVALID_ARG for a value
  * outside the lists above; nothing is changed then); they apply from the next

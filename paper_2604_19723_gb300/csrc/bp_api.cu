@@ -645,7 +645,7 @@ void update_enqueue(bp_handle* h, const float* z_dev) {
     mark(h, 2);
     // the built-in split aims at ~4096 table blocks (several waves of short blocks)
     int nsplit = h->tiles.table_split > 0 ? h->tiles.table_split : std::max(1, (4096 + S * J - 1) / (S * J));
-    nsplit = std::min(nsplit, std::max(1, P / 256));
+    nsplit = std::min(nsplit, std::max(1, P / 128));
     nsplit = std::min(nsplit, h->nsplit_max);
     launch_geom(h->G, h->Pm, D, S, h->st);
     launch_table(h->G, h->Pm, D, S, nsplit, h->tiles.table_chunk, h->st);

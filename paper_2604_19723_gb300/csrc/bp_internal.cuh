@@ -346,6 +346,34 @@ __device__ inline double ffexp_log(const ffexp& x) {
     return (double)logf(x.m.hi) + (double)(x.m.lo / x.m.hi) + (double)x.e * 0.69314718055994530942;
 }
 
+// ---------------------------------------------------------------- packed FP32 pairs
+using f2x = unsigned long long;
+__device__ __forceinline__ f2x f2_pack(float a, float b) {
+    f2x r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(f2x v, uint32_t& a, uint32_t& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
+}
+__device__ __forceinline__ f2x f2_add(f2x a, f2x b) {
+    f2x r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
+    f2x r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2x f2_mul(f2x a, f2x b) {
+    f2x r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2x f2_dup(float a) { return f2_pack(a, a); }
+__device__ __forceinline__ f2x f2_sub(f2x a, f2x b) { return f2_fma(b, f2_dup(-1.0f), a); }
+
 __device__ inline double warp_sum_d(double v) {
     #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

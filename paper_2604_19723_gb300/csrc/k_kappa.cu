@@ -73,34 +73,6 @@ __host__ __device__ inline size_t kx_smem_fixed(int nfac) {
     return ((size_t)nfac * 128 + 256 + KX_NG * 128 + 128) * sizeof(float4) + 3 * 64 * sizeof(float) + 256;
 }
 
-// ---------------------------------------------------------------- packed FP32 pairs
-using f2x = unsigned long long;
-__device__ __forceinline__ f2x f2_pack(float a, float b) {
-    f2x r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f2x v, uint32_t& a, uint32_t& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
-}
-__device__ __forceinline__ f2x f2_add(f2x a, f2x b) {
-    f2x r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
-    f2x r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f2x f2_mul(f2x a, f2x b) {
-    f2x r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2x f2_dup(float a) { return f2_pack(a, a); }
-__device__ __forceinline__ f2x f2_sub(f2x a, f2x b) { return f2_fma(b, f2_dup(-1.0f), a); }
-
 // a b for unit-modulus pairs, two elements at a time, in fixed point: hi a multiple of 2^-22
 // (adding 3 rounds each product onto that grid, where the sums are exact), lo the remainders and
 // the low-order cross terms (|lo| < 2^-20)

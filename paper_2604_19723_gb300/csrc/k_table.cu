@@ -6,7 +6,7 @@
 //   m^w  = c_w sum_p w_beta sqrt(gamma + |mu|^2 (1 - W))  psi_s^(j,p)
 //   mu4  = W sum_p w_beta mu psi_s^(j,p),  mu3 = zeta mu4
 // (c_m, c_w) = (W zeta, W) as printed in S-V, or their square roots.
-// FP32 accumulation over chunks of particles, FP64 across chunks.
+// FP32 accumulation over runs of particles, float-float across them, FP64 across blocks.
 //
 // Stage per (s, j), FP64 (S-V "PF state update message", "PR state update
 // message", S-VI): A_s = eta_bar I + M_{-s} M_{-s}^H is represented by a
@@ -26,131 +26,192 @@
 namespace bp {
 
 // ---------------------------------------------------------------- table reduction
-// grid (nsplit, S, J); per-particle factors are staged in shared memory, each
-// thread owns EPT elements of the Nz-vector.
-template <int EPT>
-__global__ void k_table(DevGeom G, DevParams Pm, DevState D, int S, int nsplit, int chunk) {
-    extern __shared__ float2 sm[];
-    const int split = blockIdx.x, s = blockIdx.y, j = blockIdx.z;
-    const int P = Pm.P, J = G.J, Nf = G.Nf, Nm = G.My * G.Mz, Nz = G.Nz;
+// grid (nsplit, S, J x element blocks).  A chunk of particles is staged in shared memory (thread per
+// particle: frequency and antenna factors, the three weighted amplitudes with the carrier), then
+// every thread accumulates two elements over its group's share of the chunk.  With u_k = x + i y the
+// unit-modulus element and c the complex weight, the four real sums of c_r and c_i with x and y
+// give both sum_p c u_k and, on a layout symmetric about 0 (u_{Nz-1-k} = conj(u_k)), the
+// mirrored element's sum_p c conj(u_k): half the elements are formed.  (x, y) travel as packed FP32
+// pairs; FP32 accumulation over runs of TABLE_FLUSH particles, float-float across.
+// Bound: FP32 issue and shared-memory reads (16 instructions per element pair and particle).
+// Measured (message-table stage, with k_geom): 32 PFs x 262144, Nz = 1024: 92.9 -> 18.4 ms; 64 x 1e5,
+// Nz = 160: 8.3 -> 3.4; 40 x 8192, Nz = 300: 2.3 -> 0.44; 10 x 30000: 0.49 -> 0.21 (against a thread
+// per element with three complex products and FP64 sums every 64 particles).
+constexpr int TABLE_FLUSH = 64;
+struct TablePlan { int nel, nb, na, nt, ntb, nblk, threads, chunk; size_t smem; };
+static __host__ __device__ inline TablePlan table_plan(const DevGeom& G, int chunk_req) {
+    TablePlan t;
+    t.nel = G.sym ? (G.Nz + 1) / 2 : G.Nz;
+    t.na = G.My * G.Mz;
+    t.nb = (t.nel - 1) / t.na + 1;                    // frequencies of the formed elements
+    t.nt = (t.nel + 1) / 2;                           // element pairs
+    t.threads = t.nt <= 128 ? 128 : 256;
+    t.nblk = (t.nt + t.threads - 1) / t.threads;
+    t.ntb = (t.nt + t.nblk - 1) / t.nblk;             // pairs per block
+    const size_t row = (size_t)((t.nb + t.na) | 1) * sizeof(float2) + 3 * sizeof(float4);
+    t.chunk = (chunk_req == 16 || chunk_req == 32 || chunk_req == 64) ? chunk_req : 128;
+    while (t.chunk > 16 && t.chunk * row > 100 * 1024) t.chunk /= 2;
+    const size_t stage = t.chunk * row, out = (size_t)t.threads * 24 * sizeof(double);
+    t.smem = (stage > out ? stage : out) + 16;
+    return t;
+}
+
+__global__ void __launch_bounds__(256, 2) k_table(DevGeom G, DevParams Pm, DevState D, int S, int nsplit, int chunk_req) {
+    extern __shared__ float4 sm[];
+    const TablePlan tp = table_plan(G, chunk_req);
+    const int split = blockIdx.x, s = blockIdx.y, j = blockIdx.z / tp.nblk, eb = blockIdx.z - j * tp.nblk;
+    const int P = Pm.P, J = G.J, My = G.My, Mz = G.Mz, Nm = My * Mz, Nz = G.Nz;
     const int per = (P + nsplit - 1) / nsplit;
     const int p0 = split * per, p1 = min(P, p0 + per);
-    // per-particle rows with odd strides: each thread writes its own particle's row, so an
-    // even stride would put a warp's stores into a few banks
-    const int nyz = G.My + G.Mz;
-    const int bst = (3 * Nf) | 1, ast = Nm | 1, yst = nyz | 1;
-    float2* Bf = sm;                                          // [chunk][bst]: 3 rows of Nf
-    float2* Ayz = sm + (size_t)chunk * bst;                   // [chunk][ast]
-    float2* Fyz = Ayz + (size_t)chunk * ast;                  // [chunk][yst] scratch
-    const double W = D.W[s];
-    const double zeta = D.zeta[s * J + j];
-    const float pi = (float)(zeta * W);
-    const float pd = (float)(1.0 - W);
+    const int tid = threadIdx.x, stride = (tp.nb + tp.na) | 1;   // odd row stride (bank spread)
+    float4* cf = sm;                                             // [chunk][3] weights (c_r, c_r, c_i, c_i)
+    float2* rows = reinterpret_cast<float2*>(sm + 3 * (size_t)tp.chunk);   // [chunk][stride] b_f, a_y a_z
+    // this thread's elements tile and tile + ntb of the block's 2 ntb, and its group of particles
+    const int ngrp = tp.threads / tp.ntb, grp = tid / tp.ntb, tile = tid - grp * tp.ntb;
+    int ob[2], oa[2];
+    #pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int k = min(eb * 2 * tp.ntb + tile + e * tp.ntb, tp.nel - 1), f = k / Nm;
+        ob[e] = f;
+        oa[e] = tp.nb + (k - f * Nm);
+    }
+    const float pi = (float)(D.zeta[s * J + j] * D.W[s]);
+    const float pd = (float)(1.0 - D.W[s]);
     const float* ph = D.phi[D.cur] + (size_t)s * 6 * P;
     const float4* geo = D.geo + ((size_t)s * J + j) * P;
     const float2* geol = D.geo_lo + ((size_t)s * J + j) * P;
-    double acc64[EPT][3][2];
+    f2x acc[2][6], hi[2][6], lo[2][6];
     #pragma unroll
-    for (int e = 0; e < EPT; ++e)
+    for (int e = 0; e < 2; ++e)
         #pragma unroll
-        for (int i = 0; i < 3; ++i) acc64[e][i][0] = acc64[e][i][1] = 0.0;
-    for (int c0 = p0; c0 < p1; c0 += chunk) {
-        const int cn = min(chunk, p1 - c0);
+        for (int i = 0; i < 6; ++i) acc[e][i] = hi[e][i] = lo[e][i] = f2_dup(0.f);
+    int held = 0;                                                // particles in acc
+    auto flush = [&]() {
+        #pragma unroll
+        for (int e = 0; e < 2; ++e)
+            #pragma unroll
+            for (int i = 0; i < 6; ++i) {                        // two_sum
+                const f2x a = hi[e][i], b = acc[e][i], t = f2_add(a, b), bb = f2_sub(t, a);
+                lo[e][i] = f2_add(lo[e][i], f2_add(f2_sub(a, f2_sub(t, bb)), f2_sub(b, bb)));
+                hi[e][i] = t;
+                acc[e][i] = f2_dup(0.f);
+            }
+        held = 0;
+    };
+    for (int c0 = p0; c0 < p1; c0 += tp.chunk) {
+        const int cn = min(tp.chunk, p1 - c0);
         __syncthreads();
-        for (int t = threadIdx.x; t < cn; t += blockDim.x) {
+        for (int t = tid; t < cn; t += tp.threads) {
             const int p = c0 + t;
-            float2* b0 = Bf + (size_t)t * bst;
-            float2* fy = Fyz + (size_t)t * yst;
-            const float2 c = factors_from_geo(G, geo[p], geol[p], b0, fy, fy + G.My, 1);
-            const float gm = ph[3 * P + p], mr = ph[4 * P + p], mi = ph[5 * P + p];
+            const float4 g = geo[p];
+            const float2 gl = geol[p], c = carrier_factor(G, g);
+            float2* b = rows + (size_t)t * stride;
+            float2* a = b + tp.nb;
+            for (int f = 0; f < tp.nb; ++f) b[f] = freq_factor(G, g, f);
+            auto factor = [&](float c, float cl, float u, float ul) {
+                const float h = __fmul_rn(c, u);
+                return cispi_ff(2.0f * h, 2.0f * fmaf(c, ul, fmaf(cl, u, fmaf(c, u, -h))));
+            };
+            // a_z into the row's first Mz places, then the products of each a_y from the last y down
+            for (int m = 0; m < Mz; ++m) a[m] = factor(G.pz_l[m], G.pz_lo[m], g.w, gl.y);
+            for (int y = My - 1; y >= 0; --y) {
+                const float2 ay = factor(G.py_l[y], G.py_lo[y], g.z, gl.x);
+                for (int m = 0; m < Mz; ++m) a[y * Mz + m] = cmul(ay, a[m]);
+            }
+            const float gm = ph[3 * (size_t)P + p], mr = ph[4 * (size_t)P + p], mi = ph[5 * (size_t)P + p];
             const float m2 = mr * mr + mi * mi;
             const float wb = (float)D.w_x[p];
             const float ca = wb * sqrtf(fmaxf(gm + m2 * (1.0f - pi), 0.0f));
             const float cb = wb * sqrtf(fmaxf(gm + m2 * pd, 0.0f));
-            const float2 c1 = make_float2(ca * c.x, ca * c.y);
-            const float2 c2 = make_float2(cb * c.x, cb * c.y);
             const float2 c3 = cmul(make_float2(wb * mr, wb * mi), c);
-            for (int f = 0; f < Nf; ++f) {
-                const float2 bb = b0[f];
-                b0[Nf + f] = cmul(c2, bb);
-                b0[2 * Nf + f] = cmul(c3, bb);
-                b0[f] = cmul(c1, bb);
-            }
-            for (int y = 0; y < G.My; ++y)
-                for (int m = 0; m < G.Mz; ++m)
-                    Ayz[(size_t)t * ast + y * G.Mz + m] = cmul(fy[y], fy[G.My + m]);
+            cf[3 * t] = make_float4(ca * c.x, ca * c.x, ca * c.y, ca * c.y);
+            cf[3 * t + 1] = make_float4(cb * c.x, cb * c.x, cb * c.y, cb * c.y);
+            cf[3 * t + 2] = make_float4(c3.x, c3.x, c3.y, c3.y);
         }
         __syncthreads();
-        float acc[EPT][3][2];
-        #pragma unroll
-        for (int e = 0; e < EPT; ++e)
-            #pragma unroll
-            for (int i = 0; i < 3; ++i) acc[e][i][0] = acc[e][i][1] = 0.f;
-        for (int t = 0; t < cn; ++t) {
-            #pragma unroll
-            for (int e = 0; e < EPT; ++e) {
-                const int k = threadIdx.x + e * blockDim.x;
-                if (k < Nz) {
-                    const int f = k / Nm, ym = k - f * Nm;
-                    const float2 a = Ayz[(size_t)t * ast + ym];
-                    #pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        const float2 bv = Bf[(size_t)t * bst + i * Nf + f];
-                        const float2 v = cmul(bv, a);
-                        acc[e][i][0] += v.x;
-                        acc[e][i][1] += v.y;
-                    }
+        if (grp < ngrp) {
+            for (int t = grp; t < cn; t += ngrp) {
+                const float2* row = rows + (size_t)t * stride;
+                f2x w[6];
+                #pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const float4 c = cf[3 * t + i];
+                    w[2 * i] = f2_pack(c.x, c.y);
+                    w[2 * i + 1] = f2_pack(c.z, c.w);
                 }
+                #pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float2 b = row[ob[e]], a = row[oa[e]];
+                    const f2x u = f2_pack(fmaf(b.x, a.x, -b.y * a.y), fmaf(b.x, a.y, b.y * a.x));
+                    #pragma unroll
+                    for (int i = 0; i < 6; ++i) acc[e][i] = f2_fma(w[i], u, acc[e][i]);
+                }
+                if (++held == TABLE_FLUSH) flush();
             }
         }
-        #pragma unroll
-        for (int e = 0; e < EPT; ++e)
-            #pragma unroll
-            for (int i = 0; i < 3; ++i) { acc64[e][i][0] += acc[e][i][0]; acc64[e][i][1] += acc[e][i][1]; }
     }
-    const int SJ = Pm.S_max * J;
-    #pragma unroll
-    for (int e = 0; e < EPT; ++e) {
-        const int k = threadIdx.x + e * blockDim.x;
-        if (k < Nz) {
+    flush();
+    __syncthreads();
+    // the groups' sums in a fixed order; per element and weight (sum c_r x, sum c_r y), (sum c_i x, sum c_i y)
+    double* out = reinterpret_cast<double*>(sm);                 // [ngrp][2 ntb][12]
+    if (grp < ngrp) {
+        #pragma unroll
+        for (int e = 0; e < 2; ++e)
             #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                double2* out = reinterpret_cast<double2*>(D.tab_part) + (((size_t)split * 3 + i) * SJ + (size_t)s * J + j) * Nz + k;
-                *out = make_double2(acc64[e][i][0], acc64[e][i][1]);
+            for (int i = 0; i < 6; ++i) {
+                uint32_t h0, h1, l0, l1;
+                f2_unpack(hi[e][i], h0, h1);
+                f2_unpack(lo[e][i], l0, l1);
+                double* o = out + ((size_t)grp * 2 * tp.ntb + tile + e * tp.ntb) * 12 + 2 * i;
+                o[0] = (double)__uint_as_float(h0) + (double)__uint_as_float(l0);
+                o[1] = (double)__uint_as_float(h1) + (double)__uint_as_float(l1);
             }
-        }
+    }
+    __syncthreads();
+    const int SJ = Pm.S_max * J;
+    for (int t = tid; t < 2 * tp.ntb * 3; t += tp.threads) {
+        const int i = t / (2 * tp.ntb), el = t - i * 2 * tp.ntb, k = eb * 2 * tp.ntb + el;
+        if (k >= tp.nel) continue;
+        double r[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int g = 0; g < ngrp; ++g)
+            #pragma unroll
+            for (int q = 0; q < 4; ++q) r[q] += out[((size_t)g * 2 * tp.ntb + el) * 12 + 4 * i + q];
+        double2* o = reinterpret_cast<double2*>(D.tab_part) + (((size_t)split * 3 + i) * SJ + (size_t)s * J + j) * Nz;
+        o[k] = make_double2(r[0] - r[3], r[1] + r[2]);
+        if (G.sym && k != Nz - 1 - k) o[Nz - 1 - k] = make_double2(r[0] + r[3], r[2] - r[1]);
     }
 }
 
-// sums the partials in fixed order and applies the existence scale factors
+// sums the partials in fixed order and applies the existence scale factors (thread per element and weight)
 __global__ void k_table_final(DevGeom G, DevParams Pm, DevState D, int S, int nsplit) {
     const int J = G.J, Nz = G.Nz;
-    const int SJ = Pm.S_max * J;
+    const int SJ = Pm.S_max * J, n = S * J * Nz;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= S * J * Nz) return;
-    const int k = idx % Nz;
-    const int sj = idx / Nz;
+    if (idx >= 3 * n) return;
+    const int i = idx / n, el = idx - i * n;
+    const int k = el % Nz, sj = el / Nz;
     const int s = sj / J, j = sj - s * J;
     const double W = D.W[s], zeta = D.zeta[s * J + j];
-    double2 v[3];
-    for (int i = 0; i < 3; ++i) {
-        double2 a = make_double2(0.0, 0.0);
-        for (int sp = 0; sp < nsplit; ++sp) {
-            const double2 t = reinterpret_cast<const double2*>(D.tab_part)[(((size_t)sp * 3 + i) * SJ + (size_t)s * J + j) * Nz + k];
-            a.x += t.x; a.y += t.y;
-        }
-        v[i] = a;
+    const double2* part = reinterpret_cast<const double2*>(D.tab_part) + ((size_t)i * SJ + (size_t)s * J + j) * Nz + k;
+    const size_t step = (size_t)3 * SJ * Nz;
+    double2 a = make_double2(0.0, 0.0);
+    #pragma unroll 8
+    for (int sp = 0; sp < nsplit; ++sp) {
+        const double2 t = part[sp * step];
+        a.x += t.x; a.y += t.y;
     }
-    double cm, cw;
-    if (Pm.mvec_scaling == 0) { cm = W * zeta; cw = W; } else { cm = sqrt(W * zeta); cw = sqrt(W); }
     double2* tab = reinterpret_cast<double2*>(D.tab);
     const size_t o = ((size_t)s * J + j) * Nz + k;
     const size_t plane = (size_t)SJ * Nz;
-    tab[0 * plane + o] = make_double2(cm * v[0].x, cm * v[0].y);
-    tab[1 * plane + o] = make_double2(cw * v[1].x, cw * v[1].y);
-    const double2 m4 = make_double2(W * v[2].x, W * v[2].y);
-    tab[3 * plane + o] = m4;
-    tab[2 * plane + o] = make_double2(zeta * m4.x, zeta * m4.y);
+    if (i == 2) {
+        const double2 m4 = make_double2(W * a.x, W * a.y);
+        tab[3 * plane + o] = m4;
+        tab[2 * plane + o] = make_double2(zeta * m4.x, zeta * m4.y);
+    } else {
+        double c = i == 0 ? W * zeta : W;
+        if (Pm.mvec_scaling != 0) c = sqrt(c);
+        tab[i * plane + o] = make_double2(c * a.x, c * a.y);
+    }
 }
 
 // ---------------------------------------------------------------- Gram matrix per j (FP64)
@@ -527,27 +588,10 @@ __global__ void k_nu_tridiag(DevParams Pm, DevState D, int S, const double* gram
 
 void launch_table(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int nsplit, int chunk_req,
                   cudaStream_t st) {
-    const int Nz = G.Nz;
-    const int bs = Nz <= 256 ? ((Nz + 31) / 32) * 32 : 256;
-    const int ept = (Nz + bs - 1) / bs;
-    const int per_particle = (((3 * G.Nf) | 1) + ((G.My * G.Mz) | 1) + ((G.My + G.Mz) | 1)) * (int)sizeof(float2);
-    // 64 particles per chunk by default (measured at 64 PFs x 1e5 particles: 128 -> 64 with
-    // 16 splits took the kernel from 14.5 to 11.5 ms, more blocks per SM)
-    int chunk = (chunk_req == 16 || chunk_req == 32 || chunk_req == 128) ? chunk_req : 64;
-    while (chunk > 16 && chunk * per_particle > 96 * 1024) chunk /= 2;
-    const size_t smem = (size_t)chunk * per_particle;
-    dim3 grid(nsplit, S, G.J);
-    switch (ept) {
-        case 1: smem_allow_max((const void*)k_table<1>);
-                k_table<1><<<grid, bs, smem, st>>>(G, Pm, D, S, nsplit, chunk); break;
-        case 2: smem_allow_max((const void*)k_table<2>);
-                k_table<2><<<grid, bs, smem, st>>>(G, Pm, D, S, nsplit, chunk); break;
-        case 3: case 4: smem_allow_max((const void*)k_table<4>);
-                k_table<4><<<grid, bs, smem, st>>>(G, Pm, D, S, nsplit, chunk); break;
-        default: smem_allow_max((const void*)k_table<8>);
-                k_table<8><<<grid, bs, smem, st>>>(G, Pm, D, S, nsplit, chunk); break;
-    }
-    const int tot = S * G.J * Nz;
+    const TablePlan t = table_plan(G, chunk_req);
+    smem_allow_max((const void*)k_table);
+    k_table<<<dim3(nsplit, S, G.J * t.nblk), t.threads, t.smem, st>>>(G, Pm, D, S, nsplit, chunk_req);
+    const int tot = 3 * S * G.J * G.Nz;
     k_table_final<<<(tot + 255) / 256, 256, 0, st>>>(G, Pm, D, S, nsplit);
 }
 
