@@ -450,6 +450,7 @@ WsPlan ws_plan(const DevGeom& G, const DevParams& Pm, int SCA, int nsplit_max) {
     w.tab_part = take((size_t)nsplit_max * 3 * SM * J * Nz * 2 * sizeof(double));
     w.kB = take(kappa_operand_bytes(G, S_max));
     w.red_part = take(nbel * 64 * RED_W * 2 * sizeof(double));
+    w.tsum = take(nbel * 256 * sizeof(double));
     w.gram = take(J * SM * SM * 2 * sizeof(double));
     w.V64 = take(SM * J * Nz * (size_t)SCA * 2 * sizeof(double));
     w.cdf = take(nbel * PP * sizeof(double));
@@ -478,6 +479,7 @@ void ws_bind(bp_handle* h, char* base) {
     D.tab_part = reinterpret_cast<double*>(base + w.tab_part);
     D.kB = reinterpret_cast<unsigned char*>(base + w.kB);
     D.red_part = reinterpret_cast<double*>(base + w.red_part);
+    D.tsum = reinterpret_cast<double*>(base + w.tsum);
     h->gram = reinterpret_cast<double*>(base + w.gram);
     h->V64 = reinterpret_cast<double*>(base + w.V64);
     h->cdf = reinterpret_cast<double*>(base + w.cdf);
@@ -531,6 +533,7 @@ bp_status handle_create(const bp_geometry* geom, const bp_params* prm, int P, in
     Pm.N_g = prm->N_g;
     Pm.key0 = (uint32_t)(seed & 0xFFFFFFFFu); Pm.key1 = (uint32_t)(seed >> 32);
     Pm.P = P; Pm.S_max = S_max;
+    for (int d = 1; d <= 6; ++d) Pm.h_opt[d] = std::pow(4.0 / (P * (d + 2.0)), 1.0 / (d + 4.0));
     h->P = P; h->S_max = S_max; h->J = geom->J; h->Nz = h->G.Nz;
     h->SCA = sc_bucket(S_max);
     h->nsplit_max = 32;
@@ -668,7 +671,7 @@ void update_enqueue(bp_handle* h, const float* z_dev) {
         cudaEventRecord(h->ev[BP_PROF_STAGES], h->st);
         for (int i = 1; i < BP_PROF_STAGES; ++i) h->ev_valid[i] = true;
     }
-    h->launches += 1 + 3 + 3 + kappa_launches + iota_launches + 1 + 5 + 3;
+    h->launches += 1 + 3 + 3 + kappa_launches + iota_launches + 1 + 5 + 2;
     h->D.cur = 1 - h->D.cur;
     h->S_upd = S;
     h->phase = 0;

@@ -24,10 +24,15 @@ __device__ inline BeliefView belief_of(int b, const DevParams& Pm, int J) {
     return BeliefView{2, b - 1 - Pm.S_max, 1};
 }
 
-__device__ inline double belief_logw(const DevState& D, const BeliefView& v, int P, int p) {
-    if (v.kind == 0) return log(D.w_x[p]) + D.lw_x[p];
-    if (v.kind == 1) return log(D.w_alpha[(size_t)v.index * P + p]) + D.lw_y[(size_t)v.index * P + p];
-    return log(D.w_eta[(size_t)v.index * P + p]) + D.lw_eta[(size_t)v.index * P + p];
+// prediction weights, log-likelihoods and (in turn) log weights / normalised weights of a belief
+__device__ inline const double* belief_w(const DevState& D, const BeliefView& v, int P) {
+    return v.kind == 0 ? D.w_x : (v.kind == 1 ? D.w_alpha : D.w_eta) + (size_t)v.index * P;
+}
+__device__ inline const double* belief_l(const DevState& D, const BeliefView& v, int P) {
+    return v.kind == 0 ? D.lw_x : (v.kind == 1 ? D.lw_y : D.lw_eta) + (size_t)v.index * P;
+}
+__device__ inline double* belief_wn(const DevState& D, const BeliefView& v, int P) {
+    return v.kind == 0 ? D.wn_x : (v.kind == 1 ? D.wn_y : D.wn_eta) + (size_t)v.index * P;
 }
 
 __device__ inline void belief_state(const DevState& D, const BeliefView& v, int P, int p, double* out) {
@@ -45,14 +50,28 @@ __device__ inline void belief_state(const DevState& D, const BeliefView& v, int 
 // active beliefs: b in {0} U {1..S} U {1+S_max .. S_max+J}
 __device__ inline int active_belief(int a, int S, int S_max) { return a <= S ? a : 1 + S_max + (a - S - 1); }
 
+// log weights of every particle (kept in the buffer of the normalised weights) and the block
+// maxima.  FP64 logarithms set the time here (GB300 issues FP64 at 1/64 of the FP32 rate): after
+// resampling a belief's weights are all equal, so the logarithm of a block's first weight serves
+// every particle that has the same one.
 __global__ void k_norm_max(DevGeom G, DevParams Pm, DevState D, int S, int NB) {
     const int b = active_belief(blockIdx.y, S, Pm.S_max);
     const BeliefView v = belief_of(b, Pm, G.J);
     const int P = Pm.P;
     const int per = (P + NB - 1) / NB;
     const int p0 = blockIdx.x * per, p1 = min(P, p0 + per);
+    const double *w = belief_w(D, v, P), *l = belief_l(D, v, P);
+    double* o = belief_wn(D, v, P);
     double m = -INFINITY;
-    for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) m = fmax(m, belief_logw(D, v, P, p));
+    if (p0 < p1) {
+        const double w0 = w[p0], lw0 = log(w0);
+        for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
+            const double wp = w[p];
+            const double t = (wp == w0 ? lw0 : log(wp)) + l[p];
+            o[p] = t;
+            m = fmax(m, t);
+        }
+    }
     __shared__ double red[32];
     m = warp_max_d(m);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
@@ -64,6 +83,9 @@ __global__ void k_norm_max(DevGeom G, DevParams Pm, DevState D, int S, int NB) {
     }
 }
 
+// Weights more than NORM_SKIP nats below the largest are left out of the sums: P e^-60 < 2^-53 for
+// every P this library takes, so they are below the rounding of a sum that is at least 1.
+constexpr double NORM_SKIP = 60.0;
 __global__ void k_norm_sum(DevGeom G, DevParams Pm, DevState D, int S, int NB, double* part) {
     const int b = active_belief(blockIdx.y, S, Pm.S_max);
     const BeliefView v = belief_of(b, Pm, G.J);
@@ -74,27 +96,32 @@ __global__ void k_norm_sum(DevGeom G, DevParams Pm, DevState D, int S, int NB, d
     belief_state(D, v, P, 0, ref);
     const int per = (P + NB - 1) / NB;
     const int p0 = blockIdx.x * per, p1 = min(P, p0 + per);
+    const double* lw = belief_wn(D, v, P);
     double acc[RED_W];
     for (int i = 0; i < RED_W; ++i) acc[i] = 0.0;
     const int d = v.dims;
     if (M > -INFINITY) {
         for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const double w = exp(belief_logw(D, v, P, p) - M);
+            const double t = lw[p] - M;
+            if (t < -NORM_SKIP) continue;
+            const double w = exp(t);
             double xs[6];
             belief_state(D, v, P, p, xs);
             for (int k = 0; k < d; ++k) xs[k] -= ref[k];
             acc[0] += w;
             for (int k = 0; k < d; ++k) acc[1 + k] += w * xs[k];
-            int t = 7;
+            int q = 7;
             for (int r = 0; r < d; ++r)
-                for (int c = r; c < d; ++c) acc[t++] += w * xs[r] * xs[c];
+                for (int c = r; c < d; ++c) acc[q++] += w * xs[r] * xs[c];
             acc[28] += w * w;
         }
     }
     __shared__ double red[32][RED_W + 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // sums of one scalar state (eta) and of idle warps are zero beyond the first entries
+    const bool any = __any_sync(0xffffffffu, acc[0] != 0.0);
     for (int i = 0; i < RED_W; ++i) {
-        const double s = warp_sum_d(acc[i]);
+        const double s = any ? warp_sum_d(acc[i]) : 0.0;
         if (lane == 0) red[wid][i] = s;
     }
     __syncthreads();
@@ -116,19 +143,24 @@ __device__ inline void pf_mask(const DevParams& Pm, int s, bool* a) {
     if (Pm.zero_mean) { a[4] = a[5] = false; }
 }
 
-// one thread per active belief: combine partials, estimates, jitter factor
+// one warp per active belief: combine the partials (lane i the i-th sum, in block order), then lane 0
+// forms estimates and the jitter factor
 __global__ void k_norm_final(DevGeom G, DevParams Pm, DevState D, int S, int NB, const double* part) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= 1 + S + G.J) return;
-    const int b = active_belief(a, S, Pm.S_max);
+    const int b = active_belief(blockIdx.x, S, Pm.S_max);
     const BeliefView v = belief_of(b, Pm, G.J);
-    const int P = Pm.P;
+    const int P = Pm.P, lane = threadIdx.x;
+    __shared__ double acc[RED_W];
     double M = -INFINITY;
-    for (int i = 0; i < NB; ++i) M = fmax(M, D.red_part[((size_t)b * NB + i) * RED_W]);
-    double acc[RED_W];
-    for (int i = 0; i < RED_W; ++i) acc[i] = 0.0;
-    for (int i = 0; i < NB; ++i)
-        for (int k = 0; k < RED_W; ++k) acc[k] += part[((size_t)b * NB + i) * RED_W + k];
+    for (int i = lane; i < NB; i += 32) M = fmax(M, D.red_part[((size_t)b * NB + i) * RED_W]);
+    M = warp_max_d(M);
+    if (lane < RED_W) {
+        double t = 0.0;
+        #pragma unroll 4
+        for (int i = 0; i < NB; ++i) t += part[((size_t)b * NB + i) * RED_W + lane];
+        acc[lane] = t;
+    }
+    __syncwarp();
+    if (lane != 0) return;
     double ref[6];
     belief_state(D, v, P, 0, ref);
     double* rec = D.bel + bel_rec(Pm.S_max, G.J, b);
@@ -180,28 +212,19 @@ __global__ void k_norm_final(DevGeom G, DevParams Pm, DevState D, int S, int NB,
             L[i][k] = s / L[k][k];
         }
     }
-    const double h = (dact > 0) ? pow(4.0 / (P * (dact + 2.0)), 1.0 / (dact + 4.0)) : 0.0;
+    const double h = Pm.h_opt[dact];
     float* Lf = D.Lchol + (size_t)b * 36;
     for (int r = 0; r < 6; ++r) for (int c = 0; c < 6; ++c) Lf[r * 6 + c] = (float)((Pm.regularize ? h : 0.0) * L[r][c]);
     rec[10] = dact;
 }
 
-// estimates, declaration, pruning map; single thread
-__global__ void k_estimate(DevGeom G, DevParams Pm, DevState D, int S) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int n = D.step[0];
-    const int J = G.J, SM = Pm.S_max;
+// estimates, declaration, pruning map: a thread per PF, the survivors numbered by ballot
+__global__ void __launch_bounds__(S_CAP_MAX) k_estimate(DevGeom G, DevParams Pm, DevState D, int S) {
+    const int J = G.J, SM = Pm.S_max, s = threadIdx.x, lane = s & 31;
     const EstLayout E{SM, J};
     double* est = D.est;
-    est[E.n()] = n;
-    est[E.S()] = S;
-    est[E.repaired()] = D.flags[0];
-    const double* r0 = D.bel + bel_rec(SM, J, 0);
-    for (int k = 0; k < 6; ++k) est[E.x_hat() + k] = r0[4 + k];
-    est[E.ess()] = 1.0 / r0[3];
-    for (int j = 0; j < J; ++j) est[E.eta_hat() + j] = (D.bel + bel_rec(SM, J, 1 + SM + j))[4];
-    int keep = 0;
-    for (int s = 0; s < S; ++s) {
+    bool kept = false;
+    if (s < S) {
         const double* rs = D.bel + bel_rec(SM, J, 1 + s);
         const double ps = D.p_s[s];
         est[E.p_s() + s] = ps;
@@ -215,11 +238,27 @@ __global__ void k_estimate(DevGeom G, DevParams Pm, DevState D, int S) {
         const double pany = 1.0 - prod;
         est[E.p_any() + s] = pany;
         est[E.declared() + s] = (ps > Pm.T_dec) ? 1.0 : 0.0;
-        const bool kept = (s == 0) || Pm.T_pru <= 0.0 || !(ps < Pm.T_pru || pany < Pm.T_pru);
-        if (kept) D.ctrl[4 + keep++] = s;
+        kept = (s == 0) || Pm.T_pru <= 0.0 || !(ps < Pm.T_pru || pany < Pm.T_pru);
     }
-    D.ctrl[1] = keep;
-    est[E.S_next()] = keep;
+    const unsigned bal = __ballot_sync(0xffffffffu, kept);
+    __shared__ int first;
+    if (s == 0) first = __popc(bal);
+    __syncthreads();
+    const int at = __popc(bal & ((1u << lane) - 1u)) + (s >= 32 ? first : 0);
+    if (kept) D.ctrl[4 + at] = s;
+    if (s == S_CAP_MAX - 1) {
+        const int keep = at + (kept ? 1 : 0);
+        D.ctrl[1] = keep;
+        est[E.S_next()] = keep;
+    }
+    if (s < J) est[E.eta_hat() + s] = (D.bel + bel_rec(SM, J, 1 + SM + s))[4];
+    if (s != 0) return;
+    const double* r0 = D.bel + bel_rec(SM, J, 0);
+    est[E.n()] = D.step[0];
+    est[E.S()] = S;
+    est[E.repaired()] = D.flags[0];
+    for (int k = 0; k < 6; ++k) est[E.x_hat() + k] = r0[4 + k];
+    est[E.ess()] = 1.0 / r0[3];
     est[E.skipped()] = D.ctrl[2];
     int status = 0;
     if (!(r0[2] > -INFINITY)) status = BP_ERR_NUMERIC;
@@ -230,163 +269,169 @@ __global__ void k_estimate(DevGeom G, DevParams Pm, DevState D, int S) {
     D.ctrl[3] = status;
 }
 
-// normalised weights of every active belief (before resampling)
-__global__ void k_norm_weights(DevGeom G, DevParams Pm, DevState D, int S) {
+// particles per tile of the cumulative weights (at most CDF_TILES tiles) and the tile count
+constexpr int CDF_SUB = 2048, CDF_TILES = 256;
+__host__ __device__ inline int cdf_tile(int P) { return CDF_SUB * ((P + CDF_SUB * CDF_TILES - 1) / (CDF_SUB * CDF_TILES)); }
+__host__ __device__ inline int cdf_tiles(int P) { return (P + cdf_tile(P) - 1) / cdf_tile(P); }
+// block sum in a fixed order, in every thread
+__device__ inline double block_sum_256(double v, double* red) {
+    v = warp_sum_d(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0.0;
+    #pragma unroll
+    for (int w = 0; w < 8; ++w) v += red[w];
+    return v;
+}
+
+// normalised weights of every active belief (before resampling), in place of the log weights, and
+// their tile sums
+__global__ void __launch_bounds__(256) k_norm_weights(DevGeom G, DevParams Pm, DevState D, int S, double* tsum) {
     const int P = Pm.P;
     const int b = active_belief(blockIdx.y, S, Pm.S_max);
     const BeliefView v = belief_of(b, Pm, G.J);
     const double logC = (D.bel + bel_rec(Pm.S_max, G.J, b))[2];
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        const double w = (logC > -INFINITY) ? exp(belief_logw(D, v, P, p) - logC) : 0.0;
-        if (v.kind == 0) D.wn_x[p] = w;
-        else if (v.kind == 1) D.wn_y[(size_t)v.index * P + p] = w;
-        else D.wn_eta[(size_t)v.index * P + p] = w;
+    double* w = belief_wn(D, v, P);
+    const int tile = cdf_tile(P), p0 = blockIdx.x * tile, p1 = min(P, p0 + tile);
+    double acc = 0.0;
+    for (int p = p0 + threadIdx.x; p < p1; p += 256) {
+        const double t = w[p] - logC;
+        // e^t is 0 in FP64 below -745.2
+        const double e = (logC > -INFINITY) ? (t < -746.0 ? 0.0 : exp(t)) : 0.0;
+        w[p] = e;
+        acc += e;
     }
+    __shared__ double red[8];
+    acc = block_sum_256(acc, red);
+    if (threadIdx.x == 0) tsum[(size_t)b * CDF_TILES + blockIdx.x] = acc;
 }
 
 int launch_normalize(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, cudaStream_t st) {
     const int P = Pm.P;
-    int NB = (P + 4095) / 4096;
+    int NB = (P + 2047) / 2048;
     if (NB > 64) NB = 64;
     const int nb = 1 + S + G.J;
     double* part = D.red_part + (size_t)bel_count(Pm.S_max, G.J) * 64 * RED_W;
     k_norm_max<<<dim3(NB, nb), 256, 0, st>>>(G, Pm, D, S, NB);
     k_norm_sum<<<dim3(NB, nb), 256, 0, st>>>(G, Pm, D, S, NB, part);
-    k_norm_final<<<(nb + 63) / 64, 64, 0, st>>>(G, Pm, D, S, NB, part);
-    k_estimate<<<1, 32, 0, st>>>(G, Pm, D, S);
-    k_norm_weights<<<dim3((P + 255) / 256 < 256 ? (P + 255) / 256 : 256, nb), 256, 0, st>>>(G, Pm, D, S);
+    k_norm_final<<<nb, 32, 0, st>>>(G, Pm, D, S, NB, part);
+    k_estimate<<<1, S_CAP_MAX, 0, st>>>(G, Pm, D, S);
+    k_norm_weights<<<dim3(cdf_tiles(P), nb), 256, 0, st>>>(G, Pm, D, S, D.tsum);
     return 5;
 }
 
 // ---------------------------------------------------------------- systematic resampling
-// one block per kept belief; CDF in FP64 (chunked per thread, block exclusive scan)
-__global__ void __launch_bounds__(1024) k_resample(DevGeom G, DevParams Pm, DevState D, int S, double* cdf_all) {
-    const int P = Pm.P, SM = Pm.S_max, J = G.J;
-    const int n = D.step[0];
-    const int S_next = D.ctrl[1];
-    const int a = blockIdx.x;   // 0: MT, 1..S_next: kept PF, then eta
-    int b, kind, index;
-    if (a == 0) { b = 0; kind = 0; index = 0; }
-    else if (a <= S_next) {
-        index = D.ctrl[4 + a - 1]; b = 1 + index; kind = 1;
-        if (!bp_in_range(index, SM, D.kerr)) return;
+// belief of resampling slot a: the MT, the kept PFs in their new order, then eta; false if idle
+struct ResampleSlot { int b, kind, index; };
+__device__ inline bool resample_slot(const DevParams& Pm, const DevState& D, int J, int a, ResampleSlot& r) {
+    const int S_next = D.ctrl[1], SM = Pm.S_max;
+    if (a == 0) { r = ResampleSlot{0, 0, 0}; return true; }
+    if (a <= S_next) {
+        const int s = D.ctrl[4 + a - 1];
+        if (!bp_in_range(s, SM, D.kerr)) return false;
+        r = ResampleSlot{1 + s, 1, s};
+        return true;
     }
-    else if (a <= S_next + J) { index = a - S_next - 1; b = 1 + SM + index; kind = 2; }
-    else return;
-    const double* w = (kind == 0) ? D.wn_x : (kind == 1) ? D.wn_y + (size_t)index * P : D.wn_eta + (size_t)index * P;
-    double* cdf = cdf_all + (size_t)a * P;
-    const int per = (P + blockDim.x - 1) / blockDim.x;
-    const int p0 = threadIdx.x * per, p1 = min(P, p0 + per);
-    double loc = 0.0;
-    for (int p = p0; p < p1; ++p) loc += w[p];
-    __shared__ double scan[1024];
-    __shared__ double total;
-    scan[threadIdx.x] = loc;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        const double t = (threadIdx.x >= (unsigned)off) ? scan[threadIdx.x - off] : 0.0;
+    if (a <= S_next + J) { const int j = a - S_next - 1; r = ResampleSlot{1 + SM + j, 2, j}; return true; }
+    return false;
+}
+
+// cumulative weights (FP64, not normalised) of every kept belief: block (tile, slot) scans its tile
+// from the sum of the tiles before it
+__global__ void __launch_bounds__(256) k_cdf(DevGeom G, DevParams Pm, DevState D, const double* tsum, double* cdf_all) {
+    const int P = Pm.P, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    ResampleSlot r;
+    if (!resample_slot(Pm, D, G.J, blockIdx.y, r)) return;
+    const double* w = belief_wn(D, BeliefView{r.kind, r.index, 0}, P);
+    double* cdf = cdf_all + (size_t)blockIdx.y * P;
+    const double* ts = tsum + (size_t)r.b * CDF_TILES;
+    __shared__ double red[8];
+    double run = block_sum_256(tid < (int)blockIdx.x ? ts[tid] : 0.0, red);
+    const int tile = cdf_tile(P), p0 = blockIdx.x * tile, p1 = min(P, p0 + tile);
+    for (int q0 = p0; q0 < p1; q0 += CDF_SUB) {
+        const int q = q0 + 8 * tid;
+        double x[8], loc = 0.0;
+        #pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            loc += (q + i < p1) ? w[q + i] : 0.0;
+            x[i] = loc;
+        }
+        double inc = loc;
+        #pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
         __syncthreads();
-        scan[threadIdx.x] += t;
+        if (lane == 31) red[wid] = inc;
         __syncthreads();
+        double off = run, tot = 0.0;
+        #pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            if (v < wid) off += red[v];
+            tot += red[v];
+        }
+        off += inc - loc;
+        #pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (q + i < p1) cdf[q + i] = off + x[i];
+        run += tot;
     }
-    if (threadIdx.x == blockDim.x - 1) total = scan[threadIdx.x];
-    __syncthreads();
-    double run = scan[threadIdx.x] - loc;
-    for (int p = p0; p < p1; ++p) { run += w[p]; cdf[p] = run; }
-    __syncthreads();
-    const double tot = total;
-    for (int p = p0; p < p1; ++p) cdf[p] = (tot > 0) ? cdf[p] / tot : (double)(p + 1) / P;
-    __syncthreads();
-    if (threadIdx.x == 0) cdf[P - 1] = 1.0;
-    __syncthreads();
-    const U4 r = draw(Pm, (uint32_t)((kind << 16) | index), n, RNG_RESAMPLE, 0, 0);
-    const double U = u32d(r.x);
-    int* idx = D.idx + (size_t)b * P;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const double u = (U + (double)i) / (double)P;
-        int lo = 0, hi = P - 1;            // first k with cdf[k] >= u
+}
+
+// resampling index, gather and jitter into the other buffer, weights of the new belief and (PFs) the PR
+// table: a thread per (output particle, slot).  Particle i takes the first k with CDF_k >= (U + i)/P.
+__global__ void __launch_bounds__(256) k_resample(DevGeom G, DevParams Pm, DevState D, const double* cdf_all) {
+    const int P = Pm.P, J = G.J, i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = D.step[0], nxt = 1 - D.cur, a = blockIdx.y;
+    ResampleSlot r;
+    if (!resample_slot(Pm, D, J, a, r)) return;
+    if (r.kind == 1 && blockIdx.x == 0 && threadIdx.x < J)
+        D.p_pr[(a - 1) * J + threadIdx.x] = D.bel[BEL_PPR + r.index * J + threadIdx.x];
+    if (i >= P) return;
+    const double* cdf = cdf_all + (size_t)a * P;
+    const double tot = cdf[P - 1];
+    const double U = u32d(draw(Pm, (uint32_t)((r.kind << 16) | r.index), n, RNG_RESAMPLE, 0, 0).x);
+    int src = i;                               // equal weights where the belief has none
+    if (tot > 0.0) {
+        const double u = (U + (double)i) / (double)P * tot;
+        int lo = 0, hi = P - 1;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
             if (cdf[mid] >= u) hi = mid; else lo = mid + 1;
         }
-        idx[i] = lo;
+        src = lo;
     }
-}
-
-// gather + jitter into the other buffer; thread per output slot
-__global__ void k_gather(DevGeom G, DevParams Pm, DevState D) {
-    const int P = Pm.P, SM = Pm.S_max, J = G.J;
-    const int n = D.step[0];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int S_next = D.ctrl[1];
-    const int nxt = 1 - D.cur;
-    if (i < P) {
-        {   // MT
-            int src = D.idx[i];
-            if (!bp_in_range(src, P, D.kerr)) src = i;
-            const float* L = D.Lchol;
-            float e[6];
-            normals8(Pm, i, n, RNG_JITTER_MT, 0, 6, e);
-            for (int r = 0; r < 6; ++r) {
-                float jit = 0.f;
-                for (int c = 0; c <= r; ++c) jit += L[r * 6 + c] * e[c];
-                D.x[nxt][(size_t)r * P + i] = D.x[D.cur][(size_t)r * P + src] + jit;
-            }
-            D.w_x[i] = 1.0 / P;
-        }
-        for (int t = 0; t < S_next; ++t) {
-            const int s = D.ctrl[4 + t];
-            if (!bp_in_range(s, SM, D.kerr)) continue;
-            int src = D.idx[(size_t)(1 + s) * P + i];
-            if (!bp_in_range(src, P, D.kerr)) src = i;
-            const float* L = D.Lchol + (size_t)(1 + s) * 36;
-            float e[6];
-            normals8(Pm, i, n, RNG_JITTER_PF, s, 6, e);
-            const float* ph = D.phi[D.cur] + (size_t)s * 6 * P;
-            float* po = D.phi[nxt] + (size_t)t * 6 * P;
-            for (int r = 0; r < 6; ++r) {
-                float jit = 0.f;
-                for (int c = 0; c <= r; ++c) jit += L[r * 6 + c] * e[c];
-                float v = ph[(size_t)r * P + src] + jit;
-                if (r == 3) v = fabsf(v);
-                po[(size_t)r * P + i] = v;
-            }
-        }
-        for (int j = 0; j < J; ++j) {
-            int src = D.idx[(size_t)(1 + SM + j) * P + i];
-            if (!bp_in_range(src, P, D.kerr)) src = i;
-            const float L = D.Lchol[(size_t)(1 + SM + j) * 36];
-            float e[1];
-            normals8(Pm, i, n, RNG_JITTER_ETA, j, 1, e);
-            D.eta[nxt][(size_t)j * P + i] = fabsf(D.eta[D.cur][(size_t)j * P + src] + L * e[0]);
-            D.w_eta[(size_t)j * P + i] = 1.0 / P;
-        }
+    D.idx[(size_t)r.b * P + i] = src;
+    if (!bp_in_range(src, P, D.kerr)) src = i;
+    const float* L = D.Lchol + (size_t)r.b * 36;
+    if (r.kind == 2) {
+        float e[1];
+        normals8(Pm, i, n, RNG_JITTER_ETA, r.index, 1, e);
+        D.eta[nxt][(size_t)r.index * P + i] = fabsf(D.eta[D.cur][(size_t)r.index * P + src] + L[0] * e[0]);
+        D.w_eta[(size_t)r.index * P + i] = 1.0 / P;
+        return;
     }
-}
-
-// weights and PR tables of the compacted PF set; runs after k_gather (reads p_s, writes w_y)
-__global__ void k_compact(DevGeom G, DevParams Pm, DevState D) {
-    const int P = Pm.P, J = G.J;
-    const int S_next = D.ctrl[1];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    __shared__ double ps_new[S_CAP_MAX];
-    if (threadIdx.x < S_next && bp_in_range(D.ctrl[4 + threadIdx.x], Pm.S_max, D.kerr))
-        ps_new[threadIdx.x] = D.p_s[D.ctrl[4 + threadIdx.x]];
-    __syncthreads();
-    if (i < P)
-        for (int t = 0; t < S_next; ++t) D.w_y[(size_t)t * P + i] = ps_new[t] / P;
-    if (blockIdx.x == 0)
-        for (int u = threadIdx.x; u < S_next * J; u += blockDim.x) {
-            const int t = u / J, j = u - t * J;
-            if (bp_in_range(D.ctrl[4 + t], Pm.S_max, D.kerr)) D.p_pr[t * J + j] = D.bel[BEL_PPR + D.ctrl[4 + t] * J + j];
-        }
+    float e[6];
+    normals8(Pm, i, n, r.kind == 0 ? RNG_JITTER_MT : RNG_JITTER_PF, r.index, 6, e);
+    const float* in = r.kind == 0 ? D.x[D.cur] : D.phi[D.cur] + (size_t)r.index * 6 * P;
+    float* out = r.kind == 0 ? D.x[nxt] : D.phi[nxt] + (size_t)(a - 1) * 6 * P;
+    for (int k = 0; k < 6; ++k) {
+        float jit = 0.f;
+        for (int c = 0; c <= k; ++c) jit += L[k * 6 + c] * e[c];
+        float v = in[(size_t)k * P + src] + jit;
+        if (r.kind == 1 && k == 3) v = fabsf(v);
+        out[(size_t)k * P + i] = v;
+    }
+    if (r.kind == 0) D.w_x[i] = 1.0 / P;
+    else D.w_y[(size_t)(a - 1) * P + i] = D.p_s[r.index] / P;
 }
 
 void launch_resample(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, double* cdf, cudaStream_t st) {
     const int nb = 1 + S + G.J;
-    k_resample<<<nb, 1024, 0, st>>>(G, Pm, D, S, cdf);
-    k_gather<<<(Pm.P + 255) / 256, 256, 0, st>>>(G, Pm, D);
-    k_compact<<<(Pm.P + 255) / 256, 256, 0, st>>>(G, Pm, D);
+    k_cdf<<<dim3(cdf_tiles(Pm.P), nb), 256, 0, st>>>(G, Pm, D, D.tsum, cdf);
+    k_resample<<<dim3((Pm.P + 255) / 256, nb), 256, 0, st>>>(G, Pm, D, cdf);
 }
 
 }  // namespace bp

@@ -71,23 +71,25 @@ __global__ void k_step_advance(DevState D) {
     if (threadIdx.x == 0 && blockIdx.x == 0) D.step[0] += 1;
 }
 
-__global__ void k_predict(DevGeom G, DevParams Pm, DevState D, int S_old, int S_new) {
+// blockIdx.y: 0 the MT (and zeta of every (s, j)), 1 .. J the noise variances, then the PFs; a thread per
+// particle.  Bound: the FP64 pipe (the Gamma draws); with one thread per particle for all its
+// beliefs a few thousand particles left most of the GPU idle (0.30 ms at 21 PFs x 5000).
+__global__ void __launch_bounds__(256) k_predict(DevGeom G, DevParams Pm, DevState D, int S_old, int S_new) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = D.step[0];
     const int P = Pm.P;
     const int J = G.J;
-    if (p < S_new * J) {   // zeta of every (s, j)
-        const int s = p / J;
-        const double pr = D.p_pr[p];
-        D.zeta[p] = (s < S_old) ? Pm.pS_pr * pr + Pm.pR_pr * (1.0 - pr) : Pm.pB_pr;
-    }
-    if (p >= P) return;
-    float* x = D.x[D.cur];
-    float* phi = D.phi[D.cur];
-    float* eta = D.eta[D.cur];
-    const float T = (float)Pm.T;
-    // MT: x = Phi_a x + Gamma w, w ~ N(0, sigma_v^2 I)
-    {
+    const int task = blockIdx.y;
+    if (task == 0) {
+        if (p < S_new * J) {
+            const int s = p / J;
+            const double pr = D.p_pr[p];
+            D.zeta[p] = (s < S_old) ? Pm.pS_pr * pr + Pm.pR_pr * (1.0 - pr) : Pm.pB_pr;
+        }
+        if (p >= P) return;
+        // MT: x = Phi_a x + Gamma w, w ~ N(0, sigma_v^2 I)
+        float* x = D.x[D.cur];
+        const float T = (float)Pm.T;
         float g[3];
         normals8(Pm, p, n, RNG_MT_PREDICT, 0, 3, g);
         const float sv = (float)Pm.sigma_v;
@@ -98,17 +100,21 @@ __global__ void k_predict(DevGeom G, DevParams Pm, DevState D, int S_old, int S_
             x[k * P + p] = pk + T * vk + 0.5f * T * T * w[k];
             x[(3 + k) * P + p] = vk + T * w[k];
         }
+        return;
     }
-    // noise variances
-    for (int j = 0; j < J; ++j) {
+    if (p >= P) return;
+    if (task <= J) {   // noise variances
+        const int j = task - 1;
+        float* eta = D.eta[D.cur];
         const double e = (double)eta[j * P + p];
         eta[j * P + p] = (float)gamma_draw(Pm, p, n, RNG_ETA_PREDICT, j, Pm.c_eta, e / Pm.c_eta);
+        return;
     }
-    // legacy PFs
-    for (int s = 0; s < S_old; ++s) {
+    const int s = task - 1 - J;
+    float* ph = D.phi[D.cur] + (size_t)s * 6 * P;
+    if (s < S_old) {   // legacy PFs
         float g[5];
         normals8(Pm, p, n, RNG_PF_GAUSS, s, 5, g);
-        float* ph = phi + (size_t)s * 6 * P;
         if (s > 0) {
             const float ss = (float)Pm.sigma_sfv;
             ph[0 * P + p] += ss * g[0];
@@ -125,30 +131,28 @@ __global__ void k_predict(DevGeom G, DevParams Pm, DevState D, int S_old, int S_
             ph[5 * P + p] += sd * g[4];
         }
         D.w_alpha[(size_t)s * P + p] = Pm.pS * D.w_y[(size_t)s * P + p];
+        return;
     }
     // births: partition q of the birth box (slabs along x)
-    for (int s = S_old; s < S_new; ++s) {
-        const int q = s - S_old;
-        const U4 a = draw(Pm, p, n, RNG_BIRTH, s, 0);
-        const U4 b = draw(Pm, p, n, RNG_BIRTH, s, 1);
-        const double u[6] = {u24d(a.x), u24d(a.y), u24d(a.z), u24d(a.w), u24d(b.x), u24d(b.y)};
-        double lo[3], hi[3];
-        for (int k = 0; k < 3; ++k) { lo[k] = 2.0 * Pm.p_min[k]; hi[k] = 2.0 * Pm.p_max[k]; }
-        const double width = (hi[0] - lo[0]) / Pm.Q;
-        lo[0] = 2.0 * Pm.p_min[0] + q * width;
-        hi[0] = lo[0] + width;
-        float* ph = phi + (size_t)s * 6 * P;
-        for (int k = 0; k < 3; ++k) ph[k * P + p] = (float)(lo[k] + (hi[k] - lo[k]) * u[k]);
-        ph[3 * P + p] = (float)(Pm.gamma_max * u[3]);
-        if (Pm.zero_mean) {
-            ph[4 * P + p] = 0.f; ph[5 * P + p] = 0.f;
-        } else {
-            const double r = Pm.mu_max * sqrt(u[4]);
-            ph[4 * P + p] = (float)(r * cospi(2.0 * u[5]));
-            ph[5 * P + p] = (float)(r * sinpi(2.0 * u[5]));
-        }
-        D.w_alpha[(size_t)s * P + p] = Pm.pB / P;
+    const int q = s - S_old;
+    const U4 a = draw(Pm, p, n, RNG_BIRTH, s, 0);
+    const U4 b = draw(Pm, p, n, RNG_BIRTH, s, 1);
+    const double u[6] = {u24d(a.x), u24d(a.y), u24d(a.z), u24d(a.w), u24d(b.x), u24d(b.y)};
+    double lo[3], hi[3];
+    for (int k = 0; k < 3; ++k) { lo[k] = 2.0 * Pm.p_min[k]; hi[k] = 2.0 * Pm.p_max[k]; }
+    const double width = (hi[0] - lo[0]) / Pm.Q;
+    lo[0] = 2.0 * Pm.p_min[0] + q * width;
+    hi[0] = lo[0] + width;
+    for (int k = 0; k < 3; ++k) ph[k * P + p] = (float)(lo[k] + (hi[k] - lo[k]) * u[k]);
+    ph[3 * P + p] = (float)(Pm.gamma_max * u[3]);
+    if (Pm.zero_mean) {
+        ph[4 * P + p] = 0.f; ph[5 * P + p] = 0.f;
+    } else {
+        const double r = Pm.mu_max * sqrt(u[4]);
+        ph[4 * P + p] = (float)(r * cospi(2.0 * u[5]));
+        ph[5 * P + p] = (float)(r * sinpi(2.0 * u[5]));
     }
+    D.w_alpha[(size_t)s * P + p] = Pm.pB / P;
 }
 
 // Per-row FP64 sums: rows 0..S-1 give W_s = sum_p w_alpha, rows S..S+J-1 give
@@ -160,11 +164,13 @@ __global__ void k_row_sums(DevParams Pm, DevState D, int S, int J) {
     double acc = 0.0;
     if (row < S) {
         const double* w = D.w_alpha + (size_t)row * P;
+        #pragma unroll 8
         for (int p = threadIdx.x; p < P; p += blockDim.x) acc += w[p];
     } else {
         const int j = row - S;
         const double* w = D.w_eta + (size_t)j * P;
         const float* e = D.eta[D.cur] + (size_t)j * P;
+        #pragma unroll 8
         for (int p = threadIdx.x; p < P; p += blockDim.x) acc += w[p] * (double)e[p];
     }
     __shared__ double red[32];
@@ -188,7 +194,7 @@ void launch_init(const DevGeom& G, const DevParams& Pm, const DevState& D, int S
 int launch_predict(const DevGeom& G, const DevParams& Pm, const DevState& D, int S_old, int S_new, cudaStream_t st) {
     const int nthr = max(Pm.P, S_new * G.J);
     k_step_advance<<<1, 32, 0, st>>>(D);
-    k_predict<<<(nthr + 255) / 256, 256, 0, st>>>(G, Pm, D, S_old, S_new);
+    k_predict<<<dim3((nthr + 255) / 256, 1 + G.J + S_new), 256, 0, st>>>(G, Pm, D, S_old, S_new);
     return 2;
 }
 
