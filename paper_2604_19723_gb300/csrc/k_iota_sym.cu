@@ -417,247 +417,331 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
 // ---------------------------------------------------------------- FP32 evaluation with an error bound
 // Every particle from 24 PFs on (the quantities, the bound and the selection are those of
 // k_iota_bulk.cu): log det A and rhs^H A^-1 rhs from one LDL^T elimination of the real A, e = z -
-// sum_s w0_s u_s element by element, |e|^2 - rhs^H A^-1 rhs.  One warp per (particle, PA); the lower
-// triangle lives in registers, lane (tr, tc) of 8 x 4 owning the entries (8 ia + tr, 4 ib + tc);
-// column k travels through shared memory (published by its owners one step ahead, one warp
-// barrier per step).
-// Bound: FP32 issue (about half of it the FMAs of Gram, elimination, e and rhs).  A block of 64
-// threads per particle on the complex matrix took 27.7 ms at 64 PFs x 1e5 particles (Nz = 160) and
-// 69 ms at 32 x 262144 (Nz = 1024).
+// sum_s w0_s u_s element by element, |e|^2 - rhs^H A^-1 rhs.  One warp per (particle, PA).
+//   * e: lanes over (y, m), two frequencies per packed FP32 pair; P and Q take 2 x 4 packed FMAs
+//     with the steering elements formed on the way.
+//   * rhs: lanes over PFs, the frequencies' factors in registers, packed the same way.
+//   * A: the lower triangle in registers, lane (tr, tc) of 8 x 4 owning (8 ia + tr, 4 ib + tc).  Panels of
+//     eight columns go through shared memory: lanes take rows, factor the panel with shuffles (the
+//     forward substitution rides along), then every lane applies the rank-8 update to its entries.
+// Bound: FP32 issue.  The whole stage at 64 PFs x 1e5 particles (Nz = 160) / 32 x 262144 (Nz = 1024):
+// 27.7 / 69 ms with a block of 64 threads per particle on the complex matrix, 15.1 / 54.4 with this
+// split but one column of the elimination at a time and unpacked e and rhs, 12.0 / 26.6 as it is.
 constexpr float IB_ERR_PER_RATIO = 4.0e-6f;    // as in k_iota_bulk.cu
 constexpr float IB_ERR_PER_ENERGY = 1.0e-6f;
 constexpr int IB_W = 4;                        // warps (PAs of a particle) per block
-constexpr int IB_FC = 4;                       // frequencies per lane and pass of the residual
-constexpr int IB_CR = 12, IB_CC = 20;          // strides of the published column (conflict-free 128-bit reads)
-struct IbPlan { size_t fac, ct, pq, col, vec, warp; int fst, cst; };
+constexpr int IB_FP = 4;                       // frequency pairs per lane and pass
+constexpr int IB_PST = 12;                     // row stride of the panel (conflict-free 128-bit accesses)
+struct IbPlan { size_t pq, pan, fx, fy, ant, vec, warp; int fp, f4, ast; };
 template <int NB>
 __host__ __device__ inline IbPlan ib_plan(const DevGeom& G, int S) {
     const IsDims d = is_dims(G);
     IbPlan p{};
-    p.fst = d.hf | 1;                          // odd row strides
-    p.cst = d.Nmh | 1;
+    p.f4 = (d.Fh + 7) & ~7;                    // frequencies, padded to a lane's four pairs
+    p.fp = p.f4 + 4;                           // row stride: 16-byte rows, 8 rows on distinct banks
+    p.ast = (d.hy + d.hz) | 1;
+    const size_t R = 8 * NB;                   // rows beyond S are zero
     size_t o = 0;
-    p.pq = o; o += (size_t)d.Fh * G.My * G.Mz * sizeof(float4);
-    p.col = o; o += 2 * (8 * IB_CR + 4 * IB_CC) * sizeof(float);
-    p.fac = o; o += (size_t)S * p.fst * sizeof(float2);
-    p.ct = o; o += (size_t)S * p.cst * sizeof(float2);
-    p.vec = o; o += (size_t)8 * NB * (sizeof(float2) + sizeof(float));
+    p.pq = o; o += (size_t)G.My * G.Mz * 4 * p.f4 * sizeof(float);
+    p.pan = o; o += R * IB_PST * sizeof(float);
+    p.fx = o; o += R * p.fp * sizeof(float);
+    p.fy = o; o += R * p.fp * sizeof(float);
+    p.vec = o; o += R * (sizeof(float4) + sizeof(float));
+    p.ant = o; o += R * p.ast * sizeof(float2);
     p.warp = (o + 15) & ~(size_t)15;
     return p;
 }
-constexpr size_t IB_FIXED = 2 * 16 * (sizeof(double) + 2 * sizeof(float));
+constexpr size_t IB_FIXED = 2 * 16 * (sizeof(double) + 2 * sizeof(float)) + 2 * 16 * sizeof(double);
 
-// registers: 168 (72 of them the triangle) up to 64 PFs, 3 blocks of four warps per SM; 80 up to 32 PFs
+// registers: 168 (72 of them the triangle) up to 64 PFs, 3 blocks of four warps per SM; 4 blocks up to 32 PFs
 template <int NB>
-__global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 6) k_iota_bulk_sym(DevGeom G, DevParams Pm, DevState D, int S, const float* __restrict__ z,
-                                                          int W) {
+__global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(DevGeom G, DevParams Pm, DevState D, int S,
+                                                                             const float* __restrict__ z, int W) {
     constexpr int NSL = NB * (NB + 1);                          // register slots (ia, ib <= 2 ia + 1)
-    static_assert(NB <= 8, "column buffer strides");
+    constexpr int NR = NB > 4 ? 2 : 1;                          // rows per lane: lane, lane + 32
     extern __shared__ float4 smb[];
     const int P = Pm.P, J = G.J, Nz = G.Nz, Nf = G.Nf, My = G.My, Mz = G.Mz, Nm = My * Mz;
     const IsDims dm = is_dims(G);
     const IbPlan pl = ib_plan<NB>(G, S);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tr = lane & 7, tc = lane >> 3;
     double* part = reinterpret_cast<double*>(smb);              // [2][16] log iota per PA (particle parity)
-    float* perr = reinterpret_cast<float*>(part + 32);          // [2][16] bound per PA
+    double* lgs = part + 32;                                    // [16] log eta_bar
+    double* ies = lgs + 16;                                     // [16] 1 / eta_bar
+    float* perr = reinterpret_cast<float*>(ies + 16);           // [2][16] bound per PA
     float* pbad = perr + 32;                                    // [2][16] breakdown per PA
     char* base = reinterpret_cast<char*>(smb) + IB_FIXED + (size_t)wid * pl.warp;
-    float4* pq = reinterpret_cast<float4*>(base + pl.pq);       // [Fh Nm] e: P, Q
-    float* col = reinterpret_cast<float*>(base + pl.col);       // [2][by row residue 8 x IB_CR | by column residue 4 x IB_CC]
-    float2* fac = reinterpret_cast<float2*>(base + pl.fac);     // [S][fst] b_f, a_y, a_z (half of each)
-    float2* ct = reinterpret_cast<float2*>(base + pl.ct);       // [S][cst] a_y a_z (half)
-    float2* ws = reinterpret_cast<float2*>(base + pl.vec);      // [8 NB] A c pi mu
+    float* pq = reinterpret_cast<float*>(base + pl.pq);         // [Nm][P re, P im, -Q re, Q im][f4] e
+    float* pan = reinterpret_cast<float*>(base + pl.pan);       // [8 NB][IB_PST] panel of eight columns
+    float* fx = reinterpret_cast<float*>(base + pl.fx);         // [8 NB][fp] Re b_f
+    float* fy = reinterpret_cast<float*>(base + pl.fy);         // [8 NB][fp] Im b_f
+    float2* ant = reinterpret_cast<float2*>(base + pl.ant);     // [8 NB][ast] a_y, a_z (half of each)
+    float4* ws = reinterpret_cast<float4*>(base + pl.vec);      // [8 NB] -2 A c pi mu, each part twice
     float* dA = reinterpret_cast<float*>(ws + 8 * NB);          // [8 NB] d_s A_s
     const float* phi = D.phi[D.cur];
     const bool odd = Nz & 1;
-    // element blocks of the residual: NL lanes over (y, m), the groups of lanes over frequencies
+    if (threadIdx.x < J) {
+        lgs[threadIdx.x] = log(D.eta_bar[threadIdx.x]);
+        ies[threadIdx.x] = 1.0 / D.eta_bar[threadIdx.x];
+    }
+    for (int i = lane; i < 8 * NB * pl.fp; i += 32) fx[i] = fy[i] = 0.f;     // rows and columns beyond S and Fh stay zero
+    for (int i = lane; i < 8 * NB * pl.ast; i += 32) ant[i] = make_float2(0.f, 0.f);
+    for (int i = lane; i < Nm * 4 * pl.f4; i += 32) pq[i] = 0.f;
+    __syncthreads();
+    // element blocks of the residual: NL lanes over (y, m), the groups of lanes over frequency pairs
     const int NL = min(Nm, 32), ngrp = 32 / NL, lg = lane / NL, ly = lane - lg * NL;
-    const int npass = (dm.Fh + ngrp * IB_FC - 1) / (ngrp * IB_FC), fc = (dm.Fh + ngrp * npass - 1) / (ngrp * npass);
+    const int np2 = (dm.Fh + 1) / 2, npass = (np2 + ngrp * IB_FP - 1) / (ngrp * IB_FP), fc = (np2 + ngrp * npass - 1) / (ngrp * npass);
+    // Gram over frequencies in pairs; the middle one of an odd count (exactly 1) may be among them
+    const int gp = (Nf / 2 + 1) / 2;
+    const float mf = (Nf & 1) ? ((Nf / 2) & 1 ? -1.0f : 1.0f) : 0.0f;
+    const float my = (My & 1) ? 1.0f : 0.0f, mz = (Mz & 1) ? 1.0f : 0.0f;
     int par = 0;
     for (int p = blockIdx.x; p < P; p += gridDim.x, par ^= 1) {
         for (int j = wid; j < J; j += W) {
             __syncwarp();
             const float ebf = (float)D.eta_bar[j];
-            for (int s = lane; s < 8 * NB; s += 32) {
-                float2 w = make_float2(0.f, 0.f);
+            #pragma unroll
+            for (int hr = 0; hr < NR; ++hr) {   // factors and weights, lanes over PFs
+                const int s = lane + 32 * hr;
+                float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
                 float d = 0.f;
                 if (s < S) {
                     const float* ph = phi + (size_t)s * 6 * P + p;
-                    const float4 g = D.geo[((size_t)s * J + j) * P + p];
+                    const size_t gi = ((size_t)s * J + j) * P + p;
+                    const float4 g = D.geo[gi];
+                    const float2 gl = D.geo_lo[gi];
+                    const float gm = ph[3 * (size_t)P], mr = ph[4 * (size_t)P], mi = ph[5 * (size_t)P];
+                    const float pi = (float)(D.zeta[s * J + j] * D.W[s]);
                     const float A = G.amp_c / (g.x + g.y);
                     float h, l;
                     ff_frac_mul2(g.x, g.y, G.inv_lam_hi, G.inv_lam_lo, h, l);
                     const float2 c = cispi_ff(-2.0f * h, -2.0f * l);
-                    const float pi = (float)(D.zeta[s * J + j] * D.W[s]);
-                    const float gm = ph[3 * (size_t)P], mr = ph[4 * (size_t)P], mi = ph[5 * (size_t)P];
                     d = A * sqrtf(fmaxf(pi * (gm + (mr * mr + mi * mi) * (1.0f - pi)), 0.0f));
-                    w = cmul(make_float2(A * pi * mr, A * pi * mi), c);
+                    const float2 w0 = cmul(make_float2(A * pi * mr, A * pi * mi), c);
+                    w = make_float4(-2.0f * w0.x, -2.0f * w0.x, -2.0f * w0.y, -2.0f * w0.y);
+                    for (int f = 0; f < dm.Fh; ++f) {
+                        const float2 b = freq_factor(G, g, f);
+                        fx[s * pl.fp + f] = b.x;
+                        fy[s * pl.fp + f] = b.y;
+                    }
+                    for (int q = 0; q < dm.hy + dm.hz; ++q) {
+                        const bool y = q < dm.hy;
+                        const int e = y ? q : q - dm.hy;
+                        const float cc = y ? G.py_l[e] : G.pz_l[e], cl = y ? G.py_lo[e] : G.pz_lo[e];
+                        const float u = y ? g.z : g.w, ul = y ? gl.x : gl.y;
+                        const float t = __fmul_rn(cc, u);
+                        ant[s * pl.ast + q] = cispi_ff(2.0f * t, 2.0f * fmaf(cc, ul, fmaf(cl, u, fmaf(cc, u, -t))));
+                    }
                 }
-                ws[s] = w;
-                dA[s] = d;
-            }
-            for (int i = lane; i < S * dm.hf; i += 32) {
-                const int s = i / dm.hf, q = i - s * dm.hf;
-                const size_t gi = ((size_t)s * J + j) * P + p;
-                const float4 g = D.geo[gi];
-                float th, tl;
-                if (q < dm.Fh) {
-                    ff_frac_mul2(g.x, g.y, G.fc_hi[q], G.fc_lo[q], th, tl);
-                    th = -th; tl = -tl;
-                } else {
-                    const float2 gl = D.geo_lo[gi];
-                    const bool y = q < dm.Fh + dm.hy;
-                    const int e = q - dm.Fh - (y ? 0 : dm.hy);
-                    const float c = y ? G.py_l[e] : G.pz_l[e], cl = y ? G.py_lo[e] : G.pz_lo[e];
-                    const float u = y ? g.z : g.w, ul = y ? gl.x : gl.y;
-                    th = __fmul_rn(c, u);
-                    tl = fmaf(c, ul, fmaf(cl, u, fmaf(c, u, -th)));
-                }
-                fac[s * pl.fst + q] = cispi_ff(2.0f * th, 2.0f * tl);
+                if (s < 8 * NB) { ws[s] = w; dA[s] = d; }
             }
             __syncwarp();
-            for (int i = lane; i < S * dm.Nmh; i += 32) {
-                const int s = i / dm.Nmh, ym = i - s * dm.Nmh, y = ym / Mz, m = ym - y * Mz;
-                const float2* fs = fac + s * pl.fst + dm.Fh;
-                bool cy, cz;
-                const int iy = is_half(y, My, dm.hy, cy), iz = is_half(m, Mz, dm.hz, cz);
-                float2 a = fs[iy], b = fs[dm.hy + iz];
-                if (cy) a.y = -a.y;
-                if (cz) b.y = -b.y;
-                ct[s * pl.cst + ym] = cmul(a, b);
-            }
-            __syncwarp();
+            // a_y a_z of element ym of row s
+            auto antenna = [&](int s, int iy, float sy, int iz, float sz) {
+                float2 a = ant[s * pl.ast + iy], b = ant[s * pl.ast + iz];
+                a.y *= sy;
+                b.y *= sz;
+                return cmul(a, b);
+            };
             // e = z - sum_s w0_s u_s as sums and differences of mirrored elements; |e|^2
             float ee = 0.f;
             for (int y0 = 0; y0 < Nm; y0 += NL) {
-                const int ym = y0 + ly;
-                bool cj = false;
-                const int ih = ym < Nm ? is_half(ym, Nm, dm.Nmh, cj) : 0;
-                const float sg = cj ? -1.0f : 1.0f;
+                const int ym = y0 + ly, y = min(ym, Nm - 1) / Mz, m = min(ym, Nm - 1) - y * Mz;
+                bool cy, cz;
+                const int iy = is_half(y, My, dm.hy, cy), iz = dm.hy + is_half(m, Mz, dm.hz, cz);
+                const float sy = cy ? -1.0f : 1.0f, sz = cz ? -1.0f : 1.0f;
                 for (int ps = 0; ps < npass; ++ps) {
-                    const int f0 = (ps * ngrp + lg) * fc;
+                    const int f0 = 2 * (ps * ngrp + lg) * fc;
                     const bool act = ym < Nm && lg < ngrp && f0 < dm.Fh;
-                    float4 a[IB_FC];
-                    #pragma unroll
-                    for (int i = 0; i < IB_FC; ++i) {
-                        const int k = (f0 + i) * Nm + ym;
-                        a[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (act && i < fc && f0 + i < dm.Fh && k < dm.Nh) {
-                            const float* za = z + 2 * ((size_t)j * Nz + k);
-                            const float* zb = z + 2 * ((size_t)j * Nz + Nz - 1 - k);
-                            a[i] = make_float4(za[0] + zb[0], za[1] + zb[1], za[0] - zb[0], za[1] - zb[1]);
-                            if (odd && k == dm.Nh - 1) a[i] = make_float4(2.0f * za[0], 2.0f * za[1], 0.f, 0.f);
-                        }
-                    }
                     const int fl = act ? f0 : 0;
-                    for (int s = 0; s < S; ++s) {
-                        float2 c = ct[s * pl.cst + ih];
-                        c.y *= sg;
-                        const float2 w = ws[s];
-                        const float2* b = fac + s * pl.fst + fl;
+                    f2x a[IB_FP][4];
+                    #pragma unroll
+                    for (int i = 0; i < IB_FP; ++i) {
+                        float v[4][2];
                         #pragma unroll
-                        for (int i = 0; i < IB_FC; ++i) {
+                        for (int q = 0; q < 2; ++q) {
+                            const int f = f0 + 2 * i + q, k = f * Nm + ym;
+                            v[0][q] = v[1][q] = v[2][q] = v[3][q] = 0.f;
+                            if (act && i < fc && f < dm.Fh && k < dm.Nh) {
+                                const float *pa = z + 2 * ((size_t)j * Nz + k), *pb = z + 2 * ((size_t)j * Nz + Nz - 1 - k);
+                                const float2 za = make_float2(pa[0], pa[1]), zb = make_float2(pb[0], pb[1]);
+                                const bool mid = odd && k == dm.Nh - 1;      // carried doubled
+                                v[0][q] = za.x + zb.x;
+                                v[1][q] = za.y + zb.y;
+                                v[2][q] = mid ? 0.f : zb.x - za.x;
+                                v[3][q] = mid ? 0.f : za.y - zb.y;
+                            }
+                        }
+                        #pragma unroll
+                        for (int c = 0; c < 4; ++c) a[i][c] = f2_pack(v[c][0], v[c][1]);
+                    }
+                    #pragma unroll 2
+                    for (int s = 0; s < S; ++s) {
+                        const float2 c = antenna(s, iy, sy, iz, sz);
+                        const float4 w = ws[s];
+                        const f2x cx = f2_dup(c.x), cyy = f2_dup(c.y), ncy = f2_dup(-c.y);
+                        const f2x wr = f2_pack(w.x, w.y), wi = f2_pack(w.z, w.w);
+                        const float2 *bx = reinterpret_cast<const float2*>(fx + s * pl.fp + fl),
+                                     *by = reinterpret_cast<const float2*>(fy + s * pl.fp + fl);
+                        #pragma unroll
+                        for (int i = 0; i < IB_FP; ++i) {
                             if (i < fc) {
-                                const float2 bb = b[i];
-                                const float x2 = 2.0f * fmaf(bb.x, c.x, -bb.y * c.y), y2 = 2.0f * fmaf(bb.x, c.y, bb.y * c.x);
-                                a[i].x = fmaf(-w.x, x2, a[i].x);
-                                a[i].y = fmaf(-w.y, x2, a[i].y);
-                                a[i].z = fmaf(w.y, y2, a[i].z);
-                                a[i].w = fmaf(-w.x, y2, a[i].w);
+                                const float2 xv = bx[i], yv = by[i];
+                                const f2x x2 = f2_pack(xv.x, xv.y), y2 = f2_pack(yv.x, yv.y);
+                                const f2x ux = f2_fma(x2, cx, f2_mul(y2, ncy)), uy = f2_fma(x2, cyy, f2_mul(y2, cx));
+                                a[i][0] = f2_fma(wr, ux, a[i][0]);
+                                a[i][1] = f2_fma(wi, ux, a[i][1]);
+                                a[i][2] = f2_fma(wi, uy, a[i][2]);       // -Q re
+                                a[i][3] = f2_fma(wr, uy, a[i][3]);
                             }
                         }
                     }
                     #pragma unroll
-                    for (int i = 0; i < IB_FC; ++i) {
-                        const int k = (f0 + i) * Nm + ym;
-                        if (act && i < fc && f0 + i < dm.Fh) {
-                            float4 v = a[i];
-                            if (k >= dm.Nh) v = make_float4(0.f, 0.f, 0.f, 0.f);
-                            const float q = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
-                            if (odd && k == dm.Nh - 1) {         // carried doubled
-                                v.x *= 0.5f; v.y *= 0.5f; v.z = 0.f; v.w = 0.f;
-                                ee += fmaf(v.x, v.x, v.y * v.y);
-                            } else {
-                                ee = fmaf(0.5f, q, ee);
+                    for (int i = 0; i < IB_FP; ++i) {
+                        if (act && i < fc && f0 + 2 * i < pl.f4) {
+                            float v[4][2];
+                            #pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                uint32_t u0, u1;
+                                f2_unpack(a[i][c], u0, u1);
+                                v[c][0] = __uint_as_float(u0);
+                                v[c][1] = __uint_as_float(u1);
                             }
-                            pq[k] = v;
+                            #pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const int f = f0 + 2 * i + q, k = f * Nm + ym;
+                                if (f >= dm.Fh || k >= dm.Nh) v[0][q] = v[1][q] = v[2][q] = v[3][q] = 0.f;
+                                float half = 0.5f;
+                                if (odd && k == dm.Nh - 1) {
+                                    v[0][q] *= 0.5f; v[1][q] *= 0.5f;
+                                    v[2][q] = v[3][q] = 0.f;
+                                    half = 1.0f;
+                                }
+                                const float e2 = fmaf(v[0][q], v[0][q], fmaf(v[1][q], v[1][q], fmaf(v[2][q], v[2][q], v[3][q] * v[3][q])));
+                                ee = fmaf(half, e2, ee);
+                            }
+                            #pragma unroll
+                            for (int c = 0; c < 4; ++c)
+                                *reinterpret_cast<float2*>(pq + (ym * 4 + c) * pl.f4 + f0 + 2 * i) = make_float2(v[c][0], v[c][1]);
                         }
                     }
                 }
             }
             ee = warp_sum_f(ee);
             __syncwarp();
-            // rhs_s = (dA)_s u_s^H e, rows lane and lane + 32: per frequency the sums over (y, m), the mirrored
-            // element's factor being the conjugate
-            float2 rhs[2];
-            #pragma unroll
-            for (int hr = 0; hr < (NB > 4 ? 2 : 1); ++hr) {
-                const int s = lane + 32 * hr;
-                float2 g = make_float2(0.f, 0.f);
-                if (s < S) {
-                    const float2 *fs = fac + s * pl.fst, *cs = ct + s * pl.cst;
-                    for (int f = 0; f < dm.Fh; ++f) {
-                        float2 al = make_float2(0.f, 0.f), be = al;
-                        const float4* ef = pq + f * Nm;
-                        auto add = [&](float2 c, float4 e) {
-                            al.x = fmaf(c.x, e.x, fmaf(c.y, e.w, al.x));
-                            al.y = fmaf(c.x, e.y, fmaf(-c.y, e.z, al.y));
-                            be.x = fmaf(c.y, e.x, fmaf(-c.x, e.w, be.x));
-                            be.y = fmaf(c.y, e.y, fmaf(c.x, e.z, be.y));
-                        };
-                        for (int ym = 0; ym < Nm / 2; ++ym) {
-                            const float2 c = cs[ym];
-                            add(c, ef[ym]);
-                            add(make_float2(c.x, -c.y), ef[Nm - 1 - ym]);
+            // rhs_s = (dA)_s u_s^H e
+            float2 rhs[NR];
+            {
+                f2x gr[NR], gi[NR];
+                #pragma unroll
+                for (int hr = 0; hr < NR; ++hr) gr[hr] = gi[hr] = f2_dup(0.f);
+                for (int f0 = 0; f0 < dm.Fh; f0 += 8) {
+                    f2x bx[NR][4], by[NR][4];
+                    #pragma unroll
+                    for (int hr = 0; hr < NR; ++hr)
+                        #pragma unroll
+                        for (int i = 0; i < 4; i += 2) {
+                            const int s = min(lane + 32 * hr, 8 * NB - 1);
+                            const float4 xv = *reinterpret_cast<const float4*>(fx + s * pl.fp + f0 + 2 * i);
+                            const float4 yv = *reinterpret_cast<const float4*>(fy + s * pl.fp + f0 + 2 * i);
+                            bx[hr][i] = f2_pack(xv.x, xv.y); bx[hr][i + 1] = f2_pack(xv.z, xv.w);
+                            by[hr][i] = f2_pack(yv.x, yv.y); by[hr][i + 1] = f2_pack(yv.z, yv.w);
                         }
-                        if (Nm & 1) add(cs[Nm / 2], ef[Nm / 2]);
-                        const float2 b = fs[f];
-                        g.x = fmaf(b.x, al.x, fmaf(-b.y, be.x, g.x));
-                        g.y = fmaf(b.x, al.y, fmaf(-b.y, be.y, g.y));
+                    const bool wide = f0 + 4 < dm.Fh;               // uniform: frequencies beyond the first four
+                    for (int y = 0; y < My; ++y) {
+                        bool cy;
+                        const int iy = is_half(y, My, dm.hy, cy);
+                        const float sy = cy ? -1.0f : 1.0f;
+                        for (int m = 0; m < Mz; ++m) {
+                            bool cz;
+                            const int iz = dm.hy + is_half(m, Mz, dm.hz, cz);
+                            const float sz = cz ? -1.0f : 1.0f;
+                            const float* e = pq + (size_t)(y * Mz + m) * 4 * pl.f4 + f0;
+                            f2x cx[NR], cyy[NR], ncy[NR];
+                            #pragma unroll
+                            for (int hr = 0; hr < NR; ++hr) {
+                                const float2 c = antenna(min(lane + 32 * hr, 8 * NB - 1), iy, sy, iz, sz);
+                                cx[hr] = f2_dup(c.x);
+                                cyy[hr] = f2_dup(c.y);
+                                ncy[hr] = f2_dup(-c.y);
+                            }
+                            #pragma unroll
+                            for (int i = 0; i < 4; i += 2) {
+                                if (i == 0 || wide) {
+                                    const float4 pr = *reinterpret_cast<const float4*>(e + 2 * i);
+                                    const float4 pi = *reinterpret_cast<const float4*>(e + pl.f4 + 2 * i);
+                                    const float4 nq = *reinterpret_cast<const float4*>(e + 2 * pl.f4 + 2 * i);
+                                    const float4 qi = *reinterpret_cast<const float4*>(e + 3 * pl.f4 + 2 * i);
+                                    #pragma unroll
+                                    for (int hr = 0; hr < NR; ++hr) {
+                                        auto two = [&](f2x x2, f2x y2, f2x epr, f2x epi, f2x enq, f2x eqi) {
+                                            const f2x ux = f2_fma(x2, cx[hr], f2_mul(y2, ncy[hr]));
+                                            const f2x uy = f2_fma(x2, cyy[hr], f2_mul(y2, cx[hr]));
+                                            gr[hr] = f2_fma(ux, epr, f2_fma(uy, eqi, gr[hr]));
+                                            gi[hr] = f2_fma(ux, epi, f2_fma(uy, enq, gi[hr]));
+                                        };
+                                        two(bx[hr][i], by[hr][i], f2_pack(pr.x, pr.y), f2_pack(pi.x, pi.y), f2_pack(nq.x, nq.y),
+                                            f2_pack(qi.x, qi.y));
+                                        two(bx[hr][i + 1], by[hr][i + 1], f2_pack(pr.z, pr.w), f2_pack(pi.z, pi.w),
+                                            f2_pack(nq.z, nq.w), f2_pack(qi.z, qi.w));
+                                    }
+                                }
+                            }
+                        }
                     }
-                    g = make_float2(dA[s] * g.x, dA[s] * g.y);
                 }
-                rhs[hr] = g;
+                #pragma unroll
+                for (int hr = 0; hr < NR; ++hr) {
+                    uint32_t r0, r1, i0, i1;
+                    f2_unpack(gr[hr], r0, r1);
+                    f2_unpack(gi[hr], i0, i1);
+                    const float d = dA[min(lane + 32 * hr, 8 * NB - 1)];
+                    rhs[hr] = make_float2(d * (__uint_as_float(r0) + __uint_as_float(r1)),
+                                          d * (__uint_as_float(i0) + __uint_as_float(i1)));
+                }
             }
-            // Gram of this lane's entries: frequencies, then the antenna factors row block by row block
+            // Gram of this lane's entries: frequencies two at a time, then the antenna factors row block by row block
             float A[NSL];
             #pragma unroll
             for (int q = 0; q < NSL; ++q) A[q] = 0.f;
-            auto ld = [&](int s, int q) { return s < S ? fac[s * pl.fst + q] : make_float2(0.f, 0.f); };
-            for (int f = 0; f < Nf / 2; ++f) {
-                float2 ra[NB];
+            for (int g = 0; g < gp; ++g) {
+                float2 rx[NB], ry[NB];
                 #pragma unroll
-                for (int ia = 0; ia < NB; ++ia) ra[ia] = ld(8 * ia + tr, f);
+                for (int ia = 0; ia < NB; ++ia) {
+                    rx[ia] = *reinterpret_cast<const float2*>(fx + (8 * ia + tr) * pl.fp + 2 * g);
+                    ry[ia] = *reinterpret_cast<const float2*>(fy + (8 * ia + tr) * pl.fp + 2 * g);
+                }
                 #pragma unroll
                 for (int ib = 0; ib < 2 * NB; ++ib) {
-                    const float2 cb = ld(4 * ib + tc, f);
+                    const float2 cx = *reinterpret_cast<const float2*>(fx + (4 * ib + tc) * pl.fp + 2 * g);
+                    const float2 cy = *reinterpret_cast<const float2*>(fy + (4 * ib + tc) * pl.fp + 2 * g);
                     #pragma unroll
                     for (int ia = ib / 2; ia < NB; ++ia) {
                         float& v = A[ia * (ia + 1) + ib];
-                        v = fmaf(ra[ia].x, cb.x, fmaf(ra[ia].y, cb.y, v));
+                        v = fmaf(rx[ia].x, cx.x, fmaf(ry[ia].x, cy.x, fmaf(rx[ia].y, cx.y, fmaf(ry[ia].y, cy.y, v))));
                     }
                 }
             }
-            const float mf = (Nf & 1) ? 1.0f : 0.0f, my = (My & 1) ? 1.0f : 0.0f, mz = (Mz & 1) ? 1.0f : 0.0f;
             #pragma unroll
             for (int ia = 0; ia < NB; ++ia) {
                 float sy[2 * NB], sz[2 * NB];
                 #pragma unroll
                 for (int ib = 0; ib <= 2 * ia + 1; ++ib) sy[ib] = sz[ib] = 0.f;
                 const int a = 8 * ia + tr;
+                const float2* ra = ant + a * pl.ast;
+                const float2* rc = ant + tc * pl.ast;
                 for (int u = 0; u < My / 2; ++u) {
-                    const float2 r = ld(a, dm.Fh + u);
+                    const float2 r = ra[u];
                     #pragma unroll
                     for (int ib = 0; ib <= 2 * ia + 1; ++ib) {
-                        const float2 cb = ld(4 * ib + tc, dm.Fh + u);
+                        const float2 cb = rc[4 * ib * pl.ast + u];
                         sy[ib] = fmaf(r.x, cb.x, fmaf(r.y, cb.y, sy[ib]));
                     }
                 }
-                for (int u = 0; u < Mz / 2; ++u) {
-                    const float2 r = ld(a, dm.Fh + dm.hy + u);
+                for (int u = dm.hy; u < dm.hy + Mz / 2; ++u) {
+                    const float2 r = ra[u];
                     #pragma unroll
                     for (int ib = 0; ib <= 2 * ia + 1; ++ib) {
-                        const float2 cb = ld(4 * ib + tc, dm.Fh + dm.hy + u);
+                        const float2 cb = rc[4 * ib * pl.ast + u];
                         sz[ib] = fmaf(r.x, cb.x, fmaf(r.y, cb.y, sz[ib]));
                     }
                 }
@@ -671,102 +755,94 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 6) k_iota_bulk_sym(Dev
                     if (a == b) v = a < S ? v + ebf : 1.0f;
                 }
             }
-            // LDL^T elimination with the forward substitution
-            float yy = 0.f, pv0 = 1.f, pv1 = 1.f;
-            auto publish = [&](int buf, int row, float v) {
-                float* c = col + buf * (8 * IB_CR + 4 * IB_CC);
-                c[(row & 7) * IB_CR + (row >> 3)] = v;
-                c[8 * IB_CR + (row & 3) * IB_CC + (row >> 2)] = v;
-            };
-            if (tc == 0) {
-                #pragma unroll
-                for (int ia = 0; ia < NB; ++ia) publish(0, 8 * ia + tr, A[ia * (ia + 1)]);
-            }
-            __syncwarp();
+            // LDL^T elimination by panels of eight columns, with the forward substitution
+            float yy = 0.f, pv[NR];
             #pragma unroll
-            for (int kb = 0; kb < 2 * NB; ++kb) {               // columns 4 kb .. 4 kb + 3: slots ib = kb
-                #pragma unroll 1
-                for (int r = 0; r < 4; ++r) {
-                    const int k = 4 * kb + r;
-                    if (k >= S) break;                          // uniform
-                    const int K = kb / 2;
-                    const float* cr = col + (k & 1) * (8 * IB_CR + 4 * IB_CC);
-                    const float* cc = cr + 8 * IB_CR;
-                    const float piv = cc[(k & 3) * IB_CC + (k >> 2)];
-                    const float ipiv = 1.0f / piv;
-                    // forward substitution: y_k = rhs_k / piv_k, rhs_i -= A_ik y_k
-                    {
-                        const float2 own = (NB > 4 && k >= 32) ? rhs[1] : rhs[0];
-                        const float2 rk = make_float2(__shfl_sync(0xffffffffu, own.x, k & 31), __shfl_sync(0xffffffffu, own.y, k & 31));
-                        const float2 y = make_float2(rk.x * ipiv, rk.y * ipiv);
-                        if (lane == (k & 31)) {
-                            yy = fmaf(fmaf(rk.x, rk.x, rk.y * rk.y), ipiv, yy);
-                            if (NB > 4 && k >= 32) pv1 = piv; else pv0 = piv;
-                        }
-                        if (lane > k && lane < S) {
-                            const float v = cr[(lane & 7) * IB_CR + (lane >> 3)];
-                            rhs[0].x = fmaf(-v, y.x, rhs[0].x);
-                            rhs[0].y = fmaf(-v, y.y, rhs[0].y);
-                        }
-                        if (NB > 4 && lane + 32 > k && lane + 32 < S) {
-                            const float v = cr[(lane & 7) * IB_CR + (lane >> 3) + 4];
-                            rhs[1].x = fmaf(-v, y.x, rhs[1].x);
-                            rhs[1].y = fmaf(-v, y.y, rhs[1].y);
-                        }
-                    }
-                    float xa[8], xc[16];
+            for (int hr = 0; hr < NR; ++hr) pv[hr] = 1.f;
+            #pragma unroll
+            for (int K = 0; K < NB; ++K) {
+                if (8 * K >= S) break;                              // uniform
+                __syncwarp();
+                #pragma unroll
+                for (int ia = K; ia < NB; ++ia) {
+                    pan[(8 * ia + tr) * IB_PST + tc] = A[ia * (ia + 1) + 2 * K];
+                    pan[(8 * ia + tr) * IB_PST + 4 + tc] = A[ia * (ia + 1) + 2 * K + 1];
+                }
+                __syncwarp();
+                float x[NR][8], ip[8];
+                #pragma unroll
+                for (int hr = 0; hr < NR; ++hr) {
+                    const float4* r = reinterpret_cast<const float4*>(pan + min(lane + 32 * hr, 8 * NB - 1) * IB_PST);
+                    const float4 v0 = r[0], v1 = r[1];
+                    x[hr][0] = v0.x; x[hr][1] = v0.y; x[hr][2] = v0.z; x[hr][3] = v0.w;
+                    x[hr][4] = v1.x; x[hr][5] = v1.y; x[hr][6] = v1.z; x[hr][7] = v1.w;
+                }
+                #pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    // row k = 8 K + c belongs to lane (8 K + c) % 32 of half (8 K) / 32; rows above k hold nothing
+                    // that is used again
+                    const int ow = (8 * K + c) & 31, hf = (8 * K) / 32;
+                    const float piv = __shfl_sync(0xffffffffu, x[hf][c], ow);
+                    ip[c] = __frcp_rn(piv);
+                    const float2 rk = make_float2(__shfl_sync(0xffffffffu, rhs[hf].x, ow), __shfl_sync(0xffffffffu, rhs[hf].y, ow));
+                    const float2 y = make_float2(rk.x * ip[c], rk.y * ip[c]);
+                    yy = fmaf(rk.x, y.x, fmaf(rk.y, y.y, yy));
+                    if (lane == ow) pv[hf] = piv;
                     #pragma unroll
-                    for (int q = 0; q < NB; q += 4) {
-                        if (q + 3 >= K) {
-                            const float4 v = *reinterpret_cast<const float4*>(cr + tr * IB_CR + q);
-                            xa[q] = v.x * -ipiv; xa[q + 1] = v.y * -ipiv; xa[q + 2] = v.z * -ipiv; xa[q + 3] = v.w * -ipiv;
-                        }
-                    }
-                    #pragma unroll
-                    for (int q = 0; q < 2 * NB; q += 4) {
-                        if (q + 3 >= kb) {
-                            const float4 v = *reinterpret_cast<const float4*>(cc + tc * IB_CC + q);
-                            xc[q] = v.x; xc[q + 1] = v.y; xc[q + 2] = v.z; xc[q + 3] = v.w;
-                        }
-                    }
-                    // the trailing entries: columns beyond k (in the slot of column k only those of larger residue)
-                    #pragma unroll
-                    for (int ia = K; ia < NB; ++ia) {
+                    for (int c2 = c + 1; c2 < 8; ++c2) {
+                        const float l = -ip[c] * __shfl_sync(0xffffffffu, x[hf][c], (8 * K + c2) & 31);
                         #pragma unroll
-                        for (int ib = kb; ib <= 2 * ia + 1; ++ib) {
+                        for (int hr = 0; hr < NR; ++hr) x[hr][c2] = fmaf(x[hr][c], l, x[hr][c2]);
+                    }
+                    #pragma unroll
+                    for (int hr = 0; hr < NR; ++hr) {
+                        rhs[hr].x = fmaf(-x[hr][c], y.x, rhs[hr].x);
+                        rhs[hr].y = fmaf(-x[hr][c], y.y, rhs[hr].y);
+                    }
+                }
+                if (K + 1 == NB) break;
+                #pragma unroll
+                for (int hr = 0; hr < NR; ++hr) {
+                    if (lane + 32 * hr < 8 * NB) {
+                        float4* r = reinterpret_cast<float4*>(pan + (lane + 32 * hr) * IB_PST);
+                        r[0] = make_float4(x[hr][0], x[hr][1], x[hr][2], x[hr][3]);
+                        r[1] = make_float4(x[hr][4], x[hr][5], x[hr][6], x[hr][7]);
+                    }
+                }
+                __syncwarp();
+                #pragma unroll
+                for (int q = 0; q < 2; ++q) {                       // the rank-8 update, four columns at a time
+                    float4 rv[NB];
+                    #pragma unroll
+                    for (int ia = K + 1; ia < NB; ++ia) {
+                        const float4 v = *reinterpret_cast<const float4*>(pan + (8 * ia + tr) * IB_PST + 4 * q);
+                        rv[ia] = make_float4(v.x * -ip[4 * q], v.y * -ip[4 * q + 1], v.z * -ip[4 * q + 2], v.w * -ip[4 * q + 3]);
+                    }
+                    #pragma unroll
+                    for (int ib = 2 * (K + 1); ib < 2 * NB; ++ib) {
+                        const float4 cv = *reinterpret_cast<const float4*>(pan + (4 * ib + tc) * IB_PST + 4 * q);
+                        #pragma unroll
+                        for (int ia = ib / 2; ia < NB; ++ia) {
                             float& v = A[ia * (ia + 1) + ib];
-                            if (ib > kb || tc > r) v = fmaf(xa[ia], xc[ib], v);
+                            v = fmaf(rv[ia].x, cv.x, fmaf(rv[ia].y, cv.y, fmaf(rv[ia].z, cv.z, fmaf(rv[ia].w, cv.w, v))));
                         }
                     }
-                    // owners of column k + 1 publish it
-                    if (r < 3) {
-                        if (tc == r + 1) {
-                            #pragma unroll
-                            for (int ia = K; ia < NB; ++ia) publish((k + 1) & 1, 8 * ia + tr, A[ia * (ia + 1) + kb]);
-                        }
-                    } else if (kb + 1 < 2 * NB) {
-                        if (tc == 0) {
-                            #pragma unroll
-                            for (int ia = (kb + 1) / 2; ia < NB; ++ia)
-                                publish((k + 1) & 1, 8 * ia + tr, A[ia * (ia + 1) + (kb + 1 < 2 * NB ? kb + 1 : kb)]);
-                        }
-                    }
-                    __syncwarp();
                 }
             }
             // log det, sum A_kk / piv_k, the smallest pivot
             float dm0 = 1.f, rsum = 0.f, pmin = 3.0e38f;
             int de = 0;
-            auto take = [&](int k, float pv) {
-                if (k >= S) return;
-                int e;
-                dm0 = frexpf(dm0 * pv, &e);
-                de += e;
-                rsum += fmaf(dA[k] * dA[k], (float)Nz, ebf) / pv;
-                pmin = fminf(pmin, pv);
-            };
-            take(lane, pv0);
-            if (NB > 4) take(lane + 32, pv1);
+            #pragma unroll
+            for (int hr = 0; hr < NR; ++hr) {
+                const int k = lane + 32 * hr;
+                if (k < S) {
+                    int e;
+                    dm0 = frexpf(dm0 * pv[hr], &e);
+                    de += e;
+                    rsum += fmaf(dA[k] * dA[k], (float)Nz, ebf) / pv[hr];
+                    pmin = fminf(pmin, pv[hr]);
+                }
+            }
             #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 int e;
@@ -775,19 +851,17 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 6) k_iota_bulk_sym(Dev
                 rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
                 pmin = fminf(pmin, __shfl_xor_sync(0xffffffffu, pmin, o));
             }
-            yy = warp_sum_f(yy);
             if (lane == 0) {
-                const double eb = D.eta_bar[j];
-                const double q = (double)ee - (double)yy;       // eta_bar e^H C^-1 e
+                const double ieb = ies[j], lgb = lgs[j];
+                const double q = ((double)ee - (double)yy) * ieb;   // e^H C^-1 e
                 const double logdet = log((double)dm0) + (double)de * 0.69314718055994530942;
-                const double lgb = log(eb);
-                const double v = -q / eb - logdet - (double)(Nz - S) * lgb - (double)Nz * IS_LOG_PI;
-                const float eq = IB_ERR_PER_ENERGY * (float)(((double)ee + (double)yy) / eb);
+                const double v = -q - logdet - (double)(Nz - S) * lgb - (double)Nz * IS_LOG_PI;
+                const float eq = IB_ERR_PER_ENERGY * (float)(((double)ee + (double)yy) * ieb);
                 part[par * 16 + j] = v;
                 perr[par * 16 + j] = IB_ERR_PER_RATIO * rsum + eq;
                 // every pivot of eta_bar I + D G D is at least eta_bar, and q >= 0: anything else is a
                 // breakdown of the FP32 elimination
-                pbad[par * 16 + j] = (!(pmin > 0.5f * ebf) || !(q / eb > -(double)eq) || !isfinite(v)) ? 1.f : 0.f;
+                pbad[par * 16 + j] = (!(pmin > 0.5f * ebf) || !(q > -(double)eq) || !isfinite(v)) ? 1.f : 0.f;
             }
         }
         __syncthreads();   // the buffers of the other parity are free again after the next one
@@ -809,7 +883,7 @@ static bool launch_bulk_sym_nb(const DevGeom& G, const DevParams& Pm, const DevS
     const size_t smem = IB_FIXED + W * warp;
     if (smem > limit) return false;
     smem_allow_max((const void*)k_iota_bulk_sym<NB>);
-    const int per_sm = max(1, min(32 / W, (int)((limit + 1024) / (smem + 1024))));
+    const int per_sm = max(1, min(16 / W, (int)((limit + 1024) / (smem + 1024))));
     k_iota_bulk_sym<NB><<<min(Pm.P, sm_count() * per_sm * 4), 32 * W, smem, st>>>(G, Pm, D, S, z, W);
     return true;
 }
@@ -818,6 +892,7 @@ static bool launch_bulk_sym_nb(const DevGeom& G, const DevParams& Pm, const DevS
 bool launch_iota_bulk_sym(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st) {
     if (!G.sym) return false;
     if (S <= 32) return launch_bulk_sym_nb<4>(G, Pm, D, S, z, st);
+    if (S <= 48) return launch_bulk_sym_nb<6>(G, Pm, D, S, z, st);
     return launch_bulk_sym_nb<8>(G, Pm, D, S, z, st);
 }
 
