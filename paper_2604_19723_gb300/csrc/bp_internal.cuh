@@ -386,7 +386,11 @@ __device__ __forceinline__ f2x f2_mul(f2x a, f2x b) {
     return r;
 }
 __device__ __forceinline__ f2x f2_dup(float a) { return f2_pack(a, a); }
-__device__ __forceinline__ f2x f2_sub(f2x a, f2x b) { return f2_fma(b, f2_dup(-1.0f), a); }
+__device__ __forceinline__ f2x f2_sub(f2x a, f2x b) {
+    f2x r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
 __device__ inline double warp_sum_d(double v) {
     #pragma unroll

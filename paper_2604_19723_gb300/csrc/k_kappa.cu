@@ -36,17 +36,19 @@
 // Im h; SW = S rounded up to 8), K = 2 Nh (Re, Im interleaved; Nh elements) in chunks of 32.  The
 // four digit slices of B lie side by side along N, and so do the accumulators, so the products
 // of A's digit i with B's digits 1 .. 5 - i are one run of 2 SW (5 - i) columns (N <= 256 per
-// instruction) onto g_{i-1} .. g_3.  One persistent block per SM: four producer groups of 128
-// threads build the A chunks (group g forms elements 4 g .. 4 g + 3 of each chunk, in registers,
-// two elements per packed FP32 instruction), one thread issues the MMAs and the bulk copies of
-// the prebuilt B chunks, and the producers read the accumulators of a finished (s, p tile, j)
-// after they have refilled the ring with the next one's first chunks, so the tensor cores wait
-// only for that read (not at all where two accumulator sets fit in TMEM, SW <= 32).
-// Bound: the producers' FP32 issue (about 45 instructions per element with its share of the factors
-// and the epilogue); the tensor pipe is next (ten products of 128 x 2 SW x 2 Nh).
-// Measured (PF likelihood stage, J = 4): 64 PFs x 1e5 particles, Nz = 160: 56.7 -> 15.6 ms; 32 PFs x
-// 262144, Nz = 1024: 401 -> 87 ms; 10 PFs x 30000, Nz = 160: 3.66 -> 0.58 ms (against the 3xTF32
-// kernel, below 33 PFs a CUDA-core kernel, with a second pass each).
+// instruction) onto g_{i-1} .. g_3.  One persistent block per SM: two teams of 256 producer threads fill
+// every other A chunk (eight elements per thread, in registers, two per packed FP32 instruction), one
+// warp copies the prebuilt B chunks, one issues the MMAs, and the producers read the accumulators of
+// a finished (s, p tile, j) after they have refilled the ring with the next one's first chunks,
+// so the tensor cores wait only for that read (not at all where two accumulator sets fit, SW <= 16).
+// Up to SW = 32 A goes through the half of tensor memory that the accumulators leave free.
+// Bound: the producers' issue slots (28 instructions per element for its digits; the factors, the loop and
+// the epilogue add as much at few elements); the tensor pipe is next (ten products of 128 x 2 SW x 2 Nh:
+// 46 % busy at 32 PFs, Nz = 1024).
+// Measured (PF likelihood stage, J = 4) with the 3xTF32 kernel (below 33 PFs a CUDA-core kernel), which
+// takes a second pass / with one thread issuing, A in shared memory and exact products by two-term
+// splits of full FP32 factors / as it is: 64 PFs x 1e5 particles, Nz = 160: 56.7 / 15.6 / 10.2 ms; 32 PFs x
+// 262144, Nz = 1024: 401 / 87 / 40.4 ms; 10 PFs x 30000, Nz = 160: 3.66 / 0.58 / 0.40 ms.
 #include "bp_internal.cuh"
 #include "bp_kernels.cuh"
 #include "tc_sm100.cuh"
@@ -54,18 +56,22 @@
 namespace bp {
 
 constexpr int KX_WAIT = 1 << 20;       // polls of a bounded wait
-constexpr int KX_NG = 4;               // producer groups (128 threads each)
+constexpr int KX_NG = 4;               // producer groups (128 threads each), two to a team
 constexpr int KX_PT = 128 * KX_NG;     // producer threads
-constexpr int KX_T = KX_PT + 32;       // + the issuing warp
+constexpr int KX_T = KX_PT + 64;       // + the issuing and the copying warp
 constexpr int KX_KC = 32;              // real K per chunk (16 elements)
 constexpr int KX_A = 4 * 128 * KX_KC * 2;   // bytes of A per chunk: 4 digits x 128 rows x KX_KC BF16
-constexpr int KX_NST_MAX = 4;
+constexpr int KX_NS_MAX = 4;           // slots of a ring
+constexpr int KX_ACOL = 256;           // first TMEM column of A (TA): slots of 4 digits x KX_KC / 2 columns
 
 __host__ __device__ inline int kx_sw(int S) { return (S + 7) & ~7; }
 __host__ __device__ inline int kx_chunks(int Nh) { return (Nh + 15) / 16; }
 __host__ __device__ inline uint32_t kx_bbytes(int SW) { return (uint32_t)(2 * SW) * KX_KC * 2 * 4; }   // 4 digits
 // elements a particle forms: half of them where the layout is symmetric
 __host__ __device__ inline int kx_elements(const DevGeom& G) { return G.sym ? (G.Nz + 1) / 2 : G.Nz; }
+__host__ __device__ inline int kx_factors(const DevGeom& G, int yz) {
+    return yz ? (G.My * G.Mz + 1) & ~1 : G.My + ((G.Mz + 1) & ~1);
+}
 __host__ __device__ inline int kx_freqs(const DevGeom& G) { return (kx_elements(G) - 1) / (G.My * G.Mz) + 1; }
 // shared memory after the ring: steering factors [nfac][128] as (hi, lo) pairs, cis table [256],
 // partial sums [KX_NG][128], u^H r0 [128] (float4 each), column scales [3][64], barriers and flags
@@ -73,9 +79,31 @@ __host__ __device__ inline size_t kx_smem_fixed(int nfac) {
     return ((size_t)nfac * 128 + 256 + KX_NG * 128 + 128) * sizeof(float4) + 3 * 64 * sizeof(float) + 256;
 }
 
-// a b for unit-modulus pairs, two elements at a time, in fixed point: hi a multiple of 2^-22
-// (adding 3 rounds each product onto that grid, where the sums are exact), lo the remainders and
-// the low-order cross terms (|lo| < 2^-20)
+// Steering factors as (h, l) with h a multiple of 2^-11 (12 bits) and |l| <= 2^-12 or so: the products of
+// the h parts and their sums are exact in FP32 (multiples of 2^-22), the cross terms are small.
+__device__ __forceinline__ void kx_grid(float hi, float lo, float& h, float& l) {
+    const float M = 6144.0f;                    // 1.5 x 2^12
+    h = __fsub_rn(__fadd_rn(__fadd_rn(hi, lo), M), M);
+    l = __fadd_rn(__fsub_rn(hi, h), lo);
+}
+__device__ __forceinline__ float4 kx_split(float4 a) {
+    float4 r;
+    kx_grid(a.x, a.z, r.x, r.z);
+    kx_grid(a.y, a.w, r.y, r.w);
+    return r;
+}
+// (a + al)(b + bl) + (c + cl)(d + dl) of split factors: hi exact, |lo| below 2^-9
+__device__ __forceinline__ void kx_dot(float a, float b, float c, float d, float al, float bl, float cl, float dl, float& hi, float& lo) {
+    hi = fmaf(c, d, __fmul_rn(a, b));
+    lo = fmaf(c, dl, fmaf(cl, d, fmaf(a, bl, fmaf(al, b, fmaf(cl, dl, __fmul_rn(al, bl))))));
+}
+__device__ __forceinline__ float4 kx_mul_split(float4 a, float4 b) {
+    float4 u;
+    kx_dot(a.x, b.x, -a.y, b.y, a.z, b.z, -a.w, b.w, u.x, u.z);
+    kx_dot(a.x, b.y, a.y, b.x, a.z, b.w, a.w, b.z, u.y, u.w);
+    return kx_split(u);
+}
+// the same, two elements at a time
 struct KxW { f2x x, y, ny, xl, yl, nyl; };     // the outer factor of each of the two elements
 struct KxU { f2x xh, yh, xl, yl; };
 __device__ __forceinline__ KxW kx_w(float4 a, float4 b) {
@@ -83,11 +111,8 @@ __device__ __forceinline__ KxW kx_w(float4 a, float4 b) {
                f2_pack(-a.w, -b.w)};
 }
 __device__ __forceinline__ void kx_dot2(f2x a, f2x b, f2x c, f2x d, f2x al, f2x bl, f2x cl, f2x dl, f2x& hi, f2x& lo) {
-    const f2x m = f2_dup(3.0f);                 // (a + al)(b + bl) + (c + cl)(d + dl)
-    const f2x t = f2_fma(a, b, m), t2 = f2_fma(c, d, t);
-    const f2x p = f2_fma(a, b, f2_sub(m, t)), q = f2_fma(c, d, f2_sub(t, t2));
-    hi = f2_sub(t2, m);
-    lo = f2_add(f2_fma(a, bl, f2_fma(al, b, p)), f2_fma(c, dl, f2_fma(cl, d, q)));
+    hi = f2_fma(c, d, f2_mul(a, b));
+    lo = f2_fma(c, dl, f2_fma(cl, d, f2_fma(a, bl, f2_fma(al, b, f2_fma(cl, dl, f2_mul(al, bl))))));
 }
 __device__ __forceinline__ KxU kx_mul(const KxW& w, const KxU& a) {
     KxU u;
@@ -95,22 +120,30 @@ __device__ __forceinline__ KxU kx_mul(const KxW& w, const KxU& a) {
     kx_dot2(w.x, a.yh, w.y, a.xh, w.xl, a.yl, w.yl, a.xl, u.yh, u.yl);
     return u;
 }
-// the four digits of two elements: adding 1.5 x 2^23 units rounds to a multiple of the unit, the
-// remainder is exact; digit i of element e in w[i][e] as the BF16 pair (Re, Im)
+// The four digits of two elements, digit i of element e in w[i][e] as the BF16 pair (Re, Im).  Adding 1.5 x
+// 2^23 units rounds to a multiple of the unit, the remainder is exact; the low part joins after the
+// first digit, where the remainder is below 2^-8 and the sum is good to 2^-33 (the second digit then
+// reaches 160 at most, still exact).  The last digit is the remainder cut to BF16: at most 2^-31 off, as far as
+// a rounded one of unit 2^-31, and its products only meet the last accumulator.
 __device__ __forceinline__ void kx_digits(const KxU& u, uint32_t (&w)[4][2]) {
-    const float M[4] = {98304.0f, 384.0f, 1.5f, 0.005859375f};   // 1.5 x 2^16, 2^8, 2^0, 2^-8
+    const float M[3] = {98304.0f, 384.0f, 1.5f};   // 1.5 x 2^16, 2^8, 2^0
     f2x rx = u.xh, ry = u.yh;
     #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const f2x m = f2_dup(M[i]), mn = f2_dup(-M[i]);
-        const f2x sx = f2_add(f2_add(rx, m), mn), sy = f2_add(f2_add(ry, m), mn);
+        f2x sx = rx, sy = ry;
+        if (i < 3) {
+            const f2x m = f2_dup(M[i]);
+            sx = f2_sub(f2_add(rx, m), m);
+            sy = f2_sub(f2_add(ry, m), m);
+            rx = f2_sub(rx, sx);
+            ry = f2_sub(ry, sy);
+        }
         uint32_t x0, x1, y0, y1;
         f2_unpack(sx, x0, x1);
         f2_unpack(sy, y0, y1);
         w[i][0] = __byte_perm(x0, y0, 0x7632);     // upper halves: the digits are exact in BF16
         w[i][1] = __byte_perm(x1, y1, 0x7632);
-        if (i < 3) { rx = f2_sub(rx, sx); ry = f2_sub(ry, sy); }
-        if (i == 1) { rx = f2_add(rx, u.xl); ry = f2_add(ry, u.yl); }
+        if (i == 0) { rx = f2_add(rx, u.xl); ry = f2_add(ry, u.yl); }
     }
 }
 // Delta of one (p, s, j): consts (1/eta_bar, zeta as pairs), amplitude A, gamma, mu, alpha_u =
@@ -269,38 +302,48 @@ __device__ __forceinline__ void kx_sts(uint32_t addr, uint32_t a, uint32_t b, ui
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-// VEC: largest of 4, 2, 1 that divides Mz (elements between possible row changes).  btab: the
-// frequency factors stay in shared memory (else they are formed when a row of elements begins).
-template <int VEC>
-__global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, DevState D, int S, int SW, int nst, int btab) {
+// The element factors split into an inner table and an outer factor: with yz the inner one is a_y a_z and the
+// outer one the frequency's (see launch_kappa), else a_z and b_f a_y.  VEC: largest of 4, 2, 1 that
+// divides the inner length (elements between possible changes of the outer factor).  btab: the
+// frequency factors stay in shared memory (else they are formed where a row of elements begins).
+// TA: A goes through tensor memory (two words per element and digit pair, the accumulators leave half of it
+// free up to 32 columns of V~), else through shared memory.  nsa, nsb: slots of the A and the B ring.
+template <int VEC, bool TA>
+__global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, DevState D, int S, int SW, int nsa, int nsb, int yz,
+                                                     int btab) {
     extern __shared__ __align__(1024) unsigned char smx[];
     const int P = Pm.P, J = G.J, Nz = G.Nz, My = G.My, Mz = G.Mz, Nm = My * Mz, Nf = G.Nf;
     const int Nh = kx_elements(G), Fh = btab ? kx_freqs(G) : 0;
     const int N1 = 2 * SW, NCk = kx_chunks(Nh);
-    const int nfac = My + ((Mz + 1) & ~1) + Fh;
-    const uint32_t bbytes = kx_bbytes(SW), stage = KX_A + bbytes;
-    // steering factors of the 128 particles: a_y [My], a_z (pairs of elements for VEC > 1), b [Fh]
-    float4* fy = reinterpret_cast<float4*>(smx + (size_t)nst * stage);
-    float4* fz = fy + (size_t)My * 128;
-    float4* fb = fz + (size_t)((Mz + 1) & ~1) * 128;
+    const int Mi = yz ? Nm : Mz, Mo = yz ? 1 : My;                       // inner and outer elements of a frequency
+    const int nfac = kx_factors(G, yz) + Fh;
+    const uint32_t bbytes = kx_bbytes(SW), bring = TA ? 0 : nsa * KX_A;
+    // steering factors of the 128 particles: a_y [My] without yz, the inner table (pairs of elements for
+    // VEC > 1), b [Fh]
+    float4* fy = reinterpret_cast<float4*>(smx + bring + (size_t)nsb * bbytes);
+    float4* fz = fy + (size_t)(yz ? 0 : My) * 128;
+    float4* fb = fz + (size_t)((Mi + 1) & ~1) * 128;
     float4* ctab = fy + (size_t)nfac * 128;                              // [256]
     float4* exs = ctab + 256;                                            // [KX_NG][128] |h|^2 (grid, rest), dev
     float4* exr = exs + KX_NG * 128;                                     // [128] u^H r0
     float* ssc = reinterpret_cast<float*>(exr + 128);                    // [3][64] column scales (unit mod 3: fetched one unit ahead, read one behind)
     uint64_t* mb = reinterpret_cast<uint64_t*>(ssc + 3 * 64);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mb + 2 * KX_NST_MAX + 4);
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(mb + 4 * KX_NS_MAX + 4);
     volatile int* sbad = reinterpret_cast<volatile int*>(tslot + 1);
-    const uint32_t mfull = tc::smem_u32(mb), mempty = mfull + 8 * KX_NST_MAX;   // slot filled; its MMAs done
-    const uint32_t maccf = mempty + 8 * KX_NST_MAX, macce = maccf + 16;         // accumulator set complete; read
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nacc = 8 * N1 <= 512 ? 2 : 1;                              // accumulator sets of 4 N1 columns
-    uint32_t ncols = 32;
+    const uint32_t afull = tc::smem_u32(mb), aempty = afull + 8 * KX_NS_MAX;   // A slot filled; its MMAs done
+    const uint32_t bfull = aempty + 8 * KX_NS_MAX, bempty = bfull + 8 * KX_NS_MAX;
+    const uint32_t maccf = bempty + 8 * KX_NS_MAX, macce = maccf + 16;         // accumulator set complete; read
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int nacc = 8 * N1 <= (TA ? KX_ACOL : 512) ? 2 : 1;             // accumulator sets of 4 N1 columns
+    uint32_t ncols = TA ? 512 : 32;
     while (ncols < (uint32_t)(nacc * 4 * N1)) ncols *= 2;
     if (warp == 0) tc::tmem_alloc(tslot, ncols);
     if (tid == 0) {
-        for (int i = 0; i < nst; ++i) {
-            tc::mbar_init(mfull + 8 * i, KX_PT / 32 + 1);    // every producer warp and the B copy
-            tc::mbar_init(mempty + 8 * i, 1);
+        for (int i = 0; i < KX_NS_MAX; ++i) {
+            tc::mbar_init(afull + 8 * i, KX_PT / 64);        // the warps of the chunk's team
+            tc::mbar_init(aempty + 8 * i, 1);
+            tc::mbar_init(bfull + 8 * i, 1);
+            tc::mbar_init(bempty + 8 * i, 1);
         }
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(maccf + 8 * i, 1);
@@ -313,90 +356,123 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
     // a wait that gives up marks the block bad: nobody waits any more, every loop runs out
     auto wait = [&](uint32_t mbar, uint32_t parity) {
-        if (*sbad) return;
-        if (!tc::mbar_wait(mbar, parity & 1u, KX_WAIT)) *sbad = 1;
+        if (tc::mbar_try(mbar, parity & 1u)) return true;
+        for (int i = 0; i < KX_WAIT; ++i) {
+            if (*sbad) return false;
+            if (tc::mbar_try(mbar, parity & 1u)) return true;
+        }
+        *sbad = 1;
+        return false;
     };
     const int ptiles = (P + 127) / 128, items = S * ptiles;
     const int nit = (int)blockIdx.x < items ? (items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int units = nit * J;                   // (item, j) in order
     const uint32_t ring = tc::smem_u32(smx);
-    if (warp == KX_PT / 32) {
-        // ---- issuing thread: B copies and MMAs
+    if (warp == KX_PT / 32 + 1) {
+        // ---- copying thread: the chunks of B, in order; those of an item are contiguous
         if (lane == 0) {
-            const int total = units * NCk;
-            int li = 0, lj = 0, lk = 0, ls = 0;  // load cursor: item, j, chunk, slot
-            auto load = [&]() {
-                const int s = (blockIdx.x + li * gridDim.x) / ptiles;
-                const unsigned char* src = D.kB + (((size_t)s * J + lj) * NCk + lk) * bbytes;
-                tc::mbar_expect_tx(mfull + 8 * ls, bbytes);
-                tc::bulk_g2s(ring + ls * stage + KX_A, src, bbytes, mfull + 8 * ls);
-                if (++ls == nst) ls = 0;
-                if (++lk == NCk) { lk = 0; if (++lj == J) { lj = 0; ++li; } }
-            };
-            int loaded = 0;
-            for (; loaded < min(nst, total); ++loaded) load();
-            int n = 0;
-            for (int u = 0; u < units && !*sbad; ++u) {
-                const int set = nacc == 2 ? (u & 1) : 0, use = nacc == 2 ? (u >> 1) : u;
-                if (use > 0) wait(macce + 8 * set, use - 1);
-                const uint32_t acc0 = tmem + (uint32_t)(set * 4 * N1);
-                for (int kc = 0; kc < NCk && !*sbad; ++kc, ++n) {
-                    const int st = n % nst;
-                    wait(mfull + 8 * st, n / nst);
-                    if (*sbad) break;
-                    tc::fence_after_sync();
-                    const uint32_t aB = ring + st * stage, bB = aB + KX_A;
-                    #pragma unroll
-                    for (int ks = 0; ks < KX_KC / 16; ++ks) {
-                        #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint64_t da = tc::smem_desc(aB + i * (128 * KX_KC * 2) + ks * 256, 128, KX_KC * 16);
-                            const int cols = (4 - i) * N1;
-                            for (int c0 = 0; c0 < cols; c0 += 256) {
-                                const int nn = min(256, cols - c0);
-                                const uint64_t db = tc::smem_desc(bB + c0 * KX_KC * 2 + ks * 256, 128, KX_KC * 16);
-                                tc::mma_bf16(acc0 + (uint32_t)(i * N1 + c0), da, db, tc::idesc_bf16_f32(128, nn),
-                                             kc > 0 || ks > 0 || i > 0);
-                            }
-                        }
-                    }
-                    tc::mma_commit(mempty + 8 * st);
-                    if (kc == NCk - 1) tc::mma_commit(maccf + 8 * set);
-                    // the slot of chunk n - 1 takes chunk n - 1 + nst once its MMAs are done
-                    if (n >= 1 && n - 1 + nst < total) {
-                        wait(mempty + 8 * ((n - 1) % nst), (n - 1) / nst);
-                        if (*sbad) break;
-                        load();
-                        ++loaded;
-                    }
+            int st = 0, use = 0, loaded = 0;
+            bool ok = true;
+            for (int it = 0; it < nit && ok; ++it) {
+                const int s = (blockIdx.x + it * gridDim.x) / ptiles;
+                const unsigned char* src = D.kB + (size_t)s * J * NCk * bbytes;
+                for (int c = 0; c < J * NCk; ++c, src += bbytes) {
+                    const uint32_t bar = bfull + 8 * st;
+                    if (use > 0 && !(ok = wait(bempty + 8 * st, use - 1))) break;
+                    tc::mbar_expect_tx(bar, bbytes);
+                    tc::bulk_g2s(ring + bring + st * bbytes, src, bbytes, bar);
+                    ++loaded;
+                    if (++st == nsb) { st = 0; ++use; }
                 }
             }
-            // after a wait that gave up: let the copies and MMAs in flight land (bounded)
-            if (*sbad) {
-                for (int m = max(0, loaded - nst); m < loaded; ++m) tc::mbar_wait(mfull + 8 * (m % nst), (m / nst) & 1, KX_WAIT);
-                for (int m = max(0, n - nst); m < n; ++m) tc::mbar_wait(mempty + 8 * (m % nst), (m / nst) & 1, KX_WAIT);
+            // after a wait that gave up: let the copies in flight land (bounded)
+            if (!ok || *sbad)
+                for (int m = max(0, loaded - nsb); m < loaded; ++m) tc::mbar_wait(bfull + 8 * (m % nsb), (m / nsb) & 1, KX_WAIT);
+        }
+        __syncwarp();
+    } else if (warp == KX_PT / 32) {
+        // ---- issuing warp.  The MMAs take their descriptors from uniform registers: the loop is uniform over
+        // the warp and one elected lane issues (a lane alone took ~180 clocks per MMA to move them)
+        {
+            // descriptors: the address is in the low word, which an offset leaves without a carry
+            const uint64_t a0 = tc::smem_desc(ring, 128, KX_KC * 16), b0 = tc::smem_desc(ring + bring, 128, KX_KC * 16);
+            const uint32_t hi = (uint32_t)(a0 >> 32);
+            auto desc = [&](uint32_t lo) { return ((uint64_t)hi << 32) | lo; };
+            // A's digit i against B's first 4 - i digit slices: at most 256 columns per MMA (a second part beyond 32
+            // columns of V~ for the first digit, beyond 40 for the second)
+            const uint32_t id0 = tc::idesc_bf16_f32(128, min(256, 4 * N1)), id1 = tc::idesc_bf16_f32(128, min(256, 3 * N1)),
+                           id2 = tc::idesc_bf16_f32(128, 2 * N1), id3 = tc::idesc_bf16_f32(128, N1),
+                           id02 = tc::idesc_bf16_f32(128, max(16, 4 * N1 - 256)), id12 = tc::idesc_bf16_f32(128, max(16, 3 * N1 - 256));
+            const bool two1 = 3 * N1 > 256;
+            int sa = 0, ua = 0, sb = 0, ub = 0, issued = 0;
+            bool ok = true;
+            // (every loop runs to its end, past a wait that gave up without issuing: it stays uniform)
+            for (int u = 0; u < units; ++u) {
+                const int set = nacc == 2 ? (u & 1) : 0, turn = nacc == 2 ? (u >> 1) : u;
+                if (turn > 0) ok = __all_sync(0xffffffffu, ok && wait(macce + 8 * set, turn - 1));
+                const uint32_t acc = tmem + (uint32_t)(set * 4 * N1), acc1 = acc + N1, acc2 = acc + 2 * N1, acc3 = acc + 3 * N1;
+                for (int kc = 0; kc < NCk; ++kc) {
+                    ok = __all_sync(0xffffffffu, ok && wait(bfull + 8 * sb, ub) && wait(afull + 8 * sa, ua));
+                    tc::fence_after_sync();
+                    const uint32_t da = (uint32_t)a0 + sa * (KX_A >> 4), db = (uint32_t)b0 + sb * (bbytes >> 4);
+                    const uint32_t ts = tmem + KX_ACOL + sa * (2 * KX_KC);
+                    if (ok && tc::elect_one()) {
+                        #pragma unroll
+                        for (int ks = 0; ks < KX_KC / 16; ++ks) {
+                            const uint64_t b = desc(db + 16 * ks), b2 = desc(db + 16 * ks + 256 * KX_KC * 2 / 16);
+                            auto mma = [&](int i, uint32_t col, uint64_t bd, uint32_t id, bool add) {
+                                if constexpr (TA) tc::mma_bf16_ta(col, ts + i * (KX_KC / 2) + 8 * ks, bd, id, add);
+                                else tc::mma_bf16(col, desc(da + i * (128 * KX_KC * 2 / 16) + 16 * ks), bd, id, add);
+                            };
+                            mma(0, acc, b, id0, kc > 0 || ks > 0);
+                            if constexpr (!TA) mma(0, acc + 256, b2, id02, kc > 0 || ks > 0);
+                            mma(1, acc1, b, id1, true);
+                            if constexpr (!TA) if (two1) mma(1, acc1 + 256, b2, id12, true);
+                            mma(2, acc2, b, id2, true);
+                            mma(3, acc3, b, id3, true);
+                        }
+                        tc::mma_commit(aempty + 8 * sa);
+                        tc::mma_commit(bempty + 8 * sb);
+                        if (kc == NCk - 1) tc::mma_commit(maccf + 8 * set);
+                    }
+                    __syncwarp();
+                    issued += ok ? 1 : 0;
+                    if (++sa == nsa) { sa = 0; ++ua; }
+                    if (++sb == nsb) { sb = 0; ++ub; }
+                }
             }
+            // after a wait that gave up: let the MMAs in flight land (bounded)
+            if (!ok || *sbad)
+                for (int m = max(0, issued - nsa); m < issued; ++m) tc::mbar_wait(aempty + 8 * (m % nsa), (m / nsa) & 1, KX_WAIT);
         }
         __syncwarp();
     } else {
         // ---- producers and epilogue
         const int grp = warp >> 2, row = tid & 127;
         const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t arow = (uint32_t)((row >> 3) * (KX_KC * 16) + (row & 7) * 16 + grp * 128);
+        const int team = grp >> 1, hh = grp & 1;  // a team fills every other chunk, eight elements per thread
+        const uint32_t arow = (uint32_t)((row >> 3) * (KX_KC * 16) + (row & 7) * 16 + hh * 256);
         float GM = 1.5f;                          // grid of the |h|^2 sum: |h|^2 <= Nz
         for (int v = 1; v < 4 * Nz; v *= 2) GM *= 2.0f;
-        // first element of this group's four in chunk 0, and the step of 16 elements, in (f, y, m)
-        const int f_0 = 4 * grp / Nm, y_0 = (4 * grp - f_0 * Nm) / Mz, m_0 = 4 * grp - f_0 * Nm - y_0 * Mz;
-        const int f_s = 16 / Nm, y_s = (16 - f_s * Nm) / Mz, m_s = 16 - f_s * Nm - y_s * Mz;
+        // two chunks (32 elements) on, in (f, outer, inner)
+        const int f_s = 32 / Nm, y_s = (32 - f_s * Nm) / Mi, m_s = 32 - f_s * Nm - y_s * Mi;
         float pA = 0.f, pDev = 0.f, pH0 = 0.f, pL0 = 0.f;   // previous unit: amplitude, |u|^2 - Nz (this group's part), carrier
         ff delta{0.f, 0.f};
-        // reads the accumulators of unit u, and one group per item evaluates Delta
+        bool dead = false;                        // a wait gave up: nothing is stored or announced any more
+        int e_it = -1, e_j = J - 1, e_s = 0, e_p = 0;   // item, PA, PF and particle of the epilogue's unit
+        // reads the accumulators of unit u (in order), and one group per item evaluates Delta
         auto epilogue = [&](int u) {
-            const int it = u / J, j = u - it * J;
-            const int item = blockIdx.x + it * gridDim.x, s = item / ptiles, p = (item - s * ptiles) * 128 + row;
+            if (++e_j == J) {
+                e_j = 0;
+                ++e_it;
+                const int item = blockIdx.x + e_it * gridDim.x;
+                e_s = item / ptiles;
+                e_p = (item - e_s * ptiles) * 128 + row;
+            }
+            const int it = e_it, j = e_j, s = e_s, p = e_p;
             const int set = nacc == 2 ? (u & 1) : 0, use = nacc == 2 ? (u >> 1) : u;
             const float* scl = ssc + (u % 3) * 64;
             const bool fin = it % KX_NG == grp;
@@ -407,7 +483,7 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
                 gm = ph[3 * (size_t)P]; mr = ph[4 * (size_t)P]; mi = ph[5 * (size_t)P];
                 kc = D.kC[s * J + j];
             }
-            wait(maccf + 8 * set, use);
+            if (!wait(maccf + 8 * set, use)) dead = true;
             __syncwarp();
             tc::fence_after_sync();
             const uint32_t acc0 = tlane + (uint32_t)(set * 4 * N1);
@@ -423,9 +499,10 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
                     auto col2 = [&](int i, int q) { return f2_pack(__uint_as_float(g[i][q]), __uint_as_float(g[i][q + 1])); };
                     #pragma unroll
                     for (int q = 0; q < 8; q += 2) {     // two columns at a time
-                        // g_0 + g_1 exactly, the rest onto its error
-                        const f2x a = col2(0, q), b = col2(1, q), t = f2_add(a, b), bb = f2_sub(t, a);
-                        const f2x e = f2_add(f2_add(f2_sub(a, f2_sub(t, bb)), f2_sub(b, bb)), f2_add(col2(2, q), col2(3, q)));
+                        // g_0 + g_1 exactly (g_0, a multiple of 2^-14, is one of g_1's last place: |g_1| < 2^10), the
+                        // rest onto the error
+                        const f2x a = col2(0, q), b = col2(1, q), t = f2_add(a, b);
+                        const f2x e = f2_add(f2_sub(b, f2_sub(t, a)), f2_add(col2(2, q), col2(3, q)));
                         if (q == 6 && c0 + 8 == SW) {    // u^H r0 (its scale in the table is zero)
                             uint32_t lo, th, eh;
                             f2_unpack(t, lo, th);
@@ -444,7 +521,7 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
             }
             tc::fence_before_sync();
             __syncwarp();
-            if (lane == 0) kx_arrive(macce + 8 * set);
+            if (lane == 0 && !dead) kx_arrive(macce + 8 * set);
             uint32_t g0, g1, r0, r1;
             f2_unpack(hg, g0, g1);
             f2_unpack(hr, r0, r1);
@@ -478,122 +555,160 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
         };
         float4 ngeo = make_float4(1.f, 0.f, 0.f, 0.f);
         float2 ngl = make_float2(0.f, 0.f);
-        auto fetch = [&](int u) {                 // geometry record of unit u
-            const int it = u / J, j = u - it * J;
-            const int item = blockIdx.x + it * gridDim.x, s = item / ptiles, p = (item - s * ptiles) * 128 + row;
+        int g_it = -1, g_j = J - 1, g_s = 0, g_p = 0;
+        auto fetch = [&](int u) {                 // geometry record of unit u (in order)
+            if (++g_j == J) {
+                g_j = 0;
+                ++g_it;
+                const int item = blockIdx.x + g_it * gridDim.x;
+                g_s = item / ptiles;
+                g_p = (item - g_s * ptiles) * 128 + row;
+            }
+            const int j = g_j, s = g_s, p = g_p;
             const size_t gi = ((size_t)s * J + j) * P + min(p, P - 1);
             ngeo = D.geo[gi];
             ngl = D.geo_lo[gi];
             if (tid < 64) ssc[(u % 3) * 64 + tid] = tid < SW - 1 ? D.kSc[((size_t)s * J + j) * 64 + tid] : 0.f;
         };
         if (units > 0) fetch(0);
-        int st = 0, use = 0;                      // ring slot and its turn
+        int st = team, use = 0;                   // A slot and its turn of this team's next chunk (nsa >= 2)
         for (int u = 0; u < units; ++u) {
             const float4 grec = ngeo;
             const float2 grl = ngl;
             const float A = G.amp_c / (grec.x + grec.y);
             float dev = 0.f;
-            // the antenna factors of a symmetric layout come in conjugate pairs
-            auto antenna = [&](int i, bool isz) {
-                const float c = isz ? G.pz_l[i] : G.py_l[i], cl = isz ? G.pz_lo[i] : G.py_lo[i];
-                const float uu = isz ? grec.w : grec.z, ul = isz ? grl.y : grl.x;
-                const float t = __fmul_rn(c, uu);
+            auto cis = [&](float c, float e) {
                 float2 hi, lo;
-                cis_pair(ctab, t, fmaf(c, ul, fmaf(cl, uu, fmaf(c, uu, -t))), hi, lo);
+                cis_pair(ctab, c, e, hi, lo);
                 return make_float4(hi.x, hi.y, lo.x, lo.y);
             };
-            auto put_z = [&](int m, float4 a) {
-                if (VEC == 1) { fz[m * 128 + row] = a; return; }
-                float* o = reinterpret_cast<float*>(fz + (m & ~1) * 128 + row) + (m & 1);   // (hx, hx', hy, hy'), then lo
-                o[0] = a.x; o[2] = a.y;
-                o[512] = a.z; o[514] = a.w;
+            auto phase = [&](bool isz, int i, float& t, float& e) {
+                const float c = isz ? G.pz_l[i] : G.py_l[i], cl = isz ? G.pz_lo[i] : G.py_lo[i];
+                const float uu = isz ? grec.w : grec.z, ul = isz ? grl.y : grl.x;
+                t = __fmul_rn(c, uu);
+                e = fmaf(c, ul, fmaf(cl, uu, fmaf(c, uu, -t)));
+            };
+            auto inner = [&](int i) {             // a_z, or a_y a_z
+                float t, e;
+                if (!yz) {
+                    phase(true, i, t, e);
+                } else {
+                    const int yi = i / Mz;
+                    float t1, e1, t2, e2;
+                    phase(false, yi, t1, e1);
+                    phase(true, i - yi * Mz, t2, e2);
+                    two_sum(t1, t2, t, e);
+                    e += e1 + e2;
+                }
+                return cis(t, e);
+            };
+            auto conj4 = [](float4 a) { return make_float4(a.x, -a.y, a.z, -a.w); };
+            auto put2 = [&](int m, float4 a, float4 b) {  // (hx, hx', hy, hy'), then the low parts
+                fz[m * 128 + row] = make_float4(a.x, b.x, a.y, b.y);
+                fz[(m + 1) * 128 + row] = make_float4(a.z, b.z, a.w, b.w);
             };
             auto freq = [&](int f) {              // b_f, without the carrier
                 float h, l;
                 ff_frac_mul2(grec.x, grec.y, G.fc_hi[f], G.fc_lo[f], h, l);
-                float2 hi, lo;
-                cis_pair(ctab, -h, -l, hi, lo);
-                return make_float4(hi.x, hi.y, lo.x, lo.y);
+                return cis(-h, -l);
             };
             auto unit_dev = [&](float4 a) { return pair_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w)); };
             const float fdup = G.sym ? 2.0f : 1.0f;
             kx_bar();                             // every group is done with the previous unit's factors
-            const int hy = G.sym ? (My + 1) / 2 : My, hz = G.sym ? (Mz + 1) / 2 : Mz;
-            for (int i = grp; i < hy + hz + Fh; i += KX_NG) {
-                if (i < hy) {
-                    const float4 a = antenna(i, false);
-                    const int i2 = My - 1 - i;
-                    const bool two = G.sym && i2 != i;
-                    fy[i * 128 + row] = a;
-                    if (two) fy[i2 * 128 + row] = make_float4(a.x, -a.y, a.z, -a.w);
+            // the antenna factors of a symmetric layout come in conjugate pairs: items of the inner table
+            // (two elements each for VEC > 1), then a_y, then b
+            constexpr int IV = VEC > 1 ? 2 : 1;
+            const int nin = Mi / IV, hin = G.sym ? (nin + 1) / 2 : nin, hy = yz ? 0 : G.sym ? (My + 1) / 2 : My;
+            const float win = (float)(Nf * Mo);
+            for (int i = grp; i < hin + hy + Fh; i += KX_NG) {
+                if (i < hin) {
+                    const int m = IV * i, m2 = Mi - IV - m;       // the mirrored item
+                    const float4 a = inner(m);
+                    float d = unit_dev(a);
+                    if (VEC > 1) {
+                        const bool self = G.sym && m2 == m;
+                        const float4 b = self ? conj4(a) : inner(m + 1);
+                        d += unit_dev(b);
+                        const float4 sa = kx_split(a), sb = kx_split(b);
+                        put2(m, sa, sb);
+                        if (G.sym && !self) { put2(m2, conj4(sb), conj4(sa)); d *= 2.0f; }
+                    } else {
+                        const float4 sa = kx_split(a);
+                        fz[m * 128 + row] = sa;
+                        if (G.sym && m2 != m) { fz[m2 * 128 + row] = conj4(sa); d *= 2.0f; }
+                    }
+                    dev = fmaf(win, d, dev);
+                } else if (i < hin + hy) {
+                    const int yi = i - hin, y2 = My - 1 - yi;
+                    float t, e;
+                    phase(false, yi, t, e);
+                    const float4 a = cis(t, e), sa = kx_split(a);
+                    const bool two = G.sym && y2 != yi;
+                    fy[yi * 128 + row] = sa;
+                    if (two) fy[y2 * 128 + row] = conj4(sa);
                     dev = fmaf((float)(Nf * Mz) * (two ? 2.0f : 1.0f), unit_dev(a), dev);
-                } else if (i < hy + hz) {
-                    const int m = i - hy, m2 = Mz - 1 - m;
-                    const float4 a = antenna(m, true);
-                    const bool two = G.sym && m2 != m;
-                    put_z(m, a);
-                    if (two) put_z(m2, make_float4(a.x, -a.y, a.z, -a.w));
-                    dev = fmaf((float)(Nf * My) * (two ? 2.0f : 1.0f), unit_dev(a), dev);
                 } else {
                     // (the middle frequency is 0: no deviation)
-                    const int f = i - hy - hz;
+                    const int f = i - hin - hy;
                     const float4 a = freq(f);
-                    fb[f * 128 + row] = a;
+                    fb[f * 128 + row] = kx_split(a);
                     dev = fmaf((float)Nm * fdup, unit_dev(a), dev);
                 }
             }
             kx_bar();
             if (u + 1 < units) fetch(u + 1);
             bool drained = u == 0;
-            int f = f_0, y = y_0, m = m_0;
-            for (int kc = 0; kc < NCk; ++kc) {
+            const int kc0 = team ^ (u & NCk & 1);  // this team's first chunk of the unit
+            int f = (16 * kc0 + 8 * hh) / Nm, m = 16 * kc0 + 8 * hh - f * Nm, y = m / Mi;
+            m -= y * Mi;
+            for (int kc = kc0; kc < NCk; kc += 2) {
                 // a slot of this unit's own ring turn frees only once the previous unit's
                 // accumulators are read
-                if (!drained && kc >= nst) { epilogue(u - 1); drained = true; }
-                if (use > 0) wait(mempty + 8 * st, use - 1);
-                const int k = 16 * kc + 4 * grp;
-                uint32_t d[4][4];                 // [digit][element]
-                #pragma unroll
-                for (int i = 0; i < 4; ++i) d[i][0] = d[i][1] = d[i][2] = d[i][3] = 0u;
+                if (!drained && kc >= nsa) { epilogue(u - 1); drained = true; }
+                const int k = 16 * kc + 8 * hh;
+                uint32_t d[4][8];                 // [digit][element]
                 if (k < Nh) {
                     int yy = y, mm = m, ff_ = f;
                     float4 b;
                     auto set_b = [&](int e) {
                         if (btab) { b = fb[ff_ * 128 + row]; return; }
                         b = freq(ff_);
-                        const int cnt = min(min((ff_ + 1) * Nm, 16 * kc + 4 * grp + 4), Nh) - (k + e);
+                        const int cnt = min(min((ff_ + 1) * Nm, k + 8), Nh) - (k + e);
                         dev = fmaf((float)cnt * fdup, unit_dev(b), dev);
+                        b = kx_split(b);
                     };
-                    auto step = [&](int e, int by) {   // to element e (by elements on); true if the row changed
+                    auto step = [&](int e, int by) {   // to element e (by elements on); true if the outer factor changed
                         mm += by;
-                        if (mm < Mz) return false;
+                        if (mm < Mi) return false;
                         mm = 0;
-                        if (++yy == My) {
+                        if (++yy == Mo) {
                             yy = 0;
                             ++ff_;
                             if (k + e < Nh) set_b(e);
                         }
-                        return true;
+                        return k + e < Nh;
                     };
+                    auto outer = [&]() { return yz ? b : kx_mul_split(b, fy[yy * 128 + row]); };
                     set_b(0);
-                    float4 w = pair_mul_fx(b, fy[yy * 128 + row]);
+                    float4 w = outer();
                     KxW w2;
                     if (VEC > 1) w2 = kx_w(w, w);
                     #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
+                    for (int q = 0; q < 4; ++q) {
                         KxU a;
                         if (VEC > 1) {
-                            if (VEC == 2 && q == 1 && step(2, 2) && k + 2 < Nh) {
-                                w = pair_mul_fx(b, fy[yy * 128 + row]);
+                            const bool at = VEC == 4 ? q == 2 : q > 0;   // the outer factor may change here
+                            if (at && step(2 * q, VEC)) {
+                                w = outer();
                                 w2 = kx_w(w, w);
                             }
-                            const int m2 = VEC == 4 ? mm + 2 * q : mm;
+                            const int m2 = VEC == 4 ? mm + 2 * (q & 1) : mm;
                             const float4 h = fz[m2 * 128 + row], l = fz[(m2 + 1) * 128 + row];
                             a = KxU{f2_pack(h.x, h.y), f2_pack(h.z, h.w), f2_pack(l.x, l.y), f2_pack(l.z, l.w)};
                         } else {
-                            if (q == 1 && step(2, 1) && k + 2 < Nh) w = pair_mul_fx(b, fy[yy * 128 + row]);
+                            if (q > 0 && step(2 * q, 1)) w = outer();
                             const float4 a0 = fz[mm * 128 + row], w0 = w;
-                            if (step(2 * q + 1, 1) && k + 2 * q + 1 < Nh) w = pair_mul_fx(b, fy[yy * 128 + row]);
+                            if (step(2 * q + 1, 1)) w = outer();
                             const float4 a1 = fz[mm * 128 + row];
                             w2 = kx_w(w0, w);
                             a = KxU{f2_pack(a0.x, a1.x), f2_pack(a0.y, a1.y), f2_pack(a0.z, a1.z), f2_pack(a0.w, a1.w)};
@@ -606,25 +721,46 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
                             d[i][2 * q + 1] = dd[i][1];
                         }
                     }
-                    if (k + 4 > Nh) {             // elements past the last one
+                    if (k + 8 > Nh) {             // elements past the last one
                         #pragma unroll
-                        for (int e = 1; e < 4; ++e)
+                        for (int e = 1; e < 8; ++e)
                             if (k + e >= Nh) d[0][e] = d[1][e] = d[2][e] = d[3][e] = 0u;
                     }
+                } else {
+                    #pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        #pragma unroll
+                        for (int e = 0; e < 8; ++e) d[i][e] = 0u;
                 }
-                const uint32_t dst = ring + st * stage + arow;
-                #pragma unroll
-                for (int i = 0; i < 4; ++i) kx_sts(dst + i * (128 * KX_KC * 2), d[i][0], d[i][1], d[i][2], d[i][3]);
-                tc::fence_async_smem();
+                // the digits are formed before the slot is free, so that the wait costs little
+                if (use > 0 && !wait(aempty + 8 * st, use - 1)) dead = true;
+                if constexpr (TA) {
+                    __syncwarp();
+                    tc::fence_after_sync();
+                    const uint32_t dst = tlane + KX_ACOL + st * (2 * KX_KC) + 8 * hh;
+                    #pragma unroll
+                    for (int i = 0; i < 4; ++i) tc::tmem_st8(dst + i * (KX_KC / 2), d[i]);
+                    tc::tmem_st_wait();
+                    tc::fence_before_sync();
+                } else {
+                    const uint32_t dst = ring + st * KX_A + arow;
+                    #pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        kx_sts(dst + i * (128 * KX_KC * 2), d[i][0], d[i][1], d[i][2], d[i][3]);
+                        kx_sts(dst + i * (128 * KX_KC * 2) + 128, d[i][4], d[i][5], d[i][6], d[i][7]);
+                    }
+                    tc::fence_async_smem();
+                }
                 __syncwarp();
-                if (lane == 0) kx_arrive(mfull + 8 * st);
-                if (++st == nst) { st = 0; ++use; }
-                // 16 elements on
+                if (lane == 0 && !dead) kx_arrive(afull + 8 * st);
+                st += 2;
+                if (st >= nsa) { st -= nsa; ++use; }
+                // two chunks on
                 m += m_s;
                 y += y_s;
                 f += f_s;
-                if (m >= Mz) { m -= Mz; ++y; }
-                if (y >= My) { y -= My; ++f; }
+                if (m >= Mi) { m -= Mi; ++y; }
+                if (y >= Mo) { y -= Mo; ++f; }
             }
             if (!drained) epilogue(u - 1);
             pA = A;
@@ -772,24 +908,36 @@ int launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S
         k_kappa_cc<<<dim3((Pm.P + KCC_T - 1) / KCC_T, S), KCC_T, smem, st>>>(G, Pm, D, S, SCA, SW, V);
         return 2;
     }
-    // Frequency factors in shared memory where several rows of four elements share one and a ring of
-    // three slots still fits; else as many slots as fit, up to four (two always do: 128 KB of
-    // ring and 80 KB of factors for the largest array and SW = 64)
-    const size_t stage = KX_A + kx_bbytes(SW), limit = 227 * 1024;
-    const int nant2 = G.My + ((G.Mz + 1) & ~1), Fh = kx_freqs(G);
-    const int btab = G.My * G.Mz > 4 && kx_smem_fixed(nant2 + Fh) + 3 * stage <= limit;
-    const size_t fixed = kx_smem_fixed(nant2 + (btab ? Fh : 0));
-    int nst = KX_NST_MAX;
-    while (nst > 2 && fixed + nst * stage > limit) --nst;
-    const size_t smem = fixed + nst * stage;
+    // Up to 32 columns A goes through tensor memory: MMAs of few columns are bound by reading A from shared
+    // memory there (128 x 256, 192, 128 and 64 columns: 333 clocks against 320 of tensor memory; 64, 48,
+    // 32 and 16: 172 against 82), and the ring leaves room for the frequency factors.
+    // The inner table holds a_y a_z where at least eight frequencies use it (its My Mz / 2 sincos per
+    // particle against a product of pairs per four elements); the frequency factors stay in shared
+    // memory where more than four elements share one.  Both only where two slots of each ring still fit,
+    // and without them two always do (128 KB of rings and 80 KB of factors for the largest array and
+    // SW = 64); the rings take what is left, up to four slots, A's first (its turn-around is longer).
+    const bool ta = SW <= 32;
+    const size_t asl = ta ? 0 : KX_A, bsl = kx_bbytes(SW), limit = 227 * 1024;
+    const int Nm = G.My * G.Mz, Fh = kx_freqs(G);
+    auto fits = [&](int yz, int fb) { return kx_smem_fixed(kx_factors(G, yz) + fb) + 2 * (asl + bsl) <= limit; };
+    const int yz = G.Nf >= 8 && fits(1, Nm > 4 ? Fh : 0);
+    const int btab = Nm > 4 && fits(yz, Fh);
+    const size_t fixed = kx_smem_fixed(kx_factors(G, yz) + (btab ? Fh : 0));
+    int nsa = KX_NS_MAX, nsb = KX_NS_MAX;
+    if (!ta) nsb = 2;
+    while (nsb > 2 && fixed + nsb * bsl > limit) --nsb;
+    while (nsa > 2 && fixed + nsa * asl + nsb * bsl > limit) --nsa;
+    while (nsb < KX_NS_MAX && fixed + nsa * asl + (nsb + 1) * bsl <= limit) ++nsb;
+    const size_t smem = fixed + nsa * asl + nsb * bsl;
     const int items = S * ((Pm.P + 127) / 128), grid = items < sm_count() ? items : sm_count();
     auto go = [&](auto kernel) {
         smem_allow_max((const void*)kernel);
-        kernel<<<grid, KX_T, smem, st>>>(G, Pm, D, S, SW, nst, btab);
+        kernel<<<grid, KX_T, smem, st>>>(G, Pm, D, S, SW, nsa, nsb, yz, btab);
     };
-    if (G.Mz % 4 == 0) go(k_kappa_x<4>);
-    else if (G.Mz % 2 == 0) go(k_kappa_x<2>);
-    else go(k_kappa_x<1>);
+    const int Mi = yz ? Nm : G.Mz;
+    if (Mi % 4 == 0) ta ? go(k_kappa_x<4, true>) : go(k_kappa_x<4, false>);
+    else if (Mi % 2 == 0) ta ? go(k_kappa_x<2, true>) : go(k_kappa_x<2, false>);
+    else ta ? go(k_kappa_x<1, true>) : go(k_kappa_x<1, false>);
     return 2;
 }
 
