@@ -48,7 +48,8 @@ __device__ __forceinline__ int is_half(int i, int n, int h, bool& c) { c = i >= 
 // steering elements as (hi, lo) pairs (~1e-9) with the products of the high parts summed exactly on
 // a grid fixed per (p, j).  Below 24 PFs every particle is evaluated (the FP32 warp kernel and the
 // block-per-particle repair of the particles it flagged took 8.7 ms at 10 PFs x 30000 particles,
-// Nz = 160; this takes 1.25 ms); from 24 PFs on the particles k_iota_select queues, with four warps
+// Nz = 160; this 1.32 ms with index divisions, a search per triangle entry and a reduction per PF, 0.99
+// without); from 24 PFs on the particles k_iota_select queues, with four warps
 // per team, since few working sets of that size fit an SM.
 // Bound: FP32 issue, the residual's ~50 instructions per (s, half element).
 constexpr int IF_WMAX = 16;
@@ -61,15 +62,23 @@ __host__ __device__ inline IfPlan if_plan(const DevGeom& G, int S) {
     p.fac = o; o += (size_t)S * d.hf * sizeof(float4);
     p.ct = o; o += (size_t)S * d.Nmh * sizeof(float4);
     p.z = o; o += (size_t)d.Nh * 2 * sizeof(float4);            // P (hi, lo), Q (hi, lo)
+    p.vec = o; o += (size_t)S * (sizeof(float4) + sizeof(float2) + sizeof(ff) + 2 * sizeof(float));   // w, g | pivots | dA, 1/L_kk
     p.K = o; o += (size_t)S * (S + 1) / 2 * sizeof(ff);
-    p.vec = o; o += (size_t)S * (2 * sizeof(float2) + sizeof(ff) + 2 * sizeof(float));   // w, g | pivots | dA, 1/L_kk
     p.L = o; o += (size_t)S * (S + 1) / 2 * sizeof(float);
     p.warp = (o + 15) & ~(size_t)15;
     return p;
 }
 constexpr int IF_TEAM_MAX = 4;           // warps of a team
+// n / d by a multiplication (n d < 2^32)
+struct IsDiv { uint32_t m, d; };
+__device__ __forceinline__ IsDiv is_div(int d) { return IsDiv{0xffffffffu / (uint32_t)d + 1u, (uint32_t)d}; }
+__device__ __forceinline__ int operator/(int n, IsDiv v) { return v.d == 1 ? n : (int)__umulhi((uint32_t)n, v.m); }
 constexpr size_t IF_FIXED = 256 * sizeof(float4) + IF_WMAX * (3 * sizeof(double) + sizeof(float)) +
                             IF_WMAX * IF_TEAM_MAX * sizeof(ff) + IF_WMAX * sizeof(float);
+// shared by the block: IF_FIXED, the elements' places [Nh], the triangle's (row, column) [S (S + 1) / 2]
+__host__ __device__ inline size_t if_fixed(const DevGeom& G, int S) {
+    return (IF_FIXED + (size_t)is_dims(G).Nh * sizeof(uint32_t) + (size_t)S * (S + 1) / 2 * sizeof(ushort) + 15) & ~(size_t)15;
+}
 
 // sum_i x_i.x y_i.x + x_i.y y_i.y of unit-modulus pairs: the high parts' products split on a grid of
 // 2^-16 (their sums below 256 exact), remainders and cross terms in FP32
@@ -114,15 +123,17 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
     float* rat = reinterpret_cast<float*>(ies + IF_WMAX);       // [J] sum of squared pivot ratios
     ff* red = reinterpret_cast<ff*>(rat + IF_WMAX) + wid * TW;  // [TW] |r|^2 of the team's warps
     float* gmS = reinterpret_cast<float*>(reinterpret_cast<ff*>(rat + IF_WMAX) + IF_WMAX * IF_TEAM_MAX) + wid;   // residual grid
+    uint32_t* kt = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(smf) + IF_FIXED);   // [Nh] f, index and conjugation of a_y a_z
+    ushort* tri = reinterpret_cast<ushort*>(kt + dm.Nh);        // [S (S + 1) / 2] row, column
     const IfPlan pl = if_plan(G, S);
-    char* base = reinterpret_cast<char*>(smf) + ((IF_FIXED + 15) & ~(size_t)15) + (size_t)wid * pl.warp;
+    char* base = reinterpret_cast<char*>(smf) + if_fixed(G, S) + (size_t)wid * pl.warp;
     float4* fac = reinterpret_cast<float4*>(base + pl.fac);     // [S][hf] b_f, a_y, a_z (half of each)
     float4* ct = reinterpret_cast<float4*>(base + pl.ct);       // [S][Nmh] a_y a_z
     float4* zp = reinterpret_cast<float4*>(base + pl.z);        // [Nh] P, then [Nh] Q, as (hi, lo)
     float4* zq = zp + dm.Nh;
     ff* K = reinterpret_cast<ff*>(base + pl.K);                 // packed lower: A, then its elimination
-    float2* ws = reinterpret_cast<float2*>(base + pl.vec);      // [S] A c pi mu, then w
-    float2* gs = ws + S;                                        // [S] u^H z
+    float4* ws = reinterpret_cast<float4*>(base + pl.vec);      // [S] (A c pi mu), then -2 w, (2 Im w, -2 Re w)
+    float2* gs = reinterpret_cast<float2*>(ws + S);             // [S] u^H z
     ff* piv = reinterpret_cast<ff*>(gs + S);                    // [S]
     float* dA = reinterpret_cast<float*>(piv + S);              // [S] d_s A_s
     float* ild = dA + S;                                        // [S] 1 / L_kk
@@ -132,7 +143,19 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
         lgs[threadIdx.x] = log(D.eta_bar[threadIdx.x]);
         ies[threadIdx.x] = 1.0 / D.eta_bar[threadIdx.x];
     }
+    for (int k = threadIdx.x; k < dm.Nh; k += blockDim.x) {
+        const int f = k / Nm;
+        bool cj;
+        const int ih = is_half(k - f * Nm, Nm, dm.Nmh, cj);
+        kt[k] = (uint32_t)f | ((uint32_t)ih << 15) | (cj ? 0x80000000u : 0u);
+    }
+    for (int t = threadIdx.x; t < S * (S + 1) / 2; t += blockDim.x) {
+        int a, b;
+        is_tri_ab(t, a, b);
+        tri[t] = (ushort)(a | (b << 8));
+    }
     __syncthreads();
+    const IsDiv by_hf = is_div(dm.hf), by_Nmh = is_div(dm.Nmh), by_Mz = is_div(Mz);
     const float* phi = D.phi[D.cur];
     const int count = all ? P : D.flags[0], npair = S * (S + 1) / 2;
     const bool odd = Nz & 1;
@@ -165,6 +188,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                 zj = j;
             }
             const double eb = D.eta_bar[j];
+            const float ebh = (float)eb, ebl = (float)(eb - (double)ebh);
             // per-PF scalars, then the factors as pairs
             for (int s = tt; s < S; s += TT) {
                 const float* ph = phi + (size_t)s * 6 * P + p;
@@ -177,10 +201,11 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                 const float pi = (float)(D.zeta[s * J + j] * D.W[s]);
                 const float gm = ph[3 * (size_t)P], mr = ph[4 * (size_t)P], mi = ph[5 * (size_t)P];
                 dA[s] = A * sqrtf(fmaxf(pi * (gm + (mr * mr + mi * mi) * (1.0f - pi)), 0.0f));
-                ws[s] = cmul(make_float2(A * pi * mr, A * pi * mi), c);
+                const float2 w0 = cmul(make_float2(A * pi * mr, A * pi * mi), c);
+                ws[s] = make_float4(w0.x, w0.y, 0.f, 0.f);
             }
             for (int i = tt; i < S * dm.hf; i += TT) {
-                const int s = i / dm.hf, q = i - s * dm.hf;
+                const int s = i / by_hf, q = i - s * dm.hf;
                 const size_t gi = ((size_t)s * J + j) * P + p;
                 const float4 g = D.geo[gi];
                 float th, tl;
@@ -202,7 +227,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
             }
             team_sync();
             for (int i = tt; i < S * dm.Nmh; i += TT) {
-                const int s = i / dm.Nmh, ym = i - s * dm.Nmh, y = ym / Mz, m = ym - y * Mz;
+                const int s = i / by_Nmh, ym = i - s * dm.Nmh, y = ym / by_Mz, m = ym - y * Mz;
                 const float4* fs = fac + s * dm.hf + dm.Fh;
                 bool cy, cz;
                 const int iy = is_half(y, My, dm.hy, cy), iz = is_half(m, Mz, dm.hz, cz);
@@ -210,34 +235,53 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
             }
             // Gram and A = eta_bar I + D G D, packed
             for (int t = tt; t < npair; t += TT) {
-                int a, b;
-                is_tri_ab(t, a, b);
+                const int a = tri[t] & 255, b = tri[t] >> 8;
                 const float4 *fa = fac + a * dm.hf, *fb = fac + b * dm.hf;
                 const ff g = ff_mul(if_sum(fa, fb, Nf), ff_mul(if_sum(fa + dm.Fh, fb + dm.Fh, My),
                                                                if_sum(fa + dm.Fh + dm.hy, fb + dm.Fh + dm.hy, Mz)));
                 ff v = ff_mul(g, ff_prod(dA[a], dA[b]));
-                if (a == b) v = ff_add(v, ff{(float)eb, (float)(eb - (double)(float)eb)});
+                if (a == b) v = ff_add(v, ff{ebh, ebl});
                 K[t] = v;
                 L[t] = g.hi;
             }
             team_sync();
             // g_s = u_s^H z (FP32: the minimiser's rounding enters at second order)
-            for (int s = wt; s < S; s += TW) {
-                const float4 *fs = fac + s * dm.hf, *cs = ct + s * dm.Nmh;
-                float gr = 0.f, gi = 0.f;
+            for (int s0 = 4 * wt; s0 < S; s0 += 4 * TW) {     // four PFs at a time
+                float g[8];
+                #pragma unroll
+                for (int q = 0; q < 8; ++q) g[q] = 0.f;
+                #pragma unroll 1
                 for (int k = lane; k < dm.Nh; k += 32) {
-                    const int f = k / Nm, ym = k - f * Nm;
-                    bool cj;
-                    const int ih = is_half(ym, Nm, dm.Nmh, cj);
-                    const float4 b = fs[f], c = conj_if(cs[ih], cj);
-                    const float x = fmaf(b.x, c.x, -b.y * c.y), y = fmaf(b.x, c.y, b.y * c.x);
+                    const uint32_t at = kt[k];
                     const float4 pv = zp[k], qv = zq[k];
-                    gr = fmaf(x, pv.x, fmaf(y, qv.y, gr));
-                    gi = fmaf(x, pv.y, fmaf(-y, qv.x, gi));
+                    const float4 *fs = fac + (at & 0x7fff), *cs = ct + ((at >> 15) & 0xffff);
+                    const float sg = (at >> 31) ? -1.0f : 1.0f;
+                    #pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int s = min(s0 + q, S - 1);
+                        const float2 b = *reinterpret_cast<const float2*>(fs + s * dm.hf);
+                        float2 c = *reinterpret_cast<const float2*>(cs + s * dm.Nmh);
+                        c.y *= sg;
+                        const float x = fmaf(b.x, c.x, -b.y * c.y), y = fmaf(b.x, c.y, b.y * c.x);
+                        g[2 * q] = fmaf(x, pv.x, fmaf(y, qv.y, g[2 * q]));
+                        g[2 * q + 1] = fmaf(x, pv.y, fmaf(-y, qv.x, g[2 * q + 1]));
+                    }
                 }
-                gr = warp_sum_f(gr);
-                gi = warp_sum_f(gi);
-                if (lane == 0) gs[s] = make_float2(gr, gi);
+                // the eight sums over lanes at once: halving the values while lanes pair up
+                #pragma unroll
+                for (int o = 16, n = 4; o >= 4; o >>= 1, n >>= 1) {
+                    const bool up = lane & o;
+                    #pragma unroll
+                    for (int q = 0; q < n; ++q) {
+                        const float keep = up ? g[q + n] : g[q], give = up ? g[q] : g[q + n];
+                        g[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                }
+                g[0] += __shfl_xor_sync(0xffffffffu, g[0], 2);
+                g[0] += __shfl_xor_sync(0xffffffffu, g[0], 1);
+                // lane bits 4, 3, 2 select value 4 b4 + 2 b3 + b2
+                const int s = s0 + (((lane >> 4) & 1) << 1) + ((lane >> 3) & 1);
+                if ((lane & 3) == 0 && s < S) reinterpret_cast<float*>(gs + s)[(lane >> 2) & 1] = g[0];
             }
             team_sync();
             // right-hand side t_a = (dA)_a (g_a - sum_b G_ab w0_b): rows lane and lane + 32
@@ -248,8 +292,9 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                 float2 acc = gs[a];
                 for (int b = 0; b < S; ++b) {
                     const float g = L[b <= a ? is_tri(a, b) : is_tri(b, a)];
-                    acc.x = fmaf(-g, ws[b].x, acc.x);
-                    acc.y = fmaf(-g, ws[b].y, acc.y);
+                    const float2 w0 = *reinterpret_cast<const float2*>(ws + b);
+                    acc.x = fmaf(-g, w0.x, acc.x);
+                    acc.y = fmaf(-g, w0.y, acc.y);
                 }
                 acc = make_float2(dA[a] * acc.x, dA[a] * acc.y);
                 if (half) r1 = acc; else r0 = acc;
@@ -270,14 +315,12 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                 if (tt == 0) {
                     piv[k] = pk;
                     ild[k] = il;
-                    const float akk = fmaf(dA[k] * dA[k], L[is_tri(k, k)], (float)eb);   // before the elimination
+                    const float akk = fmaf(dA[k] * dA[k], L[is_tri(k, k)], ebh);   // before the elimination
                     ratio2 = fmaf(akk * inv.hi, akk * inv.hi, ratio2);
                 }
                 const int n = S - k - 1;
                 for (int t = tt; t < n * (n + 1) / 2; t += TT) {
-                    int a, c;
-                    is_tri_ab(t, a, c);
-                    const int i = k + 1 + a, cc = k + 1 + c;
+                    const int i = k + 1 + (tri[t] & 255), cc = k + 1 + (tri[t] >> 8);
                     const ff x = ff_mul(K[is_tri(i, k)], inv), y = K[is_tri(cc, k)];
                     ff& v = K[is_tri(i, cc)];
                     const float pr = __fmul_rn(x.hi, y.hi);
@@ -332,8 +375,9 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                     if (a >= S) continue;
                     const float2 y = half ? r1 : r0;
                     ff_acc_sq(yy, y);
-                    const float2 w0 = ws[a], wv = make_float2(fmaf(dA[a], y.x, w0.x), fmaf(dA[a], y.y, w0.y));
-                    ws[a] = wv;
+                    const float4 w0 = ws[a];
+                    const float2 wv = make_float2(fmaf(dA[a], y.x, w0.x), fmaf(dA[a], y.y, w0.y));
+                    ws[a] = make_float4(-2.0f * wv.x, -2.0f * wv.y, 2.0f * wv.y, -2.0f * wv.x);
                     wsum += fabsf(wv.x) + fabsf(wv.y);
                 }
                 yy = warp_sum_ff(yy);
@@ -345,45 +389,50 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
             team_sync();
             const float GM = *gmS;
             ff rr{0.f, 0.f};
+            const f2x GM2 = f2_dup(GM);
+            #pragma unroll 1
             for (int k = tt; k < dm.Nh; k += TT) {
-                const int f = k / Nm, ym = k - f * Nm;
-                bool cj;
-                const int ih = is_half(ym, Nm, dm.Nmh, cj);
+                const uint32_t at = kt[k];
                 const bool mid = odd && k == dm.Nh - 1;
-                const float mul = mid ? 1.0f : 2.0f;
+                const float sg = (at >> 31) ? -1.0f : 1.0f, dbl = mid ? 2.0f : 1.0f;   // the middle element is carried doubled
                 const float4 pv = zp[k], qv = zq[k];
-                // acc: grid sum + GM; rem: what the grid left
-                float acc[4] = {__fadd_rn(pv.x, GM), __fadd_rn(pv.y, GM), __fadd_rn(qv.x, GM), __fadd_rn(qv.y, GM)};
-                float rem[4] = {__fsub_rn(pv.x, __fsub_rn(acc[0], GM)) + pv.z, __fsub_rn(pv.y, __fsub_rn(acc[1], GM)) + pv.w,
-                                __fsub_rn(qv.x, __fsub_rn(acc[2], GM)) + qv.z, __fsub_rn(qv.y, __fsub_rn(acc[3], GM)) + qv.w};
-                const float4 *fb = fac + f, *cb = ct + ih;
+                // (P re, P im), (Q re, Q im): grid sum + GM, and what the grid left
+                const f2x p2 = f2_pack(dbl * pv.x, dbl * pv.y), q2 = f2_pack(qv.x, qv.y);
+                f2x acc0 = f2_add(p2, GM2), acc1 = f2_add(q2, GM2);
+                f2x rem0 = f2_add(f2_sub(p2, f2_sub(acc0, GM2)), f2_pack(dbl * pv.z, dbl * pv.w));
+                f2x rem1 = f2_add(f2_sub(q2, f2_sub(acc1, GM2)), f2_pack(qv.z, qv.w));
+                const float4 *fb = fac + (at & 0x7fff), *cb = ct + ((at >> 15) & 0xffff);
+                #pragma unroll 2
                 for (int s = 0; s < S; ++s) {
-                    const float4 u = pair_mul_fx(fb[s * dm.hf], conj_if(cb[s * dm.Nmh], cj));
-                    const float2 wv = ws[s];
-                    const float wx = -mul * wv.x, wy = -mul * wv.y;
-                    auto mac = [&](int i, float a, float b, float bl) {
-                        const float t = fmaf(a, b, acc[i]);
-                        const float d = __fsub_rn(acc[i], t);        // minus the grid part: exact
-                        rem[i] += fmaf(a, bl, fmaf(a, b, d));
-                        acc[i] = t;
+                    float4 c = cb[s * dm.Nmh];
+                    c.y *= sg;
+                    c.w *= sg;
+                    const float4 u = pair_mul_fx(fb[s * dm.hf], c);
+                    const float4 wv = ws[s];
+                    auto mac = [&](f2x& acc, f2x& rem, f2x a, f2x b, f2x bl) {
+                        const f2x t = f2_fma(a, b, acc);
+                        const f2x d = f2_sub(acc, t);                // minus the grid part: exact
+                        rem = f2_add(rem, f2_fma(a, bl, f2_fma(a, b, d)));
+                        acc = t;
                     };
-                    mac(0, wx, u.x, u.z);
-                    mac(1, wy, u.x, u.z);
-                    mac(2, -wy, u.y, u.w);
-                    mac(3, wx, u.y, u.w);
+                    mac(acc0, rem0, f2_pack(wv.x, wv.y), f2_dup(u.x), f2_dup(u.z));
+                    mac(acc1, rem1, f2_pack(wv.z, wv.w), f2_dup(u.y), f2_dup(u.w));
                 }
                 float e = 0.f;
                 ff q{0.f, 0.f};
                 #pragma unroll
-                for (int i = 0; i < 4; i += 2) {
+                for (int i = 0; i < 2; ++i) {
+                    uint32_t g0, g1, m0, m1;
+                    f2_unpack(f2_sub(i ? acc1 : acc0, GM2), g0, g1);
+                    f2_unpack(i ? rem1 : rem0, m0, m1);
                     float hx, lx, hy, ly;
-                    two_sum(__fsub_rn(acc[i], GM), rem[i], hx, lx);
-                    two_sum(__fsub_rn(acc[i + 1], GM), rem[i + 1], hy, ly);
+                    two_sum(__uint_as_float(g0), __uint_as_float(m0), hx, lx);
+                    two_sum(__uint_as_float(g1), __uint_as_float(m1), hy, ly);
                     ff_acc_sq(q, make_float2(hx, hy));
                     e = fmaf(2.0f * hx, lx, fmaf(2.0f * hy, ly, e));
                 }
                 q.lo += e;
-                const float sc = mid ? 1.0f : 0.5f;
+                const float sc = mid ? 0.25f : 0.5f;
                 rr = ff_add(rr, ff{sc * q.hi, sc * q.lo});
             }
             rr = warp_sum_ff(rr);
@@ -898,12 +947,12 @@ bool launch_iota_bulk_sym(const DevGeom& G, const DevParams& Pm, const DevState&
 
 // whether the real form applies: a symmetric layout whose working set fits one warp
 bool iota_sym_ok(const DevGeom& G, int S) {
-    return G.sym && ((IF_FIXED + 15) & ~(size_t)15) + if_plan(G, S).warp <= 227 * 1024;
+    return G.sym && if_fixed(G, S) + if_plan(G, S).warp <= 227 * 1024;
 }
 
 // float-float log iota~ of every particle (all), or of the queued ones
 void launch_iota_ff(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, bool all, cudaStream_t st) {
-    const size_t fixed = (IF_FIXED + 15) & ~(size_t)15, warp = if_plan(G, S).warp, limit = 227 * 1024;
+    const size_t fixed = if_fixed(G, S), warp = if_plan(G, S).warp, limit = 227 * 1024;
     const int TW = all ? 1 : IF_TEAM_MAX;
     int W = min(G.J, (TW == 1 ? 8 : 16) / TW);
     while (W > 1 && fixed + W * warp > limit) --W;
