@@ -59,7 +59,7 @@ __host__ __device__ inline IfPlan if_plan(const DevGeom& G, int S) {
     const IsDims d = is_dims(G);
     IfPlan p{};
     size_t o = 0;
-    p.fac = o; o += (size_t)S * d.hf * sizeof(float4);
+    p.fac = o; o += (size_t)S * (d.hf | 1) * sizeof(float4);
     p.ct = o; o += (size_t)S * d.Nmh * sizeof(float4);
     p.z = o; o += (size_t)d.Nh * 2 * sizeof(float4);            // P (hi, lo), Q (hi, lo)
     p.vec = o; o += (size_t)S * (sizeof(float4) + sizeof(float2) + sizeof(ff) + 2 * sizeof(float));   // w, g | pivots | dA, 1/L_kk
@@ -111,6 +111,8 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
     const int P = Pm.P, J = G.J, Nz = G.Nz, Nf = G.Nf, My = G.My, Mz = G.Mz, Nm = My * Mz;
     const IsDims dm = is_dims(G);
     constexpr int TT = 32 * TW;
+    const int fst = dm.hf | 1;                                  // odd: rows on distinct banks (an even
+    // stride of 40 cost 40 PFs x 8192 of Nz = 300 0.87 ms of 3.3)
     const int lane = threadIdx.x & 31, wid = threadIdx.x / TT, tt = threadIdx.x - wid * TT, wt = tt >> 5;   // team, place in it
     auto team_sync = [&]() {
         if constexpr (TW == 1) __syncwarp();
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
     ushort* tri = reinterpret_cast<ushort*>(kt + dm.Nh);        // [S (S + 1) / 2] row, column
     const IfPlan pl = if_plan(G, S);
     char* base = reinterpret_cast<char*>(smf) + if_fixed(G, S) + (size_t)wid * pl.warp;
-    float4* fac = reinterpret_cast<float4*>(base + pl.fac);     // [S][hf] b_f, a_y, a_z (half of each)
+    float4* fac = reinterpret_cast<float4*>(base + pl.fac);     // [S][fst] b_f, a_y, a_z (half of each)
     float4* ct = reinterpret_cast<float4*>(base + pl.ct);       // [S][Nmh] a_y a_z
     float4* zp = reinterpret_cast<float4*>(base + pl.z);        // [Nh] P, then [Nh] Q, as (hi, lo)
     float4* zq = zp + dm.Nh;
@@ -223,12 +225,12 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                 }
                 float2 hi, lo;
                 cis_pair(ctab, th, tl, hi, lo);
-                fac[i] = make_float4(hi.x, hi.y, lo.x, lo.y);
+                fac[s * fst + q] = make_float4(hi.x, hi.y, lo.x, lo.y);
             }
             team_sync();
             for (int i = tt; i < S * dm.Nmh; i += TT) {
                 const int s = i / by_Nmh, ym = i - s * dm.Nmh, y = ym / by_Mz, m = ym - y * Mz;
-                const float4* fs = fac + s * dm.hf + dm.Fh;
+                const float4* fs = fac + s * fst + dm.Fh;
                 bool cy, cz;
                 const int iy = is_half(y, My, dm.hy, cy), iz = is_half(m, Mz, dm.hz, cz);
                 ct[i] = pair_mul_fx(conj_if(fs[iy], cy), conj_if(fs[dm.hy + iz], cz));
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
             // Gram and A = eta_bar I + D G D, packed
             for (int t = tt; t < npair; t += TT) {
                 const int a = tri[t] & 255, b = tri[t] >> 8;
-                const float4 *fa = fac + a * dm.hf, *fb = fac + b * dm.hf;
+                const float4 *fa = fac + a * fst, *fb = fac + b * fst;
                 const ff g = ff_mul(if_sum(fa, fb, Nf), ff_mul(if_sum(fa + dm.Fh, fb + dm.Fh, My),
                                                                if_sum(fa + dm.Fh + dm.hy, fb + dm.Fh + dm.hy, Mz)));
                 ff v = ff_mul(g, ff_prod(dA[a], dA[b]));
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                     #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const int s = min(s0 + q, S - 1);
-                        const float2 b = *reinterpret_cast<const float2*>(fs + s * dm.hf);
+                        const float2 b = *reinterpret_cast<const float2*>(fs + s * fst);
                         float2 c = *reinterpret_cast<const float2*>(cs + s * dm.Nmh);
                         c.y *= sg;
                         const float x = fmaf(b.x, c.x, -b.y * c.y), y = fmaf(b.x, c.y, b.y * c.x);
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
                     float4 c = cb[s * dm.Nmh];
                     c.y *= sg;
                     c.w *= sg;
-                    const float4 u = pair_mul_fx(fb[s * dm.hf], c);
+                    const float4 u = pair_mul_fx(fb[s * fst], c);
                     const float4 wv = ws[s];
                     auto mac = [&](f2x& acc, f2x& rem, f2x a, f2x b, f2x bl) {
                         const f2x t = f2_fma(a, b, acc);
