@@ -451,7 +451,7 @@ WsPlan ws_plan(const DevGeom& G, const DevParams& Pm, int SCA, int nsplit_max) {
     w.kB = take(kappa_operand_bytes(G, S_max));
     w.red_part = take(nbel * 64 * RED_W * 2 * sizeof(double));
     w.tsum = take(nbel * 256 * sizeof(double));
-    w.gram = take(J * SM * SM * 2 * sizeof(double));
+    w.gram = take(stage_ws_bytes(G.J, S_max, G.Nz));   // and the basis of all PFs
     w.V64 = take(SM * J * Nz * (size_t)SCA * 2 * sizeof(double));
     w.cdf = take(nbel * PP * sizeof(double));
     w.wn = take(nbel * PP * sizeof(double));
@@ -671,7 +671,7 @@ void update_enqueue(bp_handle* h, const float* z_dev) {
         cudaEventRecord(h->ev[BP_PROF_STAGES], h->st);
         for (int i = 1; i < BP_PROF_STAGES; ++i) h->ev_valid[i] = true;
     }
-    h->launches += 1 + 3 + 3 + kappa_launches + iota_launches + 1 + 5 + 2;
+    h->launches += 1 + 3 + 4 + kappa_launches + iota_launches + 1 + 5 + 2;
     h->D.cur = 1 - h->D.cur;
     h->S_upd = S;
     h->phase = 0;

@@ -239,7 +239,8 @@ void launch_row_sums(const DevParams& Pm, const DevState& D, int S, int J, cudaS
 // chunk_req: particles per shared-memory chunk (16, 32, 64, 128; 0 = 128), halved to fit
 void launch_table(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int nsplit, int chunk_req,
                   cudaStream_t st);
-// the Gram matrices, the PF basis V64 and the existence tests
+size_t stage_ws_bytes(int J, int S_max, int Nz);
+// the Gram matrices and their workspace (behind them the basis of all PFs), the PF basis V64 and the existence tests
 void launch_stage(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, const float* z,
                   double* gram, double* nu_b, double* V64, cudaStream_t st);
 // the noise likelihood's tridiagonal forms; with a side stream they run there (forked from st

@@ -199,8 +199,8 @@ __device__ __forceinline__ float4 kx_pair_mul(float4 a, float4 b) {
 // and n >= SW (Im h_{n - SW}) against k = 2 e + part, K-major core matrices:
 // [Re(v + v'), Im(v - v')] and [Im(v + v'), -Re(v - v')] for a symmetric layout (v' the mirrored
 // element's, the middle element counted once), else [Re v, Im v] and [Im v, -Re v].  Column SW - 1
-// is r0, unused columns are zero.  Bound: the FP64 conversions (82 us at 64 PFs x 4 PAs x Nz = 160).
-constexpr int KX_DSPLIT = 4;   // blocks per (s, j)
+// is r0, unused columns are zero.  Bound: the FP64 conversions (64 PFs x 4 PAs x Nz = 160: 223 us with FP64
+// maxima in four blocks per (s, j), 96 us with maxima of upper words and about four blocks per SM).
 __global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int S, int SCA, int SW,
                                                       const double2* __restrict__ V64) {
     const int s = blockIdx.x, j = blockIdx.y, J = G.J, Nz = G.Nz, K = S - 1, Nh = kx_elements(G);
@@ -227,14 +227,18 @@ __global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int
         float inv = 0.f;
         if (r0 || c < K) {
             const double2* v = V + (size_t)(r0 ? SCA - 1 : c) * Nz;
-            double m = 0.0;
+            uint32_t top = 0;                      // upper words of the magnitudes: the exponent decides
+            #pragma unroll 4
             for (int k = lane; k < Nh; k += 32) {
                 double o[4];
                 combo(v, k, o);
-                m = fmax(m, fmax(fmax(fabs(o[0]), fabs(o[1])), fmax(fabs(o[2]), fabs(o[3]))));
+                #pragma unroll
+                for (int i = 0; i < 4; ++i) top = max(top, (uint32_t)__double2hiint(o[i]) & 0x7fffffffu);
             }
-            m = warp_max_d(m) * (r0 ? 1.0 : isq);
-            if (m > 0.0 && isfinite(m)) {
+            top = __reduce_max_sync(0xffffffffu, top);
+            // the next upper word bounds the largest magnitude
+            const double m = top < 0x7ff00000u ? __hiloint2double((int)(top + 1), 0) * (r0 ? 1.0 : isq) : 0.0;
+            if (top > 0 && m > 0.0 && isfinite(m)) {
                 int e;
                 frexp(m, &e);
                 f = ldexp(r0 ? 1.0 : isq, -e);
@@ -901,7 +905,7 @@ int launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S
                  const double* V64, cudaStream_t st) {
     const int SW = kx_sw(S), nant = G.My + G.Mz;
     const double2* V = reinterpret_cast<const double2*>(V64);
-    k_kappa_digits<<<dim3(S, G.J, KX_DSPLIT), 256, 0, st>>>(G, D, S, SCA, SW, V);
+    k_kappa_digits<<<dim3(S, G.J, max(1, min(4, 4 * sm_count() / (S * G.J)))), 256, 0, st>>>(G, D, S, SCA, SW, V);
     if (!tensor) {
         const size_t smem = ((size_t)nant * KCC_T + 256 + KCC_E * KCC_C) * sizeof(float4);
         smem_allow_max((const void*)k_kappa_cc);

@@ -216,84 +216,145 @@ __global__ void k_table_final(DevGeom G, DevParams Pm, DevState D, int S, int ns
 
 // ---------------------------------------------------------------- Gram matrix per j (FP64)
 // G_j[a][b] = m_a^H m_b; also e_all = z - sum_s mu3_s, b = M^H e_all, |e_all|^2.
-__global__ void k_gram(DevGeom G, DevParams Pm, DevState D, int S, const float* z, double* gram, double* nu_b) {
+__global__ void k_gram(DevGeom G, DevParams Pm, DevState D, int S, double* gram) {
     const int j = blockIdx.y;
     const int J = G.J, Nz = G.Nz, SM = Pm.S_max;
-    const size_t plane = (size_t)SM * J * Nz;
     const double2* tab = reinterpret_cast<const double2*>(D.tab);
-    const int npair = S * (S + 1) / 2;
-    // pairs (a >= b) plus S projections of e_all plus one norm
-    const int ntask = npair + S + 1;
+    const int npair = S * (S + 1) / 2;            // pairs (a >= b)
     const int warps = blockDim.x / 32, lane = threadIdx.x & 31;
-    for (int task = blockIdx.x * warps + (threadIdx.x >> 5); task < ntask; task += gridDim.x * warps) {
+    for (int task = blockIdx.x * warps + (threadIdx.x >> 5); task < npair; task += gridDim.x * warps) {
         double2 acc = make_double2(0.0, 0.0);
-        if (task < npair) {
-            int a = (int)((sqrt(8.0 * task + 1.0) - 1.0) / 2.0);
-            while ((a + 1) * (a + 2) / 2 <= task) ++a;
-            while (a * (a + 1) / 2 > task) --a;
-            const int b = task - a * (a + 1) / 2;
-            const double2* ma = tab + ((size_t)a * J + j) * Nz;
-            const double2* mb = tab + ((size_t)b * J + j) * Nz;
-            for (int k = lane; k < Nz; k += 32) {
-                const double2 t = zmulc(ma[k], mb[k]);
-                acc.x += t.x; acc.y += t.y;
-            }
-            acc.x = warp_sum_d(acc.x); acc.y = warp_sum_d(acc.y);
-            if (lane == 0) {
-                double2* Gm = reinterpret_cast<double2*>(gram) + (size_t)j * SM * SM;
-                Gm[a * SM + b] = acc;
-                Gm[b * SM + a] = make_double2(acc.x, -acc.y);
-            }
-        } else {
-            const int a = task - npair;   // a < S: projection; a == S: norm
-            const double2* ma = tab + ((size_t)(a < S ? a : 0) * J + j) * Nz;
-            double nrm = 0.0;
-            for (int k = lane; k < Nz; k += 32) {
-                double2 e = make_double2((double)z[2 * (j * Nz + k)], (double)z[2 * (j * Nz + k) + 1]);
-                for (int t = 0; t < S; ++t) {
-                    const double2 m3 = tab[2 * plane + ((size_t)t * J + j) * Nz + k];
-                    e.x -= m3.x; e.y -= m3.y;
-                }
-                if (a < S) {
-                    const double2 t = zmulc(ma[k], e);
-                    acc.x += t.x; acc.y += t.y;
-                } else {
-                    nrm += e.x * e.x + e.y * e.y;
-                }
-            }
-            acc.x = warp_sum_d(acc.x); acc.y = warp_sum_d(acc.y); nrm = warp_sum_d(nrm);
-            if (lane == 0) {
-                double2* bv = reinterpret_cast<double2*>(nu_b) + (size_t)j * (SM + 1);
-                if (a < S) bv[a] = acc; else bv[SM] = make_double2(nrm, 0.0);
-            }
+        int a = (int)((sqrtf(8.0f * task + 1.0f) - 1.0f) * 0.5f);
+        while ((a + 1) * (a + 2) / 2 <= task) ++a;
+        while (a * (a + 1) / 2 > task) --a;
+        const int b = task - a * (a + 1) / 2;
+        const double2* ma = tab + ((size_t)a * J + j) * Nz;
+        const double2* mb = tab + ((size_t)b * J + j) * Nz;
+        #pragma unroll 4
+        for (int k = lane; k < Nz; k += 32) {
+            const double2 t = zmulc(ma[k], mb[k]);
+            acc.x += t.x; acc.y += t.y;
+        }
+        acc.x = warp_sum_d(acc.x); acc.y = warp_sum_d(acc.y);
+        if (lane == 0) {
+            double2* Gm = reinterpret_cast<double2*>(gram) + (size_t)j * SM * SM;
+            Gm[a * SM + b] = acc;
+            Gm[b * SM + a] = make_double2(acc.x, -acc.y);
         }
     }
 }
 
 // ---------------------------------------------------------------- kappa / omega stage per (s, j), FP64
-// One block per (s, j).  With B = I + M_{-s}^H M_{-s}/eta_bar = L L^H (Cholesky) the whitened
-// basis V = M_{-s} L^{-H} satisfies V V^H = M_{-s} B^{-1} M_{-s}^H, so the inversion lemma gives
+// With B = I + M_{-s}^H M_{-s}/eta_bar = L L^H (Cholesky) the whitened basis V = M_{-s} L^{-H} satisfies
+// V V^H = M_{-s} B^{-1} M_{-s}^H, so the inversion lemma gives
 // a^H A_s^{-1} b = (a^H b - (V^H a)^H (V^H b)/eta_bar)/eta_bar for every form of S-V, and
 // r0 = eta_bar A_s^{-1} e0 = e0 - V V^H e0/eta_bar.  V and r0 leave as columns of V64
 // [S][J][SCA][Nz] (r0 in column SCA - 1) for k_kappa_digits.
-// The forms of the existence test need V^H x = L^{-1} (M^H x) for x = e0, m^w, mu4 only: the
-// rows (M^H x)^H ride along the factorisation as rows K .. K + 2.
-// Bound: the FP64 pipe (2 FMA per clock and SM), 4 Nz K^2/2 FMA for V (the eigen-decomposition
-// that stood here before, which the element-wise likelihood needed for its diagonal sums, took
-// 13.4 ms at 64 PFs x 4 PAs x Nz = 160, most of it rotations and barriers; this takes 1.7 ms with
-// the Gram, and 5.6 -> 1.5 ms at 40 PFs x Nz = 300).
+// One factorisation per PA serves every PF: with all S columns B = L L^H and V_f = M L^{-H}.  Without row s
+// L is a triangle with one superdiagonal from row s on, which the unitary Q of K - s plane rotations
+// of neighbouring columns removes: (L without row s) Q = [L_s 0], and V_s = V_f Q without its last
+// column (the same basis that a factorisation of its own would give, at 12 operations per element
+// and rotation instead of K^2/2 products).  x^H V_s is x^H V_f under the same rotations.
+// Bound: the FP64 pipe (2 FMA per clock and SM) and the serial chains of pivots and rotations.
+// Measured, 4 PAs: 64 PFs x Nz = 160 1.74 -> 0.57 ms (with the Gram), 40 x 300 1.50 -> 0.43, 32 x 1024
+// 1.54 -> 0.52, 8 x 160 0.070 -> 0.068 (against a factorisation and a solve for every (s, j)).
 constexpr int STAGE_THREADS = 256;
-constexpr int STAGE_WRED = 9;   // per-warp partial sums of the omega test's scalars
-__host__ __device__ inline int stage_row(int K, int r) {   // start of row r of [L; three carried rows]
+constexpr int STAGE_WRED = 12;  // per-warp partial sums: the omega test's nine scalars, m^H e_all and |e_all|^2
+__host__ __device__ inline int stage_row(int K, int r) {   // start of row r of [L; carried rows of K]
     return r < K ? r * (r + 1) / 2 : K * (K + 1) / 2 + (r - K) * K;
 }
-__host__ __device__ inline size_t stage_kappa_smem(int K, int Nz) {
-    return ((size_t)K * (K + 1) / 2 + 3 * (size_t)K + (size_t)Nz) * sizeof(double2) +
-           ((size_t)K + STAGE_WRED * (STAGE_THREADS / 32) + 2) * sizeof(double);
+// behind the Gram matrices [J][S_max][S_max]: V_f [J][S_max][Nz], e_all [J][Nz], L [J][S_max (S_max + 1)/2]
+struct StageWs { double2 *Vf, *e, *L; };
+__host__ __device__ inline StageWs stage_ws(double* gram, int J, int SM, int Nz) {
+    StageWs w;
+    w.Vf = reinterpret_cast<double2*>(gram) + (size_t)J * SM * SM;
+    w.e = w.Vf + (size_t)J * SM * Nz;
+    w.L = w.e + (size_t)J * Nz;
+    return w;
+}
+size_t stage_ws_bytes(int J, int SM, int Nz) {
+    return ((size_t)J * SM * SM + (size_t)J * SM * Nz + (size_t)J * Nz + (size_t)J * SM * (SM + 1) / 2) * sizeof(double2);
 }
 
+// Block (j, EC elements): B, and the EC rows of M as rows S .. S + EC - 1 of a right-looking Cholesky that
+// carries them along: they leave as rows of V_f.  Every block repeats the factorisation (S^3/6 products: 46
+// us of FP64 at 64 PFs, in parallel on as many SMs); e_all = z - sum_t mu3_t of its elements on the way.
+__global__ void __launch_bounds__(STAGE_THREADS) k_stage_basis(DevGeom G, DevParams Pm, DevState D, int S, int EC, const float* z,
+                                                               double* gram) {
+    const int j = blockIdx.x, k0 = blockIdx.y * EC;
+    const int J = G.J, Nz = G.Nz, SM = Pm.S_max, ne = min(EC, Nz - k0);
+    const double eb = D.eta_bar[j];
+    const size_t plane = (size_t)SM * J * Nz;
+    const double2* tab = reinterpret_cast<const double2*>(D.tab);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = STAGE_THREADS / 32;
+    extern __shared__ double2 sh[];
+    double2* Lp = sh;                             // packed lower triangle, then ne rows of S
+    double* il = reinterpret_cast<double*>(Lp + stage_row(S, S + EC));   // 1 / L_cc
+    const double2* Gm = reinterpret_cast<const double2*>(gram) + (size_t)j * SM * SM;
+    const StageWs ws = stage_ws(gram, J, SM, Nz);
+    for (int r = wid; r < S; r += nw)
+        for (int c = lane; c <= r; c += 32) {
+            double2 g = Gm[r * SM + c];
+            g.x /= eb; g.y /= eb;
+            if (r == c) { g.x += 1.0; g.y = 0.0; }
+            Lp[stage_row(S, r) + c] = g;
+        }
+    for (int i = tid; i < S * ne; i += STAGE_THREADS) {
+        const int c = i / ne, e = i - c * ne;
+        Lp[stage_row(S, S + e) + c] = tab[((size_t)c * J + j) * Nz + k0 + e];
+    }
+    for (int e = tid; e < ne; e += STAGE_THREADS) {
+        const int k = k0 + e;
+        double2 v = make_double2((double)z[2 * (j * Nz + k)], (double)z[2 * (j * Nz + k) + 1]);
+        for (int t = 0; t < S; ++t) {
+            const double2 m3 = tab[2 * plane + ((size_t)t * J + j) * Nz + k];
+            v.x -= m3.x; v.y -= m3.y;
+        }
+        ws.e[(size_t)j * Nz + k] = v;
+    }
+    __syncthreads();
+    // Columns stay unscaled (x_rk = l_rk l_kk), so a step is one pass and one barrier: v_rc -= x_rk conj(x_ck) / p_k;
+    // whoever updates the next pivot inverts it.  Every pivot of B is at least 1.
+    if (tid == 0) il[0] = 1.0 / fmax(Lp[0].x, 1.0);
+    __syncthreads();
+    for (int k = 0; k + 1 < S; ++k) {
+        const double ip = il[k];
+        for (int r = k + 1 + (tid >> 4); r < S + ne; r += STAGE_THREADS / 16) {
+            const int row = stage_row(S, r), end = min(r, S - 1);
+            double2 x = Lp[row + k];
+            x.x *= ip; x.y *= ip;
+            for (int c = k + 1 + (tid & 15); c <= end; c += 16) {
+                const double2 u = zmulc(Lp[stage_row(S, c) + k], x);
+                double2& v = Lp[row + c];
+                v.x -= u.x; v.y -= u.y;
+                if (r == k + 1 && c == r) il[r] = 1.0 / fmax(v.x, 1.0);
+            }
+        }
+        __syncthreads();
+    }
+    for (int c = tid; c < S; c += STAGE_THREADS) il[c] = rsqrt(fmax(Lp[stage_row(S, c) + c].x, 1.0));
+    __syncthreads();
+    for (int i = tid; i < S * ne; i += STAGE_THREADS) {
+        const int c = i / ne, e = i - c * ne;
+        const double2 v = Lp[stage_row(S, S + e) + c];
+        ws.Vf[((size_t)j * SM + c) * Nz + k0 + e] = make_double2(v.x * il[c], v.y * il[c]);
+    }
+    if (blockIdx.y == 0) {
+        double2* Lg = ws.L + (size_t)j * (SM * (SM + 1) / 2);
+        for (int r = wid; r < S; r += nw)
+            for (int c = lane; c <= r; c += 32) {
+                const double2 v = Lp[stage_row(S, r) + c];
+                Lg[stage_row(S, r) + c] = r == c ? make_double2(fmax(v.x, 1.0) * il[r], 0.0) : make_double2(v.x * il[c], v.y * il[c]);
+            }
+    }
+}
+
+__host__ __device__ inline size_t stage_kappa_smem(int S, int Nz) {
+    return ((size_t)S * (S + 1) / 2 + 4 * (size_t)S + (size_t)Nz) * sizeof(double2) +
+           ((size_t)S + STAGE_WRED * (STAGE_THREADS / 32)) * sizeof(double);
+}
 __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevParams Pm, DevState D, int S, int SCA,
-                                                                  const float* z, const double* gram, double* V64) {
+                                                                  double* gram, double* nu_b, double* V64) {
     const int s = blockIdx.x, j = blockIdx.y;
     const int J = G.J, Nz = G.Nz, SM = Pm.S_max;
     const int K = S - 1;                          // columns of M_{-s}
@@ -302,33 +363,30 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
     const double2* tab = reinterpret_cast<const double2*>(D.tab);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = STAGE_THREADS / 32;
     extern __shared__ double2 sh[];
-    double2* Lp = sh;                             // packed lower triangle, then three rows of K
-    double2* E0 = Lp + stage_row(K, K + 3);       // e0 = z - sum_{t != s} mu3_t (Nz)
-    double* il = reinterpret_cast<double*>(E0 + Nz);   // 1 / L_cc (K)
-    double* wred = il + K;                        // [STAGE_WRED][nw]
-    const double2* Gm = reinterpret_cast<const double2*>(gram) + (size_t)j * SM * SM;
-    auto col = [&](int c) { return c < s ? c : c + 1; };   // column c of M_{-s} is PF col(c)
-    // B = I + G_{-s}/eb, packed
-    for (int r = wid; r < K; r += nw)
-        for (int c = lane; c <= r; c += 32) {
-            double2 g = Gm[col(r) * SM + col(c)];
-            g.x /= eb; g.y /= eb;
-            if (r == c) { g.x += 1.0; g.y = 0.0; }
-            Lp[stage_row(K, r) + c] = g;
-        }
+    double2* Lp = sh;                             // packed lower triangle of all PFs
+    double2* cr = Lp + stage_row(S, S);           // [3][S] x^H V_f, then x^H V_s, of x = e0, m^w, mu4
+    double2* qa = cr + 3 * S;                     // rotation of columns (i, i + 1), i = s .. K - 1: (a, b)
+    double2* E0 = qa + S;                         // e0 = z - sum_{t != s} mu3_t (Nz)
+    double* qb = reinterpret_cast<double*>(E0 + Nz);
+    double* wred = qb + S;                        // [STAGE_WRED][nw]
+    const StageWs ws = stage_ws(gram, J, SM, Nz);
+    const double2* Vf = ws.Vf + (size_t)j * SM * Nz;
+    const double2* mp = tab + ((size_t)s * J + j) * Nz;
+    const double2* mwp = tab + 1 * plane + ((size_t)s * J + j) * Nz;
+    const double2* m3p = tab + 2 * plane + ((size_t)s * J + j) * Nz;
+    const double2* m4p = tab + 3 * plane + ((size_t)s * J + j) * Nz;
+    {
+        const double2* Lg = ws.L + (size_t)j * (SM * (SM + 1) / 2);
+        for (int i = stage_row(S, s) + tid; i < S * (S + 1) / 2; i += STAGE_THREADS) Lp[i] = Lg[i];
+    }
     // e0 and the block sums of |e0|^2, m^H e0, |m|^2, mu4^H e0, |mu4|^2, m^H mu4 (m = m^w_s)
     {
-        double acc[STAGE_WRED] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        double acc[STAGE_WRED] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
         for (int k = tid; k < Nz; k += STAGE_THREADS) {
-            double2 e0 = make_double2((double)z[2 * (j * Nz + k)], (double)z[2 * (j * Nz + k) + 1]);
-            for (int t = 0; t < S; ++t) {
-                if (t == s) continue;
-                const double2 m3 = tab[2 * plane + ((size_t)t * J + j) * Nz + k];
-                e0.x -= m3.x; e0.y -= m3.y;
-            }
+            const double2 ea = ws.e[(size_t)j * Nz + k], m3 = m3p[k];
+            const double2 e0 = make_double2(ea.x + m3.x, ea.y + m3.y);
             E0[k] = e0;
-            const double2 mw = tab[1 * plane + ((size_t)s * J + j) * Nz + k];
-            const double2 m4 = tab[3 * plane + ((size_t)s * J + j) * Nz + k];
+            const double2 mw = mwp[k], m4 = m4p[k];
             const double2 me = zmulc(mw, e0), ue = zmulc(m4, e0), mu = zmulc(mw, m4);
             acc[0] += e0.x * e0.x + e0.y * e0.y;
             acc[1] += me.x; acc[2] += me.y;
@@ -336,6 +394,9 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
             acc[4] += ue.x; acc[5] += ue.y;
             acc[6] += m4.x * m4.x + m4.y * m4.y;
             acc[7] += mu.x; acc[8] += mu.y;
+            const double2 be = zmulc(mp[k], ea);
+            acc[9] += be.x; acc[10] += be.y;
+            acc[11] += ea.x * ea.x + ea.y * ea.y;
         }
         #pragma unroll
         for (int q = 0; q < STAGE_WRED; ++q) {
@@ -344,57 +405,76 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
         }
     }
     __syncthreads();
-    if (tid < STAGE_WRED) {
-        double v = 0.0;
-        for (int w = 0; w < nw; ++w) v += wred[tid * nw + w];
-        wred[tid * nw] = v;   // the block sum in slot 0
-    }
-    // (M^H e0)^H, (M^H m^w)^H, (M^H mu4)^H: one warp per column t
-    for (int t = wid; t < K; t += nw) {
-        const double2* mt = tab + ((size_t)col(t) * J + j) * Nz;
-        const double2* mwp = tab + 1 * plane + ((size_t)s * J + j) * Nz;
-        const double2* m4p = tab + 3 * plane + ((size_t)s * J + j) * Nz;
-        double ax = 0, ay = 0, bx = 0, by = 0, cx = 0, cy = 0;
-        for (int k = lane; k < Nz; k += 32) {
-            const double2 m = mt[k];
-            const double2 u1 = zmulc(m, E0[k]), u2 = zmulc(m, mwp[k]), u3 = zmulc(m, m4p[k]);
-            ax += u1.x; ay += u1.y; bx += u2.x; by += u2.y; cx += u3.x; cy += u3.y;
+    if (wid == 0) {
+        // the rotations: lanes over the rows i >= s of L without row s (row i was i + 1), t the entry of the
+        // column that travels.  [t_i, L_{i+1,i+1}] -> [rho, 0] with (a, b) = (t_i, L_{i+1,i+1}) / rho:
+        // (x_i, x_{i+1}) -> (x_i conj(a) + x_{i+1} b, x_{i+1} a - x_i b)
+        double2 t[2];
+        #pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = s + lane + 32 * h;
+            t[h] = i < K ? Lp[stage_row(S, i + 1) + s] : make_double2(0.0, 0.0);
         }
-        ax = warp_sum_d(ax); ay = warp_sum_d(ay);
-        bx = warp_sum_d(bx); by = warp_sum_d(by);
-        cx = warp_sum_d(cx); cy = warp_sum_d(cy);
-        if (lane == 0) {
-            Lp[stage_row(K, K) + t] = make_double2(ax, -ay);
-            Lp[stage_row(K, K + 1) + t] = make_double2(bx, -by);
-            Lp[stage_row(K, K + 2) + t] = make_double2(cx, -cy);
+        for (int c = s; c < K; ++c) {
+            const int o = c - s;
+            const double2 own = o < 32 ? t[0] : t[1];
+            double2 a = make_double2(__shfl_sync(0xffffffffu, own.x, o & 31), __shfl_sync(0xffffffffu, own.y, o & 31));
+            double b = Lp[stage_row(S, c + 1) + c + 1].x;
+            const double ir = rsqrt(fma(a.x, a.x, fma(a.y, a.y, b * b)));
+            a.x *= ir; a.y *= ir; b *= ir;
+            if (lane == 0) { qa[c] = a; qb[c] = b; }
+            #pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = s + lane + 32 * h;
+                if (i > c && i < K) {
+                    const double2 x = Lp[stage_row(S, i + 1) + c + 1], u = zmul(x, a);
+                    t[h] = make_double2(fma(-b, t[h].x, u.x), fma(-b, t[h].y, u.y));
+                }
+            }
+        }
+    } else {
+        for (int t = wid - 1; t < S; t += nw - 1) {   // one warp per column of V_f
+            const double2* vt = Vf + (size_t)t * Nz;
+            double ax = 0, ay = 0, bx = 0, by = 0, cx = 0, cy = 0;
+            for (int k = lane; k < Nz; k += 32) {
+                const double2 v = vt[k];
+                const double2 u1 = zmulc(v, E0[k]), u2 = zmulc(v, mwp[k]), u3 = zmulc(v, m4p[k]);
+                ax += u1.x; ay += u1.y; bx += u2.x; by += u2.y; cx += u3.x; cy += u3.y;
+            }
+            ax = warp_sum_d(ax); ay = warp_sum_d(ay);
+            bx = warp_sum_d(bx); by = warp_sum_d(by);
+            cx = warp_sum_d(cx); cy = warp_sum_d(cy);
+            if (lane == 0) {
+                cr[t] = make_double2(ax, -ay);
+                cr[S + t] = make_double2(bx, -by);
+                cr[2 * S + t] = make_double2(cx, -cy);
+            }
         }
     }
     __syncthreads();
-    // right-looking Cholesky of the K x K triangle with the three carried rows; every pivot of B
-    // is at least 1
-    for (int k = 0; k < K; ++k) {
-        if (tid == 0) il[k] = rsqrt(fmax(Lp[stage_row(K, k) + k].x, 1.0));
-        __syncthreads();
-        const double d = il[k];
-        for (int r = k + 1 + tid; r < K + 3; r += STAGE_THREADS) {
-            double2& v = Lp[stage_row(K, r) + k];
-            v.x *= d; v.y *= d;
+    if (tid < 3) {
+        double2* c = cr + tid * S;
+        double2 t = c[s];
+        for (int i = s; i < K; ++i) {
+            const double2 x = c[i + 1], a = qa[i], u = zmulc(a, t), w = zmul(x, a);
+            const double b = qb[i];
+            c[i] = make_double2(fma(b, x.x, u.x), fma(b, x.y, u.y));
+            t = make_double2(fma(-b, t.x, w.x), fma(-b, t.y, w.y));
         }
-        __syncthreads();
-        for (int r = k + 1 + (tid >> 4); r < K + 3; r += STAGE_THREADS / 16) {
-            const int row = stage_row(K, r), end = min(r, K - 1);
-            const double2 x = Lp[row + k];
-            for (int c = k + 1 + (tid & 15); c <= end; c += 16) {
-                const double2 u = zmulc(Lp[stage_row(K, c) + k], x);   // l_rk conj(l_ck)
-                double2& v = Lp[row + c];
-                v.x -= u.x; v.y -= u.y;
-            }
-        }
-        __syncthreads();
     }
-    const double2* ye = Lp + stage_row(K, K);     // conj of V^H e0, V^H m^w, V^H mu4
-    const double2* vm = ye + K;
-    const double2* v4 = vm + K;
+    if (tid >= 32 && tid < 32 + STAGE_WRED) {
+        double v = 0.0;
+        for (int w = 0; w < nw; ++w) v += wred[(tid - 32) * nw + w];
+        wred[(tid - 32) * nw] = v;   // the block sum in slot 0
+        // the noise likelihood's b = M^H e_all, |e_all|^2
+        double* nb = nu_b + 2 * (size_t)j * (SM + 1);
+        if (tid - 32 == 9 || tid - 32 == 10) nb[2 * s + tid - 41] = v;
+        if (s == 0 && tid - 32 == 11) { nb[2 * SM] = v; nb[2 * SM + 1] = 0.0; }
+    }
+    __syncthreads();
+    const double2* ye = cr;                       // conj of V^H e0, V^H m^w, V^H mu4
+    const double2* vm = cr + S;
+    const double2* v4 = cr + 2 * S;
     if (wid == 0) {
         double a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
         for (int c = lane; c < K; c += 32) {
@@ -431,47 +511,28 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
             D.bel[BEL_PPR + s * J + j] = pr;
         }
     }
-    // V rows v_k = m_k L^{-H} by forward substitution, eight columns at a time (finished columns
-    // are read back, coalesced, from V64); consecutive threads take consecutive elements
+    // columns of V_s: those before s are V_f's, the others rotated; r0 on the way
     double2* Vs = reinterpret_cast<double2*>(V64) + ((size_t)s * J + j) * SCA * Nz;
-    constexpr int CB = 8;
+    const double ieb = 1.0 / eb;
     for (int k = tid; k < Nz; k += STAGE_THREADS) {
-        double2 r0 = E0[k];
-        for (int c0 = 0; c0 < K; c0 += CB) {
-            double2 acc[CB];
-            #pragma unroll
-            for (int q = 0; q < CB; ++q)
-                acc[q] = c0 + q < K ? tab[((size_t)col(c0 + q) * J + j) * Nz + k] : make_double2(0.0, 0.0);
-            for (int t = 0; t < c0; ++t) {
-                const double2 v = Vs[(size_t)t * Nz + k];
-                #pragma unroll
-                for (int q = 0; q < CB; ++q) {
-                    if (c0 + q < K) {
-                        const double2 u = zmulc(Lp[stage_row(K, c0 + q) + t], v);
-                        acc[q].x -= u.x; acc[q].y -= u.y;
-                    }
-                }
-            }
-            #pragma unroll
-            for (int q = 0; q < CB; ++q) {
-                if (c0 + q < K) {
-                    const double d = il[c0 + q];
-                    acc[q].x *= d; acc[q].y *= d;
-                    Vs[(size_t)(c0 + q) * Nz + k] = acc[q];
-                    #pragma unroll
-                    for (int p = q + 1; p < CB; ++p) {
-                        if (c0 + p < K) {
-                            const double2 u = zmulc(Lp[stage_row(K, c0 + p) + c0 + q], acc[q]);
-                            acc[p].x -= u.x; acc[p].y -= u.y;
-                        }
-                    }
-                    const double2 y = make_double2(ye[c0 + q].x / eb, -ye[c0 + q].y / eb);
-                    const double2 u = zmul(acc[q], y);
-                    r0.x -= u.x; r0.y -= u.y;
-                }
-            }
+        double2 r0 = make_double2(0.0, 0.0);
+        auto put = [&](int c, double2 v) {
+            Vs[(size_t)c * Nz + k] = v;
+            const double2 u = zmulc(ye[c], v);    // v (V^H e0)_c
+            r0.x += u.x; r0.y += u.y;
+        };
+        #pragma unroll 4
+        for (int c = 0; c < s; ++c) put(c, Vf[(size_t)c * Nz + k]);
+        double2 t = Vf[(size_t)s * Nz + k];
+        #pragma unroll 4
+        for (int c = s; c < K; ++c) {
+            const double2 x = Vf[(size_t)(c + 1) * Nz + k], a = qa[c], u = zmulc(a, t), w = zmul(x, a);
+            const double b = qb[c];
+            put(c, make_double2(fma(b, x.x, u.x), fma(b, x.y, u.y)));
+            t = make_double2(fma(-b, t.x, w.x), fma(-b, t.y, w.y));
         }
-        Vs[(size_t)(SCA - 1) * Nz + k] = r0;
+        const double2 e0 = E0[k];
+        Vs[(size_t)(SCA - 1) * Nz + k] = make_double2(fma(-ieb, r0.x, e0.x), fma(-ieb, r0.y, e0.y));
     }
 }
 
@@ -597,12 +658,16 @@ void launch_table(const DevGeom& G, const DevParams& Pm, const DevState& D, int 
 
 void launch_stage(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, const float* z,
                   double* gram, double* nu_b, double* V64, cudaStream_t st) {
-    const int npair = S * (S + 1) / 2 + S + 1;
-    const int gx = min(64, (npair + 7) / 8);
-    k_gram<<<dim3(gx, G.J), 256, 0, st>>>(G, Pm, D, S, z, gram, nu_b);
-    const size_t sm = stage_kappa_smem(S - 1, G.Nz);
+    const int gx = min(128, (S * (S + 1) / 2 + 7) / 8);
+    k_gram<<<dim3(gx, G.J), 256, 0, st>>>(G, Pm, D, S, gram);
+    // element blocks of the basis: about one per SM, 8 to 64 elements
+    const int EC = min(64, max(8, (G.Nz * G.J + sm_count() - 1) / sm_count()));
+    const size_t smb = (size_t)stage_row(S, S + EC) * sizeof(double2) + S * sizeof(double);
+    smem_allow_max((const void*)k_stage_basis);
+    k_stage_basis<<<dim3(G.J, (G.Nz + EC - 1) / EC), STAGE_THREADS, smb, st>>>(G, Pm, D, S, EC, z, gram);
+    const size_t sm = stage_kappa_smem(S, G.Nz);
     smem_allow_max((const void*)k_stage_kappa);
-    k_stage_kappa<<<dim3(S, G.J), STAGE_THREADS, sm, st>>>(G, Pm, D, S, SCA, z, gram, V64);
+    k_stage_kappa<<<dim3(S, G.J), STAGE_THREADS, sm, st>>>(G, Pm, D, S, SCA, gram, nu_b, V64);
 }
 
 void launch_nu_tridiag(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const double* gram,
