@@ -269,6 +269,10 @@ __host__ __device__ inline float2 cmulc(float2 a, float2 b) {  // conj(a) * b
 }
 __host__ __device__ inline double2 zmul(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 __host__ __device__ inline double2 zmulc(double2 a, double2 b) { return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }
+// c + conj(a) b
+__device__ inline double2 zfmac(double2 a, double2 b, double2 c) {
+    return make_double2(fma(a.x, b.x, fma(a.y, b.y, c.x)), fma(a.x, b.y, fma(-a.y, b.x, c.y)));
+}
 
 // ------------------------------------------------------------------ float-float (FP32 pairs)
 // Error-free transformations (Knuth TwoSum, Dekker/FMA TwoProd) and the

@@ -97,8 +97,9 @@ __global__ void k_norm_sum(DevGeom G, DevParams Pm, DevState D, int S, int NB, d
     const int per = (P + NB - 1) / NB;
     const int p0 = blockIdx.x * per, p1 = min(P, p0 + per);
     const double* lw = belief_wn(D, v, P);
-    double acc[RED_W];
-    for (int i = 0; i < RED_W; ++i) acc[i] = 0.0;
+    double acc[32];
+    #pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.0;
     const int d = v.dims;
     if (M > -INFINITY) {
         for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
@@ -107,23 +108,42 @@ __global__ void k_norm_sum(DevGeom G, DevParams Pm, DevState D, int S, int NB, d
             const double w = exp(t);
             double xs[6];
             belief_state(D, v, P, p, xs);
-            for (int k = 0; k < d; ++k) xs[k] -= ref[k];
             acc[0] += w;
-            for (int k = 0; k < d; ++k) acc[1 + k] += w * xs[k];
-            int q = 7;
-            for (int r = 0; r < d; ++r)
-                for (int c = r; c < d; ++c) acc[q++] += w * xs[r] * xs[c];
             acc[28] += w * w;
+            if (d == 1) {
+                const double x = xs[0] - ref[0];
+                acc[1] += w * x;
+                acc[7] += w * x * x;
+                continue;
+            }
+            #pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                xs[k] -= ref[k];
+                acc[1 + k] += w * xs[k];
+            }
+            int q = 7;
+            #pragma unroll
+            for (int r = 0; r < 6; ++r)
+                #pragma unroll
+                for (int c = r; c < 6; ++c) acc[q++] += w * xs[r] * xs[c];
         }
     }
     __shared__ double red[32][RED_W + 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    // sums of one scalar state (eta) and of idle warps are zero beyond the first entries
-    const bool any = __any_sync(0xffffffffu, acc[0] != 0.0);
-    for (int i = 0; i < RED_W; ++i) {
-        const double s = any ? warp_sum_d(acc[i]) : 0.0;
-        if (lane == 0) red[wid][i] = s;
+    // the sums of a warp all at once: halving the values while the lanes pair up (31 FP64 additions instead of
+    // 145; lane i ends with the i-th sum).  An idle warp's are zero.
+    if (__any_sync(0xffffffffu, acc[0] != 0.0)) {
+        #pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const bool up = lane & o;
+            #pragma unroll
+            for (int i = 0; i < o; ++i) {
+                const double keep = up ? acc[i + o] : acc[i], give = up ? acc[i] : acc[i + o];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        }
     }
+    if (lane < RED_W) red[wid][lane] = acc[0];
     __syncthreads();
     if (threadIdx.x < RED_W) {
         double s = 0.0;
@@ -143,79 +163,93 @@ __device__ inline void pf_mask(const DevParams& Pm, int s, bool* a) {
     if (Pm.zero_mean) { a[4] = a[5] = false; }
 }
 
-// one warp per active belief: combine the partials (lane i the i-th sum, in block order), then lane 0
-// forms estimates and the jitter factor
-__global__ void k_norm_final(DevGeom G, DevParams Pm, DevState D, int S, int NB, const double* part) {
+// two warps per active belief: the first combines the partials (lane i the i-th sum, in block order), then its
+// lane 0 forms the normaliser while the second forms mean, covariance and the jitter factor, lanes over
+// their rows (one lane for everything took 36 us against 13, most of it FP64 square roots and divisions in turn)
+__global__ void __launch_bounds__(64) k_norm_final(DevGeom G, DevParams Pm, DevState D, int S, int NB, const double* part) {
     const int b = active_belief(blockIdx.x, S, Pm.S_max);
     const BeliefView v = belief_of(b, Pm, G.J);
-    const int P = Pm.P, lane = threadIdx.x;
-    __shared__ double acc[RED_W];
+    const int P = Pm.P, lane = threadIdx.x & 31;
+    __shared__ double acc[RED_W], Cs[6][6];
     double M = -INFINITY;
-    for (int i = lane; i < NB; i += 32) M = fmax(M, D.red_part[((size_t)b * NB + i) * RED_W]);
-    M = warp_max_d(M);
-    if (lane < RED_W) {
-        double t = 0.0;
-        #pragma unroll 4
-        for (int i = 0; i < NB; ++i) t += part[((size_t)b * NB + i) * RED_W + lane];
-        acc[lane] = t;
+    if (threadIdx.x < 32) {
+        for (int i = lane; i < NB; i += 32) M = fmax(M, D.red_part[((size_t)b * NB + i) * RED_W]);
+        M = warp_max_d(M);
+        if (lane < RED_W) {
+            double t = 0.0;
+            #pragma unroll 4
+            for (int i = 0; i < NB; ++i) t += part[((size_t)b * NB + i) * RED_W + lane];
+            acc[lane] = t;
+        }
     }
-    __syncwarp();
-    if (lane != 0) return;
+    __syncthreads();
+    double* rec = D.bel + bel_rec(Pm.S_max, G.J, b);
+    if (threadIdx.x < 32) {
+        if (lane != 0) return;
+        const double lse = (acc[0] > 0) ? M + log(acc[0]) : -INFINITY;
+        double logC = lse;
+        if (v.kind == 1) {
+            const double W = D.W[v.index];
+            const double ln = (W < 1.0) ? log1p(-W) : -INFINITY;
+            const double mx = fmax(lse, ln);
+            logC = (mx == -INFINITY) ? -INFINITY : mx + log(exp(lse - mx) + exp(ln - mx));
+            const double ps = (logC == -INFINITY) ? 0.0 : exp(lse - logC);
+            D.p_s[v.index] = ps;
+        }
+        rec[0] = M; rec[1] = lse; rec[2] = logC;
+        rec[3] = (acc[0] > 0) ? acc[28] / (acc[0] * acc[0]) : 1.0;   // sum of squared normalised weights
+        return;
+    }
+    const int d = v.dims;
+    const bool some = acc[0] > 0;
     double ref[6];
     belief_state(D, v, P, 0, ref);
-    double* rec = D.bel + bel_rec(Pm.S_max, G.J, b);
-    const double lse = (acc[0] > 0) ? M + log(acc[0]) : -INFINITY;
-    double logC = lse;
-    if (v.kind == 1) {
-        const double W = D.W[v.index];
-        const double ln = (W < 1.0) ? log1p(-W) : -INFINITY;
-        const double mx = fmax(lse, ln);
-        logC = (mx == -INFINITY) ? -INFINITY : mx + log(exp(lse - mx) + exp(ln - mx));
-        const double ps = (logC == -INFINITY) ? 0.0 : exp(lse - logC);
-        D.p_s[v.index] = ps;
-    }
-    rec[0] = M; rec[1] = lse; rec[2] = logC;
-    rec[3] = (acc[0] > 0) ? acc[28] / (acc[0] * acc[0]) : 1.0;   // sum of squared normalised weights
-    const int d = v.dims;
-    double mean[6] = {0, 0, 0, 0, 0, 0};
-    double C[6][6];
-    for (int r = 0; r < 6; ++r) for (int c = 0; c < 6; ++c) C[r][c] = 0.0;
-    if (acc[0] > 0) {
-        for (int k = 0; k < d; ++k) mean[k] = acc[1 + k] / acc[0];
-        int t = 7;
-        for (int r = 0; r < d; ++r)
-            for (int c = r; c < d; ++c) {
-                const double cv = acc[t++] / acc[0] - mean[r] * mean[c];
-                C[r][c] = C[c][r] = cv;
-            }
-        for (int k = 0; k < d; ++k) mean[k] += ref[k];
-    }
-    for (int k = 0; k < 6; ++k) rec[4 + k] = (k < d) ? mean[k] : 0.0;
-    // regularisation factor h_opt L (active dimensions only)
+    // lane k < 6: component k of the mean; lane t < 21: entry (r, c) of the covariance (active dimensions only)
+    double mean = 0.0;
+    if (some && lane < d) mean = acc[1 + lane] / acc[0];
     bool act[6];
     if (v.kind == 0) mt_mask(Pm, act);
     else if (v.kind == 1) pf_mask(Pm, v.index, act);
     else { act[0] = true; for (int k = 1; k < 6; ++k) act[k] = false; }
     int dact = 0;
     for (int k = 0; k < d; ++k) if (act[k]) ++dact;
-    for (int r = 0; r < 6; ++r) for (int c = 0; c < 6; ++c) if (!(r < d && c < d && act[r] && act[c])) C[r][c] = 0.0;
-    double L[6][6];
-    for (int r = 0; r < 6; ++r) for (int c = 0; c < 6; ++c) L[r][c] = 0.0;
-    for (int k = 0; k < d; ++k) {
-        double piv = C[k][k];
-        for (int m = 0; m < k; ++m) piv -= L[k][m] * L[k][m];
-        if (piv <= 0.0) continue;
-        L[k][k] = sqrt(piv);
-        for (int i = k + 1; i < d; ++i) {
-            double s = C[i][k];
-            for (int m = 0; m < k; ++m) s -= L[i][m] * L[k][m];
-            L[i][k] = s / L[k][k];
+    int r = 0, c = lane;
+    while (r < 5 && c >= 6 - r) { c -= 6 - r; ++r; }
+    c += r;
+    c = min(c, 5);
+    const double mr = __shfl_sync(0xffffffffu, mean, r), mc = __shfl_sync(0xffffffffu, mean, c);
+    if (lane < 21) {
+        bool on = some && r < d && c < d;
+        for (int k = 0; k < 6; ++k) if ((k == r || k == c) && !act[k]) on = false;
+        Cs[r][c] = Cs[c][r] = on ? acc[d == 1 ? 7 : 7 + lane] / acc[0] - mr * mc : 0.0;
+    }
+    double rk = 0.0;
+    #pragma unroll
+    for (int k = 0; k < 6; ++k) if (k == lane && k < d) rk = ref[k];
+    if (lane < 6) rec[4 + lane] = lane < d ? (some ? mean + rk : 0.0) : 0.0;
+    __syncwarp();
+    // Cholesky factor, lane i its row i (columns of non-positive pivots stay zero); h_opt L goes out
+    const int row = min(lane, 5);
+    double Lr[6] = {0, 0, 0, 0, 0, 0};
+    #pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        double x = Cs[row][k];
+        #pragma unroll
+        for (int m = 0; m < k; ++m) x -= Lr[m] * __shfl_sync(0xffffffffu, Lr[m], k);
+        const double piv = __shfl_sync(0xffffffffu, x, k);
+        if (k < d && piv > 0.0) {                 // uniform
+            const double lk = sqrt(piv);
+            if (lane == k) Lr[k] = lk;
+            else if (lane > k && lane < d) Lr[k] = x / lk;
         }
     }
     const double h = Pm.h_opt[dact];
     float* Lf = D.Lchol + (size_t)b * 36;
-    for (int r = 0; r < 6; ++r) for (int c = 0; c < 6; ++c) Lf[r * 6 + c] = (float)((Pm.regularize ? h : 0.0) * L[r][c]);
-    rec[10] = dact;
+    if (lane < 6) {
+        #pragma unroll
+        for (int k = 0; k < 6; ++k) Lf[lane * 6 + k] = (float)((Pm.regularize ? h : 0.0) * Lr[k]);
+    }
+    if (lane == 0) rec[10] = dact;
 }
 
 // estimates, declaration, pruning map: a thread per PF, the survivors numbered by ballot
@@ -315,7 +349,7 @@ int launch_normalize(const DevGeom& G, const DevParams& Pm, const DevState& D, i
     double* part = D.red_part + (size_t)bel_count(Pm.S_max, G.J) * 64 * RED_W;
     k_norm_max<<<dim3(NB, nb), 256, 0, st>>>(G, Pm, D, S, NB);
     k_norm_sum<<<dim3(NB, nb), 256, 0, st>>>(G, Pm, D, S, NB, part);
-    k_norm_final<<<nb, 32, 0, st>>>(G, Pm, D, S, NB, part);
+    k_norm_final<<<nb, 64, 0, st>>>(G, Pm, D, S, NB, part);
     k_estimate<<<1, S_CAP_MAX, 0, st>>>(G, Pm, D, S);
     k_norm_weights<<<dim3(cdf_tiles(P), nb), 256, 0, st>>>(G, Pm, D, S, D.tsum);
     return 5;

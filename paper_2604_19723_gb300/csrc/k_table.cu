@@ -232,8 +232,7 @@ __global__ void k_gram(DevGeom G, DevParams Pm, DevState D, int S, double* gram)
         const double2* mb = tab + ((size_t)b * J + j) * Nz;
         #pragma unroll 4
         for (int k = lane; k < Nz; k += 32) {
-            const double2 t = zmulc(ma[k], mb[k]);
-            acc.x += t.x; acc.y += t.y;
+            acc = zfmac(ma[k], mb[k], acc);
         }
         acc.x = warp_sum_d(acc.x); acc.y = warp_sum_d(acc.y);
         if (lane == 0) {
@@ -256,8 +255,8 @@ __global__ void k_gram(DevGeom G, DevParams Pm, DevState D, int S, double* gram)
 // column (the same basis that a factorisation of its own would give, at 12 operations per element
 // and rotation instead of K^2/2 products).  x^H V_s is x^H V_f under the same rotations.
 // Bound: the FP64 pipe (2 FMA per clock and SM) and the serial chains of pivots and rotations.
-// Measured, 4 PAs: 64 PFs x Nz = 160 1.74 -> 0.57 ms (with the Gram), 40 x 300 1.50 -> 0.43, 32 x 1024
-// 1.54 -> 0.52, 8 x 160 0.070 -> 0.068 (against a factorisation and a solve for every (s, j)).
+// Measured, 4 PAs: 64 PFs x Nz = 160 1.74 -> 0.46 ms (with the Gram), 40 x 300 1.50 -> 0.34, 32 x 1024
+// 1.54 -> 0.40, 8 x 160 0.070 -> 0.066 (against a factorisation and a solve for every (s, j)).
 constexpr int STAGE_THREADS = 256;
 constexpr int STAGE_WRED = 12;  // per-warp partial sums: the omega test's nine scalars, m^H e_all and |e_all|^2
 __host__ __device__ inline int stage_row(int K, int r) {   // start of row r of [L; carried rows of K]
@@ -322,11 +321,10 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_basis(DevGeom G, DevPar
         for (int r = k + 1 + (tid >> 4); r < S + ne; r += STAGE_THREADS / 16) {
             const int row = stage_row(S, r), end = min(r, S - 1);
             double2 x = Lp[row + k];
-            x.x *= ip; x.y *= ip;
+            x.x *= -ip; x.y *= -ip;
             for (int c = k + 1 + (tid & 15); c <= end; c += 16) {
-                const double2 u = zmulc(Lp[stage_row(S, c) + k], x);
                 double2& v = Lp[row + c];
-                v.x -= u.x; v.y -= u.y;
+                v = zfmac(Lp[stage_row(S, c) + k], x, v);
                 if (r == k + 1 && c == r) il[r] = 1.0 / fmax(v.x, 1.0);
             }
         }
@@ -435,19 +433,21 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
     } else {
         for (int t = wid - 1; t < S; t += nw - 1) {   // one warp per column of V_f
             const double2* vt = Vf + (size_t)t * Nz;
-            double ax = 0, ay = 0, bx = 0, by = 0, cx = 0, cy = 0;
+            double2 x0 = make_double2(0.0, 0.0), x1 = x0, x2 = x0;
+            #pragma unroll 4
             for (int k = lane; k < Nz; k += 32) {
                 const double2 v = vt[k];
-                const double2 u1 = zmulc(v, E0[k]), u2 = zmulc(v, mwp[k]), u3 = zmulc(v, m4p[k]);
-                ax += u1.x; ay += u1.y; bx += u2.x; by += u2.y; cx += u3.x; cy += u3.y;
+                x0 = zfmac(v, E0[k], x0);
+                x1 = zfmac(v, mwp[k], x1);
+                x2 = zfmac(v, m4p[k], x2);
             }
-            ax = warp_sum_d(ax); ay = warp_sum_d(ay);
-            bx = warp_sum_d(bx); by = warp_sum_d(by);
-            cx = warp_sum_d(cx); cy = warp_sum_d(cy);
+            x0 = make_double2(warp_sum_d(x0.x), warp_sum_d(x0.y));
+            x1 = make_double2(warp_sum_d(x1.x), warp_sum_d(x1.y));
+            x2 = make_double2(warp_sum_d(x2.x), warp_sum_d(x2.y));
             if (lane == 0) {
-                cr[t] = make_double2(ax, -ay);
-                cr[S + t] = make_double2(bx, -by);
-                cr[2 * S + t] = make_double2(cx, -cy);
+                cr[t] = make_double2(x0.x, -x0.y);
+                cr[S + t] = make_double2(x1.x, -x1.y);
+                cr[2 * S + t] = make_double2(x2.x, -x2.y);
             }
         }
     }
@@ -518,8 +518,7 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
         double2 r0 = make_double2(0.0, 0.0);
         auto put = [&](int c, double2 v) {
             Vs[(size_t)c * Nz + k] = v;
-            const double2 u = zmulc(ye[c], v);    // v (V^H e0)_c
-            r0.x += u.x; r0.y += u.y;
+            r0 = zfmac(ye[c], v, r0);             // v (V^H e0)_c
         };
         #pragma unroll 4
         for (int c = 0; c < s; ++c) put(c, Vf[(size_t)c * Nz + k]);
@@ -539,114 +538,139 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage_kappa(DevGeom G, DevPar
 // ---------------------------------------------------------------- nu: Householder tridiagonalisation per j (FP64)
 // T = Q^H G Q real symmetric tridiagonal, b' = Q^H b with b = M^H e_all; the
 // off-diagonal phases are moved into b' so that T has non-negative off-diagonals.
-__global__ void k_nu_tridiag(DevParams Pm, DevState D, int S, const double* gram, const double* nu_b) {
+// Block of 128 threads per j.  A step has one chain of square roots and divisions (the Householder vector v
+// stays unnormalised: H = I - beta v v^H, beta = 1 / (|x| (|x| + |x_0|))); its two rounds of sums over the column
+// are taken by every warp for itself (lane i the rows i and i + 32 of the trailing block), so a step
+// has four barriers.  Only the lower triangle is kept.  Bound: latency (J blocks).
+// Measured: 64 PFs 1269 -> 805 us, 8 PFs 58 -> 37 us (against block-wide sums, normalised vectors and the
+// whole matrix).
+constexpr int NU_THREADS = 128;
+__global__ void __launch_bounds__(NU_THREADS) k_nu_tridiag(DevParams Pm, DevState D, int S, const double* gram, const double* nu_b) {
     const int j = blockIdx.x;
     const int SM = Pm.S_max;
     extern __shared__ double2 sh[];
-    double2* A = sh;                 // S x S
+    double2* A = sh;                 // S x S, rows of S, lower triangle
     double2* v = A + (size_t)S * S;  // S
-    double2* pv = v + S;             // S
+    double2* pv = v + S;             // S: p = beta A v, then w
     double2* b = pv + S;             // S
-    __shared__ double red[32][3];
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-    // block sums of three values, returned to every thread
-    auto bsum3 = [&](double& x0, double& x1, double& x2) {
-        x0 = warp_sum_d(x0); x1 = warp_sum_d(x1); x2 = warp_sum_d(x2);
-        __syncthreads();
-        if (lane == 0) { red[wid][0] = x0; red[wid][1] = x1; red[wid][2] = x2; }
-        __syncthreads();
-        x0 = x1 = x2 = 0.0;
-        for (int w = 0; w < nw; ++w) { x0 += red[w][0]; x1 += red[w][1]; x2 += red[w][2]; }
-    };
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const double2* Gm = reinterpret_cast<const double2*>(gram) + (size_t)j * SM * SM;
     const double2* bv = reinterpret_cast<const double2*>(nu_b) + (size_t)j * (SM + 1);
-    for (int t = tid; t < S * S; t += nt) A[t] = Gm[(t / S) * SM + (t % S)];
-    for (int t = tid; t < S; t += nt) b[t] = bv[t];
+    for (int t = tid; t < S * S; t += NU_THREADS) A[t] = Gm[(t / S) * SM + (t % S)];
+    for (int t = tid; t < S; t += NU_THREADS) b[t] = bv[t];
     __syncthreads();
     for (int k = 0; k + 2 < S; ++k) {
-        // x = A[k+1:, k]; alpha = -ph |x| with ph the phase of x_0; v = (x - alpha e1)/|x - alpha e1|
-        double nx = 0.0, u1 = 0.0, u2 = 0.0;
-        for (int i = k + 1 + tid; i < S; i += nt) nx += A[i * S + k].x * A[i * S + k].x + A[i * S + k].y * A[i * S + k].y;
-        bsum3(nx, u1, u2);
-        nx = sqrt(nx);
-        const double2 x0 = A[(k + 1) * S + k];
-        const double ax0 = sqrt(x0.x * x0.x + x0.y * x0.y);
-        const double2 ph = ax0 > 0 ? make_double2(x0.x / ax0, x0.y / ax0) : make_double2(1.0, 0.0);
-        double vn = 0.0;
-        u1 = u2 = 0.0;
-        for (int i = k + 1 + tid; i < S; i += nt) {
-            double2 vi = A[i * S + k];
-            if (i == k + 1) { vi.x += ph.x * nx; vi.y += ph.y * nx; }
-            v[i] = vi;
-            vn += vi.x * vi.x + vi.y * vi.y;
+        const int n = S - k - 1, f = k + 1;       // trailing rows f .. S - 1
+        // x = A[f:, k]; alpha = -ph |x| with ph the phase of x_0; v = x - alpha e1
+        double2 x[2];
+        double nx2 = 0.0;
+        #pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            x[h] = i < n ? A[(f + i) * S + k] : make_double2(0.0, 0.0);
+            nx2 += x[h].x * x[h].x + x[h].y * x[h].y;
         }
-        bsum3(vn, u1, u2);
-        vn = sqrt(vn);
-        if (vn == 0.0) continue;   // the column is zero already (uniform across the block)
-        for (int i = k + 1 + tid; i < S; i += nt) { v[i].x /= vn; v[i].y /= vn; }
+        nx2 = warp_sum_d(nx2);
+        if (nx2 == 0.0) continue;                 // the column is zero already (uniform across the block)
+        const double2 x0 = A[f * S + k];
+        const double nx = sqrt(nx2), ax0 = sqrt(x0.x * x0.x + x0.y * x0.y);
+        const double beta = 1.0 / (nx * (nx + ax0)), q = ax0 > 0 ? nx / ax0 : 0.0;
+        const double2 al = ax0 > 0 ? make_double2(-x0.x * q, -x0.y * q) : make_double2(-nx, 0.0);   // alpha
+        if (lane == 0) { x[0].x -= al.x; x[0].y -= al.y; }
+        if (wid == 0) {
+            #pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (lane + 32 * h < n) v[f + lane + 32 * h] = x[h];
+        }
         __syncthreads();
-        // p = A v on the trailing block
-        for (int i = k + 1 + tid; i < S; i += nt) {
-            double2 acc = make_double2(0, 0);
-            for (int c = k + 1; c < S; ++c) {
-                const double2 u = zmul(A[i * S + c], v[c]);
-                acc.x += u.x; acc.y += u.y;
+        // p = beta A v on the trailing block: two threads per row
+        {
+            const int i = tid >> 1;
+            double2 acc = make_double2(0.0, 0.0);
+            if (i < n) {
+                const int r = f + i;
+                for (int c = f + (tid & 1); c < S; c += 2) {
+                    const double2 a = c <= r ? A[r * S + c] : A[c * S + r], vc = v[c];
+                    const double ai = c <= r ? a.y : -a.y;
+                    acc.x += a.x * vc.x - ai * vc.y;
+                    acc.y += a.x * vc.y + ai * vc.x;
+                }
             }
-            pv[i] = acc;
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+            if (i < n && !(tid & 1)) pv[f + i] = make_double2(beta * acc.x, beta * acc.y);
         }
         __syncthreads();
-        // K = v^H A v (real), v^H b
+        // K = beta/2 v^H p (real), v^H b
         double kr = 0.0, vbx = 0.0, vby = 0.0;
-        for (int i = k + 1 + tid; i < S; i += nt) {
-            kr += zmulc(v[i], pv[i]).x;
-            const double2 u = zmulc(v[i], b[i]);
-            vbx += u.x; vby += u.y;
+        double2 pr[2];
+        #pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            pr[h] = make_double2(0.0, 0.0);
+            if (i < n) {
+                pr[h] = pv[f + i];
+                kr += zmulc(x[h], pr[h]).x;
+                const double2 u = zmulc(x[h], b[f + i]);
+                vbx += u.x; vby += u.y;
+            }
         }
-        bsum3(kr, vbx, vby);
-        // w = p - K v; b <- H b = b - 2 v (v^H b)
-        for (int i = k + 1 + tid; i < S; i += nt) {
-            pv[i].x -= kr * v[i].x; pv[i].y -= kr * v[i].y;
-            const double2 u = zmul(v[i], make_double2(vbx, vby));
-            b[i].x -= 2.0 * u.x; b[i].y -= 2.0 * u.y;
+        kr = 0.5 * beta * warp_sum_d(kr);
+        vbx = beta * warp_sum_d(vbx);
+        vby = beta * warp_sum_d(vby);
+        __syncthreads();                          // p and b have been read
+        // w = p - K v; b <- H b = b - beta v (v^H b)
+        if (wid == 0) {
+            #pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = lane + 32 * h;
+                if (i < n) {
+                    pv[f + i] = make_double2(pr[h].x - kr * x[h].x, pr[h].y - kr * x[h].y);
+                    const double2 u = zmul(x[h], make_double2(vbx, vby));
+                    b[f + i].x -= u.x; b[f + i].y -= u.y;
+                }
+            }
         }
         __syncthreads();
-        // A <- A - 2 v w^H - 2 w v^H on the trailing block; column k: below-diagonal -> alpha e1
-        for (int t = tid; t < (S - k - 1) * (S - k - 1); t += nt) {
-            const int r = k + 1 + t / (S - k - 1), c = k + 1 + t % (S - k - 1);
-            const double2 a1 = zmul(v[r], make_double2(pv[c].x, -pv[c].y));
-            const double2 a2 = zmul(pv[r], make_double2(v[c].x, -v[c].y));
-            A[r * S + c].x -= 2.0 * (a1.x + a2.x);
-            A[r * S + c].y -= 2.0 * (a1.y + a2.y);
+        // A <- A - v w^H - w v^H on the trailing block; below the diagonal of column k only alpha is left
+        for (int i = tid >> 4; i < n; i += NU_THREADS / 16) {
+            const int r = f + i;
+            const double2 vr = v[r], wr = pv[r];
+            for (int c = f + (tid & 15); c <= r; c += 16) {
+                const double2 a1 = zmulc(pv[c], vr), a2 = zmulc(v[c], wr);
+                double2& a = A[r * S + c];
+                a.x -= a1.x + a2.x;
+                a.y -= a1.y + a2.y;
+            }
         }
-        const double2 al = make_double2(-ph.x * nx, -ph.y * nx);
-        for (int i = k + 1 + tid; i < S; i += nt) {
-            const double2 e = (i == k + 1) ? al : make_double2(0, 0);
-            A[i * S + k] = e;
-            A[k * S + i] = make_double2(e.x, -e.y);
-        }
+        if (tid == 0) A[f * S + k] = al;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        // make off-diagonals real non-negative: D = diag(e^{i th}), th_{k+1} = th_k + arg(e_k)
-        double* out = D.nu_T + (size_t)j * 4 * SM;   // [a(SM) | o(SM) | b'(2 SM)]
+    // make off-diagonals real non-negative: D = diag(e^{i th}), th_{k+1} = th_k + arg(e_k)
+    double* out = D.nu_T + (size_t)j * 4 * SM;    // [a(SM) | o(SM) | b'(2 SM)]
+    for (int k = tid; k + 1 < S; k += NU_THREADS) {
+        const double2 e = A[(k + 1) * S + k];
+        const double ae = sqrt(e.x * e.x + e.y * e.y);
+        out[SM + k] = ae;
+        v[k] = ae > 0 ? make_double2(e.x / ae, e.y / ae) : make_double2(1.0, 0.0);
+    }
+    __syncthreads();
+    if (tid == 0) {
         double2 ph = make_double2(1.0, 0.0);
         for (int k = 0; k < S; ++k) {
-            out[k] = A[k * S + k].x;
-            // b'' = D^H b
-            const double2 bb = zmulc(ph, b[k]);
-            out[2 * SM + 2 * k] = bb.x;
-            out[2 * SM + 2 * k + 1] = bb.y;
-            if (k + 1 < S) {
-                const double2 e = A[(k + 1) * S + k];
-                const double ae = sqrt(e.x * e.x + e.y * e.y);
-                out[SM + k] = ae;
-                if (ae > 0) ph = zmul(ph, make_double2(e.x / ae, e.y / ae));
-            }
+            pv[k] = ph;
+            if (k + 1 < S) ph = zmul(ph, v[k]);
         }
         D.nu_c[2 * j] = bv[SM].x;   // |e_all|^2
     }
+    __syncthreads();
+    for (int k = tid; k < S; k += NU_THREADS) {
+        out[k] = A[k * S + k].x;
+        const double2 bb = zmulc(pv[k], b[k]);    // b'' = D^H b
+        out[2 * SM + 2 * k] = bb.x;
+        out[2 * SM + 2 * k + 1] = bb.y;
+    }
 }
-
 void launch_table(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int nsplit, int chunk_req,
                   cudaStream_t st) {
     const TablePlan t = table_plan(G, chunk_req);
@@ -681,7 +705,7 @@ void launch_nu_tridiag(const DevGeom& G, const DevParams& Pm, const DevState& D,
     }
     const size_t sm = ((size_t)S * S + 3 * (size_t)S) * sizeof(double2);
     smem_allow_max((const void*)k_nu_tridiag);
-    k_nu_tridiag<<<G.J, 128, sm, fork ? side : st>>>(Pm, D, S, gram, nu_b);
+    k_nu_tridiag<<<G.J, NU_THREADS, sm, fork ? side : st>>>(Pm, D, S, gram, nu_b);
     if (fork) cudaEventRecord(ev_join, side);
 }
 
