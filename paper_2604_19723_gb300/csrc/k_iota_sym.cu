@@ -469,19 +469,25 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
 // Every particle from 24 PFs on (the quantities, the bound and the selection are those of
 // k_iota_bulk.cu): log det A and rhs^H A^-1 rhs from one LDL^T elimination of the real A, e = z -
 // sum_s w0_s u_s element by element, |e|^2 - rhs^H A^-1 rhs.  One warp per (particle, PA).
-//   * e: lanes over (y, m), two frequencies per packed FP32 pair; P and Q take 2 x 4 packed FMAs
-//     with the steering elements formed on the way.
-//   * rhs: lanes over PFs, the frequencies' factors in registers, packed the same way.
+//   * e: a_y a_z = c of an element (y, m) is conj(c) at the mirrored (My - 1 - y, Mz - 1 - m), so sums and
+//     differences over that pair (P+, P-, Q+, Q-) need the products b c only part by part: lanes over
+//     the pairs (groups of lanes over PFs where the pairs leave lanes idle), two frequencies per
+//     packed FP32 pair, eight packed FMAs per PF, pair and two frequencies.
+//   * rhs: lanes over PFs; per frequency the sums over the pairs in the same eight FMAs, then the
+//     frequencies' factors.
 //   * A: the lower triangle in registers, lane (tr, tc) of 8 x 4 owning (8 ia + tr, 4 ib + tc).  Panels of
 //     eight columns go through shared memory: lanes take rows, factor the panel with shuffles (the
 //     forward substitution rides along), then every lane applies the rank-8 update to its entries.
 // Bound: FP32 issue.  The whole stage at 64 PFs x 1e5 particles (Nz = 160) / 32 x 262144 (Nz = 1024):
 // 27.7 / 69 ms with a block of 64 threads per particle on the complex matrix, 15.1 / 54.4 with this
-// split but one column of the elimination at a time and unpacked e and rhs, 12.0 / 26.6 as it is.
+// split but one column of the elimination at a time and unpacked e and rhs, 12.0 / 26.7 with both packed
+// element by element and the panels unrolled, 9.5 / 22.1 as it is (instruction fetch was a fifth of the
+// stalls at 64 PFs: loops whose body is long stay rolled).
 constexpr float IB_ERR_PER_RATIO = 4.0e-6f;    // as in k_iota_bulk.cu
 constexpr float IB_ERR_PER_ENERGY = 1.0e-6f;
 constexpr int IB_W = 4;                        // warps (PAs of a particle) per block
 constexpr int IB_FP = 4;                       // frequency pairs per lane and pass
+constexpr int IB_Q = 8;                        // Re P+, Im Q-, Im P+, -Re Q-, -Re P-, Im Q+, -Im P-, -Re Q+
 constexpr int IB_PST = 12;                     // row stride of the panel (conflict-free 128-bit accesses)
 struct IbPlan { size_t pq, pan, fx, fy, ant, vec, warp; int fp, f4, ast; };
 template <int NB>
@@ -493,7 +499,7 @@ __host__ __device__ inline IbPlan ib_plan(const DevGeom& G, int S) {
     p.ast = (d.hy + d.hz) | 1;
     const size_t R = 8 * NB;                   // rows beyond S are zero
     size_t o = 0;
-    p.pq = o; o += (size_t)G.My * G.Mz * 4 * p.f4 * sizeof(float);
+    p.pq = o; o += (size_t)d.Nmh * IB_Q * p.f4 * sizeof(float);
     p.pan = o; o += R * IB_PST * sizeof(float);
     p.fx = o; o += R * p.fp * sizeof(float);
     p.fy = o; o += R * p.fp * sizeof(float);
@@ -521,26 +527,28 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
     float* perr = reinterpret_cast<float*>(ies + 16);           // [2][16] bound per PA
     float* pbad = perr + 32;                                    // [2][16] breakdown per PA
     char* base = reinterpret_cast<char*>(smb) + IB_FIXED + (size_t)wid * pl.warp;
-    float* pq = reinterpret_cast<float*>(base + pl.pq);         // [Nm][P re, P im, -Q re, Q im][f4] e
+    float* pq = reinterpret_cast<float*>(base + pl.pq);         // [Nmh][IB_Q][f4] e
     float* pan = reinterpret_cast<float*>(base + pl.pan);       // [8 NB][IB_PST] panel of eight columns
     float* fx = reinterpret_cast<float*>(base + pl.fx);         // [8 NB][fp] Re b_f
     float* fy = reinterpret_cast<float*>(base + pl.fy);         // [8 NB][fp] Im b_f
     float2* ant = reinterpret_cast<float2*>(base + pl.ant);     // [8 NB][ast] a_y, a_z (half of each)
-    float4* ws = reinterpret_cast<float4*>(base + pl.vec);      // [8 NB] -2 A c pi mu, each part twice
+    float4* ws = reinterpret_cast<float4*>(base + pl.vec);      // [8 NB] -4 A c pi mu (two parts)
     float* dA = reinterpret_cast<float*>(ws + 8 * NB);          // [8 NB] d_s A_s
     const float* phi = D.phi[D.cur];
-    const bool odd = Nz & 1;
     if (threadIdx.x < J) {
         lgs[threadIdx.x] = log(D.eta_bar[threadIdx.x]);
         ies[threadIdx.x] = 1.0 / D.eta_bar[threadIdx.x];
     }
     for (int i = lane; i < 8 * NB * pl.fp; i += 32) fx[i] = fy[i] = 0.f;     // rows and columns beyond S and Fh stay zero
     for (int i = lane; i < 8 * NB * pl.ast; i += 32) ant[i] = make_float2(0.f, 0.f);
-    for (int i = lane; i < Nm * 4 * pl.f4; i += 32) pq[i] = 0.f;
+    for (int i = lane; i < dm.Nmh * IB_Q * pl.f4; i += 32) pq[i] = 0.f;
     __syncthreads();
-    // element blocks of the residual: NL lanes over (y, m), the groups of lanes over frequency pairs
-    const int NL = min(Nm, 32), ngrp = 32 / NL, lg = lane / NL, ly = lane - lg * NL;
-    const int np2 = (dm.Fh + 1) / 2, npass = (np2 + ngrp * IB_FP - 1) / (ngrp * IB_FP), fc = (np2 + ngrp * npass - 1) / (ngrp * npass);
+    // residual: NL lanes over the element pairs, the groups of lanes over frequency pairs (gf groups of up to
+    // IB_FP) and what is left of them over PFs (gs)
+    const int np2 = (dm.Fh + 1) / 2;
+    const int NL = min(dm.Nmh, 32), ngrp = 32 / NL, gf = min(ngrp, (np2 + IB_FP - 1) / IB_FP), gs = ngrp / gf;
+    const int lg = lane / NL, ly = lane - lg * NL, fg = lg % gf, sg = min(lg / gf, gs - 1);
+    const bool first = lg < gf;                                 // the lanes that collect
     // Gram over frequencies in pairs; the middle one of an odd count (exactly 1) may be among them
     const int gp = (Nf / 2 + 1) / 2;
     const float mf = (Nf & 1) ? ((Nf / 2) & 1 ? -1.0f : 1.0f) : 0.0f;
@@ -550,7 +558,7 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
         for (int j = wid; j < J; j += W) {
             __syncwarp();
             const float ebf = (float)D.eta_bar[j];
-            #pragma unroll
+            #pragma unroll 1
             for (int hr = 0; hr < NR; ++hr) {   // factors and weights, lanes over PFs
                 const int s = lane + 32 * hr;
                 float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -568,12 +576,14 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                     const float2 c = cispi_ff(-2.0f * h, -2.0f * l);
                     d = A * sqrtf(fmaxf(pi * (gm + (mr * mr + mi * mi) * (1.0f - pi)), 0.0f));
                     const float2 w0 = cmul(make_float2(A * pi * mr, A * pi * mi), c);
-                    w = make_float4(-2.0f * w0.x, -2.0f * w0.x, -2.0f * w0.y, -2.0f * w0.y);
+                    w = make_float4(-4.0f * w0.x, -4.0f * w0.y, 0.f, 0.f);
+                    #pragma unroll 1
                     for (int f = 0; f < dm.Fh; ++f) {
                         const float2 b = freq_factor(G, g, f);
                         fx[s * pl.fp + f] = b.x;
                         fy[s * pl.fp + f] = b.y;
                     }
+                    #pragma unroll 1
                     for (int q = 0; q < dm.hy + dm.hz; ++q) {
                         const bool y = q < dm.hy;
                         const int e = y ? q : q - dm.hy;
@@ -593,86 +603,102 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                 b.y *= sz;
                 return cmul(a, b);
             };
-            // e = z - sum_s w0_s u_s as sums and differences of mirrored elements; |e|^2
+            // e = z - sum_s w0_s u_s and |e|^2
             float ee = 0.f;
-            for (int y0 = 0; y0 < Nm; y0 += NL) {
-                const int ym = y0 + ly, y = min(ym, Nm - 1) / Mz, m = min(ym, Nm - 1) - y * Mz;
+            for (int q0 = 0; q0 < dm.Nmh; q0 += NL) {
+                const int ym = q0 + ly, y = min(ym, dm.Nmh - 1) / Mz, m = min(ym, dm.Nmh - 1) - y * Mz, ym2 = Nm - 1 - ym;
+                const bool self = ym2 == ym, act = ym < dm.Nmh && first;
                 bool cy, cz;
                 const int iy = is_half(y, My, dm.hy, cy), iz = dm.hy + is_half(m, Mz, dm.hz, cz);
-                const float sy = cy ? -1.0f : 1.0f, sz = cz ? -1.0f : 1.0f;
-                for (int ps = 0; ps < npass; ++ps) {
-                    const int f0 = 2 * (ps * ngrp + lg) * fc;
-                    const bool act = ym < Nm && lg < ngrp && f0 < dm.Fh;
-                    const int fl = act ? f0 : 0;
-                    f2x a[IB_FP][4];
+                const float sy = cy ? -1.0f : 1.0f, sz = cz ? -1.0f : 1.0f, sw = self ? 0.5f : 1.0f;
+                for (int b0 = 0; b0 < np2; b0 += gf * IB_FP) {   // frequency pairs
+                    const int g0 = min(b0 + fg * IB_FP, np2), nf = min(IB_FP, np2 - g0), fl = nf > 0 ? 2 * g0 : 0;
+                    f2x a[IB_FP][IB_Q];
                     #pragma unroll
                     for (int i = 0; i < IB_FP; ++i) {
-                        float v[4][2];
+                        float v[2][IB_Q];
                         #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int f = f0 + 2 * i + q, k = f * Nm + ym;
-                            v[0][q] = v[1][q] = v[2][q] = v[3][q] = 0.f;
-                            if (act && i < fc && f < dm.Fh && k < dm.Nh) {
-                                const float *pa = z + 2 * ((size_t)j * Nz + k), *pb = z + 2 * ((size_t)j * Nz + Nz - 1 - k);
-                                const float2 za = make_float2(pa[0], pa[1]), zb = make_float2(pb[0], pb[1]);
-                                const bool mid = odd && k == dm.Nh - 1;      // carried doubled
-                                v[0][q] = za.x + zb.x;
-                                v[1][q] = za.y + zb.y;
-                                v[2][q] = mid ? 0.f : zb.x - za.x;
-                                v[3][q] = mid ? 0.f : za.y - zb.y;
+                        for (int h = 0; h < 2; ++h) {
+                            const int f = 2 * (g0 + i) + h;
+                            #pragma unroll
+                            for (int q = 0; q < IB_Q; ++q) v[h][q] = 0.f;
+                            if (act && f < dm.Fh) {
+                                auto obs = [&](int k) { return make_float2(z[2 * ((size_t)j * Nz + k)], z[2 * ((size_t)j * Nz + k) + 1]); };
+                                const float2 z0 = obs(f * Nm + ym), z1 = obs(Nz - 1 - (f * Nm + ym));
+                                const float2 P = make_float2(z0.x + z1.x, z0.y + z1.y), Q = make_float2(z0.x - z1.x, z0.y - z1.y);
+                                float2 P2 = make_float2(0.f, 0.f), Q2 = P2;
+                                if (!self) {
+                                    const float2 z2 = obs(f * Nm + ym2), z3 = obs(Nz - 1 - (f * Nm + ym2));
+                                    P2 = make_float2(z2.x + z3.x, z2.y + z3.y);
+                                    Q2 = make_float2(z2.x - z3.x, z2.y - z3.y);
+                                }
+                                v[h][0] = P.x + P2.x;
+                                v[h][2] = P.y + P2.y;
+                                v[h][5] = Q.y + Q2.y;
+                                v[h][7] = -(Q.x + Q2.x);
+                                if (!self) {
+                                    v[h][1] = Q.y - Q2.y;
+                                    v[h][3] = Q2.x - Q.x;
+                                    v[h][4] = P2.x - P.x;
+                                    v[h][6] = P2.y - P.y;
+                                }
                             }
                         }
                         #pragma unroll
-                        for (int c = 0; c < 4; ++c) a[i][c] = f2_pack(v[c][0], v[c][1]);
+                        for (int q = 0; q < IB_Q; ++q) a[i][q] = f2_pack(v[0][q], v[1][q]);
                     }
-                    #pragma unroll 2
-                    for (int s = 0; s < S; ++s) {
-                        const float2 c = antenna(s, iy, sy, iz, sz);
-                        const float4 w = ws[s];
-                        const f2x cx = f2_dup(c.x), cyy = f2_dup(c.y), ncy = f2_dup(-c.y);
-                        const f2x wr = f2_pack(w.x, w.y), wi = f2_pack(w.z, w.w);
+                    #pragma unroll 1
+                    for (int s = sg; s < S; s += gs) {
+                        float2 c = antenna(s, iy, sy, iz, sz);
+                        const float2 w = *reinterpret_cast<const float2*>(ws + s);
+                        c.x *= sw;
+                        c.y *= sw;
+                        const f2x t0 = f2_dup(w.x * c.x), t1 = f2_dup(w.y * c.x), t2 = f2_dup(w.x * c.y), t3 = f2_dup(w.y * c.y);
                         const float2 *bx = reinterpret_cast<const float2*>(fx + s * pl.fp + fl),
                                      *by = reinterpret_cast<const float2*>(fy + s * pl.fp + fl);
                         #pragma unroll
                         for (int i = 0; i < IB_FP; ++i) {
-                            if (i < fc) {
+                            if (i < nf) {
                                 const float2 xv = bx[i], yv = by[i];
                                 const f2x x2 = f2_pack(xv.x, xv.y), y2 = f2_pack(yv.x, yv.y);
-                                const f2x ux = f2_fma(x2, cx, f2_mul(y2, ncy)), uy = f2_fma(x2, cyy, f2_mul(y2, cx));
-                                a[i][0] = f2_fma(wr, ux, a[i][0]);
-                                a[i][1] = f2_fma(wi, ux, a[i][1]);
-                                a[i][2] = f2_fma(wi, uy, a[i][2]);       // -Q re
-                                a[i][3] = f2_fma(wr, uy, a[i][3]);
+                                a[i][0] = f2_fma(t0, x2, a[i][0]);
+                                a[i][1] = f2_fma(t2, x2, a[i][1]);
+                                a[i][2] = f2_fma(t1, x2, a[i][2]);
+                                a[i][3] = f2_fma(t3, x2, a[i][3]);
+                                a[i][4] = f2_fma(t2, y2, a[i][4]);
+                                a[i][5] = f2_fma(t0, y2, a[i][5]);
+                                a[i][6] = f2_fma(t3, y2, a[i][6]);
+                                a[i][7] = f2_fma(t1, y2, a[i][7]);
                             }
                         }
                     }
                     #pragma unroll
                     for (int i = 0; i < IB_FP; ++i) {
-                        if (act && i < fc && f0 + 2 * i < pl.f4) {
-                            float v[4][2];
+                        if (b0 + i >= np2) break;                 // uniform
+                        f2x t[IB_Q];                              // the groups' shares (for the first group's lanes)
+                        #pragma unroll
+                        for (int q = 0; q < IB_Q; ++q) t[q] = a[i][q];
+                        #pragma unroll 1
+                        for (int g = 1; g < gs; ++g) {
                             #pragma unroll
-                            for (int c = 0; c < 4; ++c) {
+                            for (int q = 0; q < IB_Q; ++q) t[q] = f2_add(t[q], __shfl_sync(0xffffffffu, a[i][q], lane + g * gf * NL));
+                        }
+                        const int f0 = 2 * (g0 + i);
+                        if (act && i < nf) {
+                            #pragma unroll
+                            for (int q = 0; q < IB_Q; ++q) {
                                 uint32_t u0, u1;
-                                f2_unpack(a[i][c], u0, u1);
-                                v[c][0] = __uint_as_float(u0);
-                                v[c][1] = __uint_as_float(u1);
+                                f2_unpack(t[q], u0, u1);
+                                float v0 = __uint_as_float(u0), v1 = __uint_as_float(u1);
+                                // the middle frequency holds both elements of a pair as one: half of each sum
+                                if ((Nf & 1) && f0 == dm.Fh - 1) v0 *= 0.5f;
+                                if ((Nf & 1) && f0 + 1 == dm.Fh - 1) v1 *= 0.5f;
+                                if (f0 + 1 >= dm.Fh) v1 = 0.f;
+                                const float g1 = self ? 0.5f : 0.25f;
+                                ee = fmaf(((Nf & 1) && f0 == dm.Fh - 1 ? 2.0f : 1.0f) * g1 * v0, v0, ee);
+                                ee = fmaf(((Nf & 1) && f0 + 1 == dm.Fh - 1 ? 2.0f : 1.0f) * g1 * v1, v1, ee);
+                                *reinterpret_cast<float2*>(pq + (ym * IB_Q + q) * pl.f4 + f0) = make_float2(v0, v1);
                             }
-                            #pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                const int f = f0 + 2 * i + q, k = f * Nm + ym;
-                                if (f >= dm.Fh || k >= dm.Nh) v[0][q] = v[1][q] = v[2][q] = v[3][q] = 0.f;
-                                float half = 0.5f;
-                                if (odd && k == dm.Nh - 1) {
-                                    v[0][q] *= 0.5f; v[1][q] *= 0.5f;
-                                    v[2][q] = v[3][q] = 0.f;
-                                    half = 1.0f;
-                                }
-                                const float e2 = fmaf(v[0][q], v[0][q], fmaf(v[1][q], v[1][q], fmaf(v[2][q], v[2][q], v[3][q] * v[3][q])));
-                                ee = fmaf(half, e2, ee);
-                            }
-                            #pragma unroll
-                            for (int c = 0; c < 4; ++c)
-                                *reinterpret_cast<float2*>(pq + (ym * 4 + c) * pl.f4 + f0 + 2 * i) = make_float2(v[c][0], v[c][1]);
                         }
                     }
                 }
@@ -682,78 +708,83 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
             // rhs_s = (dA)_s u_s^H e
             float2 rhs[NR];
             {
-                f2x gr[NR], gi[NR];
+                float gr[NR], gi[NR];
                 #pragma unroll
-                for (int hr = 0; hr < NR; ++hr) gr[hr] = gi[hr] = f2_dup(0.f);
+                for (int hr = 0; hr < NR; ++hr) gr[hr] = gi[hr] = 0.f;
                 for (int f0 = 0; f0 < dm.Fh; f0 += 8) {
-                    f2x bx[NR][4], by[NR][4];
+                    f2x xr[NR][4], xi[NR][4], yr[NR][4], yi[NR][4];
                     #pragma unroll
                     for (int hr = 0; hr < NR; ++hr)
                         #pragma unroll
-                        for (int i = 0; i < 4; i += 2) {
-                            const int s = min(lane + 32 * hr, 8 * NB - 1);
-                            const float4 xv = *reinterpret_cast<const float4*>(fx + s * pl.fp + f0 + 2 * i);
-                            const float4 yv = *reinterpret_cast<const float4*>(fy + s * pl.fp + f0 + 2 * i);
-                            bx[hr][i] = f2_pack(xv.x, xv.y); bx[hr][i + 1] = f2_pack(xv.z, xv.w);
-                            by[hr][i] = f2_pack(yv.x, yv.y); by[hr][i + 1] = f2_pack(yv.z, yv.w);
+                        for (int i = 0; i < 4; ++i) xr[hr][i] = xi[hr][i] = yr[hr][i] = yi[hr][i] = f2_dup(0.f);
+                    const bool wide = f0 + 4 < dm.Fh, full = f0 + 6 < dm.Fh;   // uniform: the later frequencies of the eight
+                    int y = 0, m = 0;
+                    #pragma unroll 1
+                    for (int ym = 0; ym < dm.Nmh; ++ym) {
+                        bool cy, cz;
+                        const int iy = is_half(y, My, dm.hy, cy), iz = dm.hy + is_half(m, Mz, dm.hz, cz);
+                        const float sy = cy ? -1.0f : 1.0f, sz = cz ? -1.0f : 1.0f;
+                        const float* e = pq + (size_t)ym * IB_Q * pl.f4 + f0;
+                        f2x cx[NR], cyy[NR];
+                        #pragma unroll
+                        for (int hr = 0; hr < NR; ++hr) {
+                            const float2 c = antenna(min(lane + 32 * hr, 8 * NB - 1), iy, sy, iz, sz);
+                            cx[hr] = f2_dup(c.x);
+                            cyy[hr] = f2_dup(c.y);
                         }
-                    const bool wide = f0 + 4 < dm.Fh;               // uniform: frequencies beyond the first four
-                    for (int y = 0; y < My; ++y) {
-                        bool cy;
-                        const int iy = is_half(y, My, dm.hy, cy);
-                        const float sy = cy ? -1.0f : 1.0f;
-                        for (int m = 0; m < Mz; ++m) {
-                            bool cz;
-                            const int iz = dm.hy + is_half(m, Mz, dm.hz, cz);
-                            const float sz = cz ? -1.0f : 1.0f;
-                            const float* e = pq + (size_t)(y * Mz + m) * 4 * pl.f4 + f0;
-                            f2x cx[NR], cyy[NR], ncy[NR];
+                        auto acc = [&](int i, int q, f2x (&o)[NR][4], const f2x (&c)[NR]) {   // two frequency pairs of one sum
+                            const float4 v = *reinterpret_cast<const float4*>(e + q * pl.f4 + 2 * i);
                             #pragma unroll
                             for (int hr = 0; hr < NR; ++hr) {
-                                const float2 c = antenna(min(lane + 32 * hr, 8 * NB - 1), iy, sy, iz, sz);
-                                cx[hr] = f2_dup(c.x);
-                                cyy[hr] = f2_dup(c.y);
-                                ncy[hr] = f2_dup(-c.y);
+                                o[hr][i] = f2_fma(c[hr], f2_pack(v.x, v.y), o[hr][i]);
+                                if (i == 0 || full) o[hr][i + 1] = f2_fma(c[hr], f2_pack(v.z, v.w), o[hr][i + 1]);
                             }
-                            #pragma unroll
-                            for (int i = 0; i < 4; i += 2) {
-                                if (i == 0 || wide) {
-                                    const float4 pr = *reinterpret_cast<const float4*>(e + 2 * i);
-                                    const float4 pi = *reinterpret_cast<const float4*>(e + pl.f4 + 2 * i);
-                                    const float4 nq = *reinterpret_cast<const float4*>(e + 2 * pl.f4 + 2 * i);
-                                    const float4 qi = *reinterpret_cast<const float4*>(e + 3 * pl.f4 + 2 * i);
-                                    #pragma unroll
-                                    for (int hr = 0; hr < NR; ++hr) {
-                                        auto two = [&](f2x x2, f2x y2, f2x epr, f2x epi, f2x enq, f2x eqi) {
-                                            const f2x ux = f2_fma(x2, cx[hr], f2_mul(y2, ncy[hr]));
-                                            const f2x uy = f2_fma(x2, cyy[hr], f2_mul(y2, cx[hr]));
-                                            gr[hr] = f2_fma(ux, epr, f2_fma(uy, eqi, gr[hr]));
-                                            gi[hr] = f2_fma(ux, epi, f2_fma(uy, enq, gi[hr]));
-                                        };
-                                        two(bx[hr][i], by[hr][i], f2_pack(pr.x, pr.y), f2_pack(pi.x, pi.y), f2_pack(nq.x, nq.y),
-                                            f2_pack(qi.x, qi.y));
-                                        two(bx[hr][i + 1], by[hr][i + 1], f2_pack(pr.z, pr.w), f2_pack(pi.z, pi.w),
-                                            f2_pack(nq.z, nq.w), f2_pack(qi.z, qi.w));
-                                    }
-                                }
+                        };
+                        #pragma unroll
+                        for (int i = 0; i < 4; i += 2) {
+                            if (i == 0 || wide) {
+                                acc(i, 0, xr, cx);
+                                acc(i, 1, xr, cyy);
+                                acc(i, 2, xi, cx);
+                                acc(i, 3, xi, cyy);
+                                acc(i, 4, yr, cyy);
+                                acc(i, 5, yr, cx);
+                                acc(i, 6, yi, cyy);
+                                acc(i, 7, yi, cx);
                             }
                         }
+                        if (++m == Mz) { m = 0; ++y; }
+                    }
+                    #pragma unroll
+                    for (int hr = 0; hr < NR; ++hr) {
+                        const int s = min(lane + 32 * hr, 8 * NB - 1);
+                        f2x r2 = f2_dup(0.f), i2 = r2;
+                        #pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float2 xv = *reinterpret_cast<const float2*>(fx + s * pl.fp + f0 + 2 * i);
+                            const float2 yv = *reinterpret_cast<const float2*>(fy + s * pl.fp + f0 + 2 * i);
+                            const f2x bx = f2_pack(xv.x, xv.y), by = f2_pack(yv.x, yv.y);
+                            r2 = f2_fma(bx, xr[hr][i], f2_fma(by, yr[hr][i], r2));
+                            i2 = f2_fma(bx, xi[hr][i], f2_fma(by, yi[hr][i], i2));
+                        }
+                        uint32_t r0, r1, i0, i1;
+                        f2_unpack(r2, r0, r1);
+                        f2_unpack(i2, i0, i1);
+                        gr[hr] += __uint_as_float(r0) + __uint_as_float(r1);
+                        gi[hr] += __uint_as_float(i0) + __uint_as_float(i1);
                     }
                 }
                 #pragma unroll
                 for (int hr = 0; hr < NR; ++hr) {
-                    uint32_t r0, r1, i0, i1;
-                    f2_unpack(gr[hr], r0, r1);
-                    f2_unpack(gi[hr], i0, i1);
                     const float d = dA[min(lane + 32 * hr, 8 * NB - 1)];
-                    rhs[hr] = make_float2(d * (__uint_as_float(r0) + __uint_as_float(r1)),
-                                          d * (__uint_as_float(i0) + __uint_as_float(i1)));
+                    rhs[hr] = make_float2(d * gr[hr], d * gi[hr]);
                 }
             }
             // Gram of this lane's entries: frequencies two at a time, then the antenna factors row block by row block
             float A[NSL];
             #pragma unroll
             for (int q = 0; q < NSL; ++q) A[q] = 0.f;
+            #pragma unroll 1
             for (int g = 0; g < gp; ++g) {
                 float2 rx[NB], ry[NB];
                 #pragma unroll
@@ -780,6 +811,7 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                 const int a = 8 * ia + tr;
                 const float2* ra = ant + a * pl.ast;
                 const float2* rc = ant + tc * pl.ast;
+                #pragma unroll 1
                 for (int u = 0; u < My / 2; ++u) {
                     const float2 r = ra[u];
                     #pragma unroll
@@ -788,6 +820,7 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                         sy[ib] = fmaf(r.x, cb.x, fmaf(r.y, cb.y, sy[ib]));
                     }
                 }
+                #pragma unroll 1
                 for (int u = dm.hy; u < dm.hy + Mz / 2; ++u) {
                     const float2 r = ra[u];
                     #pragma unroll
@@ -810,14 +843,19 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
             float yy = 0.f, pv[NR];
             #pragma unroll
             for (int hr = 0; hr < NR; ++hr) pv[hr] = 1.f;
-            #pragma unroll
-            for (int K = 0; K < NB; ++K) {
-                if (8 * K >= S) break;                              // uniform
+            // (one copy of the panel's code for every panel: unrolled, instruction fetch set the time)
+            #pragma unroll 1
+            for (int K = 0; 8 * K < S; ++K) {
                 __syncwarp();
                 #pragma unroll
-                for (int ia = K; ia < NB; ++ia) {
-                    pan[(8 * ia + tr) * IB_PST + tc] = A[ia * (ia + 1) + 2 * K];
-                    pan[(8 * ia + tr) * IB_PST + 4 + tc] = A[ia * (ia + 1) + 2 * K + 1];
+                for (int q = 0; q < NB; ++q) {
+                    if (q == K) {
+                        #pragma unroll
+                        for (int ia = q; ia < NB; ++ia) {
+                            pan[(8 * ia + tr) * IB_PST + tc] = A[ia * (ia + 1) + 2 * q];
+                            pan[(8 * ia + tr) * IB_PST + 4 + tc] = A[ia * (ia + 1) + 2 * q + 1];
+                        }
+                    }
                 }
                 __syncwarp();
                 float x[NR][8], ip[8];
@@ -828,20 +866,24 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                     x[hr][0] = v0.x; x[hr][1] = v0.y; x[hr][2] = v0.z; x[hr][3] = v0.w;
                     x[hr][4] = v1.x; x[hr][5] = v1.y; x[hr][6] = v1.z; x[hr][7] = v1.w;
                 }
+                const bool up = NR > 1 && K >= 4;                   // row k = 8 K + c belongs to lane k % 32 of half k / 32
+                const int ow = (8 * K) & 31;
                 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    // row k = 8 K + c belongs to lane (8 K + c) % 32 of half (8 K) / 32; rows above k hold nothing
-                    // that is used again
-                    const int ow = (8 * K + c) & 31, hf = (8 * K) / 32;
-                    const float piv = __shfl_sync(0xffffffffu, x[hf][c], ow);
+                    // (rows above k hold nothing that is used again)
+                    const float xc = up ? x[NR - 1][c] : x[0][c];
+                    const float2 rc = up ? rhs[NR - 1] : rhs[0];
+                    const float piv = __shfl_sync(0xffffffffu, xc, ow + c);
                     ip[c] = __frcp_rn(piv);
-                    const float2 rk = make_float2(__shfl_sync(0xffffffffu, rhs[hf].x, ow), __shfl_sync(0xffffffffu, rhs[hf].y, ow));
+                    const float2 rk = make_float2(__shfl_sync(0xffffffffu, rc.x, ow + c), __shfl_sync(0xffffffffu, rc.y, ow + c));
                     const float2 y = make_float2(rk.x * ip[c], rk.y * ip[c]);
                     yy = fmaf(rk.x, y.x, fmaf(rk.y, y.y, yy));
-                    if (lane == ow) pv[hf] = piv;
+                    if (lane == ow + c) {
+                        if (up) pv[NR - 1] = piv; else pv[0] = piv;
+                    }
                     #pragma unroll
                     for (int c2 = c + 1; c2 < 8; ++c2) {
-                        const float l = -ip[c] * __shfl_sync(0xffffffffu, x[hf][c], (8 * K + c2) & 31);
+                        const float l = -ip[c] * __shfl_sync(0xffffffffu, xc, ow + c2);
                         #pragma unroll
                         for (int hr = 0; hr < NR; ++hr) x[hr][c2] = fmaf(x[hr][c], l, x[hr][c2]);
                     }
@@ -851,7 +893,6 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                         rhs[hr].y = fmaf(-x[hr][c], y.y, rhs[hr].y);
                     }
                 }
-                if (K + 1 == NB) break;
                 #pragma unroll
                 for (int hr = 0; hr < NR; ++hr) {
                     if (lane + 32 * hr < 8 * NB) {
@@ -862,20 +903,24 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                 }
                 __syncwarp();
                 #pragma unroll
-                for (int q = 0; q < 2; ++q) {                       // the rank-8 update, four columns at a time
-                    float4 rv[NB];
+                for (int KK = 0; KK + 1 < NB; ++KK) {               // the rank-8 update, four columns at a time
+                    if (KK != K) continue;
                     #pragma unroll
-                    for (int ia = K + 1; ia < NB; ++ia) {
-                        const float4 v = *reinterpret_cast<const float4*>(pan + (8 * ia + tr) * IB_PST + 4 * q);
-                        rv[ia] = make_float4(v.x * -ip[4 * q], v.y * -ip[4 * q + 1], v.z * -ip[4 * q + 2], v.w * -ip[4 * q + 3]);
-                    }
-                    #pragma unroll
-                    for (int ib = 2 * (K + 1); ib < 2 * NB; ++ib) {
-                        const float4 cv = *reinterpret_cast<const float4*>(pan + (4 * ib + tc) * IB_PST + 4 * q);
+                    for (int q = 0; q < 2; ++q) {
+                        float4 rv[NB];
                         #pragma unroll
-                        for (int ia = ib / 2; ia < NB; ++ia) {
-                            float& v = A[ia * (ia + 1) + ib];
-                            v = fmaf(rv[ia].x, cv.x, fmaf(rv[ia].y, cv.y, fmaf(rv[ia].z, cv.z, fmaf(rv[ia].w, cv.w, v))));
+                        for (int ia = KK + 1; ia < NB; ++ia) {
+                            const float4 v = *reinterpret_cast<const float4*>(pan + (8 * ia + tr) * IB_PST + 4 * q);
+                            rv[ia] = make_float4(v.x * -ip[4 * q], v.y * -ip[4 * q + 1], v.z * -ip[4 * q + 2], v.w * -ip[4 * q + 3]);
+                        }
+                        #pragma unroll
+                        for (int ib = 2 * (KK + 1); ib < 2 * NB; ++ib) {
+                            const float4 cv = *reinterpret_cast<const float4*>(pan + (4 * ib + tc) * IB_PST + 4 * q);
+                            #pragma unroll
+                            for (int ia = ib / 2; ia < NB; ++ia) {
+                                float& v = A[ia * (ia + 1) + ib];
+                                v = fmaf(rv[ia].x, cv.x, fmaf(rv[ia].y, cv.y, fmaf(rv[ia].z, cv.z, fmaf(rv[ia].w, cv.w, v))));
+                            }
                         }
                     }
                 }
