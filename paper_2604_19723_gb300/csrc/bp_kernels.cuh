@@ -129,21 +129,29 @@ __device__ inline float factors_from_geo_folded(const DevGeom& G, float4 g, floa
 }
 
 // e^{i 2 pi t} for a phase t = th + tl in cycles, as an unevaluated pair hi + lo good to
-// ~1e-9: the nearest 1/256 of a cycle from a table of FP64-rounded (hi, lo) values, turned
+// ~3e-11: the nearest 1/256 of a cycle from a table of FP64-rounded (hi, lo) values, turned
 // by the remainder angle phi (|phi| <= pi/256) through the angle-addition formulas with
-// cos phi - 1 and sin phi from their Taylor series (terms beyond phi^5 below 1e-14)
+// cos phi - 1 and sin phi from their Taylor series (terms beyond phi^5 below 1e-14).  phi and its products
+// with the table's high parts are carried as pairs: in plain FP32 they leave 1e-9, which a log ratio
+// of 1e6 nats (30 dB, 384 elements) shows as 1e-3.
 __device__ inline void cis_pair(const float4* tab, float th, float tl, float2& hi, float2& lo) {
     const float n = rintf(th * 256.0f);
-    const float rem = __fadd_rn(__fsub_rn(th, n * 0.00390625f), tl);   // th - n/256 is exact
     const float4 T = tab[((int)n) & 255];                                // cos hi, cos lo, sin hi, sin lo
-    const float ph = 6.28318530717958648f * rem;
+    float rh, rl;
+    two_sum(__fsub_rn(th, n * 0.00390625f), tl, rh, rl);                 // th - n/256 is exact
+    const float c1 = 6.28318548f, c2 = -1.74845553e-7f;                  // 2 pi
+    const float ph = __fmul_rn(c1, rh), pl = fmaf(c1, rh, -ph) + fmaf(c2, rh, c1 * rl);
     const float p2 = ph * ph;
     const float cm1 = p2 * fmaf(p2, 1.0f / 24.0f, -0.5f);
-    const float sp = ph * fmaf(p2, fmaf(p2, 1.0f / 120.0f, -1.0f / 6.0f), 1.0f);
-    const float cr = fmaf(T.x, cm1, fmaf(-T.z, sp, T.y));
-    const float ci = fmaf(T.z, cm1, fmaf(T.x, sp, T.w));
-    fast_two_sum(T.x, cr, hi.x, lo.x);   // |cr| <= |T.x| unless T.x == 0
-    fast_two_sum(T.z, ci, hi.y, lo.y);
+    const float sl = fmaf(ph, p2 * fmaf(p2, 1.0f / 120.0f, -1.0f / 6.0f), pl);   // sin phi = ph + sl
+    const float qc = __fmul_rn(T.z, ph), qs = __fmul_rn(T.x, ph);
+    const float ec = fmaf(T.x, cm1, fmaf(-T.z, sl, fmaf(-T.w, ph, __fsub_rn(T.y, fmaf(T.z, ph, -qc)))));
+    const float es = fmaf(T.z, cm1, fmaf(T.x, sl, fmaf(T.y, ph, __fadd_rn(T.w, fmaf(T.x, ph, -qs)))));
+    float h, l;
+    two_sum(T.x, -qc, h, l);
+    fast_two_sum(h, __fadd_rn(l, ec), hi.x, lo.x);
+    two_sum(T.z, qs, h, l);
+    fast_two_sum(h, __fadd_rn(l, es), hi.y, lo.y);
 }
 // the table: e^{i 2 pi n / 256}, n = 0..255, in FP64 and split into FP32 pairs
 __device__ inline void cis_table_fill(float4* tab, int tid, int nthreads) {

@@ -13,7 +13,7 @@
 // alpha is a small difference where the others' span holds most of psi (PFs that nearly
 // coincide), and Delta reaches ~1e3 nats, so h is needed to ~1e-10 of |u||V_c|, far beyond FP32.
 //
-// Precision on the tensor cores.  u (as a (hi, lo) FP32 pair, ~1e-9) and the columns of V~ and
+// Precision on the tensor cores.  u (as a (hi, lo) FP32 pair, ~1e-10) and the columns of V~ and
 // r0 (scaled by a power of two to just below 1) are written in fixed point as four signed
 // base-256 digits of units 2^-7, 2^-15, 2^-23, 2^-31.  A digit has at most 8 bits, so it is exact
 // in BF16, and a product of two digits is an integer multiple of its unit; the sums of the
@@ -47,8 +47,8 @@
 // 46 % busy at 32 PFs, Nz = 1024).
 // Measured (PF likelihood stage, J = 4) with the 3xTF32 kernel (below 33 PFs a CUDA-core kernel), which
 // takes a second pass / with one thread issuing, A in shared memory and exact products by two-term
-// splits of full FP32 factors / as it is: 64 PFs x 1e5 particles, Nz = 160: 56.7 / 15.6 / 10.2 ms; 32 PFs x
-// 262144, Nz = 1024: 401 / 87 / 40.4 ms; 10 PFs x 30000, Nz = 160: 3.66 / 0.58 / 0.40 ms.
+// splits of full FP32 factors / as it is: 64 PFs x 1e5 particles, Nz = 160: 56.7 / 15.6 / 10.3 ms; 32 PFs x
+// 262144, Nz = 1024: 401 / 87 / 41 ms; 10 PFs x 30000, Nz = 160: 3.66 / 0.58 / 0.42 ms.
 #include "bp_internal.cuh"
 #include "bp_kernels.cuh"
 #include "tc_sm100.cuh"
@@ -168,7 +168,7 @@ __device__ inline ff kx_delta(float4 kc, float A, float gm, float mr, float mi, 
     return out;
 }
 
-// steering factors of one (particle, s, j) as (hi, lo) pairs (cis_pair, ~1e-9)
+// steering factors of one (particle, s, j) as (hi, lo) pairs (cis_pair, ~3e-11)
 struct KxPath {
     float dh, dl, h0, l0;   // distance, carrier cycles (float-float)
     float uy, uz, uyl, uzl; // direction cosines
