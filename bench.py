@@ -369,8 +369,8 @@ def run_gpu(args, rank, world):
         ms, fl = per_kernel[name]
         a = fl / (ms * 1e-3) / 1e12
         label = name if name != "k_iota_blk" else (
-            "k_iota_bulk (FP32, every particle) + k_iota_select + k_iota_blk (float-float, queued particles)"
-            if S >= 24 else "k_iota (FP32) + k_iota_blk (flagged particles)")
+            "k_iota_bulk_sym (FP32, every particle) + k_iota_select + k_iota_ff (float-float, queued particles)"
+            if S >= 24 else "k_iota_ff (float-float, every particle)")
         r = {"bound": "alu", "kernel": label, "achieved": a, "peak": peak_alu, "unit": "TFLOP/s",
              "frac": a / peak_alu, "traffic": traffic_for(name, args.workload, P), "ms_per_launch": ms,
              "peak_basis": f"FP32 FMA lanes: {SMS} SMs x {FP32_LANES_PER_SM} x 2 flop x {sm_mhz:.0f} MHz "
@@ -617,7 +617,7 @@ def run_batched(args, rank, world):
                            "how": "same scenarios, one stream, direct launches, " +
                                   ("the tuned tiles" if args.sequential_tiles and tile_res else "built-in tiles")}
                           if seq_ms else None),
-           "roofline": {"bound": "alu", "kernel": "k_kappa + k_iota/k_iota_blk of every scenario (whole step time)",
+           "roofline": {"bound": "alu", "kernel": "k_kappa_x + k_iota_ff / k_iota_bulk_sym of every scenario (whole step time)",
                         "achieved": ach, "peak": peak_alu, "unit": "TFLOP/s", "frac": ach / peak_alu,
                         "traffic": None,
                         "peak_basis": f"FP32 FMA lanes: {SMS} SMs x {FP32_LANES_PER_SM} x 2 flop x {sm_mhz:.0f} MHz"},

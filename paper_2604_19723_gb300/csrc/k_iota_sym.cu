@@ -45,7 +45,7 @@ __device__ __forceinline__ int is_half(int i, int n, int h, bool& c) { c = i >= 
 // A team of TW warps per (particle, PA), the PAs of a particle in one block.  log det from a Cholesky
 // factorisation of A in float-float (pivots of nearly coinciding columns keep ~1e-13), the quadratic
 // form in its variational form |r|^2/eta_bar + |y|^2 at an FP32 minimiser y, the residual r from
-// steering elements as (hi, lo) pairs (~1e-9) with the products of the high parts summed exactly on
+// steering elements as (hi, lo) pairs (~1e-10) with the products of the high parts summed exactly on
 // a grid fixed per (p, j).  Below 24 PFs every particle is evaluated (the FP32 warp kernel and the
 // block-per-particle repair of the particles it flagged took 8.7 ms at 10 PFs x 30000 particles,
 // Nz = 160; this 1.32 ms with index divisions, a search per triangle entry and a reduction per PF, 0.99
