@@ -481,8 +481,9 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
 // Bound: FP32 issue.  The whole stage at 64 PFs x 1e5 particles (Nz = 160) / 32 x 262144 (Nz = 1024):
 // 27.7 / 69 ms with a block of 64 threads per particle on the complex matrix, 15.1 / 54.4 with this
 // split but one column of the elimination at a time and unpacked e and rhs, 12.0 / 26.7 with both packed
-// element by element and the panels unrolled, 9.5 / 22.1 as it is (instruction fetch was a fifth of the
-// stalls at 64 PFs: loops whose body is long stay rolled).
+// element by element and the panels unrolled, 9.4 / 22.1 over mirrored pairs with long loops rolled
+// (instruction fetch was a fifth of the stalls), 8.9 / 19.8 as it is (panel in the residual's place, Re and
+// Im of the factors in one row: 13.7 instead of 16 KB per warp, 16 instead of 12 warps per SM, at 32 PFs).
 constexpr float IB_ERR_PER_RATIO = 4.0e-6f;    // as in k_iota_bulk.cu
 constexpr float IB_ERR_PER_ENERGY = 1.0e-6f;
 constexpr int IB_W = 4;                        // warps (PAs of a particle) per block
@@ -495,14 +496,14 @@ __host__ __device__ inline IbPlan ib_plan(const DevGeom& G, int S) {
     const IsDims d = is_dims(G);
     IbPlan p{};
     p.f4 = (d.Fh + 7) & ~7;                    // frequencies, padded to a lane's four pairs
-    p.fp = p.f4 + 4;                           // row stride: 16-byte rows, 8 rows on distinct banks
+    p.fp = 2 * p.f4 + 4;                       // stride of a row (Re b, Im b): 16-byte rows, 8 rows on distinct banks
     p.ast = (d.hy + d.hz) | 1;
     const size_t R = 8 * NB;                   // rows beyond S are zero
     size_t o = 0;
-    p.pq = o; o += (size_t)d.Nmh * IB_Q * p.f4 * sizeof(float);
-    p.pan = o; o += R * IB_PST * sizeof(float);
-    p.fx = o; o += R * p.fp * sizeof(float);
-    p.fy = o; o += R * p.fp * sizeof(float);
+    // the panel takes the residual's place, which the elimination no longer needs
+    const size_t pq = (size_t)d.Nmh * IB_Q * p.f4 * sizeof(float), pan = R * IB_PST * sizeof(float);
+    p.pq = p.pan = o; o += pq > pan ? pq : pan;
+    p.fx = o; p.fy = o + p.f4 * sizeof(float); o += R * p.fp * sizeof(float);
     p.vec = o; o += R * (sizeof(float4) + sizeof(float));
     p.ant = o; o += R * p.ast * sizeof(float2);
     p.warp = (o + 15) & ~(size_t)15;
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
     float* pq = reinterpret_cast<float*>(base + pl.pq);         // [Nmh][IB_Q][f4] e
     float* pan = reinterpret_cast<float*>(base + pl.pan);       // [8 NB][IB_PST] panel of eight columns
     float* fx = reinterpret_cast<float*>(base + pl.fx);         // [8 NB][fp] Re b_f
-    float* fy = reinterpret_cast<float*>(base + pl.fy);         // [8 NB][fp] Im b_f
+    float* fy = reinterpret_cast<float*>(base + pl.fy);         // [8 NB][fp] Im b_f (in the same rows)
     float2* ant = reinterpret_cast<float2*>(base + pl.ant);     // [8 NB][ast] a_y, a_z (half of each)
     float4* ws = reinterpret_cast<float4*>(base + pl.vec);      // [8 NB] -4 A c pi mu (two parts)
     float* dA = reinterpret_cast<float*>(ws + 8 * NB);          // [8 NB] d_s A_s
@@ -539,9 +540,8 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
         lgs[threadIdx.x] = log(D.eta_bar[threadIdx.x]);
         ies[threadIdx.x] = 1.0 / D.eta_bar[threadIdx.x];
     }
-    for (int i = lane; i < 8 * NB * pl.fp; i += 32) fx[i] = fy[i] = 0.f;     // rows and columns beyond S and Fh stay zero
+    for (int i = lane; i < 8 * NB * pl.fp; i += 32) fx[i] = 0.f;     // (fy with it) rows and columns beyond S and Fh stay zero
     for (int i = lane; i < 8 * NB * pl.ast; i += 32) ant[i] = make_float2(0.f, 0.f);
-    for (int i = lane; i < dm.Nmh * IB_Q * pl.f4; i += 32) pq[i] = 0.f;
     __syncthreads();
     // residual: NL lanes over the element pairs, the groups of lanes over frequency pairs (gf groups of up to
     // IB_FP) and what is left of them over PFs (gs)
@@ -703,6 +703,9 @@ __global__ void __launch_bounds__(32 * IB_W, NB > 4 ? 3 : 4) k_iota_bulk_sym(Dev
                     }
                 }
             }
+            // (read below where the last pair is the first of four frequencies)
+            if (2 * np2 < pl.f4)
+                for (int i = lane; i < dm.Nmh * IB_Q; i += 32) *reinterpret_cast<float2*>(pq + i * pl.f4 + 2 * np2) = make_float2(0.f, 0.f);
             ee = warp_sum_f(ee);
             __syncwarp();
             // rhs_s = (dA)_s u_s^H e
