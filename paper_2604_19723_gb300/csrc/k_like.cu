@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(32 * NCG, IOTA_BLK_PER_SM) k_iota_blk(DevGeom 
             __syncthreads();
             // residual r = z - sum_s w_s (b' kron a_y kron a_z)_s, w_s = A_s (pi mu + d y)_s.  Its
             // energy reaches ~1e4 noise units, so the steering values enter as (hi, lo) pairs
-            // (~1e-9), the products of the high parts are summed exactly on a grid fixed for
+            // (~1e-10), the products of the high parts are summed exactly on a grid fixed for
             // this (p, j) (2^E > 4 (max_k |z_k| + sum_s |w_s|) bounds every partial sum), and
             // the remainders and the low-part cross terms are summed in FP32
             if (wid == 1) {

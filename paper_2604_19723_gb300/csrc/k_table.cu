@@ -215,7 +215,7 @@ __global__ void k_table_final(DevGeom G, DevParams Pm, DevState D, int S, int ns
 }
 
 // ---------------------------------------------------------------- Gram matrix per j (FP64)
-// G_j[a][b] = m_a^H m_b; also e_all = z - sum_s mu3_s, b = M^H e_all, |e_all|^2.
+// G_j[a][b] = m_a^H m_b, a warp per pair.
 __global__ void k_gram(DevGeom G, DevParams Pm, DevState D, int S, double* gram) {
     const int j = blockIdx.y;
     const int J = G.J, Nz = G.Nz, SM = Pm.S_max;
