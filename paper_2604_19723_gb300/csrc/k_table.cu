@@ -561,21 +561,33 @@ __global__ void __launch_bounds__(NU_THREADS) k_nu_tridiag(DevParams Pm, DevStat
     __syncthreads();
     for (int k = 0; k + 2 < S; ++k) {
         const int n = S - k - 1, f = k + 1;       // trailing rows f .. S - 1
-        // x = A[f:, k]; alpha = -ph |x| with ph the phase of x_0; v = x - alpha e1
+        // x = A[f:, k], scaled by a power of two to a largest part in [1, 2) so that its squares stay in range
+        // (products of small existence weights do not); alpha = -ph |x| with ph the phase of x_0; v = x - alpha e1
         double2 x[2];
-        double nx2 = 0.0;
+        uint32_t top = 0;                         // upper words of the magnitudes
         #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = lane + 32 * h;
             x[h] = i < n ? A[(f + i) * S + k] : make_double2(0.0, 0.0);
+            top = max(top, max((uint32_t)__double2hiint(x[h].x) & 0x7fffffffu, (uint32_t)__double2hiint(x[h].y) & 0x7fffffffu));
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        if (top < 0x00100000u) continue;          // the column is zero already (uniform across the block)
+        const int ex = min((int)(top >> 20), 2045);
+        const double up = __hiloint2double((2046 - ex) << 20, 0), down = __hiloint2double(ex << 20, 0);
+        double nx2 = 0.0;
+        #pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            x[h].x *= up; x[h].y *= up;
             nx2 += x[h].x * x[h].x + x[h].y * x[h].y;
         }
         nx2 = warp_sum_d(nx2);
-        if (nx2 == 0.0) continue;                 // the column is zero already (uniform across the block)
-        const double2 x0 = A[f * S + k];
-        const double nx = sqrt(nx2), ax0 = sqrt(x0.x * x0.x + x0.y * x0.y);
-        const double beta = 1.0 / (nx * (nx + ax0)), q = ax0 > 0 ? nx / ax0 : 0.0;
-        const double2 al = ax0 > 0 ? make_double2(-x0.x * q, -x0.y * q) : make_double2(-nx, 0.0);   // alpha
+        const double2 x0 = make_double2(up * A[f * S + k].x, up * A[f * S + k].y);
+        const double a2 = x0.x * x0.x + x0.y * x0.y;
+        const bool ph = a2 > 1e-200;              // below, x_0 is nothing beside |x| >= 1: any phase will do
+        const double nx = sqrt(nx2), ax0 = ph ? sqrt(a2) : 0.0;
+        const double beta = 1.0 / (nx * (nx + ax0)), q = ph ? nx / ax0 : 0.0;
+        const double2 al = ph ? make_double2(-x0.x * q, -x0.y * q) : make_double2(-nx, 0.0);   // alpha
         if (lane == 0) { x[0].x -= al.x; x[0].y -= al.y; }
         if (wid == 0) {
             #pragma unroll
@@ -643,16 +655,18 @@ __global__ void __launch_bounds__(NU_THREADS) k_nu_tridiag(DevParams Pm, DevStat
                 a.y -= a1.y + a2.y;
             }
         }
-        if (tid == 0) A[f * S + k] = al;
+        if (tid == 0) A[f * S + k] = make_double2(down * al.x, down * al.y);
         __syncthreads();
     }
     // make off-diagonals real non-negative: D = diag(e^{i th}), th_{k+1} = th_k + arg(e_k)
     double* out = D.nu_T + (size_t)j * 4 * SM;    // [a(SM) | o(SM) | b'(2 SM)]
     for (int k = tid; k + 1 < S; k += NU_THREADS) {
+        // (off-diagonals near the end of the range, whose phases are lost, are nothing beside eta)
         const double2 e = A[(k + 1) * S + k];
-        const double ae = sqrt(e.x * e.x + e.y * e.y);
-        out[SM + k] = ae;
-        v[k] = ae > 0 ? make_double2(e.x / ae, e.y / ae) : make_double2(1.0, 0.0);
+        const double ae = hypot(e.x, e.y);
+        const bool on = !(ae <= 1e-290);
+        out[SM + k] = on ? ae : 0.0;
+        v[k] = on ? make_double2(e.x / ae, e.y / ae) : make_double2(1.0, 0.0);
     }
     __syncthreads();
     if (tid == 0) {
