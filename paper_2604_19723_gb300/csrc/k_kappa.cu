@@ -16,9 +16,12 @@
 // Precision on the tensor cores.  u (as a (hi, lo) FP32 pair, ~1e-10) and the columns of V~ and
 // r0 (scaled by a power of two to just below 1) are written in fixed point as four signed
 // base-256 digits of units 2^-7, 2^-15, 2^-23, 2^-31.  A digit has at most 8 bits, so it is exact
-// in BF16, and a product of two digits is an integer multiple of its unit; the sums of the
-// products of one total weight stay below 2^24 of that unit, so the FP32 accumulator of
-// tcgen05.mma kind::f16 holds them exactly.  The digit products (i, k) with i + k <= 5 (ten of
+// in BF16, and a product of two digits is an integer multiple of its unit.  The FP32 accumulator of
+// tcgen05.mma kind::f16 holds sums up to 2^24 of that unit exactly.  The products of the first digits
+// reach 1.43 x 2^14 units per element where u and a column are aligned (nearly coinciding PFs, r0 of a strong
+// one), that is 717 elements; beyond, the columns are scaled one or two powers of two lower
+// (kx_headroom; without, 2048 elements left 0.3 nats on log ratios of 1e5 and 10 on those of PFs
+// millimetres apart).  The second digits change sign along the array, and their sums stay lower.  The digit products (i, k) with i + k <= 5 (ten of
 // sixteen; the rest is below 2^-35 of |u||V_c|) go to four accumulators g_{i+k-2}, which the
 // epilogue adds as an FP32 pair.  The earlier kernel (3xTF32, FP32 accumulation) needed a second
 // contraction V conj(h) and an element-wise float-float residual to make the error of h
@@ -69,6 +72,11 @@ __host__ __device__ inline int kx_chunks(int Nh) { return (Nh + 15) / 16; }
 __host__ __device__ inline uint32_t kx_bbytes(int SW) { return (uint32_t)(2 * SW) * KX_KC * 2 * 4; }   // 4 digits
 // elements a particle forms: half of them where the layout is symmetric
 __host__ __device__ inline int kx_elements(const DevGeom& G) { return G.sym ? (G.Nz + 1) / 2 : G.Nz; }
+// Powers of two r between the largest part of a scaled column and 1.  For the first digits |u_1| <= 1 + sqrt(2)/256
+// and |v_1| <= sqrt(2) (2^-r + 1/256), and Nh |u_1| |v_1| 2^14 is to stay below 2^24.  (The columns are
+// rounded at 2^-32; beside the steering elements' 2^-31 the lost bits do not show: log ratios of 2048
+// elements agree with the CUDA-core kernel's to 1e-4, as at r = 0.)
+__host__ __device__ inline int kx_headroom(int Nh) { return Nh <= 717 ? 0 : Nh <= 1429 ? 1 : 2; }
 __host__ __device__ inline int kx_factors(const DevGeom& G, int yz) {
     return yz ? (G.My * G.Mz + 1) & ~1 : G.My + ((G.Mz + 1) & ~1);
 }
@@ -195,7 +203,7 @@ __device__ __forceinline__ float4 kx_pair_mul(float4 a, float4 b) {
 
 // ---------------------------------------------------------------- operand digits of V~ and r0
 // Block (s, j, part of the chunks): the columns' power-of-two scales (largest part in [1/2, 1)
-// after scaling), then the four digit slices of its chunks of 16 elements as rows n < SW (Re h_n)
+// after scaling, less kx_headroom), then the four digit slices of its chunks of 16 elements as rows n < SW (Re h_n)
 // and n >= SW (Im h_{n - SW}) against k = 2 e + part, K-major core matrices:
 // [Re(v + v'), Im(v - v')] and [Im(v + v'), -Re(v - v')] for a symmetric layout (v' the mirrored
 // element's, the middle element counted once), else [Re v, Im v] and [Im v, -Re v].  Column SW - 1
@@ -241,6 +249,7 @@ __global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int
             if (top > 0 && m > 0.0 && isfinite(m)) {
                 int e;
                 frexp(m, &e);
+                e += kx_headroom(Nh);
                 f = ldexp(r0 ? 1.0 : isq, -e);
                 inv = ldexpf(1.0f, e);
             }
