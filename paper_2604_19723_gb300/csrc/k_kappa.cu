@@ -246,7 +246,9 @@ __global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int
             top = __reduce_max_sync(0xffffffffu, top);
             // the next upper word bounds the largest magnitude
             const double m = top < 0x7ff00000u ? __hiloint2double((int)(top + 1), 0) * (r0 ? 1.0 : isq) : 0.0;
-            if (top > 0 && m > 0.0 && isfinite(m)) {
+            if (!(m < INFINITY) || top >= 0x7ff00000u) {
+                inv = NAN;                         // an observation that is not finite: neither are the log ratios
+            } else if (top > 0 && m > 0.0) {
                 int e;
                 frexp(m, &e);
                 e += kx_headroom(Nh);
