@@ -31,12 +31,12 @@ int launch_birth_proposal(const DevGeom& G, const DevParams& Pm, const DevState&
 
 // Largest dynamic shared memory a block may opt in to on the current device.
 int smem_optin();
-// Streaming multiprocessors of the device.
+// Streaming multiprocessors of the current device.
 int sm_count();
 // Raises a kernel's dynamic shared-memory limit to the opt-in maximum less its static
-// shared memory (once per kernel), not to one launch's need: launches of one kernel
-// with different sizes from several streams, or replayed from a captured graph, then
-// never meet a limit set for a smaller launch.
+// shared memory (once per kernel and device, from any thread), not to one launch's need:
+// launches of one kernel with different sizes from several streams, or replayed from a
+// captured graph, then never meet a limit set for a smaller launch.
 void smem_allow_max(const void* kernel);
 
 

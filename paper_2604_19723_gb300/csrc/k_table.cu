@@ -18,10 +18,9 @@
 // nu (S-V "Noise variance update message"): G = M^H M is reduced once per j
 // to a real symmetric tridiagonal T = Q^H G Q (Householder), with b = Q^H M^H e;
 // each particle then needs O(S) work (k_like.cu).
-#include <vector>
-
 #include "bp_internal.cuh"
 #include "bp_kernels.cuh"
+#include "per_device.cuh"
 
 namespace bp {
 
@@ -723,36 +722,36 @@ void launch_nu_tridiag(const DevGeom& G, const DevParams& Pm, const DevState& D,
     if (fork) cudaEventRecord(ev_join, side);
 }
 
+static int current_device() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev;
+}
+static int device_attribute(int dev, cudaDeviceAttr attr, int fallback) {
+    int a = 0;
+    cudaDeviceGetAttribute(&a, attr, dev);
+    return a > 0 ? a : fallback;
+}
+
 void smem_allow_max(const void* kernel) {
-    static std::vector<const void*> done;
-    for (const void* k : done)
-        if (k == kernel) return;
-    cudaFuncAttributes a{};
-    cudaFuncGetAttributes(&a, kernel);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - (int)a.sharedSizeBytes);
-    done.push_back(kernel);
+    static OncePerDevice done;
+    done.run(current_device(), kernel, [&] {
+        cudaFuncAttributes a{};
+        cudaFuncGetAttributes(&a, kernel);
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - (int)a.sharedSizeBytes);
+    });
 }
 
 int sm_count() {
-    static int v = 0;
-    if (v == 0) {
-        int dev = 0, a = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&a, cudaDevAttrMultiProcessorCount, dev);
-        v = a > 0 ? a : 1;
-    }
-    return v;
+    static NumberPerDevice v;
+    const int dev = current_device();
+    return v.get(dev, [&] { return device_attribute(dev, cudaDevAttrMultiProcessorCount, 1); });
 }
 
 int smem_optin() {
-    static int v = 0;
-    if (v == 0) {
-        int dev = 0, a = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&a, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        v = a > 0 ? a : 48 * 1024;
-    }
-    return v;
+    static NumberPerDevice v;
+    const int dev = current_device();
+    return v.get(dev, [&] { return device_attribute(dev, cudaDevAttrMaxSharedMemoryPerBlockOptin, 48 * 1024); });
 }
 
 }  // namespace bp
