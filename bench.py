@@ -75,6 +75,7 @@ def iota_flops(P, S, J, Nf, My, Mz):
 # value.
 TRAFFIC_RECORDS = {}
 KERNEL_SOURCES = ("paper_2604_19723_gb300/csrc/k_kappa.cu", "paper_2604_19723_gb300/csrc/k_like.cu",
+                  "paper_2604_19723_gb300/csrc/k_iota_sym.cu", "paper_2604_19723_gb300/csrc/k_iota_bulk.cu",
                   "paper_2604_19723_gb300/csrc/bp_kernels.cuh", "paper_2604_19723_gb300/csrc/bp_internal.cuh",
                   "paper_2604_19723_gb300/csrc/tc_sm100.cuh")
 
@@ -408,7 +409,8 @@ def run_gpu(args, rank, world):
            "e2e": {"value": world * P * g.J / (t_e2e * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                    "d2h_bytes_per_step": d2h, "ms_per_step": t_e2e},
            "gpu_launches": int(launches), "clocks": clocks,
-           "iota_floatfloat_particles_per_step": float(np.mean(repaired)) if repaired else 0.0}
+           # below 24 PFs (symmetric layout) every particle is evaluated in float-float
+           "iota_floatfloat_particles_per_step": float(P) if S < 24 else float(np.mean(repaired)) if repaired else 0.0}
     if rank == 0 and not args.no_cpu_baseline:
         out["cpu_baseline"] = cpu_baseline(wl, g, prm, scn, args.cpu_particles, z_all[:1].cpu().numpy())
     f.close()

@@ -127,7 +127,10 @@ typedef struct {
     double* phi_hat;
     double* p_pr;
     int* declared;
-    int iota_repaired;   /* particles whose MT likelihood was recomputed in FP64 (ill-conditioned) */
+    int iota_repaired;   /* particles whose FP32 MT likelihood does not do: ill-conditioned (up to 23 PFs), or
+                            their error bound reaches the largest weight (from 24 PFs on).  They are
+                            evaluated in float-float; on layouts symmetric about 0 with up to 23 PFs so
+                            are all the others */
 } bp_estimate_out;
 
 /* Creates a filter: validates, copies the geometry and parameters, allocates

@@ -267,10 +267,11 @@ void launch_cis_table(const DevState& D, cudaStream_t st);
 bool iota_sym_ok(const DevGeom& G, int S);
 bool launch_iota_bulk_sym(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st);
 void launch_iota_ff(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, bool all, cudaStream_t st);
-// MT likelihood of every particle (returns its launches): the FP32 warp kernel with
-// ratio flags below IOTA_FF_ALL_S PFs, else k_iota_bulk and the selection of the particles
-// whose weights need the float-float evaluation; launch_iota_repair then evaluates the
-// flagged particles in float-float
+// MT likelihood of every particle (returns its launches).  Below IOTA_FF_ALL_S PFs: float-float for all
+// of them on symmetric layouts, else the FP32 warp kernel with ratio flags.  From there on:
+// k_iota_bulk_sym or k_iota_bulk, and the selection of the particles whose weights need the
+// float-float evaluation.  launch_iota_repair then evaluates the flagged or selected ones in
+// float-float (nothing is left for it where all were)
 int launch_iota(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st);
 int launch_iota_bulk(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st);
 size_t iota_bulk_smem_bytes(const DevGeom& G, int S);

@@ -695,7 +695,8 @@ __global__ void k_nu(DevGeom G, DevParams Pm, DevState D, int S) {
     D.lw_eta[(size_t)j * P + p] = lnu;
 }
 
-// S below which the FP32 path runs first and only flagged particles are redone
+// S below which every particle is evaluated in float-float (symmetric layouts), or in FP32 with only
+// the ill-conditioned ones redone; from it on the FP32 bulk kernels and the selection by error bounds
 constexpr int IOTA_FF_ALL_S = 24;
 
 int launch_iota(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, const float* z, cudaStream_t st) {
