@@ -176,29 +176,17 @@ __device__ inline ff kx_delta(float4 kc, float A, float gm, float mr, float mi, 
     return out;
 }
 
-// steering factors of one (particle, s, j) as (hi, lo) pairs (cis_pair, ~3e-11)
-struct KxPath {
-    float dh, dl, h0, l0;   // distance, carrier cycles (float-float)
-    float uy, uz, uyl, uzl; // direction cosines
-};
-__device__ __forceinline__ KxPath kx_path(const DevGeom& G, float4 g, float2 gl) {
-    KxPath t{g.x, g.y, 0.f, 0.f, g.z, g.w, gl.x, gl.y};
-    ff_frac_mul2(g.x, g.y, G.inv_lam_hi, G.inv_lam_lo, t.h0, t.l0);
-    return t;
-}
-// antenna factor i < My: a_y, else a_z of element i - My
-__device__ __forceinline__ float4 kx_antenna(const DevGeom& G, const float4* tab, const KxPath& t, int i) {
+// antenna factor i < My: a_y, else a_z of element i - My, of a geometry record and its low parts, as a
+// (hi, lo) pair (cis_pair, ~3e-11)
+__device__ __forceinline__ float4 kx_antenna(const DevGeom& G, const float4* tab, float4 g, float2 gl, int i) {
     const bool y = i < G.My;
     const float c = y ? G.py_l[i] : G.pz_l[i - G.My], cl = y ? G.py_lo[i] : G.pz_lo[i - G.My];
-    const float u = y ? t.uy : t.uz, ul = y ? t.uyl : t.uzl;
+    const float u = y ? g.z : g.w, ul = y ? gl.x : gl.y;
     const float p = __fmul_rn(c, u);
     const float e = fmaf(c, ul, fmaf(cl, u, fmaf(c, u, -p)));
     float2 hi, lo;
     cis_pair(tab, p, e, hi, lo);
     return make_float4(hi.x, hi.y, lo.x, lo.y);
-}
-__device__ __forceinline__ float4 kx_pair_mul(float4 a, float4 b) {
-    return cpair_mul(make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y), make_float2(b.z, b.w));
 }
 
 // ---------------------------------------------------------------- operand digits of V~ and r0
@@ -209,7 +197,10 @@ __device__ __forceinline__ float4 kx_pair_mul(float4 a, float4 b) {
 // element's, the middle element counted once), else [Re v, Im v] and [Im v, -Re v].  Column SW - 1
 // is r0, unused columns are zero.  Bound: the FP64 conversions (64 PFs x 4 PAs x Nz = 160: 223 us with FP64
 // maxima in four blocks per (s, j), 96 us with maxima of upper words and about four blocks per SM).
-__global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int S, int SCA, int SW,
+// With `whole` (the CUDA-core kernel's operand) the fixed-point numbers themselves go out instead of their
+// digits, in units of 2^-29 of a column scaled to [1/2, 1): per chunk [16][SW] the factors of Re u and Im u
+// in Re h, then in Im h.
+__global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int S, int SCA, int SW, bool whole,
                                                       const double2* __restrict__ V64) {
     const int s = blockIdx.x, j = blockIdx.y, J = G.J, Nz = G.Nz, K = S - 1, Nh = kx_elements(G);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -281,10 +272,14 @@ __global__ void __launch_bounds__(256) k_kappa_digits(DevGeom G, DevState D, int
         if (k < Nh && sc[c] != 0.0) {
             double o[4];
             combo(V + (size_t)(c == SW - 1 ? SCA - 1 : c) * Nz, k, o);
-            const double f = sc[c] * 2147483648.0;
+            const double f = sc[c] * (whole ? ldexp(1.0, 29 + kx_headroom(Nh)) : 2147483648.0);
             #pragma unroll
             for (int i = 0; i < 4; ++i) q[i] = __double2ll_rn(o[i] * f);
             q[3] = -q[3];
+        }
+        if (whole) {
+            reinterpret_cast<int4*>(out + (size_t)kc * 4 * slice)[e * SW + c] = make_int4((int)q[0], (int)q[1], (int)q[2], (int)q[3]);
+            continue;
         }
         unsigned char* o = out + (size_t)kc * 4 * slice;
         const uint32_t o1 = (uint32_t)tc::core_off16(c, 2 * e, KX_KC), o2 = (uint32_t)tc::core_off16(SW + c, 2 * e, KX_KC);
@@ -795,113 +790,202 @@ __global__ void __launch_bounds__(KX_T, 1) k_kappa_x(DevGeom G, DevParams Pm, De
 }
 
 // ---------------------------------------------------------------- CUDA-core kernel
-// The same closed form without the tensor cores (a tile request can ask for it): thread per
-// particle, the columns eight at a time, each product split on a grid fixed per (s, j) so that
-// the grid parts add exactly (2^E > 4 Nz bounds every partial sum of the scaled columns) and the
-// remainders and low-part cross terms in FP32.  Issue bound: 24 instructions per complex product.
-constexpr int KCC_T = 128, KCC_C = 8, KCC_E = 32;   // threads, columns per pass, staged elements
+// The same closed form without the tensor cores (a tile request can ask for it), in integers.  With the
+// steering elements in units of 2^-30 and the columns of 2^-29 a sum of eight elements' products fits 64 bits
+// exactly; every eight elements it is added, in units of 2^-47, to the column's running sum.
+// Block: 64 particles of one PF, a warp per four columns, lane i the particles 2 i and 2 i + 1 (16 sums in
+// registers).  While a chunk of 16 elements is multiplied, the next one's steering elements are formed (a
+// thread per particle and row of Mz elements) and its columns fetched, in the other half of the
+// buffers.  Bound: the integer multiply-adds (four per complex product) and the shared-memory reads of
+// their operands.
+// Measured (PF likelihood stage, J = 4, symmetric / general layout), and a thread per particle with the products as
+// FP32 pairs over all elements: 10 PFs x 30000, Nz = 160: 1.19 / 2.21 ms (4.26); 64 x 20000: 22.6 / 40.3 (69.5);
+// 32 x 20000, Nz = 1024: 29.0 / 56.9 (110).
+constexpr int KCC_P = 64, KCC_E = 16, KCC_Q = 4;   // particles per block, elements per chunk, columns per warp
+struct KccPlan { int quads, rows, dev; size_t smem; };
+__host__ __device__ inline KccPlan kcc_plan(const DevGeom& G, int S) {
+    KccPlan t;
+    t.quads = (S + KCC_Q - 1) / KCC_Q;
+    t.rows = (KCC_E - 1) / G.Mz + 2;               // rows of Mz elements that a chunk can touch
+    t.dev = 2 * t.rows > G.My + G.Mz ? 2 * t.rows : G.My + G.Mz;
+    t.smem = ((size_t)(G.My + G.Mz + 2) * KCC_P + 256 + 2 * (size_t)KCC_E * KCC_Q * t.quads) * sizeof(float4) +
+             (2 * (size_t)KCC_E + t.quads + 1) * KCC_P * sizeof(float2) + (size_t)(t.dev + 1) * KCC_P * sizeof(float);
+    return t;
+}
 
-__global__ void __launch_bounds__(KCC_T) k_kappa_cc(DevGeom G, DevParams Pm, DevState D, int S, int SCA, int SW,
-                                                    const double2* __restrict__ V64) {
+__global__ void __launch_bounds__(32 * S_CAP_MAX / KCC_Q, 1) k_kappa_cc(DevGeom G, DevParams Pm, DevState D, int S, int SW) {
     extern __shared__ float4 smc[];
+    const KccPlan pl = kcc_plan(G, S);
     const int P = Pm.P, J = G.J, Nz = G.Nz, My = G.My, Mz = G.Mz, Nm = My * Mz, nant = My + Mz, K = S - 1;
-    float4* fa = smc;                              // [nant][KCC_T]
-    float4* ctab = fa + (size_t)nant * KCC_T;      // [256]
-    float4* vs = ctab + 256;                       // [KCC_E][KCC_C] scaled columns (re, im hi; re, im lo)
-    const int s = blockIdx.y, tid = threadIdx.x, p = blockIdx.x * KCC_T + tid, pp = min(p, P - 1);
-    for (int i = tid; i < 256; i += KCC_T) ctab[i] = D.ctab[i];
+    const int Nh = kx_elements(G), NCk = kx_chunks(Nh), NC = KCC_Q * pl.quads;
+    float4* fa = smc;                              // [nant][KCC_P] a_y, a_z, split
+    float4* ctab = fa + (size_t)nant * KCC_P;      // [256]
+    int4* vs = reinterpret_cast<int4*>(ctab + 256);   // [2][KCC_E][NC] factors of Re u and Im u in Re h, in Im h
+    float4* sgeo = reinterpret_cast<float4*>(vs + 2 * (size_t)KCC_E * NC);   // [KCC_P]
+    float4* exr = sgeo + KCC_P;                    // [KCC_P] u^H r0
+    int2* us = reinterpret_cast<int2*>(exr + KCC_P);   // [2][KCC_E][KCC_P] u
+    float2* ex = reinterpret_cast<float2*>(us + 2 * (size_t)KCC_E * KCC_P);  // [quads][KCC_P] |h|^2 (grid, rest)
+    float2* sdl = ex + (size_t)pl.quads * KCC_P;   // [KCC_P] Delta over the PAs
+    float* dv = reinterpret_cast<float*>(sdl + KCC_P);   // |.|^2 - 1: [nant][KCC_P] of factors, then [2][rows][KCC_P] of the rows' b_f
+    float* sdv = dv + (size_t)pl.dev * KCC_P;      // [KCC_P] |u|^2 - Nz
+    const int s = blockIdx.y, tid = threadIdx.x, T = blockDim.x, lane = tid & 31, quad = tid >> 5, p0 = blockIdx.x * KCC_P;
+    for (int i = tid; i < 256; i += T) ctab[i] = D.ctab[i];
     const float* ph = D.phi[D.cur] + (size_t)s * 6 * P;
+    const size_t chunk = kx_bbytes(SW);
+    const float back = ldexpf(1.0f, -47 - kx_headroom(Nh)), dbl = G.sym ? 2.0f : 1.0f;
     float GM = 1.5f;
     for (int v = 1; v < 4 * Nz; v *= 2) GM *= 2.0f;
-    ff delta{0.f, 0.f};
     for (int j = 0; j < J; ++j) {
         const size_t sj = (size_t)s * J + j;
-        const double2* V = V64 + sj * SCA * Nz;
+        const unsigned char* B = D.kB + sj * NCk * chunk;
         const float* scl = D.kSc + sj * 64;
-        const double isq = 1.0 / sqrt(D.eta_bar[j]);
-        const float4 grec = D.geo[sj * P + pp];
-        const KxPath path = kx_path(G, grec, D.geo_lo[sj * P + pp]);
         __syncthreads();
-        float dev = 0.f, sg = 0.f, sr = 0.f;
-        for (int i = 0; i < nant; ++i) {
-            const float4 a = kx_antenna(G, ctab, path, i);
-            dev = fmaf((float)(i < My ? G.Nf * Mz : G.Nf * My), pair_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w)), dev);
-            fa[i * KCC_T + tid] = a;
+        for (int t = tid; t < nant * KCC_P; t += T) {
+            const int i = t / KCC_P, q = t % KCC_P;
+            const size_t gi = sj * P + min(p0 + q, P - 1);
+            const float4 grec = D.geo[gi];
+            const float4 a = kx_antenna(G, ctab, grec, D.geo_lo[gi], i);
+            dv[t] = (float)(i < My ? G.Nf * Mz : G.Nf * My) * pair_unit_dev(make_float2(a.x, a.y), make_float2(a.z, a.w));
+            fa[t] = kx_split(a);
+            if (i == 0) sgeo[q] = grec;
         }
-        cff pr{ff{0.f, 0.f}, ff{0.f, 0.f}};
-        for (int c0 = 0; c0 < SW; c0 += KCC_C) {
-            float ar[KCC_C], ai[KCC_C], lr[KCC_C], li[KCC_C];
-            #pragma unroll
-            for (int q = 0; q < KCC_C; ++q) ar[q] = ai[q] = lr[q] = li[q] = 0.f;
-            float4 b = make_float4(0.f, 0.f, 0.f, 0.f), w = b;
-            for (int k0 = 0; k0 < Nz; k0 += KCC_E) {
-                const int nk = min(KCC_E, Nz - k0);
-                __syncthreads();
-                for (int t = tid; t < KCC_C * KCC_E; t += KCC_T) {
-                    const int e = t % KCC_E, q = t / KCC_E, c = c0 + q;
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const bool r0 = c == SW - 1;
-                    if (e < nk && (r0 || c < K) && scl[c] != 0.f) {
-                        const double f = (r0 ? 1.0 : isq) / (double)scl[c];
-                        const double2 x = V[(size_t)(r0 ? SCA - 1 : c) * Nz + k0 + e];
-                        v.x = (float)(x.x * f);
-                        v.y = (float)(x.y * f);
-                        v.z = (float)(x.x * f - (double)v.x);
-                        v.w = (float)(x.y * f - (double)v.y);
-                    }
-                    vs[e * KCC_C + q] = v;
-                }
-                __syncthreads();
-                for (int e = 0; e < nk; ++e) {
-                    const int k = k0 + e, f = k / Nm, ym = k - f * Nm, y = ym / Mz, m = ym - y * Mz;
-                    if (ym == 0 || e == 0) {
-                        float2 hi, lo;
-                        bprime_pair(G, ctab, path.dh, path.dl, path.h0, path.l0, f, hi, lo);
-                        b = make_float4(hi.x, hi.y, lo.x, lo.y);
-                        if (c0 == 0 && ym == 0) dev = fmaf((float)Nm, pair_unit_dev(hi, lo), dev);
-                    }
-                    if (m == 0 || e == 0) w = kx_pair_mul(b, fa[y * KCC_T + tid]);
-                    const float4 u = kx_pair_mul(w, fa[(My + m) * KCC_T + tid]);
-                    #pragma unroll
-                    for (int q = 0; q < KCC_C; ++q) {
-                        const float4 v = vs[e * KCC_C + q];
-                        auto mac = [&](float& g, float& l, float x, float xl, float c, float cl) {
-                            const float t = __fsub_rn(fmaf(x, c, GM), GM);
-                            g = __fadd_rn(g, t);
-                            l += fmaf(x, cl, fmaf(xl, c, fmaf(x, c, -t)));
-                        };
-                        mac(ar[q], lr[q], u.x, u.z, v.x, v.z);
-                        mac(ar[q], lr[q], u.y, u.w, v.y, v.w);
-                        mac(ai[q], li[q], u.x, u.z, v.y, v.w);
-                        mac(ai[q], li[q], -u.y, -u.w, v.x, v.z);
-                    }
+        __syncthreads();
+        for (int q = tid; q < KCC_P; q += T) {
+            float d = 0.f;
+            for (int i = 0; i < nant; ++i) d += dv[i * KCC_P + q];
+            sdv[q] = d;
+        }
+        __syncthreads();
+        // the steering elements (in units of 2^-30) and the columns of chunk kc
+        auto fill = [&](int kc) {
+            const int k0 = kc * KCC_E, k1 = min(k0 + KCC_E, Nh), r0 = k0 / Mz, nr = (k1 - 1) / Mz - r0 + 1;
+            int2* u = us + (kc & 1) * KCC_E * KCC_P;
+            float* d = dv + (kc & 1) * pl.rows * KCC_P;
+            int4* v = vs + (kc & 1) * KCC_E * NC;
+            const int4* src = reinterpret_cast<const int4*>(B + kc * chunk);
+            for (int t = tid; t < KCC_E * NC; t += T) {
+                const int e = t / NC, c = t - e * NC;
+                v[t] = c < S ? src[e * SW + (c < K ? c : SW - 1)] : make_int4(0, 0, 0, 0);
+            }
+            for (int t = tid; t < nr * KCC_P; t += T) {
+                const int r = r0 + t / KCC_P, q = t % KCC_P, f = r / My, y = r - f * My, ka = max(r * Mz, k0), kb = min(r * Mz + Mz, k1);
+                const float4 g = sgeo[q];
+                float h, l;
+                float2 hi, lo;
+                ff_frac_mul2(g.x, g.y, G.fc_hi[f], G.fc_lo[f], h, l);
+                cis_pair(ctab, -h, -l, hi, lo);
+                // once per frequency (a half-used middle frequency is 0: no deviation)
+                d[t] = y == 0 && r * Mz >= k0 ? (float)Nm * dbl * pair_unit_dev(hi, lo) : 0.f;
+                const float4 w = kx_mul_split(kx_split(make_float4(hi.x, hi.y, lo.x, lo.y)), fa[y * KCC_P + q]);
+                for (int k = ka; k < kb; ++k) {
+                    const float4 a = fa[(My + k - r * Mz) * KCC_P + q];
+                    float4 x;
+                    kx_dot(w.x, a.x, -w.y, a.y, w.z, a.z, -w.w, a.w, x.x, x.z);
+                    kx_dot(w.x, a.y, w.y, a.x, w.z, a.w, w.w, a.z, x.y, x.w);
+                    u[(k - k0) * KCC_P + q] = make_int2(__float2int_rn(x.x * 1073741824.0f) + __float2int_rn(x.z * 1073741824.0f),
+                                                        __float2int_rn(x.y * 1073741824.0f) + __float2int_rn(x.w * 1073741824.0f));
                 }
             }
+            for (int t = tid + (k1 - k0) * KCC_P; t < KCC_E * KCC_P; t += T) u[t] = make_int2(0, 0);
+        };
+        long long tot[2][KCC_Q][2];
+        #pragma unroll
+        for (int i = 0; i < 2; ++i)
             #pragma unroll
-            for (int q = 0; q < KCC_C; ++q) {
-                const int c = c0 + q;
-                const float sc = scl[c];
-                    cff h;
-            two_sum(ar[q], lr[q], h.re.hi, h.re.lo);
-            two_sum(ai[q], li[q], h.im.hi, h.im.lo);
-            h = cff{ff_mulf(h.re, sc), ff_mulf(h.im, sc)};
-                if (c == SW - 1) { pr = h; continue; }
-                const float v[2] = {h.re.hi, h.im.hi}, vl[2] = {h.re.lo, h.im.lo};
+            for (int q = 0; q < KCC_Q; ++q) tot[i][q][0] = tot[i][q][1] = 0;
+        fill(0);
+        __syncthreads();
+        for (int kc = 0; kc < NCk; ++kc) {
+            if (kc + 1 < NCk) fill(kc + 1);
+            {   // deviations of this chunk's rows
+                const int k0 = kc * KCC_E, nr = (min(k0 + KCC_E, Nh) - 1) / Mz - k0 / Mz + 1;
+                const float* d = dv + (kc & 1) * pl.rows * KCC_P;
+                for (int q = tid; q < KCC_P; q += T) {
+                    float v = sdv[q];
+                    for (int r = 0; r < nr; ++r) v += d[r * KCC_P + q];
+                    sdv[q] = v;
+                }
+            }
+            const int2* u2 = us + (kc & 1) * KCC_E * KCC_P + 2 * lane;
+            const int4* v2 = vs + (kc & 1) * KCC_E * NC + quad * KCC_Q;
+            #pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                long long acc[2][KCC_Q][2];
                 #pragma unroll
-                for (int part = 0; part < 2; ++part) {
-                    const float t = __fsub_rn(fmaf(v[part], v[part], GM), GM);
+                for (int i = 0; i < 2; ++i)
+                    #pragma unroll
+                    for (int q = 0; q < KCC_Q; ++q) acc[i][q][0] = acc[i][q][1] = 0;
+                #pragma unroll 2
+                for (int e = 0; e < KCC_E / 2; ++e) {
+                    const int4 u = *reinterpret_cast<const int4*>(u2 + (half * (KCC_E / 2) + e) * KCC_P);
+                    #pragma unroll
+                    for (int q = 0; q < KCC_Q; ++q) {
+                        const int4 v = v2[(half * (KCC_E / 2) + e) * NC + q];
+                        acc[0][q][0] += (long long)u.x * v.x + (long long)u.y * v.y;
+                        acc[0][q][1] += (long long)u.x * v.z + (long long)u.y * v.w;
+                        acc[1][q][0] += (long long)u.z * v.x + (long long)u.w * v.y;
+                        acc[1][q][1] += (long long)u.z * v.z + (long long)u.w * v.w;
+                    }
+                }
+                #pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    #pragma unroll
+                    for (int q = 0; q < KCC_Q; ++q) {
+                        tot[i][q][0] += acc[i][q][0] >> 12;
+                        tot[i][q][1] += acc[i][q][1] >> 12;
+                    }
+            }
+            __syncthreads();
+        }
+        #pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float sg = 0.f, sr = 0.f;
+            #pragma unroll
+            for (int q = 0; q < KCC_Q; ++q) {
+                const int c = quad * KCC_Q + q;
+                if (c >= S) break;
+                const float sc = scl[c < K ? c : SW - 1];
+                float hi[2], lo[2];
+                #pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const float t = __ll2float_rn(tot[i][q][v]);
+                    hi[v] = t * back * sc;
+                    lo[v] = __ll2float_rn(tot[i][q][v] - __float2ll_rn(t)) * back * sc;
+                }
+                if (c == K) { exr[2 * lane + i] = make_float4(hi[0], hi[1], lo[0], lo[1]); continue; }
+                #pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const float t = __fsub_rn(fmaf(hi[v], hi[v], GM), GM);
                     sg = __fadd_rn(sg, t);
-                    sr += fmaf(2.0f * v[part], vl[part], fmaf(v[part], v[part], -t));
+                    sr += fmaf(2.0f * hi[v], lo[v], fmaf(hi[v], hi[v], -t));
                 }
             }
+            ex[quad * KCC_P + 2 * lane + i] = make_float2(sg, sr);
         }
-        ff au;
-        two_sum(__fsub_rn((float)Nz, sg), dev - sr, au.hi, au.lo);
-        if (!(au.hi > 0.f)) au = ff{0.f, 0.f};
-        delta = ff_add(delta, kx_delta(D.kC[sj], G.amp_c / (grec.x + grec.y), ph[3 * (size_t)P + pp],
-                                       ph[4 * (size_t)P + pp], ph[5 * (size_t)P + pp], au, pr));
+        __syncthreads();
+        for (int q = tid; q < KCC_P; q += T) {
+            const int p = p0 + q, pp = min(p, P - 1);
+            float sg = 0.f, sr = 0.f;
+            for (int c = 0; c < pl.quads; ++c) {
+                sg = __fadd_rn(sg, ex[c * KCC_P + q].x);   // multiples of the grid: exact
+                sr += ex[c * KCC_P + q].y;
+            }
+            ff au;
+            two_sum(__fsub_rn((float)Nz, sg), sdv[q] - sr, au.hi, au.lo);
+            if (!(au.hi > 0.f)) au = ff{0.f, 0.f};
+            const float4 g = sgeo[q], r = exr[q];
+            float h0, l0;                          // the carrier: conj(e^{-i 2 pi d / lambda})
+            ff_frac_mul2(g.x, g.y, G.inv_lam_hi, G.inv_lam_lo, h0, l0);
+            float2 ch, cl;
+            cis_pair(ctab, h0, l0, ch, cl);
+            const cff pr = cff_mul(cff{ff{r.x, r.z}, ff{r.y, r.w}}, cff{ff{ch.x, cl.x}, ff{ch.y, cl.y}});
+            const ff d = kx_delta(D.kC[sj], G.amp_c / (g.x + g.y), ph[3 * (size_t)P + pp], ph[4 * (size_t)P + pp],
+                                  ph[5 * (size_t)P + pp], au, pr);
+            const ff all = j == 0 ? d : ff_add(ff{sdl[q].x, sdl[q].y}, d);
+            sdl[q] = make_float2(all.hi, all.lo);
+            if (j == J - 1 && p < P) D.lw_y[(size_t)s * P + p] = ff_to_d(all);
+        }
     }
-    if (p < P) D.lw_y[(size_t)s * P + p] = ff_to_d(delta);
 }
 
 // the (hi, lo) cis table of the steering factors, once per handle
@@ -914,13 +998,13 @@ size_t kappa_operand_bytes(const DevGeom& G, int S_max) {
 
 int launch_kappa(const DevGeom& G, const DevParams& Pm, const DevState& D, int S, int SCA, bool tensor,
                  const double* V64, cudaStream_t st) {
-    const int SW = kx_sw(S), nant = G.My + G.Mz;
+    const int SW = kx_sw(S);
     const double2* V = reinterpret_cast<const double2*>(V64);
-    k_kappa_digits<<<dim3(S, G.J, max(1, min(4, 4 * sm_count() / (S * G.J)))), 256, 0, st>>>(G, D, S, SCA, SW, V);
+    k_kappa_digits<<<dim3(S, G.J, max(1, min(4, 4 * sm_count() / (S * G.J)))), 256, 0, st>>>(G, D, S, SCA, SW, !tensor, V);
     if (!tensor) {
-        const size_t smem = ((size_t)nant * KCC_T + 256 + KCC_E * KCC_C) * sizeof(float4);
+        const KccPlan t = kcc_plan(G, S);
         smem_allow_max((const void*)k_kappa_cc);
-        k_kappa_cc<<<dim3((Pm.P + KCC_T - 1) / KCC_T, S), KCC_T, smem, st>>>(G, Pm, D, S, SCA, SW, V);
+        k_kappa_cc<<<dim3((Pm.P + KCC_P - 1) / KCC_P, S), 32 * t.quads, t.smem, st>>>(G, Pm, D, S, SW);
         return 2;
     }
     // Up to 32 columns A goes through tensor memory: MMAs of few columns are bound by reading A from shared

@@ -51,7 +51,11 @@ CASES = [("corner", dict(J=1, Nf=10, My=4, Mz=4), 1, 131), ("corner", dict(J=2, 
          ("corner", dict(J=2, Nf=10, My=4, Mz=4), 24, 130), ("irregular", dict(J=2, Nf=8, My=2, Mz=3), 26, 130),
          ("irregular", dict(J=2, Nf=75, My=2, Mz=2), 33, 130), ("corner", dict(J=2, Nf=10, My=4, Mz=4), 40, 130),
          ("irregular", dict(J=2, Nf=10, My=4, Mz=4), 60, 130), ("corner", dict(J=1, Nf=9, My=9, Mz=5), 6, 66),
-         ("irregular", dict(J=1, Nf=16, My=8, Mz=8), 25, 66)]
+         ("irregular", dict(J=1, Nf=16, My=8, Mz=8), 25, 66),
+         # (for the CUDA-core PF likelihood: middle elements, one antenna, one frequency, all columns)
+         ("symmetric", dict(J=2, Nf=9, My=3, Mz=3), 21, 130), ("symmetric", dict(J=2, Nf=7, My=1, Mz=1), 4, 63),
+         ("symmetric", dict(J=2, Nf=1, My=3, Mz=5), 3, 65), ("symmetric", dict(J=2, Nf=10, My=4, Mz=4), 64, 64),
+         ("irregular", dict(J=1, Nf=37, My=1, Mz=1), 5, 129)]
 
 # up to the largest array, the last two PFs millimetres apart: sums of the steering vectors' products over all elements
 LARGE = [(kind, geom_kw, 5, 66, True) for kind in ("corner", "irregular", "symmetric")
@@ -62,10 +66,18 @@ LARGE = [(kind, geom_kw, 5, 66, True) for kind in ("corner", "irregular", "symme
 def check(kind, geom_kw, S, P, twins=False):
     g, prm, z, pred = problem(kind, geom_kw, S, P, 300 + S, twins)
     f = bp.Filter(g, prm, P=P, S_max=16 if S <= 16 else 64, seed=9)
-    f.set_predicted(pred.n, pred.S, pred.x, pred.phi, pred.eta, pred.w_beta, pred.w_alpha, pred.w_xi, pred.zeta)
-    f.update(torch.from_numpy(np.ascontiguousarray(z)).cuda())
+    zd = torch.from_numpy(np.ascontiguousarray(z)).cuda()
+
+    def update(**tiles):
+        f.set_tiles(**tiles)
+        f.set_predicted(pred.n, pred.S, pred.x, pred.phi, pred.eta, pred.w_beta, pred.w_alpha, pred.w_xi, pred.zeta)
+        f.update(zd)
+        return f.diag_loglik(S)
+
+    cuda_cores = update(kappa_tc=-1)
+    ll = update(kappa_tc=0)
     msg = messages_woodbury.update_messages(pred, prm, g, z.astype(np.complex128))
-    tab, ll, gw = f.diag_table(S), f.diag_loglik(S), f.diag_weights(S)
+    tab, gw = f.diag_table(S), f.diag_weights(S)
     for key in ("m", "mw", "mu3", "mu4"):
         ref = getattr(msg.table, key)
         assert np.max(np.abs(tab[key] - ref)) <= 1e-5 * max(np.max(np.abs(ref)), 1e-300), key
@@ -78,7 +90,8 @@ def check(kind, geom_kw, S, P, twins=False):
         tol_i = np.where(rest, np.maximum(tol_i, di["err"]), tol_i)
     tol_k = 2e-3 + 1e-6 * np.abs(dk)
     assert np.all(np.abs(ll["log_iota"] - li) <= tol_i), np.max(np.abs(ll["log_iota"] - li) / tol_i)
-    assert np.all(np.abs(ll["delta_kappa"] - dk) <= tol_k), np.max(np.abs(ll["delta_kappa"] - dk) / tol_k)
+    for got in (ll["delta_kappa"], cuda_cores["delta_kappa"]):
+        assert np.all(np.abs(got - dk) <= tol_k), np.max(np.abs(got - dk) / tol_k)
     w_eta = beliefs.beliefs(pred, msg).w_eta
     for j in range(g.J):
         assert np.max(np.abs(gw["w_eta"][j] - w_eta[j])) < 1e-4 * np.max(w_eta[j]), j
