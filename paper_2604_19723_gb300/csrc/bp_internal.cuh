@@ -102,10 +102,8 @@ __device__ inline U4 draw(const DevParams& P, uint32_t item, uint32_t n, uint32_
     return philox(item, n, (purpose << 16) | (sub & 0xFFFFu), block, P.key0, P.key1);
 }
 
-// ((x >> 8) + 1/2) 2^-24: uniform in (0,1), exact in FP32
-__device__ inline float u24(uint32_t x) { return ((float)(x >> 8) + 0.5f) * 5.9604644775390625e-8f; }
-// the same uniform exactly, ((x >> 8) + 1/2) 2^-24 in FP64 (the FP32 form above rounds the
-// half away for x >= 2^31: within FP32 rounding of the draws it feeds)
+// ((x >> 8) + 1/2) 2^-24: uniform in (0,1), exact in FP64 (FP32 would round the half away for
+// x >= 2^31)
 __device__ inline double u24d(uint32_t x) { return ((double)(x >> 8) + 0.5) * 5.9604644775390625e-8; }
 // (x + 1/2) 2^-32: uniform in (0,1), exact in FP64
 __host__ __device__ inline double u32d(uint32_t x) { return ((double)x + 0.5) * 2.3283064365386963e-10; }
@@ -230,19 +228,9 @@ __device__ inline double2 steer_elem(const DevGeom& G, const PathGeo& g, int f, 
 // fractional part in [-1/2, 1/2]
 __device__ inline double frac_c(double t) { return t - rint(t); }
 
-// Fractional part (in [-1/2, 1/2]) of the float-float product (ah + al)(bh + bl),
-// with the leading product split exactly by FMA (Dekker/Ogita two-product):
-// about 1e-8 absolute accuracy for products up to ~1e3 cycles, all in FP32.
-__device__ inline float ff_frac_mul(float ah, float al, float bh, float bl) {
-    const float p = ah * bh;
-    const float e = fmaf(ah, bh, -p);
-    const float n = rintf(p);
-    const float t = e + ah * bl + al * bh;
-    return (p - n) + t;
-}
-
-// The same fraction as an unevaluated pair hi + lo (hi = p - rint(p) exactly, lo the
-// low-order terms), for a phase kept beyond FP32 rounding.
+// Fractional part (in [-1/2, 1/2]) of the float-float product (ah + al)(bh + bl), with the
+// leading product p split exactly by FMA (Dekker/Ogita two-product), as an unevaluated pair
+// hi + lo (hi = p - rint(p) exactly, lo the low-order terms): a phase beyond FP32 rounding.
 __device__ inline void ff_frac_mul2(float ah, float al, float bh, float bl, float& hi, float& lo) {
     const float p = __fmul_rn(ah, bh);
     const float e = fmaf(ah, bh, -p);
@@ -324,18 +312,8 @@ __device__ inline ff ff_div(ff x, ff y) {              // one Newton correction
     return out;
 }
 struct cff { ff re, im; };
-__device__ inline cff cff_add(cff a, cff b) { return cff{ff_add(a.re, b.re), ff_add(a.im, b.im)}; }
-__device__ inline cff cff_sub(cff a, cff b) { return cff{ff_add(a.re, ff_neg(b.re)), ff_add(a.im, ff_neg(b.im))}; }
 __device__ inline cff cff_mul(cff a, cff b) {
     return cff{ff_add(ff_mul(a.re, b.re), ff_neg(ff_mul(a.im, b.im))), ff_add(ff_mul(a.re, b.im), ff_mul(a.im, b.re))};
-}
-__device__ inline cff cff_mulc(cff a, cff b) {         // conj(a) * b
-    return cff{ff_add(ff_mul(a.re, b.re), ff_mul(a.im, b.im)), ff_add(ff_mul(a.re, b.im), ff_neg(ff_mul(a.im, b.re)))};
-}
-__device__ inline cff cff_from(float2 v) { return cff{ff{v.x, 0.f}, ff{v.y, 0.f}}; }
-// exact conj(a) * b of two FP32 complex numbers
-__device__ inline cff cff_prodc(float2 a, float2 b) {
-    return cff{ff_add(ff_prod(a.x, b.x), ff_prod(a.y, b.y)), ff_add(ff_prod(a.x, b.y), ff_neg(ff_prod(a.y, b.x)))};
 }
 
 // acc += |v|^2 with exact squares; acc.lo is left unnormalised

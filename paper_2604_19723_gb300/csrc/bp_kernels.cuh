@@ -187,15 +187,6 @@ __device__ inline float factors_from_geo_pairs(const DevGeom& G, const float4* t
     }
     return G.amp_c / d;
 }
-// the frequency factor b'_f of factors_from_geo_pairs alone, from the record's distance
-// (dh + dl) and its carrier cycle count (h0 + l0, from ff_frac_mul2 with 1/lambda)
-__device__ inline void bprime_pair(const DevGeom& G, const float4* tab, float dh, float dl, float h0, float l0, int f,
-                                   float2& hi, float2& lo) {
-    float hf, lf, h, e;
-    ff_frac_mul2(dh, dl, G.fc_hi[f], G.fc_lo[f], hf, lf);
-    two_sum(h0, hf, h, e);
-    cis_pair(tab, -h, -(e + l0 + lf), hi, lo);
-}
 
 // (ah + al)(bh + bl) as hi + lo: exact products of the high parts, the rounding of their
 // sum, and the first-order cross terms

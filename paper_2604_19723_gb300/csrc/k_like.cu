@@ -262,24 +262,6 @@ __device__ inline cff fx_dotc(const float2* x, const float2* y, int n) {
     return r;
 }
 
-// A -= x1 y1 + x2 y2 in float-float: exact high products, first-order cross terms,
-// both roundings of the high sum captured; A.lo is left unnormalised.
-__device__ inline void ff_sub_dot2(ff& A, ff x1, ff y1, ff x2, ff y2) {
-    const float p1 = __fmul_rn(x1.hi, y1.hi), e1 = fmaf(x1.hi, y1.hi, -p1);
-    const float p2 = __fmul_rn(x2.hi, y2.hi), e2 = fmaf(x2.hi, y2.hi, -p2);
-    float s, t1, t2;
-    two_sum(A.hi, -p1, s, t1);
-    two_sum(s, -p2, A.hi, t2);
-    const float cross = fmaf(x1.hi, y1.lo, fmaf(x1.lo, y1.hi, fmaf(x2.hi, y2.lo, __fmul_rn(x2.lo, y2.hi))));
-    A.lo = __fadd_rn(A.lo, __fsub_rn(__fadd_rn(t1, t2), __fadd_rn(__fadd_rn(e1, e2), cross)));
-}
-// A -= l conj(a)
-__device__ inline void cff_sub_mulc(cff& A, const cff& l, const cff& a) {
-    ff_sub_dot2(A.re, l.re, a.re, l.im, a.im);
-    ff_sub_dot2(A.im, l.im, a.re, ff_neg(l.re), a.im);
-}
-__device__ inline ff ff_norm(ff x) { ff r; two_sum(x.hi, x.lo, r.hi, r.lo); return r; }
-__device__ inline cff cff_norm(cff x) { return cff{ff_norm(x.re), ff_norm(x.im)}; }
 __device__ inline ff ff_recip(ff x) {
     const float r = __frcp_rn(x.hi);
     const float e = __fsub_rn(fmaf(-x.hi, r, 1.0f), __fmul_rn(x.lo, r));   // 1 - x r

@@ -1,12 +1,12 @@
 // Inline-PTX building blocks for the fifth-generation tensor cores (tcgen05) and
 // the bulk-copy engine of sm_100-class GPUs: shared-memory matrix descriptors,
-// the TF32 and BF16 instruction descriptors, tensor-memory (TMEM) allocation, MMA issue and
+// the BF16 instruction descriptor, tensor-memory (TMEM) allocation, MMA issue and
 // commit, bounded mbarrier waits, bulk global->shared copies and TMEM loads.
 //
 // Operand layout used throughout: K-major, no swizzle.  A tile of R rows x Kt
-// 4-byte elements is stored as "core matrices" of 8 rows x 16 bytes (8 x 4
+// 2-byte elements is stored as "core matrices" of 8 rows x 16 bytes (8 x 8
 // elements, rows 16 B apart); core matrices adjacent along K are LBO = 128 B
-// apart, consecutive groups of 8 rows SBO = (Kt/4) * 128 B apart.
+// apart, consecutive groups of 8 rows SBO = (Kt/8) * 128 B apart.
 #pragma once
 #include <cstdint>
 
@@ -15,11 +15,6 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// byte offset of element (r, k) in the layout above
-__host__ __device__ inline int core_off(int r, int k, int Kt) {
-    return (r >> 3) * (Kt >> 2) * 128 + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4;
 }
 
 // shared-memory matrix descriptor: start address, leading (K) and stride (8-row)
@@ -32,31 +27,16 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
     return d;
 }
 
-// instruction descriptor of kind::tf32 with an F32 accumulator, both operands
-// K-major, dense: D format (bits 4-5) = F32, A/B formats (bits 7-9, 10-12) = TF32,
-// N/8 at bits 17-22, M/16 at bits 24-28
-__host__ __device__ constexpr uint32_t idesc_tf32_f32(int m, int n) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
 // instruction descriptor of kind::f16 with BF16 A and B (the same type for both) and
-// an F32 accumulator, both operands K-major, dense: A/B format code 1 = BF16
+// an F32 accumulator, both operands K-major, dense: D format (bits 4-5) = F32, A/B formats
+// (bits 7-9, 10-12) = BF16, N/8 at bits 17-22, M/16 at bits 24-28
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// byte offset of element (r, k) of a tile of R rows x Kt 2-byte elements, K-major, no
-// swizzle: core matrices of 8 rows x 16 bytes (8 x 8 elements), LBO = 128 B along K,
-// SBO = (Kt/8) * 128 B between groups of 8 rows
+// byte offset of element (r, k) in the layout above
 __host__ __device__ inline int core_off16(int r, int k, int Kt) {
     return (r >> 3) * (Kt >> 3) * 128 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
-}
-
-// round to TF32 (10 explicit mantissa bits), nearest with ties away from zero
-__device__ __forceinline__ float tf32_rn(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
 }
 
 // TMEM allocation by one whole warp; the base address is written to *slot
@@ -74,13 +54,8 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p != 0;
 }
-// D (+)= A B^T for M x K and N x K tiles in shared memory, issued by one thread
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool acc) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc ? 1u : 0u));
-}
-// D (+)= A B^T, BF16 operands (K = 16 per instruction), F32 accumulator
+// D (+)= A B^T for M x K and N x K tiles in shared memory, BF16 operands (K = 16 per
+// instruction), F32 accumulator, issued by one thread
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool acc) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
@@ -162,18 +137,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
                  : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// 32 consecutive 32-bit TMEM columns of this thread's lane written from registers (shape
-// 32x32b, as tmem_ld32); tmem_st_wait makes them visible to this thread's later loads
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-                 "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
-                 :: "r"(taddr),
-                   "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-                   "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
-                   "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
-                   "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-                 : "memory");
-}
 
 }  // namespace tc
 }  // namespace bp
