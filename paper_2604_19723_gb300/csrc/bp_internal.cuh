@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include "../../include/bp.h"
+#include "gamma_accept.cuh"
 
 namespace bp {
 
@@ -150,32 +151,18 @@ __device__ inline void normals8(const DevParams& P, uint32_t item, uint32_t n, u
     }
 }
 
-// Marsaglia & Tsang (2000) Gamma(shape >= 1, scale) in FP64; attempt a uses block a.  The acceptance
-// test is decided in FP32 where its two sides are further apart than FP32 can err (they are
-// within ~1e-5 sqrt(shape) of exact, for |g| < 7), which spares two FP64 logarithms in all but
-// ~1e-3 of the draws; the decision is the same.
+// Marsaglia & Tsang (2000) Gamma(shape >= 1, scale) in FP64; attempt a uses block a
 __device__ inline double gamma_draw(const DevParams& P, uint32_t item, uint32_t n, uint32_t purpose, uint32_t sub,
                                     double shape, double scale) {
     const double d = shape - 1.0 / 3.0;
     const double c = 1.0 / sqrt(9.0 * d);
-    const float df = (float)d, margin = 2.0e-4f + 2.0e-4f * sqrtf(df);
     for (int a = 0; a < MAX_GAMMA_ATTEMPTS; ++a) {
         const U4 r = draw(P, item, n, purpose, sub, (uint32_t)a);
         const double g = sqrt(-2.0 * log(u32d(r.x))) * cospi(2.0 * u32d(r.y));
         const double t = 1.0 + c * g;
         const double v = t * t * t;
         if (v <= 0.0) continue;
-        // g^2/2 + d (1 - v + log v) - log u with v = (1 + w)^3
-        const float w = (float)(c * g), gf = (float)g;
-        const float gap = fmaf(0.5f * gf, gf, df * (3.0f * log1pf(w) - w * fmaf(w, w + 3.0f, 3.0f))) - logf((float)u32d(r.z));
-        bool ok;
-        if (fabsf(gap) > margin) {
-            ok = gap > 0.0f;
-        } else {
-            const double u = u32d(r.z);
-            ok = log(u) < 0.5 * g * g + d - d * v + d * log(v);
-        }
-        if (ok) return d * v * scale;
+        if (gamma_accept(g, t, c, d, u32d(r.z))) return d * v * scale;
     }
     return shape * scale;
 }
