@@ -51,7 +51,9 @@ typedef enum {
 /* Array and signal constants (Sec. II-B).  f_k = -B/2 + k B/(Nf-1).
  * R_pa: J rotation matrices, row-major 3x3, columns = local PA axes in
  * global coordinates (local vector r' = R^T r, eq. rangep).  p_y, p_z:
- * template URA element positions, symmetric about 0.
+ * template URA element positions, any; the paper's are symmetric about 0, and
+ * layouts whose positions are so to 1e-13 of the largest take kernels that form
+ * half of the elements.
  * Limits: 1 <= J <= 16, Nf <= 128, My <= 16, Mz <= 16, Nz <= 2048. */
 typedef struct {
     int J, Nf, My, Mz;

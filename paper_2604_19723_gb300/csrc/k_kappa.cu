@@ -47,7 +47,7 @@
 // Up to SW = 32 A goes through the half of tensor memory that the accumulators leave free.
 // Bound: the producers' issue slots (28 instructions per element for its digits; the factors, the loop and
 // the epilogue add as much at few elements); the tensor pipe is next (ten products of 128 x 2 SW x 2 Nh:
-// 46 % busy at 32 PFs, Nz = 1024).
+// 44 % busy at 32 PFs, Nz = 1024).
 // Measured (PF likelihood stage, J = 4) with the 3xTF32 kernel (below 33 PFs a CUDA-core kernel), which
 // takes a second pass / with one thread issuing, A in shared memory and exact products by two-term
 // splits of full FP32 factors / as it is: 64 PFs x 1e5 particles, Nz = 160: 56.7 / 15.6 / 10.3 ms; 32 PFs x
