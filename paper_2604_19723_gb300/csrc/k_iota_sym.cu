@@ -456,7 +456,11 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 512, TW == 1 ? 3 : 1) k_iota_f
             float r2 = 0.f;
             for (int j = 0; j < J; ++j) { t += part[j]; r2 += rat[j]; }
             D.lw_x[p] = t;
-            if (all && sqrtf(r2) > IF_RATIO_MAX) atomicAdd(&D.flags[0], 1);   // counted only: nothing is left to repair
+            // nothing is left to repair, but the ill-conditioned ones are counted, and listed for the diagnostics
+            if (all && sqrtf(r2) > IF_RATIO_MAX) {
+                const int slot = atomicAdd(&D.flags[0], 1);
+                if (bp_in_range(slot, P, D.kerr)) D.flags[1 + slot] = p;
+            }
         }
         __syncthreads();
     }

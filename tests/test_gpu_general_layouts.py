@@ -101,3 +101,19 @@ def check(kind, geom_kw, S, P, twins=False):
 @pytest.mark.parametrize("case", CASES + LARGE, ids=lambda c: "%s-%dx%dx%d-S%d" % (c[0], c[1]["Nf"], c[1]["My"], c[1]["Mz"], c[2]))
 def test_update_on_a_general_layout(case):
     check(*case)
+
+
+@pytest.mark.parametrize("kind", ["symmetric", "corner"])
+def test_the_ill_conditioned_particles_are_counted_and_listed(kind):
+    """Below 24 PFs: particles in which the last two PFs nearly coincide, on both layouts' routes."""
+    P, S = 200, 5
+    g, prm, z, pred = problem(kind, dict(J=2, Nf=10, My=4, Mz=4), S, P, 305, True)
+    pred.phi[S - 1, :3, ::2] += np.float32(0.5)      # every other particle apart
+    f = bp.Filter(g, prm, P=P, S_max=16, seed=9)
+    f.set_predicted(pred.n, pred.S, pred.x, pred.phi, pred.eta, pred.w_beta, pred.w_alpha, pred.w_xi, pred.zeta)
+    f.update(torch.from_numpy(np.ascontiguousarray(z)).cuda())
+    listed = f.diag_iota()["selected"]
+    assert len(listed) == f.estimate()["iota_repaired"] > 50
+    assert len(np.unique(listed)) == len(listed) and listed[0] >= 0 and listed[-1] < P
+    assert np.mean(listed % 2) > 0.9
+    f.close()
